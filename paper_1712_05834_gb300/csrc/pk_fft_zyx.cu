@@ -1,0 +1,941 @@
+// pk_fft_zyx.cu -- the library's own 3D r2c transform of FP32 meshes for sizes
+// where it beats both cuFFT and the packed transform of pk_fft.cu, with its
+// last axis fused into the bin pass (the transform of Sec. 3.3.1; the binning
+// of Sec. 3.4.1, Eq. window-deconvolution).  In place, in the padded r2c
+// layout (rows of N/2 + 1 complex), two kernels per compute:
+//
+//   k_fft_zy     z and y axes in one pass over device memory.  Persistent CTAs
+//                take work items in ticket order: "z" items read a block of
+//                real rows of one x plane, transform them (length-N/2 complex
+//                FFT of the pairs d[2n] + i d[2n+1] and the real-input split
+//                  D[l] = (C[l] + conj C[M-l]) / 2
+//                         - (i/2) W_N^l (C[l] - conj C[M-l]),  M = N/2)
+//                and write them back; "y" items transform a tile of columns
+//                of a plane whose z items are done.  A plane's y items follow
+//                its z items Cfg::LAG planes later, so they read the rows from
+//                L2 (129 MB) and overwrite them there: device memory sees one
+//                read and one write for two axes (512^3: 2.1 GB counted, where
+//                two passes move 4.3).
+//   k_fft_xbin   x axis and the bin pass: one CTA per tile of columns (ky, l0 ..)
+//                (two interlaced meshes share a tile) takes the length-N FFTs
+//                along x in shared memory and bins the modes from there:
+//                interlace combine, sinc^p compensation, k bin, mu bin,
+//                Legendre sums.  The r2c transform itself is never written.
+//   k_fft_x      the x axis alone, written back in place, for the passes that
+//                read the transform after a compute (cross, projected power).
+//
+// Only modes with m = |n|^2 < mhi enter a bin: columns l with l^2 >= mhi are
+// neither transformed along y nor read, the y pass does not write rows ky with
+// ky^2 + l0^2 >= mhi, and the x pass reads only tiles below mhi (21 % less
+// traffic for kmax = k_N).  What they leave in the mesh is never read.
+//
+// All transforms are forward (e^{-2 pi i jk/n}), unnormalized, decimation in
+// frequency in the radix order of radix_of; twiddles come from one table
+// W_N^e (e < N) computed in FP64 on the host.
+//
+// The file is compiled once per group of sizes (PK_ZYX_GROUP), so that the
+// groups build in parallel.
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "pk_internal.h"
+
+namespace pk {
+
+namespace {
+
+// Complex sums as one packed FP32x2 instruction each.
+__device__ __forceinline__ float2 c_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 c_sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
+__device__ __forceinline__ float2 c_mul(float2 a, float2 b) {
+    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+__device__ __forceinline__ float2 c_mi(float2 a) { return make_float2(a.y, -a.x); }   // a * (-i)
+
+// In-register DFT of R points: v[k] <- sum_j v[j] W_R^{jk}.
+template <int R>
+__device__ __forceinline__ void dft(float2 *v);
+
+template <>
+__device__ __forceinline__ void dft<2>(float2 *v) {
+    const float2 a = v[0];
+    v[0] = c_add(a, v[1]);
+    v[1] = c_sub(a, v[1]);
+}
+
+template <>
+__device__ __forceinline__ void dft<4>(float2 *v) {
+    const float2 a = c_add(v[0], v[2]), b = c_sub(v[0], v[2]);
+    const float2 c = c_add(v[1], v[3]), d = c_sub(v[1], v[3]);
+    v[0] = c_add(a, c);
+    v[2] = c_sub(a, c);
+    v[1] = make_float2(b.x + d.y, b.y - d.x);                  // b -+ i d
+    v[3] = make_float2(b.x - d.y, b.y + d.x);
+}
+
+template <>
+__device__ __forceinline__ void dft<3>(float2 *v) {
+    const float h = 0.86602540378443865f;                      // sqrt(3) / 2
+    const float2 s = c_add(v[1], v[2]), d = c_sub(v[1], v[2]);
+    const float2 m = make_float2(v[0].x - 0.5f * s.x, v[0].y - 0.5f * s.y);
+    v[0] = c_add(v[0], s);
+    v[1] = make_float2(m.x + h * d.y, m.y - h * d.x);          // W_3 = -1/2 - i sqrt(3)/2
+    v[2] = make_float2(m.x - h * d.y, m.y + h * d.x);
+}
+
+// c1, c2 = cos(2 pi/5), cos(4 pi/5); s1, s2 the sines: outputs k and 5 - k
+// share the cosine sum and take +- the sine sum.
+template <>
+__device__ __forceinline__ void dft<5>(float2 *v) {
+    const float c1 = 0.30901699437494742f, c2 = -0.80901699437494742f;
+    const float s1 = 0.95105651629515357f, s2 = 0.58778525229247313f;
+    const float2 p1 = c_add(v[1], v[4]), q1 = c_sub(v[1], v[4]);
+    const float2 p2 = c_add(v[2], v[3]), q2 = c_sub(v[2], v[3]);
+    const float2 a = make_float2(v[0].x + c1 * p1.x + c2 * p2.x, v[0].y + c1 * p1.y + c2 * p2.y);
+    const float2 b = make_float2(v[0].x + c2 * p1.x + c1 * p2.x, v[0].y + c2 * p1.y + c1 * p2.y);
+    const float2 s = make_float2(s1 * q1.x + s2 * q2.x, s1 * q1.y + s2 * q2.y);
+    const float2 t = make_float2(s2 * q1.x - s1 * q2.x, s2 * q1.y - s1 * q2.y);
+    v[0] = c_add(v[0], c_add(p1, p2));
+    v[1] = make_float2(a.x + s.y, a.y - s.x);
+    v[4] = make_float2(a.x - s.y, a.y + s.x);
+    v[2] = make_float2(b.x + t.y, b.y - t.x);
+    v[3] = make_float2(b.x - t.y, b.y + t.x);
+}
+
+// Split into the even and odd outputs: X[2k] = DFT4(v[j] + v[j+4]),
+// X[2k+1] = DFT4((v[j] - v[j+4]) W_8^j).
+template <>
+__device__ __forceinline__ void dft<8>(float2 *v) {
+    const float h = 0.70710678118654752f;
+    float2 u[4], w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        u[j] = c_add(v[j], v[j + 4]);
+        w[j] = c_sub(v[j], v[j + 4]);
+    }
+    w[1] = make_float2(h * (w[1].x + w[1].y), h * (w[1].y - w[1].x));    // * W_8 = (1 - i)/sqrt 2
+    w[2] = c_mi(w[2]);                                                   // * W_8^2 = -i
+    w[3] = make_float2(h * (w[3].y - w[3].x), -h * (w[3].x + w[3].y));   // * W_8^3 = -(1 + i)/sqrt 2
+    dft<4>(u);
+    dft<4>(w);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[2 * k] = u[k];
+        v[2 * k + 1] = w[k];
+    }
+}
+
+// 4 x 4: X[k + 4 q] = sum_j W_4^{jq} W_16^{jk} (DFT4 over v[j], v[j+4], v[j+8], v[j+12])[k].
+template <>
+__device__ __forceinline__ void dft<16>(float2 *v) {
+    const float h = 0.70710678118654752f, c = 0.92387953251128676f, s = 0.38268343236508977f;
+    float2 u[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) u[j][q] = v[j + 4 * q];
+        dft<4>(u[j]);
+    }
+    const auto w8 = [&](float2 a) { return make_float2(h * (a.x + a.y), h * (a.y - a.x)); };      // * W_16^2
+    const auto w83 = [&](float2 a) { return make_float2(h * (a.y - a.x), -h * (a.x + a.y)); };    // * W_16^6
+    u[1][1] = c_mul(u[1][1], make_float2(c, -s));
+    u[1][2] = w8(u[1][2]);
+    u[1][3] = c_mul(u[1][3], make_float2(s, -c));
+    u[2][1] = w8(u[2][1]);
+    u[2][2] = c_mi(u[2][2]);
+    u[2][3] = w83(u[2][3]);
+    u[3][1] = c_mul(u[3][1], make_float2(s, -c));
+    u[3][2] = w83(u[3][2]);
+    u[3][3] = c_mul(u[3][3], make_float2(-c, s));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        float2 t[4] = {u[0][k], u[1][k], u[2][k], u[3][k]};
+        dft<4>(t);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[k + 4 * q] = t[q];
+    }
+}
+
+// Radix 2 H as two radix-H transforms of the even and odd outputs (H odd):
+// X[2k] = DFT_H(v[j] + v[j+H]), X[2k+1] = DFT_H((v[j] - v[j+H]) W_2H^j).
+template <int H>
+__device__ __forceinline__ void dft_2h(float2 *v, const float2 *w2h) {
+    float2 u[H], w[H];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+        u[j] = c_add(v[j], v[j + H]);
+        w[j] = c_sub(v[j], v[j + H]);
+        if (j) w[j] = c_mul(w[j], w2h[j]);
+    }
+    dft<H>(u);
+    dft<H>(w);
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+        v[2 * k] = u[k];
+        v[2 * k + 1] = w[k];
+    }
+}
+
+template <>
+__device__ __forceinline__ void dft<6>(float2 *v) {
+    const float2 w[3] = {{1.0f, 0.0f}, {0.5f, -0.86602540378443865f}, {-0.5f, -0.86602540378443865f}};
+    dft_2h<3>(v, w);
+}
+
+template <>
+__device__ __forceinline__ void dft<10>(float2 *v) {
+    const float2 w[5] = {{1.0f, 0.0f},
+                         {0.80901699437494742f, -0.58778525229247313f},
+                         {0.30901699437494742f, -0.95105651629515357f},
+                         {-0.30901699437494742f, -0.95105651629515357f},
+                         {-0.80901699437494742f, -0.58778525229247313f}};
+    dft_2h<5>(v, w);
+}
+
+// Radix of the decimation-in-frequency step over blocks of S points: 10 and 6
+// take the factors 5 and 3 out first (20: 5, then 4; 12: 4, then 3), then 8 and
+// 16 so that a power of two takes the fewest steps (1024: 16, 8, 8; 2048: 16,
+// 16, 8; measured against 8, 8, 4, 4 and 8, 8, 8, 4: both kernels 6 % faster).
+__host__ __device__ constexpr int radix_of(int S) {
+    return S <= 6 || S == 10              ? S
+           : S == 12                      ? 4
+           : S == 20                      ? 5
+           : S % 10 == 0                  ? 10
+           : S % 6 == 0                   ? 6
+           : S % 5 == 0                   ? 5
+           : S % 3 == 0                   ? 3
+           : S == 16 ? 4
+           : S == 128 || S == 1024 || S == 2048 || S == 256 ? 16
+                                          : 8;
+}
+
+// Radix order of the z FFTs: as radix_of, but 4 for the blocks of 32.
+__host__ __device__ constexpr int zradix_of(int S) { return S == 32 ? 4 : radix_of(S); }
+
+// Frequency at position p (< S) after all steps over a block of S points:
+// a step of radix R puts output k of the butterfly at n + (S/R) k, so the
+// digits of p, most significant first, are the frequency's digits from the
+// least significant up.
+template <int S, int MUL, bool Z = false>
+__device__ __forceinline__ int dif_freq(int p) {
+    if constexpr (S == 1) {
+        return 0;
+    } else {
+        constexpr int R = Z ? zradix_of(S) : radix_of(S), Q = S / R;
+        return (p / Q) * MUL + dif_freq<Q, MUL * R, Z>(p % Q);
+    }
+}
+
+// Shapes per mesh size.  T threads of k_fft_zy (CTAS per SM, 64 registers a
+// thread), NBY columns per y tile, TX threads of the x kernels (CTASX per SM), NX
+// columns per x tile.  About 12 to 16 complex values per thread.  At N = 2048
+// and 1024 the x tiles take 128 KB and one CTA of 1024 threads, since their runs
+// along z come from device memory (64-byte runs at 1024: 9.0 against 4.1 ms
+// interlaced), while the y tiles are read from L2, where short runs cost little.
+// LAG: planes between a plane's z and y items (1024 interlaced, k_fft_zy: 8.4,
+// 7.4 and 7.6 ms at 3, 6 and 12 planes; 2048: 36.2, 36.6 and 39.4 at 1, 2 and 3).
+template <int N>
+struct Shape;
+template <int T_, int CTAS_, int NBY_, int TX_, int CTASX_, int NX_, int LAG_>
+struct ShapeOf {
+    static constexpr int T = T_, CTAS = CTAS_, NBY = NBY_, TX = TX_, CTASX = CTASX_, NX = NX_, LAG = LAG_;
+};
+template <> struct Shape<320> : ShapeOf<256, 4, 8, 256, 4, 8, 32> {};
+template <> struct Shape<384> : ShapeOf<384, 2, 8, 384, 2, 8, 32> {};
+template <> struct Shape<400> : ShapeOf<320, 3, 8, 320, 3, 8, 32> {};
+template <> struct Shape<480> : ShapeOf<384, 2, 8, 384, 2, 8, 24> {};
+template <> struct Shape<500> : ShapeOf<416, 2, 8, 416, 2, 8, 24> {};
+template <> struct Shape<600> : ShapeOf<480, 2, 8, 480, 2, 8, 16> {};
+template <> struct Shape<640> : ShapeOf<512, 2, 8, 512, 2, 8, 16> {};
+template <> struct Shape<768> : ShapeOf<512, 2, 8, 512, 2, 8, 10> {};
+template <> struct Shape<800> : ShapeOf<512, 2, 8, 512, 2, 8, 10> {};
+template <> struct Shape<1024> : ShapeOf<512, 2, 8, 1024, 1, 16, 6> {};
+template <> struct Shape<2048> : ShapeOf<512, 2, 4, 1024, 1, 8, 1> {};
+
+template <int N>
+struct Cfg : Shape<N> {
+    static constexpr int M = N / 2, Nh = M + 1;
+    // z rows: NT threads share NR rows of M complex (about 16 per thread)
+    static constexpr int NT = M >= 1024 ? 64 : 32;
+    static constexpr int NR = M > 256 ? 1 : 2;
+    static constexpr int RS = (M & (M - 1)) == 0 ? M : M + 16;   // shared slots per row
+    static constexpr int GROUPS = Shape<N>::T / NT;              // row groups per CTA (named barriers 1 .. GROUPS)
+    static constexpr int RPI = GROUPS * NR;                      // rows per z item
+    static constexpr int ZI = (N + RPI - 1) / RPI;               // z items per plane
+    static_assert(NT == 32 || GROUPS <= 15, "named barriers are 1 .. 15");
+};
+
+// ---------------------------------------------------------------------------
+// Column FFTs: a tile of LEN rows x NC columns in shared memory, element (r, c)
+// at slot(r, c).  The first step takes its inputs from ld(r, c), the last hands
+// its outputs to st(frequency, c, value); the steps in between stay in place.
+// NC threads cover one row.  Slots: rows of 16 columns are conflict-free as
+// they are; rows of 8 are swapped in pairs so that butterflies 8 rows apart
+// (the last step) and the bin pass's runs of 4 rows reach both halves of the
+// banks.  IL tiles (two meshes side by side) swap the halves of a row instead.
+template <int NC, bool IL>
+struct Tile {
+    __device__ static __forceinline__ int slot(int r, int c) {
+        if constexpr (NC == 16) {
+            return r * NC + (IL ? c ^ (((r >> 2) & 1) << 3) : c);
+        } else if constexpr (NC == 8) {
+            if constexpr (IL) return (r ^ ((r >> 3) & 1)) * NC + (c ^ (((r >> 2) & 1) << 2));
+            else return (r ^ (((r >> 2) ^ (r >> 3)) & 1)) * NC + c;
+        } else {
+            return r * NC + c;
+        }
+    }
+};
+
+template <int LEN, int NC, int T, bool IL, int S, bool FIRST, bool TOSM, typename Ld, typename St>
+__device__ __forceinline__ void col_step(float2 *buf, const float2 *tw, int c, int grp, const Ld &ld, const St &st) {
+    constexpr int R = radix_of(S), Q = S / R;
+    constexpr int NG = T / NC;                  // thread groups (one per butterfly)
+    constexpr int NBF = LEN / R;
+    constexpr int PER = (NBF + NG - 1) / NG;    // butterflies per thread
+    constexpr bool EVEN = NBF % NG == 0;
+    using Tl = Tile<NC, IL>;
+    // all of a thread's inputs loaded before the first butterfly, unless that
+    // takes more than half of the 64 registers (a butterfly then goes at a time:
+    // it reads and writes the same places, except in a last step to shared
+    // memory, whose reordered writes come after every read)
+    constexpr bool REORDER = Q == 1 && TOSM;
+    constexpr bool HOLD = PER * R <= 16 || REORDER;
+    constexpr int NV = HOLD ? PER : 1;
+    float2 v[NV][R];
+    const auto load = [&](int s) {
+        const int beta = grp + NG * s;
+        if (EVEN || beta < NBF) {
+            const int base = (beta / Q) * S + beta % Q;
+#pragma unroll
+            for (int j = 0; j < R; ++j)
+                v[HOLD ? s : 0][j] = FIRST ? ld(base + Q * j, c) : buf[Tl::slot(base + Q * j, c)];
+        }
+    };
+    if constexpr (HOLD) {
+#pragma unroll
+        for (int s = 0; s < PER; ++s) load(s);
+    }
+    if constexpr (REORDER) __syncthreads();
+    const auto work = [&](int s) {
+        float2 *w = v[HOLD ? s : 0];
+        const int beta = grp + NG * s;
+        if (EVEN || beta < NBF) {
+            const int n = beta % Q, base = (beta / Q) * S + n;
+            dft<R>(w);
+            if constexpr (Q > 1) {
+                constexpr int E = LEN / S;
+                float2 ww[R];
+                ww[1] = tw[n * E];
+                if constexpr (R == 16) {
+                    ww[2] = tw[2 * n * E];
+                    ww[4] = tw[4 * n * E];
+                    ww[8] = tw[8 * n * E];
+                    ww[3] = c_mul(ww[2], ww[1]);
+#pragma unroll
+                    for (int k = 5; k < 8; ++k) ww[k] = c_mul(ww[4], ww[k - 4]);
+#pragma unroll
+                    for (int k = 9; k < 16; ++k) ww[k] = c_mul(ww[8], ww[k - 8]);
+                } else if constexpr (R == 8) {
+                    ww[4] = tw[4 * n * E];
+                    ww[2] = c_mul(ww[1], ww[1]);
+                    ww[3] = c_mul(ww[2], ww[1]);
+                    ww[5] = c_mul(ww[4], ww[1]);
+                    ww[6] = c_mul(ww[4], ww[2]);
+                    ww[7] = c_mul(ww[4], ww[3]);
+                } else {
+#pragma unroll
+                    for (int k = 2; k < R; ++k) ww[k] = tw[k * n * E];
+                }
+#pragma unroll
+                for (int k = 1; k < R; ++k) w[k] = c_mul(w[k], ww[k]);
+#pragma unroll
+                for (int k = 0; k < R; ++k) buf[Tl::slot(base + Q * k, c)] = w[k];
+            } else {
+                const int f0 = dif_freq<LEN, 1>(base);
+#pragma unroll
+                for (int k = 0; k < R; ++k) st(f0 + k * (LEN / R), c, w[k]);
+            }
+        }
+    };
+    if constexpr (HOLD) {
+#pragma unroll
+        for (int s = 0; s < PER; ++s) work(s);
+    } else {
+#pragma unroll 1
+        for (int s = 0; s < PER; ++s) {
+            load(s);
+            work(s);
+        }
+    }
+    if constexpr (Q > 1) {
+        __syncthreads();
+        col_step<LEN, NC, T, IL, Q, false, TOSM>(buf, tw, c, grp, ld, st);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// z rows.  NT threads transform NR rows; position p of a row sits in slot
+// p ^ ((p >> 2) & 15), a bijection on [0, M] that keeps the FFT steps and the
+// natural-order write free of bank conflicts, except the reads of the last
+// step of the length-256 FFT (two-way).
+__host__ __device__ constexpr int zslot(int p) { return p ^ ((p >> 2) & 15); }
+
+// Slot of position base + off, off a multiple of Q with base % Q < Q and no bit
+// in common (power-of-two lengths): zslot is linear over bits, so the slot of
+// base is shifted by a constant and its low four bits flipped by another.
+template <bool POW2>
+__device__ __forceinline__ int zslot_at(int zbase, int base, int off) {
+    if constexpr (POW2) return (zbase ^ (zslot(off) & 15)) + (off & ~15);
+    else return zslot(base + off);
+}
+
+// Twiddles of the z FFT steps, one table per step with block size S (from M
+// down): entry (k - 1) Q + n = W_S^{nk} (Q = S/R, n < Q, 1 <= k < R), so the
+// lanes of a step read consecutive or equal entries.
+__host__ __device__ constexpr int ztw_offset(int M, int S) {
+    int off = 0;
+    for (int s = M; s > S; s /= zradix_of(s)) {
+        const int q = s / zradix_of(s);
+        off += q > 1 ? (zradix_of(s) - 1) * q : 0;
+    }
+    return off;
+}
+
+__device__ __forceinline__ void fill_ztw(float2 *ztw, const float2 *__restrict__ twg, int M) {
+    for (int s = M; s > 1; s /= zradix_of(s)) {
+        const int R = zradix_of(s), Q = s / R, off = ztw_offset(M, s);
+        if (Q == 1) continue;
+        for (int e = threadIdx.x; e < (R - 1) * Q; e += blockDim.x) {
+            const int k = e / Q + 1, n = e % Q;
+            ztw[off + e] = twg[2 * n * k * (M / s)];     // W_N^{2nk M/S} = W_S^{nk}
+        }
+    }
+}
+
+// Barrier of the NT threads that share rows: a warp, or the aligned pair of
+// warps `grp` on named barrier 1 + grp (0 is __syncthreads').
+template <int NT>
+__device__ __forceinline__ void row_sync(int grp) {
+    if constexpr (NT == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(NT) : "memory");
+}
+
+// One step over blocks of S points of the FFTs of rows [0, nrow) (FIRST: read
+// from g, rows gs complex apart).  The last step writes in natural order.
+template <int M, int NR, int NT, int RS, int S, bool FIRST>
+__device__ __forceinline__ void zrow_step(float2 *rows, const float2 *g, long long gs, int nrow, const float2 *ztw,
+                                          int lane, int grp) {
+    constexpr int R = zradix_of(S), Q = S / R;
+    constexpr int BPR = M / R;                    // butterflies per row
+    constexpr int TOT = NR * BPR;
+    constexpr int PER = (TOT + NT - 1) / NT;
+    constexpr int TW = ztw_offset(M, S);
+    constexpr bool POW2 = (M & (M - 1)) == 0;
+    constexpr bool HOLD = (POW2 && PER * R <= 16) || Q == 1;
+    constexpr int NV = HOLD ? PER : 1;
+    float2 v[NV][R];
+    const auto load = [&](int s) {
+        const int beta = lane + NT * s;
+        const int r = beta / BPR, b = beta % BPR;
+        if ((TOT % NT == 0 || beta < TOT) && r < nrow) {
+            const int base = (b / Q) * S + b % Q;
+            if (FIRST) {
+                const float2 *src = g + r * gs + base;
+#pragma unroll
+                for (int j = 0; j < R; ++j) v[HOLD ? s : 0][j] = __ldcs(src + Q * j);
+            } else {
+#pragma unroll
+                for (int j = 0; j < R; ++j) v[HOLD ? s : 0][j] = rows[r * RS + zslot_at<POW2>(zslot(base), base, Q * j)];
+            }
+        }
+    };
+    if constexpr (HOLD) {
+#pragma unroll
+        for (int s = 0; s < PER; ++s) load(s);
+    }
+    // the last step writes other positions than it reads: all reads first
+    if constexpr (Q == 1) row_sync<NT>(grp);
+    const auto work = [&](int s) {
+        float2 *w = v[HOLD ? s : 0];
+        const int beta = lane + NT * s;
+        const int r = beta / BPR, b = beta % BPR;
+        if ((TOT % NT == 0 || beta < TOT) && r < nrow) {
+            const int n = b % Q, base = (b / Q) * S + n;
+            dft<R>(w);
+            if constexpr (Q > 1) {
+#pragma unroll
+                for (int k = 1; k < R; ++k) w[k] = c_mul(w[k], ztw[TW + (k - 1) * Q + n]);   // W_S^{nk}
+#pragma unroll
+                for (int k = 0; k < R; ++k) rows[r * RS + zslot_at<POW2>(zslot(base), base, Q * k)] = w[k];
+            } else {
+                const int f0 = dif_freq<M, 1, true>(base), zf = zslot(f0);
+#pragma unroll
+                for (int k = 0; k < R; ++k)         // output k: frequency f0 + k M / R
+                    rows[r * RS + zslot_at<POW2>(zf, f0, k * (M / R))] = w[k];
+            }
+        }
+    };
+    if constexpr (HOLD) {
+#pragma unroll
+        for (int s = 0; s < PER; ++s) work(s);
+    } else {
+#pragma unroll 1
+        for (int s = 0; s < PER; ++s) {
+            load(s);
+            work(s);
+        }
+    }
+    row_sync<NT>(grp);
+    if constexpr (Q > 1) zrow_step<M, NR, NT, RS, Q, false>(rows, g, gs, nrow, ztw, lane, grp);
+}
+
+// D[l] and D[M-l] from u = C[l], v = C[M-l] and w = W_N^l: with s = u + conj v
+// and q = i w (u - conj v), D[l] = (s - q) / 2 and D[M-l] = conj(s + q) / 2.
+__device__ __forceinline__ void split_real(float2 u, float2 v, float2 w, float2 *dl, float2 *dm) {
+    const float2 s = make_float2(0.5f * (u.x + v.x), 0.5f * (u.y - v.y));
+    const float ox = u.x - v.x, oy = u.y + v.y;
+    const float qx = -(w.x * oy + w.y * ox), qy = w.x * ox - w.y * oy;
+    *dl = make_float2(fmaf(-0.5f, qx, s.x), fmaf(-0.5f, qy, s.y));
+    *dm = make_float2(fmaf(0.5f, qx, s.x), -fmaf(0.5f, qy, s.y));
+}
+
+// Waits of y items for their plane's z items.  A CTA holds its current item and
+// the ticket of its next one.  The unfinished item with the lowest ticket is
+// always some running CTA's current one (were it a next one, that CTA's
+// current item would have a lower ticket), and it does not wait: z items never
+// do, and a y item's z items have lower tickets.  So every wait ends; the limit
+// (about a second) only bounds it if that were ever wrong.
+constexpr int kMaxPolls = 1 << 20;
+
+// sync[0]: next ticket; sync[1 + p]: z items done in plane p.  Zero at launch;
+// the kernel that takes the x axis clears them again.  err: 4 if a wait gave up.
+template <int N>
+__global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::CTAS)
+k_fft_zy(float2 *__restrict__ mesh, int planes, int ncol, int mcut, const float2 *__restrict__ twg,
+         unsigned *__restrict__ sync, int *__restrict__ err) {
+    using K = Cfg<N>;
+    constexpr int M = K::M, Nh = K::Nh, T = K::T, NBY = K::NBY, LAG = K::LAG;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ unsigned s_ticket;
+    float2 *tw = reinterpret_cast<float2 *>(smraw);
+    float2 *ztw = tw + N;
+    float2 *buf = ztw + (ztw_offset(M, 1) + 1) / 2 * 2;
+    for (int e = threadIdx.x; e < N; e += T) tw[e] = twg[e];
+    fill_ztw(ztw, twg, M);
+    const unsigned ytiles = (unsigned)(ncol + NBY - 1) / NBY;
+    const unsigned per = K::ZI + ytiles;
+    const unsigned total = (unsigned)(planes + LAG) * per;
+    const long long plane_c = (long long)N * Nh;
+    unsigned next = threadIdx.x == 0 ? atomicAdd(sync, 1u) : 0u;
+    for (;;) {
+        __syncthreads();                        // the previous item is done with buf and s_ticket
+        if (threadIdx.x == 0) s_ticket = next;
+        __syncthreads();
+        const unsigned t = s_ticket;
+        if (t >= total) return;
+        if (threadIdx.x == 0) next = atomicAdd(sync, 1u);    // in flight during this item
+        const int step = (int)(t / per);
+        const unsigned idx = t - (unsigned)step * per;
+        if (idx < K::ZI) {
+            if (step >= planes) continue;
+            const int lane = threadIdx.x % K::NT, grp = threadIdx.x / K::NT;
+            const int row0 = (int)idx * K::RPI + grp * K::NR;
+            const int nrow = grp < K::GROUPS ? min(K::NR, N - row0) : 0;
+            float2 *g = mesh + (long long)step * plane_c + (long long)row0 * Nh;
+            if (nrow > 0) {
+                float2 *rows = buf + (size_t)grp * K::NR * K::RS;
+                zrow_step<M, K::NR, K::NT, K::RS, M, true>(rows, g, Nh, nrow, ztw, lane, grp);
+                for (int r = 0; r < nrow; ++r) {
+                    const float2 *C = rows + r * K::RS;
+                    float2 *d = g + (long long)r * Nh;
+                    for (int l = lane; l <= M / 2; l += K::NT) {
+                        float2 dl, dm;
+                        split_real(C[zslot(l)], C[zslot(l ? M - l : 0)], tw[l], &dl, &dm);
+                        if (l < ncol) d[l] = dl;
+                        if (M - l < ncol && l != M - l) d[M - l] = dm;
+                    }
+                }
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {             // the CTA's rows, seen through the barrier, then the count
+                __threadfence();
+                atomicAdd(sync + 1 + step, 1u);
+            }
+        } else {
+            const int plane = step - LAG;
+            if (plane < 0 || plane >= planes) continue;
+            if (threadIdx.x == 0) {
+                unsigned *flag = sync + 1 + plane, done;
+                int polls = 0;
+                do {
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(done) : "l"(flag) : "memory");
+                    if (done >= K::ZI) break;
+                    __nanosleep(64);
+                } while (++polls < kMaxPolls);
+                if (done < K::ZI) atomicOr(err, 4);
+            }
+            __syncthreads();
+            const int c0 = (int)(idx - K::ZI) * NBY;
+            float2 *g = mesh + (long long)plane * plane_c + c0;
+            const int nc = ncol - c0;           // valid columns of the tile
+            const auto ld = [&](int r, int c) {
+                return c < nc ? __ldcg(g + (long long)r * Nh + c) : make_float2(0.0f, 0.0f);
+            };
+            const int l2 = c0 * c0;
+            const auto st = [&](int f, int c, float2 v) {
+                const int jp = f < M ? f : f - N;
+                if (c < nc && jp * jp + l2 < mcut) g[(long long)f * Nh + c] = v;
+            };
+            col_step<N, NBY, T, false, N, true, false>(buf, tw, threadIdx.x % NBY, threadIdx.x / NBY, ld, st);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// x axis.  tiles[t] = ky index * 65536 + column block (the tiles that hold a
+// mode below mcut).
+
+// Clear the z / y pass's tickets and counters for the next compute.
+__device__ __forceinline__ void clear_sync(unsigned *sync, int n) {
+    if (blockIdx.x == 0 && blockIdx.y == 0)
+        for (int k = threadIdx.x; k < n; k += blockDim.x) sync[k] = 0u;
+}
+
+template <int N>
+__global__ void __launch_bounds__(Cfg<N>::TX, Cfg<N>::CTASX)
+k_fft_x(float2 *__restrict__ mesh, long long mesh_c, int ncol, int mcut, const int *__restrict__ tiles,
+        const float2 *__restrict__ twg, unsigned *__restrict__ sync, int nsync) {
+    using K = Cfg<N>;
+    constexpr int M = K::M, Nh = K::Nh, NX = K::NX;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float2 *tw = reinterpret_cast<float2 *>(smraw);
+    float2 *buf = tw + N;
+    for (int e = threadIdx.x; e < N; e += K::TX) tw[e] = twg[e];
+    clear_sync(sync, nsync);
+    __syncthreads();
+    const int tile = tiles[blockIdx.x];
+    const int j = tile >> 16, c0 = (tile & 0xffff) * NX;
+    const int jp = j < M ? j : j - N, nc = ncol - c0, r2 = jp * jp + c0 * c0;
+    float2 *g = mesh + (long long)blockIdx.y * mesh_c + (long long)j * Nh + c0;
+    const long long ps = (long long)N * Nh;
+    const auto ld = [&](int r, int c) { return c < nc ? __ldcs(g + r * ps + c) : make_float2(0.0f, 0.0f); };
+    const auto st = [&](int f, int c, float2 v) {
+        const int ip = f < M ? f : f - N;
+        if (c < nc && ip * ip + r2 < mcut) g[f * ps + c] = v;
+    };
+    col_step<N, NX, K::TX, false, N, true, false>(buf, tw, threadIdx.x % NX, threadIdx.x / NX, ld, st);
+}
+
+// Shared memory of k_fft_xbin: the twiddles, the tile, then the histogram,
+// the cw and phase tables and the k-bin edges.
+template <int N>
+struct XSmem {
+    __host__ __device__ static constexpr size_t al(size_t x) { return (x + 15) / 16 * 16; }
+    __host__ __device__ static constexpr size_t off_buf() { return al(sizeof(float2) * N); }
+    __host__ __device__ static constexpr size_t off_hist() { return off_buf() + al(sizeof(float2) * N * Cfg<N>::NX); }
+    __host__ __device__ static size_t off_cw(const BinGeom &g) { return off_hist() + al(sizeof(float) * g.nh); }
+    __host__ __device__ static size_t off_ph(const BinGeom &g) { return off_cw(g) + al(sizeof(float) * Cfg<N>::Nh); }
+    __host__ __device__ static size_t off_edge(const BinGeom &g) { return off_ph(g) + al(sizeof(float2) * Cfg<N>::Nh); }
+    __host__ __device__ static size_t bytes(const BinGeom &g) { return off_edge(g) + al(sizeof(int2) * g.nk); }
+};
+
+// x FFT + bin over the tiles of one catalog per blockIdx.y.  Bin pass: a
+// thread takes one column l and runs of four kx with their mirror images -kx:
+// both modes have the same m, k bin, mu bin and Legendre weights, so the key
+// arithmetic is done once for the pair, and a run is summed in registers until
+// its key changes.  |kx| = 0 and N/2 occur once.
+template <int N, bool IL, bool TWOD, bool POLES>
+__global__ void __launch_bounds__(Cfg<N>::TX, Cfg<N>::CTASX)
+k_fft_xbin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g, int ncol,
+           const int *__restrict__ tiles, int ntiles, const float *__restrict__ cw, const float2 *__restrict__ ph,
+           const float2 *__restrict__ twg, const int *__restrict__ kedge, float *__restrict__ partial,
+           unsigned *__restrict__ sync, int nsync) {
+    using K = Cfg<N>;
+    using SM = XSmem<N>;
+    constexpr int M = K::M, Nh = K::Nh, NX = K::NX, TX = K::TX, CM = IL ? NX / 2 : NX;
+    using Tl = Tile<NX, IL>;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    float2 *tw = reinterpret_cast<float2 *>(smraw);
+    float2 *buf = reinterpret_cast<float2 *>(smraw + SM::off_buf());
+    float *hist = reinterpret_cast<float *>(smraw + SM::off_hist());
+    float *scw = reinterpret_cast<float *>(smraw + SM::off_cw(g));
+    float2 *sph = reinterpret_cast<float2 *>(smraw + SM::off_ph(g));
+    int2 *sedge = reinterpret_cast<int2 *>(smraw + SM::off_edge(g));
+    for (int e = threadIdx.x; e < N; e += TX) tw[e] = twg[e];
+    for (int k = threadIdx.x; k < g.nh; k += TX) hist[k] = 0.0f;
+    for (int k = threadIdx.x; k < Nh; k += TX) {
+        scw[k] = cw[k];                          // cw[N/2] = the Nyquist index
+        sph[k] = ph[k + M];                      // e^{+i pi k / N}
+    }
+    for (int k = threadIdx.x; k < g.nk; k += TX) sedge[k] = make_int2(kedge[k], kedge[k + 1]);
+    clear_sync(sync, nsync);
+
+    const int nk = g.nk, nmu = g.nmu, hbase = g.hbase;
+    const float kscale = g.kscale, koff = g.koff;
+    const long long ps = (long long)N * Nh;
+    const float2 *base = mesh + (long long)blockIdx.y * item_stride_c;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int tile = tiles[t];
+        const int j = tile >> 16, c0 = (tile & 0xffff) * CM, nc = ncol - c0;
+        const float2 *gt = base + (long long)j * Nh + c0;
+        __syncthreads();                         // tables filled; the previous tile is binned
+        const auto ld = [&](int r, int c) {
+            const int cc = IL ? c % CM : c;
+            const float2 *p = gt + r * ps + cc;
+            if (IL && c >= CM) p += mesh_stride_c;
+            return cc < nc ? __ldcs(p) : make_float2(0.0f, 0.0f);
+        };
+        const auto st = [&](int f, int c, float2 v) { buf[Tl::slot(f, c)] = v; };
+        col_step<N, NX, TX, IL, N, true, true>(buf, tw, threadIdx.x % NX, threadIdx.x / NX, ld, st);
+        __syncthreads();
+
+        const int c = threadIdx.x % CM, l = c0 + c;
+        const int jp = j < M ? j : j - N, ja = j < M ? j : N - j;
+        const int r2 = jp * jp + l * l;
+        if (c < nc && r2 < g.mhi) {
+            const float rowcw = scw[ja] * scw[l] * (IL ? 0.25f : 1.0f) * ((l != 0 && l != M) ? 2.0f : 1.0f);
+            float2 rph = make_float2(1.0f, 0.0f);
+            if (IL) {
+                const float2 py = sph[ja];
+                rph = c_mul(make_float2(py.x, jp < 0 ? -py.y : py.y), sph[l]);
+            }
+            const unsigned rhs = (unsigned)(nmu * nmu) * (unsigned)(l * l);
+            for (int i0 = 4 * (threadIdx.x / CM); i0 <= M; i0 += 4 * (TX / CM)) {
+                if (i0 * i0 + r2 >= g.mhi) break;
+                int cur2 = -1, cur1 = -1;                 // open register runs
+                float run2 = 0.0f, runm2 = 0.0f, runm4 = 0.0f;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const int i = min(i0 + v, M);
+                    const int m = r2 + i * i;
+                    const bool live = i0 + v <= M && m < g.mhi && m >= g.mlo && m != 0;
+                    // k bin: FP32 estimate, then one exact step against the edges
+                    const float rsm = rsqrtf((float)max(m, 1));
+                    int b = (int)((float)m * rsm * kscale - koff);
+                    b = min(max(b, 0), nk - 1);
+                    {
+                        const int2 e = sedge[b];
+                        b += (int)(m >= e.y) - (int)(m < e.x);
+                        b = min(max(b, 0), nk - 1);
+                    }
+                    const int ib = i ? N - i : 0;          // row of -kx (row N/2: kx = -N/2)
+                    float2 zp = buf[Tl::slot(i == M ? 0 : i, c)], zm = buf[Tl::slot(ib, c)];
+                    if (IL) {
+                        const float2 yp = buf[Tl::slot(i == M ? 0 : i, c + CM)], ym = buf[Tl::slot(ib, c + CM)];
+                        const float2 px = sph[i];
+                        const float2 tp = c_mul(rph, px), tm = c_mul(rph, make_float2(px.x, -px.y));
+                        zp.x += yp.x * tp.x - yp.y * tp.y;
+                        zp.y += yp.x * tp.y + yp.y * tp.x;
+                        zm.x += ym.x * tm.x - ym.y * tm.y;
+                        zm.y += ym.x * tm.y + ym.y * tm.x;
+                    }
+                    float pw = i != M ? zp.x * zp.x + zp.y * zp.y : 0.0f;
+                    if (i != 0) pw += zm.x * zm.x + zm.y * zm.y;
+                    pw = live ? pw * (rowcw * scw[i]) : 0.0f;
+                    int key = b;
+                    if (TWOD) {
+                        // mu bin: FP32 estimate, then one exact integer step each way
+                        int q = (int)((float)(nmu * l) * rsm);
+                        q = min(max(q, 0), nmu - 1);
+                        if (g.mu32) {
+                            q -= (int)(q > 0 && (unsigned)(q * q) * (unsigned)m > rhs);
+                            q += (int)(q < nmu - 1 && (unsigned)((q + 1) * (q + 1)) * (unsigned)m <= rhs);
+                        } else {
+                            const long long rl = (long long)nmu * nmu * l * l;
+                            q -= (int)(q > 0 && (long long)q * q * m > rl);
+                            q += (int)(q < nmu - 1 && (long long)(q + 1) * (q + 1) * m <= rl);
+                        }
+                        key = b * nmu + q;
+                    }
+                    const bool new2 = key != cur2;
+                    if (new2 && cur2 >= 0) atomicAdd(hist + cur2, run2);
+                    run2 = new2 ? pw : run2 + pw;
+                    cur2 = key;
+                    if (POLES) {
+                        const float mu = (float)l * rsm;
+                        const float mu2 = mu * mu;
+                        const float t2 = pw * (1.5f * mu2 - 0.5f);
+                        const float t4 = pw * ((4.375f * mu2 - 3.75f) * mu2 + 0.375f);
+                        const bool new1 = b != cur1;
+                        if (new1 && cur1 >= 0) {
+                            atomicAdd(hist + hbase + cur1, runm2);
+                            atomicAdd(hist + hbase + nk + cur1, runm4);
+                        }
+                        runm2 = new1 ? t2 : runm2 + t2;
+                        runm4 = new1 ? t4 : runm4 + t4;
+                        cur1 = b;
+                    }
+                }
+                atomicAdd(hist + cur2, run2);
+                if (POLES) {
+                    atomicAdd(hist + hbase + cur1, runm2);
+                    atomicAdd(hist + hbase + nk + cur1, runm4);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    float *out = partial + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * g.nh;
+    for (int k = threadIdx.x; k < g.nh; k += TX) out[k] = hist[k];
+}
+
+// ---------------------------------------------------------------- host --
+
+template <int N>
+constexpr size_t zy_smem() {
+    using K = Cfg<N>;
+    const size_t z = (size_t)K::RPI * K::RS, y = (size_t)N * K::NBY;
+    return sizeof(float2) * (N + (ztw_offset(K::M, 1) + 1) / 2 * 2 + (z > y ? z : y));
+}
+
+template <typename F>
+cudaError_t allow_smem(F kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <int N>
+cudaError_t zy_inst(float2 *mesh, int planes, int ncol, int mcut, const float2 *tw, unsigned *sync, int *err, int nsm,
+                    cudaStream_t st) {
+    using K = Cfg<N>;
+    constexpr size_t smem = zy_smem<N>();
+    cudaError_t e = allow_smem(k_fft_zy<N>, smem);
+    if (e != cudaSuccess) return e;
+    const long long items = (long long)(planes + K::LAG) * (K::ZI + (ncol + K::NBY - 1) / K::NBY);
+    if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const unsigned grid = (unsigned)std::min<long long>((long long)nsm * K::CTAS, items);
+    k_fft_zy<N><<<grid, K::T, smem, st>>>(mesh, planes, ncol, mcut, tw, sync, err);
+    return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t x_inst(float2 *mesh, int nmesh, long long mesh_c, int ncol, int mcut, const int *tiles, int ntiles,
+                   const float2 *tw, unsigned *sync, int nsync, cudaStream_t st) {
+    using K = Cfg<N>;
+    const size_t smem = sizeof(float2) * (N + (size_t)N * K::NX);
+    cudaError_t e = allow_smem(k_fft_x<N>, smem);
+    if (e != cudaSuccess) return e;
+    k_fft_x<N><<<dim3(ntiles, nmesh), K::TX, smem, st>>>(mesh, mesh_c, ncol, mcut, tiles, tw, sync, nsync);
+    return cudaGetLastError();
+}
+
+struct XbinArgs {
+    const float2 *mesh;
+    long long is, ms;
+    int nitems, G, ncol;
+    const int *tiles;
+    int ntiles;
+    const float *cw;
+    const float2 *ph, *tw;
+    const int *kedge;
+    float *partial;
+    unsigned *sync;
+    int nsync;
+};
+
+template <int N, bool IL, bool TWOD, bool POLES>
+cudaError_t xbin_inst(const XbinArgs &a, const BinGeom &g, cudaStream_t st) {
+    const size_t smem = XSmem<N>::bytes(g);
+    cudaError_t e = allow_smem(k_fft_xbin<N, IL, TWOD, POLES>, smem);
+    if (e != cudaSuccess) return e;
+    k_fft_xbin<N, IL, TWOD, POLES><<<dim3(a.G, a.nitems), Cfg<N>::TX, smem, st>>>(
+        a.mesh, a.is, a.ms, g, a.ncol, a.tiles, a.ntiles, a.cw, a.ph, a.tw, a.kedge, a.partial, a.sync, a.nsync);
+    return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t xbin_dispatch(const XbinArgs &a, int il, const BinGeom &g, cudaStream_t st) {
+    const int key = (il ? 4 : 0) | (g.twod ? 2 : 0) | (g.poles ? 1 : 0);
+    switch (key) {
+    case 0: return xbin_inst<N, false, false, false>(a, g, st);
+    case 1: return xbin_inst<N, false, false, true>(a, g, st);
+    case 2: return xbin_inst<N, false, true, false>(a, g, st);
+    case 3: return xbin_inst<N, false, true, true>(a, g, st);
+    case 4: return xbin_inst<N, true, false, false>(a, g, st);
+    case 5: return xbin_inst<N, true, false, true>(a, g, st);
+    case 6: return xbin_inst<N, true, true, false>(a, g, st);
+    default: return xbin_inst<N, true, true, true>(a, g, st);
+    }
+}
+
+template <int N>
+int xbin_occ(const BinGeom &g, int il) {
+    const size_t smem = XSmem<N>::bytes(g);
+    const void *k = il ? reinterpret_cast<const void *>(k_fft_xbin<N, true, true, true>)
+                       : reinterpret_cast<const void *>(k_fft_xbin<N, false, true, true>);
+    int n = 0;
+    if (smem > 227 * 1024 ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, Cfg<N>::TX, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+// One size's launchers.
+template <int N>
+struct OpsOf final : ZyxOps {
+    int tile_columns(int interlaced) const override { return interlaced ? Cfg<N>::NX / 2 : Cfg<N>::NX; }
+    cudaError_t zy(void *mesh, int planes, int ncol, int mcut, const void *tw, unsigned *sync, int *err, int nsm,
+                   cudaStream_t st) const override {
+        return zy_inst<N>(reinterpret_cast<float2 *>(mesh), planes, ncol, mcut, reinterpret_cast<const float2 *>(tw),
+                          sync, err, nsm, st);
+    }
+    cudaError_t x(void *mesh, int nmesh, long long mesh_c, int ncol, int mcut, const int *tiles, int ntiles,
+                  const void *tw, unsigned *sync, int nsync, cudaStream_t st) const override {
+        return x_inst<N>(reinterpret_cast<float2 *>(mesh), nmesh, mesh_c, ncol, mcut, tiles, ntiles,
+                         reinterpret_cast<const float2 *>(tw), sync, nsync, st);
+    }
+    int xbin_ctas_per_sm(const BinGeom &g, int interlaced) const override { return xbin_occ<N>(g, interlaced); }
+    cudaError_t xbin(const void *mesh, int interlaced, long long item_stride_c, long long mesh_stride_c, int nitems,
+                     int ctas_per_item, const BinGeom &g, int ncol, const int *tiles, int ntiles, const void *cw,
+                     const void *ph, const void *tw, const int *kedge, void *partial, unsigned *sync, int nsync,
+                     cudaStream_t st) const override {
+        const XbinArgs a{reinterpret_cast<const float2 *>(mesh), item_stride_c, mesh_stride_c, nitems, ctas_per_item,
+                         ncol, tiles, ntiles, reinterpret_cast<const float *>(cw), reinterpret_cast<const float2 *>(ph),
+                         reinterpret_cast<const float2 *>(tw), kedge, reinterpret_cast<float *>(partial), sync, nsync};
+        return xbin_dispatch<N>(a, interlaced, g, st);
+    }
+};
+
+template <int N>
+const ZyxOps *ops_of() {
+    static const OpsOf<N> ops;
+    return &ops;
+}
+
+}  // namespace
+
+#ifndef PK_ZYX_GROUP
+#error "compile with -DPK_ZYX_GROUP=0 .. 3"
+#endif
+#define PK_ZYX_NAME2(g) zyx_ops_group##g
+#define PK_ZYX_NAME(g) PK_ZYX_NAME2(g)
+
+const ZyxOps *PK_ZYX_NAME(PK_ZYX_GROUP)(int N) {
+    switch (N) {
+#if PK_ZYX_GROUP == 0
+    case 320: return ops_of<320>();
+    case 384: return ops_of<384>();
+    case 400: return ops_of<400>();
+#elif PK_ZYX_GROUP == 1
+    case 480: return ops_of<480>();
+    case 500: return ops_of<500>();
+    case 600: return ops_of<600>();
+#elif PK_ZYX_GROUP == 2
+    case 640: return ops_of<640>();
+    case 768: return ops_of<768>();
+    case 800: return ops_of<800>();
+#else
+    case 1024: return ops_of<1024>();
+    case 2048: return ops_of<2048>();
+#endif
+    default: return nullptr;
+    }
+}
+
+}  // namespace pk

@@ -802,6 +802,11 @@ __device__ __forceinline__ void flush_tile(const unsigned *lo, const unsigned *h
     }
 }
 
+// Words of the cell area (two per cell), rounded up so that the float4 staging
+// area behind it is 16-byte aligned for odd tile edges too (2 T^3 words are a
+// multiple of 4 only when T is even).
+__host__ __device__ constexpr int paint_cell_words(int T) { return (2 * T * T * T + 3) & ~3; }
+
 // TC > 0: the tile edge is the compile-time constant TC (index math in shifts).
 template <int P, int NM, typename M, int TC>
 __global__ void __launch_bounds__(kPaintThreads)
@@ -814,7 +819,7 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
     const int T = TC > 0 ? TC : g.T, T3 = T * T * T;
     unsigned *lo = smu, *hi = smu + T3;
     unsigned long long *acc64 = reinterpret_cast<unsigned long long *>(smu);
-    float4 *cand = reinterpret_cast<float4 *>(smu + 2 * T3);
+    float4 *cand = reinterpret_cast<float4 *>(smu + paint_cell_words(T));
 
     // item * ntiles + tile (the launch keeps the block count below 2^31, so
     // 32-bit unsigned division suffices: 64-bit division is a long software
@@ -1607,7 +1612,7 @@ cudaError_t launch_scan64(const unsigned long long *in, int64_t n, unsigned long
 }
 
 size_t paint_smem_bytes(int T, int window, int nmesh) {
-    const size_t general = (size_t)2 * T * T * T * sizeof(unsigned) + (size_t)kStage * sizeof(float4);
+    const size_t general = (size_t)paint_cell_words(T) * sizeof(unsigned) + (size_t)kStage * sizeof(float4);
     const size_t padded = T != 16 ? 0
                           : window == 4 ? (size_t)nmesh * SweepLayout<4>::Words * sizeof(unsigned)
                           : window == 3 ? (size_t)nmesh * SweepLayout<3>::Words * sizeof(unsigned) : 0;
