@@ -69,8 +69,8 @@ typedef enum {
 /* Mesh / transform precision.  Both paint into int64 fixed point (so the
  * mesh is bit-identical run to run) and form the catalog weight sums in FP64
  * in a fixed order (also bit-identical run to run).
- * PK_MESH_F32: the library's own r2c transform at nmesh 128, 192, 256, 512
- * and 2048 (cuFFT R2C otherwise; see pk_use_own_fft); bins summed per CTA in
+ * PK_MESH_F32: the library's own r2c transform at the sizes it has kernels for
+ * (cuFFT R2C otherwise; see pk_use_own_fft); bins summed per CTA in
  * FP32 with shared-memory atomics, whose order (and so the last bits of
  * P(k)) can vary between runs, then across CTAs in FP64.
  * PK_MESH_F64: cuFFT D2Z; bins summed in FP64. */
@@ -271,26 +271,28 @@ pk_status pk_mesh(pk_plan_t plan, int item, int mesh, void *dst);
 
 /* Choose the 3D r2c transform of pk_compute (the Fourier transform of the
  * painted field, Sec. 3.3.1; the binning it feeds, Sec. 3.4.1).  on = 1: the
- * library's own FFT kernels -- length-N complex FFTs along y and x of the mesh
- * with each z row read as N/2 complex pairs (d[2n] + i d[2n+1], in place),
- * then one pass that takes the length-N/2 FFTs along z, splits the packed
- * transform into the r2c transform and bins it without writing it.  on = 0:
- * cuFFT's in-place R2C, then the bin pass.  Both give the same result within
- * FP32 rounding.  It applies to the FP32 mesh form with nmesh 128, 192, 256,
- * 512, 1024 or 2048 and is the default at all but 1024 (where cuFFT measured
- * faster).  After a compute with it, pk_cross
- * and pk_projected first write the r2c transform into the meshes (one extra
- * pass).  Takes effect at the next pk_compute.
- * Errors: PK_EINVAL (on = 1 where the own transform does not apply). */
+ * library's own FFT kernels, in place, the FP32 mesh form's default at the
+ * sizes they exist for: nmesh 128, 192, 256, 512 (length-N complex FFTs along y
+ * and x of the mesh with each z row read as N/2 complex pairs, then one pass
+ * that takes the length-N/2 FFTs along z, splits the packed transform into the
+ * r2c transform and bins it without writing it) and 320, 384, 400, 480, 500,
+ * 600, 640, 768, 800, 1024, 2048 (z and y in one pass over device memory, then
+ * x, at 1024 and 2048 in the bin pass).  on = 0: cuFFT's in-place R2C, then the
+ * bin pass.  Both give the same result within FP32 rounding.  After a compute
+ * that did not write the transform itself, pk_cross and pk_projected first
+ * write it into the meshes (one extra pass).  Takes effect at the next
+ * pk_compute.
+ * Errors: PK_EINVAL (on = 1 other than for the FP32 mesh form with nmesh 128,
+ * 192, 256, 512, 1024 or 2048). */
 pk_status pk_use_own_fft(pk_plan_t plan, int on);
 
 /* Stages whose device time pk_stage_times reports. */
 typedef enum {
     PK_STAGE_SORT = 0,    /* tile count + scan + scatter (pk_paint)             */
     PK_STAGE_PAINT = 1,   /* shared-memory tile paint (pk_paint)                */
-    PK_STAGE_FFT = 2,     /* r2c of every mesh: cuFFT, or the own y and x passes */
-    PK_STAGE_BIN = 3,     /* compensate + interlace + bin (own transform: with   */
-                          /* the z FFTs and the r2c split)                       */
+    PK_STAGE_FFT = 2,     /* r2c of every mesh: cuFFT, or the own passes         */
+    PK_STAGE_BIN = 3,     /* compensate + interlace + bin (with the own          */
+                          /* transform's last axis where that is fused into it)  */
     PK_STAGE_FINAL = 4,   /* histogram reduce + normalize + multipoles          */
     PK_NSTAGES = 5
 } pk_stage;

@@ -1,6 +1,6 @@
 """Build libpk.so in-tree with nvcc for sm_103a (GB300).
 
-Two translation units are compiled in parallel and linked against cuFFT; the
+The translation units are compiled in parallel and linked against cuFFT; the
 CUDA runtime is linked statically.  The result lands next to this file and is
 loaded by the binding in ``__init__.py``.  Rebuilds only when a source or the
 public header is newer than the library.
@@ -16,7 +16,9 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libpk.so")
-SOURCES = ["pk_kernels.cu", "pk_api.cu", "pk_static.cu", "pk_lognormal.cu", "pk_survey.cu", "pk_fft.cu"]
+SOURCES = ["pk_kernels.cu", "pk_api.cu", "pk_static.cu", "pk_lognormal.cu", "pk_survey.cu", "pk_fft.cu", "pk_fft_zyx.cu"]
+# sources compiled several times, once per group of template instances
+GROUPS = {"pk_fft_zyx.cu": ["-DPK_ZYX_GROUP=%d" % g for g in range(3)]}
 HEADERS = [os.path.join(ROOT, "include", "pk.h"), os.path.join(CSRC, "pk_internal.h"),
            os.path.join(CSRC, "pk_plan.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -54,10 +56,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
                      "-I", os.path.join(ROOT, "include")]
     procs = []
     objs = []
-    for src in SOURCES:
-        obj = os.path.join(OUT_DIR, src.replace(".cu", ".o"))
+    units = [(src, g, flag) for src in SOURCES for g, flag in enumerate(GROUPS.get(src, [None]))]
+    for src, g, flag in units:
+        obj = os.path.join(OUT_DIR, src.replace(".cu", "%s.o" % ("" if flag is None else "_%d" % g)))
         objs.append(obj)
-        cmd = [nvcc] + common + ["-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [nvcc] + common + ([] if flag is None else [flag]) + ["-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             print(" ".join(cmd), file=sys.stderr)
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

@@ -428,15 +428,39 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
         PK_CUDA(P, cudaMemcpy(P->d_kedge, P->kedge.data(), sizeof(int) * (nk + 1), cudaMemcpyHostToDevice));
     }
 
-    // ---- own transform: FP32 meshes of the supported sizes (the default at all but 1024) ----
-    if (!P->f64 && own_fft_supported(P->N)) {
+    // ---- own transform: FP32 meshes of the sizes it has kernels for ----
+    if (!P->f64) P->zyx = zyx_ops(P->N);
+    if (!P->f64 && (P->zyx || own_fft_packed(P->N))) {
         std::vector<float> tw(2 * (size_t)P->N);
         own_fft_twiddles(P->N, tw.data());
         PK_CUDA(P, dev_alloc(&P->d_tw, sizeof(float) * tw.size()));
         PK_CUDA(P, cudaMemcpy(P->d_tw, tw.data(), sizeof(float) * tw.size(), cudaMemcpyHostToDevice));
-        // one wave of k_zbin CTAs, within the partial histograms k_bin's grid sized
-        P->G_own = std::min(P->G_total, P->nsm * zbin_ctas_per_sm(bg, c.interlaced));
-        P->own_fft = own_fft_default(P->N) ? 1 : 0;
+        // one wave of fused last-axis CTAs, within the partial histograms k_bin's grid sized
+        P->own_fft = 1;
+        P->own_selectable = !P->zyx || P->N == 1024 || P->N == 2048;
+        if (!P->zyx) {
+            P->G_own = std::min(P->G_total, P->nsm * zbin_ctas_per_sm(bg, c.interlaced));
+        } else {
+            P->nsync = 1 + P->B * P->nm * P->N;
+            PK_CUDA(P, dev_alloc(&P->d_sync, sizeof(unsigned) * P->nsync));
+            PK_CUDA(P, cudaMemset(P->d_sync, 0, sizeof(unsigned) * P->nsync));
+            while (P->fft_ncol < P->Nh && (long long)P->fft_ncol * P->fft_ncol < bg.mhi) ++P->fft_ncol;
+            std::vector<int> tiles;
+            const auto add_tiles = [&](int w) {
+                const int before = (int)tiles.size();
+                for (int j = 0; j < P->N; ++j) {
+                    const long long jp = j < P->N / 2 ? j : P->N - j;
+                    for (int b = 0; b * w < P->fft_ncol; ++b)
+                        if (jp * jp + (long long)b * w * b * w < bg.mhi) tiles.push_back(j << 16 | b);
+                }
+                return (int)tiles.size() - before;
+            };
+            P->nxbin = add_tiles(P->zyx->tile_columns(c.interlaced));
+            P->nx = c.interlaced ? add_tiles(P->zyx->tile_columns(0)) : P->nxbin;
+            PK_CUDA(P, dev_alloc(&P->d_xtiles, sizeof(int) * tiles.size()));
+            PK_CUDA(P, cudaMemcpy(P->d_xtiles, tiles.data(), sizeof(int) * tiles.size(), cudaMemcpyHostToDevice));
+            P->G_own = std::min(std::min(P->G_total, P->nsm * P->zyx->xbin_ctas_per_sm(bg, c.interlaced)), P->nxbin);
+        }
     }
 
     // ---- geometry-only bin data: exact counts, mean k, mean mu ----
@@ -546,7 +570,7 @@ static pk_status paint_atomic(pk_plan_s *P, const void *dpos, int dtype, const f
     P->launches += launches;
     P->npainted = nitems;
     P->transformed = 0;
-    P->zpacked = 0;
+    P->unfinished = 0;
     return PK_OK;
 }
 
@@ -655,7 +679,7 @@ static pk_status paint_impl(pk_plan_s *P, const void *pos, int dtype, const floa
     P->launches += launches;
     P->npainted = nitems;
     P->transformed = 0;
-    P->zpacked = 0;
+    P->unfinished = 0;
     return PK_OK;
 }
 
@@ -685,6 +709,23 @@ pk_status pk_paint_values(pk_plan_t P, const void *pos, int dtype, const float *
     return paint_impl(P, pos, dtype, weights, values, offsets, nitems, 0);
 }
 
+// After a compute on the own transform the meshes of its nitems catalogs lack
+// the last axis; the passes that read the transform itself get it taken in
+// place first (once per compute).
+static pk_status finish_transform(pk_plan_s *P, int nitems) {
+    if (!P->unfinished) return PK_OK;
+    if (P->zyx)
+        PK_CUDA(P, P->zyx->x(P->mesh, nitems * P->nm, P->mesh_reals / 2, P->fft_ncol, P->bg.mhi,
+                             P->cfg.interlaced ? P->d_xtiles + P->nxbin : P->d_xtiles, P->nx, P->d_tw, P->d_sync,
+                             P->nsync, P->st));
+    else
+        PK_CUDA(P, launch_zfinish(P->mesh, P->cfg.interlaced, (long long)P->nm * P->mesh_reals / 2, P->mesh_reals / 2,
+                                  nitems, P->N, P->d_tw, P->nsm, P->st));
+    P->launches += 1;
+    P->unfinished = 0;
+    return PK_OK;
+}
+
 pk_status pk_compute(pk_plan_t P) {
     if (!P) return PK_EINVAL;
     P->err.clear();
@@ -699,16 +740,36 @@ pk_status pk_compute(pk_plan_t P) {
     int G = std::max(1, P->G_total / nitems);
     pk_status s_ = PK_OK;
     if (P->own_fft) {
-        // x and y passes, then z fused into the bin pass: the meshes end up
-        // holding the x/y transforms of the packed z rows (zpacked)
-        G = std::max(1, P->G_own / nitems);
-        PK_CUDA(P, launch_fft_xy(P->mesh, nitems * P->nm, mesh_c, P->N, P->d_tw, st));
         P->transformed = 1;
-        P->zpacked = 1;
-        if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
-        PK_CUDA(P, launch_zbin(P->mesh, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->d_cw, P->d_ph,
-                               P->d_tw, P->d_kedge, P->d_partial, st));
-        P->launches += 2;   // the two axis passes
+        P->unfinished = 1;
+        if (!P->zyx) {
+            // y and x passes, then z fused into the bin pass: the meshes end up
+            // holding the x/y transforms of the packed z rows
+            G = std::max(1, P->G_own / nitems);
+            PK_CUDA(P, launch_fft_xy(P->mesh, nitems * P->nm, mesh_c, P->N, P->d_tw, st));
+            if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
+            PK_CUDA(P, launch_zbin(P->mesh, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->d_cw, P->d_ph,
+                                   P->d_tw, P->d_kedge, P->d_partial, st));
+            P->launches += 2;   // the two axis passes
+        } else {
+            // z and y axes, then x fused into the bin pass (or, where its
+            // histogram does not fit beside a tile, x in place and k_bin)
+            PK_CUDA(P, P->zyx->zy(P->mesh, nitems * P->nm * P->N, P->fft_ncol, P->bg.mhi, P->d_tw, P->d_sync,
+                                  P->d_err, P->nsm, st));
+            P->launches += 1;
+            if (P->G_own > 0) {
+                if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
+                G = std::max(1, P->G_own / nitems);
+                PK_CUDA(P, P->zyx->xbin(P->mesh, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->fft_ncol,
+                                        P->d_xtiles, P->nxbin, P->d_cw, P->d_ph, P->d_tw, P->d_kedge, P->d_partial,
+                                        P->d_sync, P->nsync, st));
+            } else {
+                if (pk_status s = finish_transform(P, nitems); s != PK_OK) return s;
+                if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
+                PK_CUDA(P, launch_bin(P->mesh, P->f64, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->d_cw,
+                                      P->d_ph, P->d_kedge, P->d_partial, st));
+            }
+        }
     } else if ((s_ = ensure_cufft(P)) != PK_OK) {
         return s_;
     } else if (P->fft_single) {
@@ -737,7 +798,7 @@ pk_status pk_compute(pk_plan_t P) {
     }
     if (!P->own_fft) {
         P->transformed = 1;
-        P->zpacked = 0;
+        P->unfinished = 0;
         if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
         PK_CUDA(P, launch_bin(P->mesh, P->f64, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg,
                               P->d_cw, P->d_ph, P->d_kedge, P->d_partial, st));
@@ -763,23 +824,10 @@ pk_status pk_compute(pk_plan_t P) {
 
 static pk_status fill_view(pk_plan_s *P, const double *r, pk_result_view *out);
 
-// After a compute on the own transform the meshes hold the x/y transforms of
-// the packed z rows; the passes that read the r2c transform itself get it
-// written in place first (once per compute).
-static pk_status finish_transform(pk_plan_s *P) {
-    if (!P->zpacked) return PK_OK;
-    const long long item_c = (long long)P->nm * P->mesh_reals / 2;
-    PK_CUDA(P, launch_zfinish(P->mesh, P->cfg.interlaced, item_c, P->mesh_reals / 2, P->computed, P->N, P->d_tw,
-                              P->nsm, P->st));
-    P->launches += 1;
-    P->zpacked = 0;
-    return PK_OK;
-}
-
 pk_status pk_use_own_fft(pk_plan_t P, int on) {
     if (!P) return PK_EINVAL;
     P->err.clear();
-    if (on && !P->d_tw)
+    if (on && !P->own_selectable)
         return fail(P, PK_EINVAL, "the own transform needs the FP32 mesh form and nmesh 128, 192, 256, 512, 1024 or 2048");
     if (!on) {
         if (pk_status s = ensure_cufft(P); s != PK_OK) return s;
@@ -805,7 +853,7 @@ pk_status pk_cross(pk_plan_t P, int item_a, int item_b) {
     if (item_a < 0 || item_a >= P->computed || item_b < 0 || item_b >= P->computed)
         return fail(P, PK_EINVAL, "item out of range");
     const cudaStream_t st = P->st;
-    if (pk_status s = finish_transform(P); s != PK_OK) return s;
+    if (pk_status s = finish_transform(P, P->computed); s != PK_OK) return s;
     const long long item_c = (long long)P->nm * P->mesh_reals / 2;   // complex elements per catalog
     const long long mesh_c = P->mesh_reals / 2;
     const size_t csz = 2 * P->esz;
@@ -845,7 +893,7 @@ pk_status pk_projected(pk_plan_t P, int item, unsigned keep_axes, pk_projected_v
     if (!P->transformed || P->computed < 1) return fail(P, PK_ESTATE, "pk_projected needs a pk_compute first");
     if (item < 0 || item >= P->computed) return fail(P, PK_EINVAL, "item out of range");
     const cudaStream_t st = P->st;
-    if (pk_status s = finish_transform(P); s != PK_OK) return s;
+    if (pk_status s = finish_transform(P, P->computed); s != PK_OK) return s;
     const int nk = P->bg.nk;
     const size_t csz = 2 * P->esz;
     const size_t item_bytes = (size_t)P->nm * P->mesh_reals * P->esz;
@@ -910,6 +958,7 @@ static pk_status fill_view(pk_plan_s *P, const double *r, pk_result_view *out) {
     out->w2sum = r[rl.w2sum];
     const int flags = (int)r[rl.flags];
     if (flags & 2) return fail(P, PK_ECUDA, "internal: tile sort saw more copies than it counted");
+    if (flags & 4) return fail(P, PK_ETIMEOUT, "internal: a wait inside the transform gave up");
     if (flags & 1) return fail(P, PK_EOVERFLOW, "sum |w| * 2^S exceeded 2^62: lower fixed_scale_log2");
     return PK_OK;
 }

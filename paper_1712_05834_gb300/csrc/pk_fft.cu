@@ -24,7 +24,7 @@
 //                    transform after a compute (cross and projected power).
 // All transforms are forward (e^{-2 pi i jk/n}), unnormalized, radix-8
 // decimation in frequency with radix-4 and radix-3 steps where the length
-// needs them (N = 2^k, 128 <= N <= 2048, and N = 192);
+// needs them (N = 128, 192, 256, 512);
 // twiddles come from one table W_N^e (e < N) computed in FP64 on the host
 // (the x and y passes read W^n and W^{4n} of a butterfly from it and form
 // its other twiddles as products, a few ulp each).
@@ -126,17 +126,14 @@ __device__ __forceinline__ int dif_freq(int p) {
 // the first step's registers, kept in shared memory between steps
 // (buf[a * NB + c]: NB threads cover one row of buf) and written back from
 // the last step's registers in natural order.  Tile shapes per line length:
-// 16 columns (128-byte runs of each line) where the tile fits twice per SM
-// (N <= 512: 512 threads, two CTAs per SM); 16 columns in one CTA of 1024
-// threads at N = 1024 (136 KB); 8 columns at N = 2048 (144 KB: 16 would not
-// fit).  Measured: at N = 2048 the x lines' 64-byte runs stream at 2.9 TB/s
-// where 128-byte ones reach 5 TB/s.
+// 16 columns (128-byte runs of each line), where the tile fits twice per SM at
+// 512 (512 threads, two CTAs per SM).
 template <int LEN>
 struct AxisCfg {
-    static constexpr int NB = LEN >= 2048 ? 8 : 16;        // columns per tile
+    static constexpr int NB = 16;                          // columns per tile
     // threads per CTA (for 192 lines: 8 butterfly groups divide 24 and 64)
-    static constexpr int T = LEN >= 1024 ? 1024 : (LEN >= 256 ? 512 : (LEN == 192 ? 128 : 256));
-    static constexpr int MINB = LEN >= 1024 ? 1 : (LEN >= 256 ? 2 : (LEN == 192 ? 8 : 4));   // CTAs per SM
+    static constexpr int T = LEN >= 256 ? 512 : (LEN == 192 ? 128 : 256);
+    static constexpr int MINB = LEN >= 256 ? 2 : (LEN == 192 ? 8 : 4);   // CTAs per SM
 };
 
 template <int LEN, int NB, int S, bool FIRST>
@@ -246,16 +243,13 @@ cudaError_t axis_inst(float2 *mesh, int nmesh, long long mesh_c, const float2 *t
 // same slots.
 __device__ __forceinline__ int zslot(int p) { return p ^ ((p >> 2) & 15); }
 
-// A pair is handled by one warp up to M = 256 (eight pairs per CTA at a
-// time), by the whole CTA above (its four rows of M complex are 16 or 32 KB).
+// A pair is handled by one warp, eight pairs per CTA at a time.
 template <int M>
 struct ZRows {
     // slots per row: positions 0..M, even (zslot(M) = M for M = 2^k >= 64;
     // up to M + 15 otherwise)
     static constexpr int RS = (M & (M - 1)) == 0 ? M + 2 : M + 16;
     static constexpr int WPB = 8;                 // warps per CTA
-    static constexpr int NT = M >= 512 ? 256 : 32;   // threads per pair
-    static constexpr int PPC = 256 / NT;          // pairs in flight per CTA
 };
 
 // Twiddles of the z FFT steps, one table per step with block size S (from M
@@ -288,30 +282,23 @@ __device__ __forceinline__ const float2 *pair_row(const float2 *m1, const float2
     return ((r >> 1) ? m2 : m1) + ((r & 1) ? offB : offA);
 }
 
-// Barrier of the NT threads that share a pair: the warp, or the whole CTA.
-template <int NT>
-__device__ __forceinline__ void pair_sync() {
-    if constexpr (NT == 32) __syncwarp();
-    else __syncthreads();
-}
-
 // One step over blocks of S points of the length-M FFTs of the NR rows of a
-// pair, by NT threads (FIRST: read from the mesh).  The last step writes the
+// pair, by one warp (FIRST: read from the mesh).  The last step writes the
 // outputs in natural order.
-template <int M, int NR, int S, bool FIRST, int NT = 32>
+template <int M, int NR, int S, bool FIRST>
 __device__ __forceinline__ void zfft_step(float2 *rows, const float2 *m1, const float2 *m2, long long offA,
                                           long long offB, const float2 *ztw, int lane) {
     constexpr int RS = ZRows<M>::RS;
     constexpr int R = zradix_of(S), Q = S / R;
     constexpr int BPR = M / R;                    // butterflies per row
     constexpr int TOT = NR * BPR;
-    constexpr int PER = (TOT + NT - 1) / NT;
+    constexpr int PER = (TOT + 32 - 1) / 32;
     constexpr int TW = ztw_offset(M, S);
     float2 v[PER][R];
 #pragma unroll
     for (int s = 0; s < PER; ++s) {
-        const int beta = lane + NT * s;
-        if (TOT % NT == 0 || beta < TOT) {
+        const int beta = lane + 32 * s;
+        if (TOT % 32 == 0 || beta < TOT) {
             const int r = beta / BPR, b = beta % BPR;
             const int base = (b / Q) * S + b % Q;
             if (FIRST) {
@@ -325,11 +312,11 @@ __device__ __forceinline__ void zfft_step(float2 *rows, const float2 *m1, const 
         }
     }
     // the last step writes other positions than it reads: all reads first
-    if constexpr (Q == 1) pair_sync<NT>();
+    if constexpr (Q == 1) __syncwarp();
 #pragma unroll
     for (int s = 0; s < PER; ++s) {
-        const int beta = lane + NT * s;
-        if (TOT % NT == 0 || beta < TOT) {
+        const int beta = lane + 32 * s;
+        if (TOT % 32 == 0 || beta < TOT) {
             const int r = beta / BPR, b = beta % BPR;
             const int n = b % Q, base = (b / Q) * S + n;
             dft<R>(v[s]);
@@ -344,8 +331,8 @@ __device__ __forceinline__ void zfft_step(float2 *rows, const float2 *m1, const 
             }
         }
     }
-    pair_sync<NT>();
-    if constexpr (Q > 1) zfft_step<M, NR, Q, false, NT>(rows, m1, m2, offA, offB, ztw, lane);
+    __syncwarp();
+    if constexpr (Q > 1) zfft_step<M, NR, Q, false>(rows, m1, m2, offA, offB, ztw, lane);
 }
 
 // 2 D[l] from u = C[l] and v = C'[M-l] (w = W_N^l):
@@ -386,7 +373,7 @@ struct ZSmem {
     __host__ __device__ static size_t off_wl() { return al(sizeof(float2) * ztw_offset(M, 1)); }
     __host__ __device__ static size_t off_rows() { return off_wl() + al(sizeof(float2) * ZRows<M>::RS); }
     __host__ __device__ static size_t off_hist() {
-        return off_rows() + al(sizeof(float2) * (size_t)ZRows<M>::PPC * NR * ZRows<M>::RS);
+        return off_rows() + al(sizeof(float2) * (size_t)ZRows<M>::WPB * NR * ZRows<M>::RS);
     }
     __host__ __device__ static size_t off_cw(const BinGeom &g) { return off_hist() + al(sizeof(float) * g.nh); }
     __host__ __device__ static size_t off_ph(const BinGeom &g) {
@@ -414,7 +401,7 @@ __device__ __forceinline__ void fill_z_tables(unsigned char *smraw, const float2
 // same r2 = kx'^2 + ky'^2 and so, mode by mode, the same m, k bin, mu bin and
 // Legendre weights: each key is computed once and takes the sum of both
 // rows' powers (the partner's is left out for a row that is its own partner).
-template <bool IL, bool TWOD, bool POLES, bool MU32, int M, int NT = 32>
+template <bool IL, bool TWOD, bool POLES, bool MU32, int M>
 __device__ __forceinline__ void bin_pair(const float2 *rows, int i, int j, int pi, int pj, int r2, int llo,
                                          int lhi, const BinGeom &g, const float *__restrict__ cw,
                                          const float2 *__restrict__ ph, const float *scw, const float2 *sph,
@@ -435,7 +422,7 @@ __device__ __forceinline__ void bin_pair(const float2 *rows, int i, int j, int p
         phA = c_mul(ph[ip + M], ph[jp + M]);
         phB = c_mul(ph[pip + M], ph[pjp + M]);
     }
-    for (int l0 = llo + kZVec * lane; l0 < lhi; l0 += NT * kZVec) {
+    for (int l0 = llo + kZVec * lane; l0 < lhi; l0 += 32 * kZVec) {
         const int cnt = lhi - l0;
         int cur2 = -1, cur1 = -1;
         float run2 = 0.0f, runm2 = 0.0f, runm4 = 0.0f;
@@ -516,7 +503,7 @@ __global__ void __launch_bounds__(32 * ZRows<M>::WPB)
 k_zbin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
        const float *__restrict__ cw, const float2 *__restrict__ ph, const float2 *__restrict__ twg,
        const int *__restrict__ kedge, float *__restrict__ partial) {
-    constexpr int NR = IL ? 4 : 2, RS = ZRows<M>::RS, NT = ZRows<M>::NT, PPC = ZRows<M>::PPC, N = 2 * M,
+    constexpr int NR = IL ? 4 : 2, RS = ZRows<M>::RS, PPC = ZRows<M>::WPB, N = 2 * M,
                   Nh = M + 1;
     using SM = ZSmem<M, NR>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -526,7 +513,7 @@ k_zbin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_
     float *scw = reinterpret_cast<float *>(smraw + SM::off_cw(g));
     float2 *sph = reinterpret_cast<float2 *>(smraw + SM::off_ph(g));
     int2 *sedge = reinterpret_cast<int2 *>(smraw + SM::off_edge(g));
-    const int lane = threadIdx.x % NT, grp = threadIdx.x / NT;
+    const int lane = threadIdx.x % 32, grp = threadIdx.x / 32;
     float2 *rows = reinterpret_cast<float2 *>(smraw + SM::off_rows()) + (size_t)grp * NR * RS;
     fill_z_tables<M, NR>(smraw, twg);
     for (int k = threadIdx.x; k < g.nh; k += blockDim.x) hist[k] = 0.0f;
@@ -552,9 +539,9 @@ k_zbin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_
         if (llo >= lhi) continue;
         const int pi = i == 0 ? 0 : N - i, pj = j == 0 ? 0 : N - j;
         const long long offA = ((long long)i * N + j) * Nh, offB = ((long long)pi * N + pj) * Nh;
-        pair_sync<NT>();    // the previous pair's bin reads are done
-        zfft_step<M, NR, M, true, NT>(rows, m1, m2, offA, offB, ztw, lane);
-        bin_pair<IL, TWOD, POLES, MU32, M, NT>(rows, i, j, pi, pj, r2, llo, lhi, g, cw, ph, scw, sph, swl, sedge,
+        __syncwarp();    // the previous pair's bin reads are done
+        zfft_step<M, NR, M, true>(rows, m1, m2, offA, offB, ztw, lane);
+        bin_pair<IL, TWOD, POLES, MU32, M>(rows, i, j, pi, pj, r2, llo, lhi, g, cw, ph, scw, sph, swl, sedge,
                                                hist, lane);
     }
     __syncthreads();
@@ -568,12 +555,12 @@ template <int M, int NR>
 __global__ void __launch_bounds__(32 * ZRows<M>::WPB)
 k_zfinish(float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c,
           const float2 *__restrict__ twg) {
-    constexpr int RS = ZRows<M>::RS, NT = ZRows<M>::NT, PPC = ZRows<M>::PPC, N = 2 * M, Nh = M + 1;
+    constexpr int RS = ZRows<M>::RS, PPC = ZRows<M>::WPB, N = 2 * M, Nh = M + 1;
     using SM = ZSmem<M, NR>;
     extern __shared__ __align__(16) unsigned char smraw[];
     const float2 *ztw = reinterpret_cast<const float2 *>(smraw);
     const float2 *swl = reinterpret_cast<const float2 *>(smraw + SM::off_wl());
-    const int lane = threadIdx.x % NT, grp = threadIdx.x / NT;
+    const int lane = threadIdx.x % 32, grp = threadIdx.x / 32;
     float2 *rows = reinterpret_cast<float2 *>(smraw + SM::off_rows()) + (size_t)grp * NR * RS;
     fill_z_tables<M, NR>(smraw, twg);
     __syncthreads();
@@ -585,8 +572,8 @@ k_zfinish(float2 *__restrict__ mesh, long long item_stride_c, long long mesh_str
         pair_rows(p, N, &i, &j);
         const int pi = i == 0 ? 0 : N - i, pj = j == 0 ? 0 : N - j;
         const long long offA = ((long long)i * N + j) * Nh, offB = ((long long)pi * N + pj) * Nh;
-        pair_sync<NT>();
-        zfft_step<M, NR, M, true, NT>(rows, m1, m2, offA, offB, ztw, lane);
+        __syncwarp();
+        zfft_step<M, NR, M, true>(rows, m1, m2, offA, offB, ztw, lane);
         // every row pair's transform is in shared memory before any store:
         // the stores below overwrite only this pair's rows
         const bool self = pi == i && pj == j;
@@ -594,7 +581,7 @@ k_zfinish(float2 *__restrict__ mesh, long long item_stride_c, long long mesh_str
         for (int q = 0; q < NR / 2; ++q) {
             float2 *dst = q ? m2 : m1;
             const float2 *ra = rows + (2 * q) * RS, *rb = ra + RS;
-            for (int l = lane; l < Nh; l += NT) {
+            for (int l = lane; l < Nh; l += 32) {
                 const int sl = zslot(l), la = zslot(l == M ? 0 : l), lb = zslot(l == 0 ? 0 : M - l);
                 const float2 w = swl[sl];
                 const float2 dA = split2(ra[la], rb[lb], w);
@@ -665,14 +652,12 @@ cudaError_t zfinish_inst(void *mesh, long long is, long long ms, int nitems, int
 
 }  // namespace
 
-bool own_fft_supported(int N) { return N == 128 || N == 192 || N == 256 || N == 512 || N == 1024 || N == 2048; }
-
 // Measured on a GB300 (FFT + bin): 32 catalogs of 128^3 0.40 against 0.56 ms
-// with cuFFT, 24 of 192^3 1.07 against 1.35 ms, 512^3 1.25 against 1.84 ms,
-// 2048^3 121 against 234 ms; at 1024^3 13.4 against 12.7 ms (the CTA-per-pair
-// z pass is latency-bound at 16 warps per SM), so 1024 keeps cuFFT unless the
-// caller asks for the own transform.
-bool own_fft_default(int N) { return N == 128 || N == 192 || N == 256 || N == 512 || N == 2048; }
+// with cuFFT, 24 of 192^3 1.07 against 1.35 ms, 512^3 1.24 against 1.84 ms.
+// Against the z-and-y-in-one-pass form of pk_fft_zyx.cu (interlaced at 512^3
+// 1.24 against 1.28 ms, one mesh of 256^3 0.099 against 0.144 ms): these sizes
+// stay packed, where the fused z pass works warp by warp without CTA barriers.
+bool own_fft_packed(int N) { return N == 128 || N == 192 || N == 256 || N == 512; }
 
 void own_fft_twiddles(int N, float *tw) {
     for (int e = 0; e < N; ++e) {
@@ -695,8 +680,6 @@ cudaError_t launch_fft_xy(void *mesh, int nmesh, long long mesh_c, int N, const 
     case 192: return axis_inst<192>(m, nmesh, mesh_c, t, st);
     case 256: return axis_inst<256>(m, nmesh, mesh_c, t, st);
     case 512: return axis_inst<512>(m, nmesh, mesh_c, t, st);
-    case 1024: return axis_inst<1024>(m, nmesh, mesh_c, t, st);
-    case 2048: return axis_inst<2048>(m, nmesh, mesh_c, t, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -707,8 +690,6 @@ size_t zbin_smem_bytes(const BinGeom &g, int interlaced) {
     case 192: return interlaced ? ZSmem<96, 4>::bytes(g) : ZSmem<96, 2>::bytes(g);
     case 256: return interlaced ? ZSmem<128, 4>::bytes(g) : ZSmem<128, 2>::bytes(g);
     case 512: return interlaced ? ZSmem<256, 4>::bytes(g) : ZSmem<256, 2>::bytes(g);
-    case 1024: return interlaced ? ZSmem<512, 4>::bytes(g) : ZSmem<512, 2>::bytes(g);
-    case 2048: return interlaced ? ZSmem<1024, 4>::bytes(g) : ZSmem<1024, 2>::bytes(g);
     default: return 0;
     }
 }
@@ -730,10 +711,8 @@ int zbin_ctas_per_sm(const BinGeom &g, int interlaced) {
         PK_ZK(128)
     } else if (g.N == 512) {
         PK_ZK(256)
-    } else if (g.N == 1024) {
-        PK_ZK(512)
     } else {
-        PK_ZK(1024)
+        return 1;
     }
 #undef PK_ZK
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
@@ -764,12 +743,6 @@ cudaError_t launch_zbin(const void *mesh, int interlaced, long long item_stride_
     case 512:
         return zbin_dispatch<256>(mesh, interlaced, item_stride_c, mesh_stride_c, nitems, ctas_per_item, g, cw,
                                   ph, tw, kedge, partial, st);
-    case 1024:
-        return zbin_dispatch<512>(mesh, interlaced, item_stride_c, mesh_stride_c, nitems, ctas_per_item, g, cw,
-                                  ph, tw, kedge, partial, st);
-    case 2048:
-        return zbin_dispatch<1024>(mesh, interlaced, item_stride_c, mesh_stride_c, nitems, ctas_per_item, g, cw,
-                                   ph, tw, kedge, partial, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -789,12 +762,6 @@ cudaError_t launch_zfinish(void *mesh, int interlaced, long long item_stride_c, 
     case 512:
         return interlaced ? zfinish_inst<256, 4>(mesh, item_stride_c, mesh_stride_c, nitems, nsm, tw, st)
                           : zfinish_inst<256, 2>(mesh, item_stride_c, mesh_stride_c, nitems, nsm, tw, st);
-    case 1024:
-        return interlaced ? zfinish_inst<512, 4>(mesh, item_stride_c, mesh_stride_c, nitems, nsm, tw, st)
-                          : zfinish_inst<512, 2>(mesh, item_stride_c, mesh_stride_c, nitems, nsm, tw, st);
-    case 2048:
-        return interlaced ? zfinish_inst<1024, 4>(mesh, item_stride_c, mesh_stride_c, nitems, nsm, tw, st)
-                          : zfinish_inst<1024, 2>(mesh, item_stride_c, mesh_stride_c, nitems, nsm, tw, st);
     default: return cudaErrorInvalidValue;
     }
 }

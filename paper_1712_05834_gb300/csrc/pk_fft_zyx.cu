@@ -16,13 +16,18 @@
 //                L2 (129 MB) and overwrite them there: device memory sees one
 //                read and one write for two axes (512^3: 2.1 GB counted, where
 //                two passes move 4.3).
-//   k_fft_xbin   x axis and the bin pass: one CTA per tile of columns (ky, l0 ..)
+//   k_fft_x      the x axis, written back in place; k_bin then bins the modes.
+//   k_fft_xbin   (N = 1024, 2048, unless a pass needs the transform itself) x
+//                axis and the bin pass: one CTA per tile of columns (ky, l0 ..)
 //                (two interlaced meshes share a tile) takes the length-N FFTs
 //                along x in shared memory and bins the modes from there:
 //                interlace combine, sinc^p compensation, k bin, mu bin,
-//                Legendre sums.  The r2c transform itself is never written.
-//   k_fft_x      the x axis alone, written back in place, for the passes that
-//                read the transform after a compute (cross, projected power).
+//                Legendre sums; the r2c transform is never written.  Measured
+//                against k_fft_x + k_bin (ms, with k_fft_zy): 1024 interlaced
+//                11.1 against 12.0, 2048 58.3 against 62.1; 640 interlaced 4.5
+//                against 4.1, 480 1.96 against 1.74 (its bin pass idles half
+//                of the threads at the edge of the sphere), so the smaller
+//                sizes take the two kernels.
 //
 // Only modes with m = |n|^2 < mhi enter a bin: columns l with l^2 >= mhi are
 // neither transformed along y nor read, the y pass does not write rows ky with
@@ -243,10 +248,10 @@ template <int T_, int CTAS_, int NBY_, int TX_, int CTASX_, int NX_, int LAG_>
 struct ShapeOf {
     static constexpr int T = T_, CTAS = CTAS_, NBY = NBY_, TX = TX_, CTASX = CTASX_, NX = NX_, LAG = LAG_;
 };
-template <> struct Shape<320> : ShapeOf<256, 4, 8, 256, 4, 8, 32> {};
-template <> struct Shape<384> : ShapeOf<384, 2, 8, 384, 2, 8, 32> {};
+template <> struct Shape<320> : ShapeOf<256, 4, 8, 320, 2, 16, 32> {};
+template <> struct Shape<384> : ShapeOf<384, 2, 8, 384, 2, 16, 32> {};
 template <> struct Shape<400> : ShapeOf<320, 3, 8, 320, 3, 8, 32> {};
-template <> struct Shape<480> : ShapeOf<384, 2, 8, 384, 2, 8, 24> {};
+template <> struct Shape<480> : ShapeOf<384, 2, 8, 384, 2, 16, 24> {};
 template <> struct Shape<500> : ShapeOf<416, 2, 8, 416, 2, 8, 24> {};
 template <> struct Shape<600> : ShapeOf<480, 2, 8, 480, 2, 8, 16> {};
 template <> struct Shape<640> : ShapeOf<512, 2, 8, 512, 2, 8, 16> {};
@@ -266,6 +271,7 @@ struct Cfg : Shape<N> {
     static constexpr int RPI = GROUPS * NR;                      // rows per z item
     static constexpr int ZI = (N + RPI - 1) / RPI;               // z items per plane
     static_assert(NT == 32 || GROUPS <= 15, "named barriers are 1 .. 15");
+    static constexpr bool FUSE = N >= 1024;                      // k_fft_xbin
 };
 
 // ---------------------------------------------------------------------------
@@ -890,7 +896,10 @@ struct OpsOf final : ZyxOps {
         return x_inst<N>(reinterpret_cast<float2 *>(mesh), nmesh, mesh_c, ncol, mcut, tiles, ntiles,
                          reinterpret_cast<const float2 *>(tw), sync, nsync, st);
     }
-    int xbin_ctas_per_sm(const BinGeom &g, int interlaced) const override { return xbin_occ<N>(g, interlaced); }
+    int xbin_ctas_per_sm(const BinGeom &g, int interlaced) const override {
+        if constexpr (Cfg<N>::FUSE) return xbin_occ<N>(g, interlaced);
+        else return 0;
+    }
     cudaError_t xbin(const void *mesh, int interlaced, long long item_stride_c, long long mesh_stride_c, int nitems,
                      int ctas_per_item, const BinGeom &g, int ncol, const int *tiles, int ntiles, const void *cw,
                      const void *ph, const void *tw, const int *kedge, void *partial, unsigned *sync, int nsync,
@@ -898,7 +907,8 @@ struct OpsOf final : ZyxOps {
         const XbinArgs a{reinterpret_cast<const float2 *>(mesh), item_stride_c, mesh_stride_c, nitems, ctas_per_item,
                          ncol, tiles, ntiles, reinterpret_cast<const float *>(cw), reinterpret_cast<const float2 *>(ph),
                          reinterpret_cast<const float2 *>(tw), kedge, reinterpret_cast<float *>(partial), sync, nsync};
-        return xbin_dispatch<N>(a, interlaced, g, st);
+        if constexpr (Cfg<N>::FUSE) return xbin_dispatch<N>(a, interlaced, g, st);
+        else return cudaErrorInvalidValue;
     }
 };
 
@@ -911,7 +921,7 @@ const ZyxOps *ops_of() {
 }  // namespace
 
 #ifndef PK_ZYX_GROUP
-#error "compile with -DPK_ZYX_GROUP=0 .. 3"
+#error "compile with -DPK_ZYX_GROUP=0 .. 2"
 #endif
 #define PK_ZYX_NAME2(g) zyx_ops_group##g
 #define PK_ZYX_NAME(g) PK_ZYX_NAME2(g)
@@ -922,16 +932,15 @@ const ZyxOps *PK_ZYX_NAME(PK_ZYX_GROUP)(int N) {
     case 320: return ops_of<320>();
     case 384: return ops_of<384>();
     case 400: return ops_of<400>();
-#elif PK_ZYX_GROUP == 1
     case 480: return ops_of<480>();
     case 500: return ops_of<500>();
     case 600: return ops_of<600>();
-#elif PK_ZYX_GROUP == 2
     case 640: return ops_of<640>();
     case 768: return ops_of<768>();
     case 800: return ops_of<800>();
-#else
+#elif PK_ZYX_GROUP == 1
     case 1024: return ops_of<1024>();
+#else
     case 2048: return ops_of<2048>();
 #endif
     default: return nullptr;

@@ -124,10 +124,9 @@ cudaError_t launch_plane_bin(const void *m1, const void *m2, int f64, int N, int
                              const void *ph, const int *kedge, int nk, double kF, double *sums, int nsm,
                              cudaStream_t st);
 
-// ---- own FFT path (pk_fft.cu), FP32 meshes with N in {128, 192, 256, 512, 1024, 2048} ----
+// ---- own FFT path (pk_fft.cu), FP32 meshes with N in {128, 192, 256, 512} ----
 // The meshes' z rows are read as N/2 complex values (packed real pairs).
-bool own_fft_supported(int N);
-bool own_fft_default(int N);                      // pk_compute uses it unless told otherwise
+bool own_fft_packed(int N);
 void own_fft_twiddles(int N, float *tw);          // tw[2e], tw[2e+1] = W_N^e, e < N
 // length-N FFTs along y, then along x, of nmesh packed meshes mesh_c complex apart
 cudaError_t launch_fft_xy(void *mesh, int nmesh, long long mesh_c, int N, const void *tw, cudaStream_t st);
@@ -141,6 +140,42 @@ int zbin_ctas_per_sm(const BinGeom &g, int interlaced);
 // z transform + r2c split written back in place (the meshes then hold the r2c transform)
 cudaError_t launch_zfinish(void *mesh, int interlaced, long long item_stride_c, long long mesh_stride_c,
                            int nitems, int N, const void *tw, int nsm, cudaStream_t st);
+
+// ---- own FFT path (pk_fft_zyx.cu): z and y axes in one pass, then x ----
+struct ZyxOps {
+    // Columns l of one x tile (per mesh) of the fused bin pass; tile lists hold
+    // ky index * 65536 + column block for the tiles with a mode m < mhi.
+    virtual int tile_columns(int interlaced) const = 0;
+    // z and y axes of `planes` consecutive x planes; only columns l < ncol and
+    // rows with ky^2 + l^2 below mcut are transformed.  sync: 1 + planes
+    // counters, zero on entry, cleared by the next x or xbin.  err: 4 if a wait
+    // gave up.
+    virtual cudaError_t zy(void *mesh, int planes, int ncol, int mcut, const void *tw, unsigned *sync, int *err,
+                           int nsm, cudaStream_t st) const = 0;
+    // x axis of nmesh meshes in place (tiles: tile_columns(0) wide).
+    virtual cudaError_t x(void *mesh, int nmesh, long long mesh_c, int ncol, int mcut, const int *tiles, int ntiles,
+                          const void *tw, unsigned *sync, int nsync, cudaStream_t st) const = 0;
+    // x axis + the bin pass of launch_bin, partial histograms as launch_bin
+    // writes them.
+    virtual cudaError_t xbin(const void *mesh, int interlaced, long long item_stride_c, long long mesh_stride_c,
+                             int nitems, int ctas_per_item, const BinGeom &g, int ncol, const int *tiles, int ntiles,
+                             const void *cw, const void *ph, const void *tw, const int *kedge, void *partial,
+                             unsigned *sync, int nsync, cudaStream_t st) const = 0;
+    virtual int xbin_ctas_per_sm(const BinGeom &g, int interlaced) const = 0;   // 0: no xbin (or its shared memory does not fit)
+
+protected:
+    ~ZyxOps() = default;
+};
+const ZyxOps *zyx_ops_group0(int N);
+const ZyxOps *zyx_ops_group1(int N);
+const ZyxOps *zyx_ops_group2(int N);
+// The launchers of size N (static storage), or NULL.
+inline const ZyxOps *zyx_ops(int N) {
+    const ZyxOps *o = zyx_ops_group0(N);
+    if (!o) o = zyx_ops_group1(N);
+    if (!o) o = zyx_ops_group2(N);
+    return o;
+}
 
 cudaError_t launch_geom_hist(const BinGeom &g, unsigned long long *H, unsigned long long *HL,
                              cudaStream_t st);

@@ -1374,7 +1374,7 @@ __global__ void k_finalize(const double *__restrict__ sums2, int nchunk, int nsu
         r[rl.shot] = shot;
         r[rl.wsum] = wsum;
         r[rl.w2sum] = w2sum;
-        r[rl.flags] = (double)(((wabs > f.headroom) ? 1 : 0) | (*err & 2));
+        r[rl.flags] = (double)(((wabs > f.headroom) ? 1 : 0) | (*err & 6));
     }
 }
 

@@ -32,11 +32,19 @@ struct pk_plan_s {
     std::vector<cufftHandle> fft;
     int fft_single = 0;              // one single-mesh plan, one call per mesh (large meshes)
     void *fft_work = nullptr;
-    // Own transform (pk_fft.cu): y and x passes, then z fused into the bin.
+    // Own transform: packed (pk_fft.cu: y and x passes, then z fused into the bin)
+    // or zyx (pk_fft_zyx.cu: z and y in one pass, then x fused into the bin).
     int own_fft = 0;                 // pk_compute uses it (FP32 form, supported N)
-    int zpacked = 0;                 // meshes hold the x/y transforms of packed z rows
-    int G_own = 0;                   // k_zbin CTAs for one catalog
+    int own_selectable = 0;          // pk_use_own_fft(plan, 1) accepts it
+    const pk::ZyxOps *zyx = nullptr; // zyx form; NULL: packed
+    int unfinished = 0;              // meshes hold the transform without its last axis
+    int G_own = 0;                   // fused last-axis CTAs for one catalog (zyx: 0 = x, then k_bin)
     void *d_tw = nullptr;            // W_N^e, e < N (float2)
+    unsigned *d_sync = nullptr;      // zyx: ticket and plane counters of the z / y pass
+    int nsync = 0;
+    int fft_ncol = 0;                // zyx: columns l that hold a binned mode
+    int *d_xtiles = nullptr;         // zyx: tiles of the x axis, fused pass then plain pass
+    int nxbin = 0, nx = 0;
 
     uint32_t *d_count = nullptr;     // objects per (tile, class) key
     uint32_t *d_off = nullptr;       // exclusive scan of d_count (+ total)
