@@ -309,6 +309,7 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
     pg.invHd = (double)P->N / c.box_size;
     pg.N = P->N;
     pg.T = T;
+    pg.inv_T = ((1u << 20) + T - 1) / T;
     pg.ntx = P->N / T;
     pg.lo = rlo;
     pg.hi = rhi;
@@ -666,11 +667,11 @@ static pk_status paint_impl(pk_plan_s *P, const void *pos, int dtype, const floa
                                  P->d_wsums, P->d_wpart, P->d_wmax, st));
     if (dw != nullptr || dv != nullptr || dtype == PK_F32X4) launches += 1;   // the weight sums' reduce
     PK_CUDA(P, launch_scan(P->d_count, nkeys, P->d_off, P->d_scan_tmp, &launches, st));
-    PK_CUDA(P, launch_sort_scatter(dpos, dtype, dw, dv, P->d_item_off, nitems, max_n, P->pg, P->d_off,
-                                   P->d_count, P->d_sorted, P->d_err, st));
+    PK_CUDA(P, launch_sort_scatter(dpos, dtype, dw, dv, P->d_item_off, nitems, max_n, P->pg, P->d_count,
+                                   P->d_sorted, (uint32_t)ntot, P->d_err, st));
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[1], st));
     const int unit_weights = dw == nullptr && dv == nullptr && dtype != PK_F32X4;
-    PK_CUDA(P, launch_paint_tiles(P->d_sorted, P->d_off, nitems, P->pg, P->p, P->nm, P->S, P->f64,
+    PK_CUDA(P, launch_paint_tiles(P->d_sorted, P->d_off, P->d_count, P->d_err, nitems, P->pg, P->p, P->nm, P->S, P->f64,
                                   P->d_wmax, unit_weights, P->mesh, P->nm * P->mesh_reals,
                                   P->mesh_reals, accumulate, st));
     launches += 1;

@@ -23,6 +23,8 @@ struct PaintGeom {
     double invHd;       // N / L in FP64
     int N;              // cells per side
     int T;              // tile edge (divides N, T >= hi - lo)
+    unsigned inv_T;     // ceil(2^20 / T): cell / T = cell * inv_T >> 20 exactly for
+                        // cell < 4096 (the excess, below 2^-8, is less than 1 / T)
     int ntx;            // tiles per side = N / T
     int lo, hi;         // reach of the window support relative to floor(s)
     long long ntiles;   // ntx^3 tiles per catalog
@@ -70,16 +72,18 @@ cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const 
                               uint32_t *count, double *wsums, double *wpart, unsigned *wmax, cudaStream_t st);
 // Doubles of the per-block weight-sum rows (wpart) for nitems catalogs.
 size_t wsum_partial_elems(int nitems);
-cudaError_t launch_scan(const uint32_t *in, int64_t n, uint32_t *out, uint32_t *tmp, int *launches,
+// exclusive scan into out (total in out[n]) and, in place of the counts, into in
+cudaError_t launch_scan(uint32_t *in, int64_t n, uint32_t *out, uint32_t *tmp, int *launches,
                         cudaStream_t st);
 cudaError_t launch_scan64(const unsigned long long *in, int64_t n, unsigned long long *out,
                           unsigned long long *tmp, int *launches, cudaStream_t st);
 cudaError_t launch_sort_scatter(const void *pos, int dtype, const float *w, const float *vals,
                                 const int64_t *item_off, int nitems, int64_t max_n, const PaintGeom &g,
-                                const uint32_t *off, uint32_t *count, float4 *sorted, int *err,
-                                cudaStream_t st);
-cudaError_t launch_paint_tiles(const float4 *sorted, const uint32_t *off, int nitems,
-                               const PaintGeom &g, int window, int nmesh, int S, int f64,
+                                uint32_t *cursor, float4 *sorted, uint32_t ntot, int *err, cudaStream_t st);
+// off, cursor: the scan's offsets and their copy as the scatter left it (err: 2
+// if a cursor is not at the next key's offset).
+cudaError_t launch_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *err,
+                               int nitems, const PaintGeom &g, int window, int nmesh, int S, int f64,
                                const unsigned *wmax, int unit_weights, void *mesh,
                                long long item_stride, long long mesh_stride, int accumulate,
                                cudaStream_t st);

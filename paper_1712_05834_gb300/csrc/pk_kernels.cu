@@ -11,10 +11,11 @@
 //                   added in a fixed order (run-to-run identical sums).
 //   k_scan_*        exclusive scan of the key counts (uint32).
 //   k_sort_scatter  write one float4 (home-tile-local x, y, z, w) per object
-//                   at offset[key] + (its key's count, decremented): the
-//                   order inside a key is whatever order the decrements are
+//                   at its key's cursor, advanced by the write (the scan
+//                   leaves the offsets in the counts' place, too): the
+//                   order inside a key is whatever order the cursors are
 //                   served in, which the paint's integer deposits do not
-//                   see; the counts end at zero.  No per-object rank array.
+//                   see.  No per-object rank array.
 //   k_paint_tiles   one CTA per tile: gather the tile's own objects and the
 //                   boundary classes of its 26 neighbours whose window reaches
 //                   into it, deposit B-spline weights into shared memory as
@@ -100,10 +101,15 @@ __device__ __forceinline__ float wrap_cells(float x, float invH, float invH_lo, 
     }
     return s;
 }
+// The range tests compare the bit patterns of non-negative doubles as integers:
+// this part runs FP64 at 1/64 of the FP32 rate, and the count and scatter of
+// FP64 positions are bound by it (count and scatter of 1e6
+// weighted objects 54 + 44 -> 47 + 33 us).
 __device__ __forceinline__ double wrap_cells(double x, double invH, int N) {
     const double n = (double)N;
     double s = __dmul_rn(x, invH);
-    if (!(s >= 0.0 && s < n)) {
+    // sign bit clear and s < n (NaN and infinities are not)
+    if ((unsigned long long)__double_as_longlong(s) >= (unsigned long long)__double_as_longlong(n)) {
         s = __dsub_rn(s, __dmul_rn(n, floor(__ddiv_rn(s, n))));
         if (s < 0.0) s = __dadd_rn(s, n);
         if (s >= n) s = __dsub_rn(s, n);
@@ -163,8 +169,8 @@ __device__ __forceinline__ void home_key(const Obj<R> &o, const PaintGeom &g, in
     int c = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int cell = min((int)floor(o.s[a]), g.N - 1);
-        const int t = cell / g.T;
+        const int cell = min((int)o.s[a], g.N - 1);        // s >= 0: truncation is the floor
+        const int t = (int)(((unsigned)cell * g.inv_T) >> 20);      // cell / T (see PaintGeom)
         const int cl = cell - t * g.T;
         tile3[a] = t;
         c = c * 3 + (cl < -g.lo ? 0 : (cl >= g.T - g.hi ? 2 : 1));
@@ -282,16 +288,19 @@ k_sort_count(const void *__restrict__ pos, const float *__restrict__ w, const fl
     flush_wsums(sw, sw2, swa, mw, WEIGHTED, item, end - beg, wsums, wpart, wmax);
 }
 
-// Tile sort, pass 2: each object takes the last free slot of its key's range
-// (the key's count, decremented: objects of the key not yet placed, this one
-// included).  Measured: both passes are bound by the L2's atomic rate, not by
-// its latency (two, four or eight objects per thread with every load and
-// atomic issued before the first use ran 4 %, 10 % and 23 % slower).
+// Tile sort, pass 2: each object takes the slot at its key's cursor (the scan's
+// offsets, copied over the counts) and advances it.  Two scattered accesses per
+// object, the returning atomic and the 16-byte write: the L1 takes one 128-byte
+// line of a scattered warp access per clock, and the offset and its successor
+// read beside a decremented count were two more (1e7 objects at 512^3: 200 -> 176
+// us; 1.3e8 at 1024^3: 4.66 -> 3.72 ms).  k_paint_tiles checks that every cursor
+// ends at the next key's offset.  More objects per thread with every load and atomic
+// issued before the first use ran slower (two, four, eight: 4, 10, 23 %).
 template <int DT>
 __global__ void __launch_bounds__(kCountThreads)
 k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
-               const int64_t *__restrict__ item_off, PaintGeom g, const uint32_t *__restrict__ off,
-               uint32_t *__restrict__ count, float4 *__restrict__ sorted, int *__restrict__ err) {
+               const int64_t *__restrict__ item_off, PaintGeom g, uint32_t *__restrict__ cursor,
+               float4 *__restrict__ sorted, uint32_t ntot, int *__restrict__ err) {
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
     const int64_t beg = item_off[item], end = item_off[item + 1];
@@ -301,15 +310,14 @@ k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const 
         const Obj<R> o = load_obj<DT>(pos, w, vals, i, g);
         int t3[3];
         const int64_t key = sort_key<R>(o, g, kbase, t3);
-        const uint32_t left = atomicSub(count + key, 1u);
-        const uint32_t first = off[key];
-        if (left == 0 || left > off[key + 1] - first) {   // count and scatter disagree: never write
+        const uint32_t slot = atomicAdd(cursor + key, 1u);
+        if (slot >= ntot) {                      // count and scatter disagree: never write
             atomicOr(err, 2);
             continue;
         }
-        sorted[first + left - 1] = make_float4((float)(o.s[0] - (R)(t3[0] * g.T)) + o.e[0],
-                                               (float)(o.s[1] - (R)(t3[1] * g.T)) + o.e[1],
-                                               (float)(o.s[2] - (R)(t3[2] * g.T)) + o.e[2], o.a);
+        sorted[slot] = make_float4((float)(o.s[0] - (R)(t3[0] * g.T)) + o.e[0],
+                                   (float)(o.s[1] - (R)(t3[1] * g.T)) + o.e[1],
+                                   (float)(o.s[2] - (R)(t3[2] * g.T)) + o.e[2], o.a);
     }
 }
 
@@ -342,10 +350,11 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T *total) {
     return before;
 }
 
-// out may alias in: every thread reads its own elements before writing them.
+// out and copy (a second place for the results, or NULL) may alias in: every
+// thread reads its own elements before writing them.
 template <typename T>
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_blocks(const T *in, int64_t n, T *out, T *bsum) {
+k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
     T v[kScanPer];
     T s = 0;
@@ -358,7 +367,10 @@ k_scan_blocks(const T *in, int64_t n, T *out, T *bsum) {
     T run = block_exclusive_scan<T>(s, &total);
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
-        if (base + k < n) out[base + k] = run;
+        if (base + k < n) {
+            out[base + k] = run;
+            if (copy) copy[base + k] = run;
+        }
         run += v[k];
     }
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
@@ -366,12 +378,16 @@ k_scan_blocks(const T *in, int64_t n, T *out, T *bsum) {
 
 template <typename T>
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb) {
+k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T *__restrict__ copy) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
     const T add = bsum[blockIdx.x];
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k)
-        if (base + k < n) out[base + k] += add;
+        if (base + k < n) {
+            const T v = out[base + k] + add;
+            out[base + k] = v;
+            if (copy) copy[base + k] = v;
+        }
     if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = bsum[nb];
 }
 
@@ -810,8 +826,8 @@ __host__ __device__ constexpr int paint_cell_words(int T) { return (2 * T * T * 
 // TC > 0: the tile edge is the compile-time constant TC (index math in shifts).
 template <int P, int NM, typename M, int TC>
 __global__ void __launch_bounds__(kPaintThreads)
-k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ off, PaintGeom g,
-              int S, const unsigned *__restrict__ wmax_bits, float wmax_deposit, M *__restrict__ mesh,
+k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ off,
+              const uint32_t *__restrict__ cursor, int *__restrict__ err, PaintGeom g, int S, const unsigned *__restrict__ wmax_bits, float wmax_deposit, M *__restrict__ mesh,
               long long item_stride, long long mesh_stride, int accumulate) {
     extern __shared__ __align__(16) unsigned smu[];   // lo[T^3], hi[T^3] or acc64[T^3]; cand[kStage]
     __shared__ uint32_t s_beg[kSegments];
@@ -854,6 +870,10 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
         const uint32_t b = off[kb + cz0], e = off[kb + cz1 + 1];
         s_beg[s] = b;
         s_pre[s + 1] = e - b;
+    } else if (threadIdx.x >= 96 && threadIdx.x < 96 + kClasses) {
+        // the scatter left every cursor of this tile's keys at the next key's offset
+        const int64_t key = ((int64_t)item * g.ntiles + t) * kClasses + (threadIdx.x - 96);
+        if (cursor[key] != off[key + 1]) atomicOr(err, 2);
     }
     __syncthreads();
     if (threadIdx.x < 32) {                          // warp scan of the 75 lengths
@@ -1538,13 +1558,12 @@ size_t wsum_partial_elems(int nitems) { return (size_t)nitems * kWsumBlocks * 3;
 
 cudaError_t launch_sort_scatter(const void *pos, int dtype, const float *w, const float *vals,
                                 const int64_t *item_off, int nitems, int64_t max_n, const PaintGeom &g,
-                                const uint32_t *off, uint32_t *count, float4 *sorted, int *err,
-                                cudaStream_t st) {
+                                uint32_t *cursor, float4 *sorted, uint32_t ntot, int *err, cudaStream_t st) {
     dim3 grid(grid_for(max_n, kCountThreads, 1u << 20), nitems);
     switch (dtype) {
-    case PK_F32: k_sort_scatter<PK_F32><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, off, count, sorted, err); break;
-    case PK_F64: k_sort_scatter<PK_F64><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, off, count, sorted, err); break;
-    default: k_sort_scatter<PK_F32X4><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, off, count, sorted, err); break;
+    case PK_F32: k_sort_scatter<PK_F32><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, cursor, sorted, ntot, err); break;
+    case PK_F64: k_sort_scatter<PK_F64><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, cursor, sorted, ntot, err); break;
+    default: k_sort_scatter<PK_F32X4><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, cursor, sorted, ntot, err); break;
     }
     return cudaGetLastError();
 }
@@ -1583,32 +1602,32 @@ size_t scan_tmp_elems(int64_t n) {
 }
 
 template <typename T>
-static cudaError_t scan_impl(const T *in, int64_t n, T *out, T *tmp, int *launches, cudaStream_t st) {
+static cudaError_t scan_impl(const T *in, int64_t n, T *out, T *tmp, T *copy, int *launches, cudaStream_t st) {
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb <= 1) {
-        k_scan_blocks<T><<<1, kScanThreads, 0, st>>>(in, n, out, out + n);
+        k_scan_blocks<T><<<1, kScanThreads, 0, st>>>(in, n, out, out + n, copy);
         *launches += 1;
         return cudaGetLastError();
     }
     if (nb > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_scan_blocks<T><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, out, tmp);
+    k_scan_blocks<T><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, out, tmp, nullptr);
     *launches += 1;
-    cudaError_t e = scan_impl<T>(tmp, nb, tmp, tmp + nb + 1, launches, st);
+    cudaError_t e = scan_impl<T>(tmp, nb, tmp, tmp + nb + 1, nullptr, launches, st);
     if (e != cudaSuccess) return e;
-    k_scan_add<T><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb);
+    k_scan_add<T><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
     *launches += 1;
     return cudaGetLastError();
 }
 
-// out[0 .. n) = exclusive scan of in, out[n] = total.  tmp: scan_tmp_elems(n).
-cudaError_t launch_scan(const uint32_t *in, int64_t n, uint32_t *out, uint32_t *tmp, int *launches,
-                        cudaStream_t st) {
-    return scan_impl<uint32_t>(in, n, out, tmp, launches, st);
+// out[0 .. n) = exclusive scan of in, out[n] = total; in[0 .. n) gets a copy of
+// out[0 .. n).  tmp: scan_tmp_elems(n).
+cudaError_t launch_scan(uint32_t *in, int64_t n, uint32_t *out, uint32_t *tmp, int *launches, cudaStream_t st) {
+    return scan_impl<uint32_t>(in, n, out, tmp, in, launches, st);
 }
 
 cudaError_t launch_scan64(const unsigned long long *in, int64_t n, unsigned long long *out,
                           unsigned long long *tmp, int *launches, cudaStream_t st) {
-    return scan_impl<unsigned long long>(in, n, out, tmp, launches, st);
+    return scan_impl<unsigned long long>(in, n, out, tmp, nullptr, launches, st);
 }
 
 size_t paint_smem_bytes(int T, int window, int nmesh) {
@@ -1620,7 +1639,7 @@ size_t paint_smem_bytes(int T, int window, int nmesh) {
 }
 
 template <int P, int NM, typename M>
-static cudaError_t paint_inst(const float4 *sorted, const uint32_t *off, int nitems,
+static cudaError_t paint_inst(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *err, int nitems,
                               const PaintGeom &g, int S, const unsigned *wmax, float wmax_deposit,
                               void *mesh, long long item_stride, long long mesh_stride, int accumulate,
                               cudaStream_t st) {
@@ -1631,14 +1650,14 @@ static cudaError_t paint_inst(const float4 *sorted, const uint32_t *off, int nit
     auto kern = g.T == 16 ? k_paint_tiles<P, NM, M, 16> : k_paint_tiles<P, NM, M, 0>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)nblocks, kPaintThreads, smem, st>>>(sorted, off, g, S, wmax, wmax_deposit,
+    kern<<<(unsigned)nblocks, kPaintThreads, smem, st>>>(sorted, off, cursor, err, g, S, wmax, wmax_deposit,
                                                          reinterpret_cast<M *>(mesh), item_stride,
                                                          mesh_stride, accumulate);
     return cudaGetLastError();
 }
 
-cudaError_t launch_paint_tiles(const float4 *sorted, const uint32_t *off, int nitems,
-                               const PaintGeom &g, int window, int nmesh, int S, int f64,
+cudaError_t launch_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *err,
+                               int nitems, const PaintGeom &g, int window, int nmesh, int S, int f64,
                                const unsigned *wmax, int unit_weights, void *mesh,
                                long long item_stride, long long mesh_stride, int accumulate,
                                cudaStream_t st) {
@@ -1646,13 +1665,13 @@ cudaError_t launch_paint_tiles(const float4 *sorted, const uint32_t *off, int ni
     const float wdep = !unit_weights ? 0.0f : (window == 2 ? 1.0f : window == 3 ? 0.421875f : 0.2962963f);
 #define PK_PAINT_CASE(P)                                                                              \
     if (window == P) {                                                                                \
-        if (f64) return nmesh == 2 ? paint_inst<P, 2, double>(sorted, off, nitems, g, S, wmax, wdep, mesh, \
+        if (f64) return nmesh == 2 ? paint_inst<P, 2, double>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh, \
                                                               item_stride, mesh_stride, accumulate, st) \
-                                   : paint_inst<P, 1, double>(sorted, off, nitems, g, S, wmax, wdep, mesh, \
+                                   : paint_inst<P, 1, double>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh, \
                                                               item_stride, mesh_stride, accumulate, st); \
-        return nmesh == 2 ? paint_inst<P, 2, float>(sorted, off, nitems, g, S, wmax, wdep, mesh,     \
+        return nmesh == 2 ? paint_inst<P, 2, float>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh,     \
                                                     item_stride, mesh_stride, accumulate, st)         \
-                          : paint_inst<P, 1, float>(sorted, off, nitems, g, S, wmax, wdep, mesh,     \
+                          : paint_inst<P, 1, float>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh,     \
                                                     item_stride, mesh_stride, accumulate, st);        \
     }
     PK_PAINT_CASE(2)
