@@ -377,7 +377,7 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
     PK_CUDA(P, dev_alloc(&P->d_item_off, sizeof(int64_t) * (P->B + 1)));
     PK_CUDA(P, dev_alloc(&P->d_wsums, sizeof(double) * 4 * P->B));
     PK_CUDA(P, dev_alloc(&P->d_wpart, sizeof(double) * wsum_partial_elems(P->B)));
-    PK_CUDA(P, dev_alloc(&P->d_wmax, sizeof(unsigned) * P->B));
+    PK_CUDA(P, dev_alloc(&P->d_wmax, sizeof(uint4) * P->B));
     PK_CUDA(P, dev_alloc(&P->d_err, sizeof(int)));
     PK_CUDA(P, cudaMemset(P->d_err, 0, sizeof(int)));
     PK_CUDA(P, dev_alloc(&P->d_cw, P->esz * P->N));
@@ -558,7 +558,7 @@ static pk_status paint_atomic(pk_plan_s *P, const void *dpos, int dtype, const f
     PK_CUDA(P, launch_upload_i64(P->d_item_off, offsets, nitems + 1, &launches, st));
     if (!accumulate) {
         PK_CUDA(P, cudaMemsetAsync(P->d_wsums, 0, sizeof(double) * 4 * nitems, st));
-        PK_CUDA(P, cudaMemsetAsync(P->d_wmax, 0, sizeof(unsigned) * nitems, st));
+        PK_CUDA(P, cudaMemsetAsync(P->d_wmax, 0, sizeof(uint4) * nitems, st));
     }
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[1], st));   // no sort stage
     PK_CUDA(P, launch_paint_atomic(dpos, dtype, dw, dv, P->d_item_off, nitems, max_n, P->pg, P->p, P->nm, P->S,
@@ -661,7 +661,7 @@ static pk_status paint_impl(pk_plan_s *P, const void *pos, int dtype, const floa
     PK_CUDA(P, cudaMemsetAsync(P->d_count, 0, sizeof(uint32_t) * nkeys, st));
     if (!accumulate) {
         PK_CUDA(P, cudaMemsetAsync(P->d_wsums, 0, sizeof(double) * 4 * nitems, st));
-        PK_CUDA(P, cudaMemsetAsync(P->d_wmax, 0, sizeof(unsigned) * nitems, st));
+        PK_CUDA(P, cudaMemsetAsync(P->d_wmax, 0, sizeof(uint4) * nitems, st));
     }
     PK_CUDA(P, launch_sort_count(dpos, dtype, dw, dv, P->d_item_off, nitems, max_n, P->pg, P->d_count,
                                  P->d_wsums, P->d_wpart, P->d_wmax, st));
@@ -672,8 +672,8 @@ static pk_status paint_impl(pk_plan_s *P, const void *pos, int dtype, const floa
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[1], st));
     const int unit_weights = dw == nullptr && dv == nullptr && dtype != PK_F32X4;
     PK_CUDA(P, launch_paint_tiles(P->d_sorted, P->d_off, P->d_count, P->d_err, nitems, P->pg, P->p, P->nm, P->S, P->f64,
-                                  P->d_wmax, unit_weights, P->mesh, P->nm * P->mesh_reals,
-                                  P->mesh_reals, accumulate, st));
+                                  P->d_wmax, unit_weights, P->mesh,
+                                  P->nm * P->mesh_reals, P->mesh_reals, accumulate, st));
     launches += 1;
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[2], st));
     P->tev_paint = tm;

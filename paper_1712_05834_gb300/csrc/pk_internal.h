@@ -69,7 +69,7 @@ cudaError_t launch_upload_i64(int64_t *dst, const int64_t *src, int n, int *laun
 // each object deposits W V and the sums keep sum W, sum (W V)^2, sum |W V|.
 cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const float *vals,
                               const int64_t *item_off, int nitems, int64_t max_n, const PaintGeom &g,
-                              uint32_t *count, double *wsums, double *wpart, unsigned *wmax, cudaStream_t st);
+                              uint32_t *count, double *wsums, double *wpart, uint4 *wmax, cudaStream_t st);
 // Doubles of the per-block weight-sum rows (wpart) for nitems catalogs.
 size_t wsum_partial_elems(int nitems);
 // exclusive scan into out (total in out[n]) and, in place of the counts, into in
@@ -84,16 +84,15 @@ cudaError_t launch_sort_scatter(const void *pos, int dtype, const float *w, cons
 // if a cursor is not at the next key's offset).
 cudaError_t launch_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *err,
                                int nitems, const PaintGeom &g, int window, int nmesh, int S, int f64,
-                               const unsigned *wmax, int unit_weights, void *mesh,
-                               long long item_stride, long long mesh_stride, int accumulate,
-                               cudaStream_t st);
+                               const uint4 *wmax, int unit_weights, void *mesh, long long item_stride, long long mesh_stride,
+                               int accumulate, cudaStream_t st);
 
 // Direct atomic paint into dense int64 accumulators (nitems x nmesh x N^3,
 // zero on entry), then conversion into the r2c mesh layout (clears them).
 cudaError_t launch_paint_atomic(const void *pos, int dtype, const float *w, const float *vals,
                                 const int64_t *item_off, int nitems, int64_t max_n, const PaintGeom &g,
                                 int window, int nmesh, int S, unsigned long long *acc, double *wsums,
-                                double *wpart, unsigned *wmax, cudaStream_t st);
+                                double *wpart, uint4 *wmax, cudaStream_t st);
 cudaError_t launch_acc_to_mesh(unsigned long long *acc, int nitems, int nmesh, int N, int S, int f64,
                                void *mesh, long long item_stride, long long mesh_stride, int accumulate,
                                int nsm, cudaStream_t st);

@@ -23,11 +23,11 @@
 //                   (the split point is chosen per tile so the low word can
 //                   never carry; shared 32-bit atomics are ~5x faster than
 //                   64-bit ones here), then write the tile once, coalesced,
-//                   into the in-place r2c layout.  Unit weights: one sweep
-//                   over the candidates deposits both interlaced meshes (one
-//                   32-bit word per cell each), branch-free in sparse tiles;
-//                   weighted objects: one mesh per pass over staged
-//                   candidates.  Integer adds are order-free: the mesh is
+//                   into the in-place r2c layout.  Where a 32-bit word holds
+//                   every cell of the tile, one sweep over the candidates
+//                   deposits both interlaced meshes, branch-free in sparse
+//                   tiles; else one mesh per pass over staged candidates.
+//                   Integer adds are order-free: the mesh is
 //                   bit-identical run to run and for any object order.
 //   k_paint_atomic  the variant without a sort: one thread per object adds
 //                   each deposit with a 64-bit global atomic into a dense
@@ -193,12 +193,13 @@ __device__ __forceinline__ float warp_max(float v) {
 // Block reduction of the weight sums: sum W, sum (W V)^2, sum |W V| of the
 // block's objects into its row wpart[(item * gridDim.x + block) * 3 + k]
 // (summed over the blocks in a fixed order by k_wsum_reduce, so the sums do
-// not depend on which block finishes first); wmax[item] = max |W V| (float
+// not depend on which block finishes first); wmax[item].x = max |W V| (float
 // bits, order-free), with W the weight and W V the painted amplitude.
-// Unweighted: wsums[4 * item + {0,1,2}] += n, wmax = 1.
-__device__ __forceinline__ void flush_wsums(double sw, double sw2, double swa, float mw, bool weighted,
+// .y = 1 if any W V is negative.  Unweighted: wsums[4 * item + {0,1,2}] += n,
+// max = 1.
+__device__ __forceinline__ void flush_wsums(double sw, double sw2, double swa, float mw, bool neg, bool weighted,
                                             int item, int64_t n_item, double *__restrict__ wsums,
-                                            double *__restrict__ wpart, unsigned *__restrict__ wmax) {
+                                            double *__restrict__ wpart, uint4 *__restrict__ wmax) {
     if (weighted) {
         __shared__ double red[3][kCountThreads / 32];
         __shared__ float redm[kCountThreads / 32];
@@ -213,7 +214,7 @@ __device__ __forceinline__ void flush_wsums(double sw, double sw2, double swa, f
             red[2][wid] = swa;
             redm[wid] = mw;
         }
-        __syncthreads();
+        const int any_neg = __syncthreads_or(neg);
         if (threadIdx.x < 3) {
             double t = 0.0;
             for (int k = 0; k < kCountThreads / 32; ++k) t += red[threadIdx.x][k];
@@ -221,19 +222,23 @@ __device__ __forceinline__ void flush_wsums(double sw, double sw2, double swa, f
         } else if (threadIdx.x == 3) {
             float m = 0.0f;
             for (int k = 0; k < kCountThreads / 32; ++k) m = fmaxf(m, redm[k]);
-            atomicMax(wmax + item, __float_as_uint(m));
+            atomicMax(&wmax[item].x, __float_as_uint(m));
+        } else if (threadIdx.x == 4 && any_neg) {
+            atomicOr(&wmax[item].y, 1u);
         }
     } else if (blockIdx.x == 0 && threadIdx.x < 3) {
         atomicAdd(wsums + 4 * item + threadIdx.x, (double)n_item);   // exact below 2^53
-        if (threadIdx.x == 0) atomicMax(wmax + item, __float_as_uint(1.0f));
+        if (threadIdx.x == 0) atomicMax(&wmax[item].x, __float_as_uint(1.0f));
     }
 }
 
 // Fixed-order sum of the blocks' weight-sum rows of catalog blockIdx.x:
 // thread t adds rows t, t + 256, ... in turn, then a fixed tree; the result
-// is added to wsums[4 * item + k] (one writer per value).
+// is added to wsums[4 * item + k] (one writer per value).  wmax[item].z: the
+// mean |W V| (float bits), from which the tile paint guesses a tile's sum.
 __global__ void __launch_bounds__(256)
-k_wsum_reduce(const double *__restrict__ wpart, int nblk, double *__restrict__ wsums) {
+k_wsum_reduce(const double *__restrict__ wpart, int nblk, const int64_t *__restrict__ item_off,
+              double *__restrict__ wsums, uint4 *__restrict__ wmax) {
     __shared__ double red[3][256];
     const int item = blockIdx.x, t = threadIdx.x;
     double a[3] = {0.0, 0.0, 0.0};
@@ -250,6 +255,10 @@ k_wsum_reduce(const double *__restrict__ wpart, int nblk, double *__restrict__ w
         __syncthreads();
     }
     if (t < 3) wsums[4 * item + t] += red[t][0];
+    if (t == 3) {
+        const float n = (float)(item_off[item + 1] - item_off[item]);
+        wmax[item].z = __float_as_uint(n > 0.0f ? (float)red[2][0] / n : 0.0f);
+    }
 }
 
 // Key of an object: (catalog, home tile, boundary class).
@@ -265,13 +274,14 @@ template <int DT, bool WEIGHTED>
 __global__ void __launch_bounds__(kCountThreads)
 k_sort_count(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
              const int64_t *__restrict__ item_off, PaintGeom g, uint32_t *__restrict__ count,
-             double *__restrict__ wsums, double *__restrict__ wpart, unsigned *__restrict__ wmax) {
+             double *__restrict__ wsums, double *__restrict__ wpart, uint4 *__restrict__ wmax) {
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
     const int64_t beg = item_off[item], end = item_off[item + 1];
     const int64_t kbase = (int64_t)item * g.ntiles * kClasses;
     double sw = 0.0, sw2 = 0.0, swa = 0.0;
     float mw = 0.0f;
+    bool neg = false;
     for (int64_t i = beg + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end;
          i += (int64_t)gridDim.x * blockDim.x) {
         const Obj<R> o = load_obj<DT>(pos, w, vals, i, g);
@@ -283,9 +293,10 @@ k_sort_count(const void *__restrict__ pos, const float *__restrict__ w, const fl
             sw2 += ad * ad;
             swa += fabs(ad);
             mw = fmaxf(mw, fabsf(o.a));
+            neg |= o.a < 0.0f;
         }
     }
-    flush_wsums(sw, sw2, swa, mw, WEIGHTED, item, end - beg, wsums, wpart, wmax);
+    flush_wsums(sw, sw2, swa, mw, neg, WEIGHTED, item, end - beg, wsums, wpart, wmax);
 }
 
 // Tile sort, pass 2: each object takes the slot at its key's cursor (the scan's
@@ -350,9 +361,9 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T *total) {
     return before;
 }
 
-// out and copy (a second place for the results, or NULL) may alias in: every
+// out and copy (COPY: a second place for the results) may alias in: every
 // thread reads its own elements before writing them.
-template <typename T>
+template <typename T, bool COPY>
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
@@ -369,14 +380,14 @@ k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
     for (int k = 0; k < kScanPer; ++k) {
         if (base + k < n) {
             out[base + k] = run;
-            if (copy) copy[base + k] = run;
+            if constexpr (COPY) copy[base + k] = run;
         }
         run += v[k];
     }
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 
-template <typename T>
+template <typename T, bool COPY>
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T *__restrict__ copy) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
@@ -386,7 +397,7 @@ k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T
         if (base + k < n) {
             const T v = out[base + k] + add;
             out[base + k] = v;
-            if (copy) copy[base + k] = v;
+            if constexpr (COPY) copy[base + k] = v;
         }
     if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = bsum[nb];
 }
@@ -432,15 +443,23 @@ struct Split {
     unsigned twoB_u;  // 2^B as an integer
     float inv2B;      // 2^-B
     float hi_scale;   // 2^(B - S): weight units of one hi count
-    int fast;         // 2: no deposit needs a split; 1: split when needed;
-                      // 0: this tile uses 64-bit shared atomics instead
+    int fast;         // 1: split when needed; 0: this tile uses 64-bit shared atomics instead
 };
 
-// MODE 2: every deposit is known to satisfy 0 <= round(v) < 2^B (unit
-// weights): one FMA, one subtract, one 32-bit shared atomic per cell.
-// MODE 1: as 2, with a split into hi * 2^B + lo for the rare large or
-// negative deposit.  MODE 0: 64-bit shared atomics (dense tiles).
-template <int P, int MODE, int TC = 0>
+// round(vxy wz) as a two's complement word.  UNIT: in [0, 2^23), by one FMA
+// against 2^23, whose bits hold the integer; else any |v| < 2^31, by a conversion
+// (16 lanes a clock on this part, hidden behind the shared atomics).
+template <bool UNIT>
+__device__ __forceinline__ unsigned quantize(float vxy, float wz) {
+    if constexpr (UNIT) return __float_as_uint(fmaf(vxy, wz, 8388608.0f)) - 0x4B000000u;
+    else return (unsigned)__float2int_rn(vxy * wz);
+}
+
+// MODE 2: the tile's cells fit one word each (see the sweep in k_paint_tiles):
+// one rounding and one 32-bit shared atomic per cell.  MODE 1: lo words with a
+// split into hi * 2^B + lo for the rare large or negative deposit.  MODE 0:
+// 64-bit shared atomics (dense tiles).
+template <int P, int MODE, int TC = 0, bool UNIT = true>
 __device__ __forceinline__ void deposit(unsigned *lo, unsigned *hi, unsigned long long *acc64,
                                         const Split &sp, int T, float x, float y, float z, float ws) {
     int bx, by, bz;
@@ -464,7 +483,7 @@ __device__ __forceinline__ void deposit(unsigned *lo, unsigned *hi, unsigned lon
                 const int cz = bz + c;
                 if ((unsigned)cz >= (unsigned)T) continue;
                 if (MODE == 2) {
-                    atomicAdd(lo + row + cz, __float_as_uint(fmaf(vxy, wz[c], 8388608.0f)) - 0x4B000000u);
+                    atomicAdd(lo + row + cz, quantize<UNIT>(vxy, wz[c]));
                 } else if (MODE == 1) {
                     // 2^23 + round(v) in one FMA; its bits minus 0x4B000000 are
                     // round(v) whenever 0 <= round(v) < 2^B (B <= 22): the
@@ -496,7 +515,7 @@ __device__ __forceinline__ void deposit(unsigned *lo, unsigned *hi, unsigned lon
 // min((unsigned)sum, trash) sends it to the lane's scratch word sm[trash]
 // (never read); the lanes of a warp never split on tile bounds.  cell0: the
 // first word of the mesh's cells in sm.
-template <int P, int TC>
+template <int P, int TC, bool UNIT>
 __device__ __forceinline__ void deposit_flat(unsigned *sm, int cell0, unsigned trash, int T, float x, float y,
                                              float z, float ws) {
     int bx, by, bz;
@@ -526,8 +545,7 @@ __device__ __forceinline__ void deposit_flat(unsigned *sm, int cell0, unsigned t
             const int oab = ox[a] + oy[b];
 #pragma unroll
             for (int c = 0; c < P; ++c) {
-                const unsigned q = __float_as_uint(fmaf(vxy, wz[c], 8388608.0f)) - 0x4B000000u;
-                atomicAdd(sm + min((unsigned)(oab + oz[c]), trash), q);
+                atomicAdd(sm + min((unsigned)(oab + oz[c]), trash), quantize<UNIT>(vxy, wz[c]));
             }
         }
     }
@@ -571,7 +589,7 @@ struct SweepLayout {
 // ws already scaled by 2^S) into the mesh whose first word is sm.  A first
 // node bz outside [BzMin, BzMax] only occurs for a window lying wholly
 // outside the tile along z: it deposits nothing.
-template <int P, bool SKIP_PLANES>
+template <int P, bool UNIT>
 __device__ __forceinline__ void sweep_deposit(unsigned *sm, float x, float y, float z, float ws) {
     using Lay = SweepLayout<P>;
     constexpr int kOut = 1 << 20;                     // > Words: marks a row outside the tile
@@ -590,7 +608,6 @@ __device__ __forceinline__ void sweep_deposit(unsigned *sm, float x, float y, fl
     }
 #pragma unroll
     for (int a = 0; a < P; ++a) {
-        if (SKIP_PLANES && ox[a] == kOut) continue;
         const float vxw = ws * wx[a];
 #pragma unroll
         for (int b = 0; b < P; ++b) {
@@ -600,17 +617,24 @@ __device__ __forceinline__ void sweep_deposit(unsigned *sm, float x, float y, fl
                 unsigned *row = sm + ro;
 #pragma unroll
                 for (int c = 0; c < P; ++c)
-                    atomicAdd(row + c, __float_as_uint(fmaf(vxy, wz[c], 8388608.0f)) - 0x4B000000u);
+                    atomicAdd(row + c, quantize<UNIT>(vxy, wz[c]));
             }
         }
     }
 }
 
+// Value of a one-word cell: two's complement where deposits can be negative.
+template <typename M, bool UNIT>
+__device__ __forceinline__ M word_value(unsigned w, bool sgn) {
+    if constexpr (UNIT) return (M)w;
+    else return sgn ? (M)(int)w : (M)w;
+}
+
 // Write mesh words of the padded layout (cells of the tile only) to the r2c
 // mesh: two cells per thread and store, as flush_tile (two 32-bit loads: the
 // odd strides leave a pair of cells 4-byte aligned only).
-template <typename M, int P>
-__device__ __forceinline__ void sweep_flush(const unsigned *sm, float inv_scale, M *__restrict__ dst0, int N,
+template <typename M, int P, bool UNIT>
+__device__ __forceinline__ void sweep_flush(const unsigned *sm, bool sgn, float inv_scale, M *__restrict__ dst0, int N,
                                             long long pitch, int accumulate) {
     using Lay = SweepLayout<P>;
     using M2 = typename std::conditional<sizeof(M) == 4, float2, double2>::type;
@@ -626,10 +650,9 @@ __device__ __forceinline__ void sweep_flush(const unsigned *sm, float inv_scale,
     const long long gstep = (long long)planes * N * pitch;
 #pragma unroll 2
     for (int k = 0; k < T / planes; ++k, w += planes * Lay::XS, dst += gstep) {
-        const uint2 l2 = make_uint2(sm[w], sm[w + 1]);
         M2 v;
-        v.x = (M)l2.x * (M)inv_scale;
-        v.y = (M)l2.y * (M)inv_scale;
+        v.x = word_value<M, UNIT>(sm[w], sgn) * (M)inv_scale;
+        v.y = word_value<M, UNIT>(sm[w + 1], sgn) * (M)inv_scale;
         M2 *d2 = reinterpret_cast<M2 *>(dst);
         if (accumulate) {
             const M2 o = *d2;
@@ -728,20 +751,42 @@ __device__ __forceinline__ void deposit_staged(const float4 *cand, uint32_t n, u
 template <int P, int TC>
 __device__ __forceinline__ void deposit_any(const float4 *cand, uint32_t n, unsigned *lo, unsigned *hi,
                                             unsigned long long *acc64, const Split &sp, int T, float sh) {
-    if (sp.fast == 2) deposit_staged<P, 2, TC>(cand, n, lo, hi, acc64, sp, T, sh);
-    else if (sp.fast == 1) deposit_staged<P, 1, TC>(cand, n, lo, hi, acc64, sp, T, sh);
+    if (sp.fast) deposit_staged<P, 1, TC>(cand, n, lo, hi, acc64, sp, T, sh);
     else deposit_staged<P, 0, TC>(cand, n, lo, hi, acc64, sp, T, sh);
 }
 
 // Write one tile's cells to the mesh (r2c layout, rows of T cells along z at
-// the given pitch).  Sources: lo alone (no split), lo + hi (split), or acc64
-// (64-bit cells).  Even T: two cells per thread with 8- (FP32) or 16-byte
+// the given pitch).  Sources: lo alone
+// (one-word cells), lo + hi (split), or acc64 (64-bit cells).  Even T: two cells per thread with 8- (FP32) or 16-byte
 // (FP64) stores; the row pitch and tile origin are even, so they are aligned.
-template <typename M, int TC>
+template <typename M, int TC, bool UNIT>
 __device__ __forceinline__ void flush_tile(const unsigned *lo, const unsigned *hi, const unsigned long long *acc64,
-                                           const Split &sp, float inv_scale, M *__restrict__ mb, int T, int N,
+                                           const Split &sp, bool sgn, float inv_scale, M *__restrict__ mb, int T, int N,
                                            long long pitch, int accumulate) {
     using M2 = typename std::conditional<sizeof(M) == 4, float2, double2>::type;
+    const auto cell = [&](int c) -> M {
+        if (acc64) return cell_value<M>(0u, 0u, acc64[c], sp, inv_scale);
+        if (hi) return cell_value<M>(lo[c], hi[c], 0ull, sp, inv_scale);
+        return word_value<M, UNIT>(lo[c], sgn) * (M)inv_scale;
+    };
+    const auto pair = [&](int c) -> M2 {        // cells c, c + 1 (c even)
+        M2 v;
+        if (acc64) {
+            v.x = cell_value<M>(0u, 0u, acc64[c], sp, inv_scale);
+            v.y = cell_value<M>(0u, 0u, acc64[c + 1], sp, inv_scale);
+        } else {
+            const uint2 l2 = *reinterpret_cast<const uint2 *>(lo + c);
+            if (hi) {
+                const uint2 h2 = *reinterpret_cast<const uint2 *>(hi + c);
+                v.x = cell_value<M>(l2.x, h2.x, 0ull, sp, inv_scale);
+                v.y = cell_value<M>(l2.y, h2.y, 0ull, sp, inv_scale);
+            } else {
+                v.x = word_value<M, UNIT>(l2.x, sgn) * (M)inv_scale;
+                v.y = word_value<M, UNIT>(l2.y, sgn) * (M)inv_scale;
+            }
+        }
+        return v;
+    };
     constexpr int kPlane = TC > 0 ? (TC / 2) * TC : 1;                 // cell pairs per x-plane
     constexpr bool kFixed = TC > 0 && TC % 2 == 0 && kPaintThreads % kPlane == 0 &&
                             TC % (kPaintThreads / kPlane) == 0;
@@ -759,16 +804,7 @@ __device__ __forceinline__ void flush_tile(const unsigned *lo, const unsigned *h
         const long long gstep = (long long)planes * N * pitch;
 #pragma unroll 2
         for (int k = 0; k < TC / planes; ++k, c += planes * TC * TC, dst += gstep) {
-            M2 v;
-            if (acc64) {
-                v.x = cell_value<M>(0u, 0u, acc64[c], sp, inv_scale);
-                v.y = cell_value<M>(0u, 0u, acc64[c + 1], sp, inv_scale);
-            } else {
-                const uint2 l2 = *reinterpret_cast<const uint2 *>(lo + c);
-                const uint2 h2 = hi ? *reinterpret_cast<const uint2 *>(hi + c) : make_uint2(0u, 0u);
-                v.x = cell_value<M>(l2.x, h2.x, 0ull, sp, inv_scale);
-                v.y = cell_value<M>(l2.y, h2.y, 0ull, sp, inv_scale);
-            }
+            M2 v = pair(c);
             M2 *d2 = reinterpret_cast<M2 *>(dst);
             if (accumulate) {
                 const M2 o = *d2;
@@ -786,16 +822,7 @@ __device__ __forceinline__ void flush_tile(const unsigned *lo, const unsigned *h
             const int cx = TC > 0 ? r / TC : r / T;
             const int cy = r - cx * T;
             const int c = r * T + cz;
-            M2 v;
-            if (acc64) {
-                v.x = cell_value<M>(0u, 0u, acc64[c], sp, inv_scale);
-                v.y = cell_value<M>(0u, 0u, acc64[c + 1], sp, inv_scale);
-            } else {
-                const uint2 l2 = *reinterpret_cast<const uint2 *>(lo + c);
-                const uint2 h2 = hi ? *reinterpret_cast<const uint2 *>(hi + c) : make_uint2(0u, 0u);
-                v.x = cell_value<M>(l2.x, h2.x, 0ull, sp, inv_scale);
-                v.y = cell_value<M>(l2.y, h2.y, 0ull, sp, inv_scale);
-            }
+            M2 v = pair(c);
             M2 *dst = reinterpret_cast<M2 *>(mb + ((long long)cx * N + cy) * pitch + cz);
             if (accumulate) {
                 const M2 o = *dst;
@@ -809,8 +836,7 @@ __device__ __forceinline__ void flush_tile(const unsigned *lo, const unsigned *h
         for (int c = threadIdx.x; c < n; c += blockDim.x) {
             const int r = c / T, cz = c - r * T;
             const int cx = r / T, cy = r - cx * T;
-            const M val = acc64 ? cell_value<M>(0u, 0u, acc64[c], sp, inv_scale)
-                                : cell_value<M>(lo[c], hi ? hi[c] : 0u, 0ull, sp, inv_scale);
+            const M val = cell(c);
             M *dst = mb + ((long long)cx * N + cy) * pitch + cz;
             if (accumulate) *dst += val;
             else *dst = val;
@@ -824,10 +850,10 @@ __device__ __forceinline__ void flush_tile(const unsigned *lo, const unsigned *h
 __host__ __device__ constexpr int paint_cell_words(int T) { return (2 * T * T * T + 3) & ~3; }
 
 // TC > 0: the tile edge is the compile-time constant TC (index math in shifts).
-template <int P, int NM, typename M, int TC>
+template <int P, int NM, typename M, int TC, bool UNIT>
 __global__ void __launch_bounds__(kPaintThreads)
 k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ off,
-              const uint32_t *__restrict__ cursor, int *__restrict__ err, PaintGeom g, int S, const unsigned *__restrict__ wmax_bits, float wmax_deposit, M *__restrict__ mesh,
+              const uint32_t *__restrict__ cursor, int *__restrict__ err, PaintGeom g, int S, const uint4 *__restrict__ wmaxs, float wdep, M *__restrict__ mesh,
               long long item_stride, long long mesh_stride, int accumulate) {
     extern __shared__ __align__(16) unsigned smu[];   // lo[T^3], hi[T^3] or acc64[T^3]; cand[kStage]
     __shared__ uint32_t s_beg[kSegments];
@@ -848,6 +874,7 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
     const int tz = (int)(t - tq * ntx);
     const int tx = (int)(tq / ntx);
     const int ty = (int)(tq - (unsigned)tx * ntx);
+    const uint4 wm = wmaxs[item];
 
     // Segments: neighbour offset d (per axis -1, 0, +1) with the classes of
     // that neighbour whose window reaches this tile: d = -1 -> class 2,
@@ -898,6 +925,111 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
     __syncthreads();
     const uint32_t total = s_pre[kSegments];
 
+    // Largest deposit of the tile's catalog in fixed-point units (wdep: the
+    // window's largest weight).
+    const float wmax = __uint_as_float(wm.x);
+    const float scale = pow2f(S);
+    const float inv_scale = pow2f(-S);
+    const float dmax = wmax * wdep * scale;
+    const long long pitch = 2LL * (g.N / 2 + 1);
+    M *base = mesh + item * item_stride;
+    const long long tile_off = ((long long)tx * T * g.N + (long long)ty * T) * pitch + (long long)tz * T;
+
+    // Sweep: cells of one word.  The tile is painted in one pass over its
+    // candidates, each read once straight from the sorted copy (nothing to
+    // stage), both interlaced meshes together (lo: mesh 0, hi: mesh 1).
+    // Unit weights: deposits below 2^23 whose sum cannot reach 2^32.  Other
+    // weights: the sum of the candidates' |W V| bounds every cell; it is taken
+    // during the sweep, and a tile whose cells might pass 2^31, or 2^32 where no
+    // W V is negative (S = 22: sum |W V| above 1022 for CIC, 2424 for TSC, 3451
+    // for PCS), is painted again the general way.  A tile that the catalog's
+    // mean |W V| says will not fit skips the sweep.
+    //
+    // Weighted catalogs used to stage their candidates and take one pass per
+    // mesh; unit weights needed deposits below the general path's 2^B, so at
+    // most 1024 candidates, and CIC never qualified.  1e7 log-normal objects,
+    // interlaced at 512^3, us: CIC 516 -> 444, weighted CIC 516 -> 438, TSC 985 ->
+    // 535, PCS 2604 -> 948; 1.3e8 at 1024^3, ms: CIC 5.8 -> 3.8, TSC 6.5 -> 5.5,
+    // PCS 20.9 -> 10.7, weighted CIC 5.7 -> 4.1, TSC 11.0 -> 5.7, PCS 29.4 -> 10.9.
+    const float ncf = (float)total;
+    bool sweep = UNIT ? dmax < 8388607.0f && ncf * (dmax + 1.0f) < 4.29e9f : dmax < 1.07e9f;
+    const bool sgn = !UNIT && wm.y != 0u;
+    const float cell_max = sgn ? 2.145e9f : 4.29e9f;      // 2^31, 2^32, less 1e-3 for rounding
+    if (!UNIT && ncf * __uint_as_float(wm.z) * wdep * scale > 0.9f * cell_max) sweep = false;
+    if (sweep) {
+        // TSC and PCS sweeps of 16^3 tiles deposit into the padded layout
+        // (SweepLayout); CIC keeps the compact one
+        constexpr bool kPadded = TC == 16 && (P == 4 || P == 3);
+        {
+            uint4 *z4 = reinterpret_cast<uint4 *>(smu);
+            const int nw = kPadded ? NM * SweepLayout<P>::Words : (NM == 1 ? T3 : 2 * T3);
+            const int n4 = nw / 4;
+            for (int c = threadIdx.x; c < n4; c += blockDim.x) z4[c] = make_uint4(0u, 0u, 0u, 0u);
+            for (int c = 4 * n4 + threadIdx.x; c < nw; c += blockDim.x) smu[c] = 0u;
+        }
+        __syncthreads();
+        float sum_abs = 0.0f;
+        if (kPadded) {
+            for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
+                const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
+                if (!UNIT) sum_abs += fabsf(v.w);
+                sweep_deposit<P, UNIT>(smu, v.x, v.y, v.z, v.w);
+                if (NM == 2)
+                    sweep_deposit<P, UNIT>(smu + SweepLayout<P>::Words, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
+            }
+        } else {
+            // the staging area is unused here: its first 32 words are the lanes' scratch
+            const unsigned trash = (unsigned)(2 * T3) + (threadIdx.x & 31);
+            const bool flat = total <= (uint32_t)kFlatMaxCand;
+            for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
+                const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
+                if (!UNIT) sum_abs += fabsf(v.w);
+                if (flat) {
+                    deposit_flat<P, TC, UNIT>(smu, 0, trash, T, v.x, v.y, v.z, v.w);
+                    if (NM == 2) deposit_flat<P, TC, UNIT>(smu, T3, trash, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
+                } else {
+                    const Split none{};
+                    deposit<P, 2, TC, UNIT>(lo, nullptr, nullptr, none, T, v.x, v.y, v.z, v.w);
+                    if (NM == 2)
+                        deposit<P, 2, TC, UNIT>(hi, nullptr, nullptr, none, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
+                }
+            }
+        }
+        bool fits = true;
+        if constexpr (UNIT) {
+            __syncthreads();
+        } else {
+            __shared__ float s_abs[kPaintThreads / 32];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum_abs += __shfl_down_sync(0xffffffffu, sum_abs, o);
+            if ((threadIdx.x & 31) == 0) s_abs[threadIdx.x >> 5] = sum_abs;
+            __syncthreads();
+            float t = 0.0f;
+#pragma unroll
+            for (int k = 0; k < kPaintThreads / 32; ++k) t += s_abs[k];
+            // every cell: sum of round(w W V 2^S) <= wdep sum |W V| 2^S + candidates / 2
+            fits = t * wdep + ncf < cell_max;
+        }
+        if (fits) {
+            const Split none{};
+            if (kPadded) {
+                sweep_flush<M, P, UNIT>(smu, sgn, inv_scale, base + tile_off, g.N, pitch, accumulate);
+                if (NM == 2)
+                    sweep_flush<M, P, UNIT>(smu + SweepLayout<P>::Words, sgn, inv_scale, base + mesh_stride + tile_off, g.N,
+                                            pitch, accumulate);
+            } else {
+                flush_tile<M, TC, UNIT>(lo, nullptr, nullptr, none, sgn, inv_scale, base + tile_off, T, g.N, pitch,
+                                        accumulate);
+                if (NM == 2)
+                    flush_tile<M, TC, UNIT>(hi, nullptr, nullptr, none, sgn, inv_scale, base + mesh_stride + tile_off, T,
+                                            g.N, pitch, accumulate);
+            }
+            return;
+        }
+        __syncthreads();                                  // s_abs read; the cells are zeroed again below
+    }
+
+    // General path: one mesh per pass over staged candidates.
     Split sp;
     {
         const unsigned nc = total > 0u ? total : 1u;
@@ -906,67 +1038,22 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
         sp.twoB_u = 1u << max(sp.B, 0);
         sp.inv2B = __uint_as_float((unsigned)(127 - max(sp.B, 0)) << 23);
         sp.hi_scale = pow2f(sp.B - S);
-        const float wmax = __uint_as_float(wmax_bits[item]);
         const float hmax = wmax * pow2f(S - sp.B);
         sp.fast = sp.B >= 1 && hmax < 4194304.0f && (float)nc * (hmax + 1.0f) < 2.0e9f;
-        // wmax_deposit > 0: all weights are in [0, wmax_deposit / max W]; then
-        // no deposit reaches 2^B if wmax_deposit 2^S < 2^B - 1
-        if (sp.fast && wmax_deposit > 0.0f && wmax_deposit * pow2f(S) < (float)(sp.twoB_u - 1u)) sp.fast = 2;
     }
-    const float scale = pow2f(S);
-    const float inv_scale = pow2f(-S);
-    // With no split needed (unit weights, sparse tile) the tile is painted in
-    // one sweep over its candidates, each read once straight from the sorted
-    // copy (nothing to stage), with branch-free deposits; an interlaced pair
-    // goes into lo (mesh 0) and hi (mesh 1) together.
-    const bool sweep = sp.fast == 2;
-    // TSC and PCS sweeps of 16^3 tiles deposit into the padded layout
-    // (SweepLayout); CIC keeps the compact one (its padded layout with even
-    // strides measured 0.69 against 0.54 ms)
-    const bool kPadded = sweep && TC == 16 && (P == 4 || P == 3);
     const bool staged_once = total <= (uint32_t)kStage;
-    if (staged_once && !sweep) stage_candidates(sorted, s_beg, s_pre, T, 0u, total, scale, cand);
-    const long long pitch = 2LL * (g.N / 2 + 1);
-    M *base = mesh + item * item_stride;
-
-    const int passes = sweep ? 1 : NM;
-    const long long tile_off = ((long long)tx * T * g.N + (long long)ty * T) * pitch + (long long)tz * T;
+    if (staged_once) stage_candidates(sorted, s_beg, s_pre, T, 0u, total, scale, cand);
 #pragma unroll 1
-    for (int m = 0; m < passes; ++m) {
+    for (int m = 0; m < NM; ++m) {
         {
             uint4 *z4 = reinterpret_cast<uint4 *>(smu);
-            const int nw = kPadded ? NM * SweepLayout<P>::Words
-                                   : ((sweep && NM == 1) ? T3 : 2 * T3);   // a single unsplit mesh uses lo only
-            const int n4 = nw / 4;
+            const int nw = 2 * T3, n4 = nw / 4;
             for (int c = threadIdx.x; c < n4; c += blockDim.x) z4[c] = make_uint4(0u, 0u, 0u, 0u);
             for (int c = 4 * n4 + threadIdx.x; c < nw; c += blockDim.x) smu[c] = 0u;
         }
         __syncthreads();
         const float sh = m ? 0.5f : 0.0f;
-        if (kPadded) {
-            // one-sweep deposits into the padded layout (SweepLayout), both meshes
-            for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
-                const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
-                sweep_deposit<P, false>(smu, v.x, v.y, v.z, v.w);
-                if (NM == 2)
-                    sweep_deposit<P, false>(smu + SweepLayout<P>::Words, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f,
-                                             v.w);
-            }
-        } else if (sweep) {
-            // the staging area is unused here: its first 32 words are the lanes' scratch
-            const unsigned trash = (unsigned)(2 * T3) + (threadIdx.x & 31);
-            const bool flat = total <= (uint32_t)kFlatMaxCand;
-            for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
-                const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
-                if (flat) {
-                    deposit_flat<P, TC>(smu, 0, trash, T, v.x, v.y, v.z, v.w);
-                    if (NM == 2) deposit_flat<P, TC>(smu, T3, trash, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
-                } else {
-                    deposit<P, 2, TC>(lo, nullptr, nullptr, sp, T, v.x, v.y, v.z, v.w);
-                    if (NM == 2) deposit<P, 2, TC>(hi, nullptr, nullptr, sp, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
-                }
-            }
-        } else if (staged_once) {
+        if (staged_once) {
             deposit_any<P, TC>(cand, total, lo, hi, acc64, sp, T, sh);
         } else {
             for (uint32_t k0 = 0; k0 < total; k0 += kStage) {     // dense tile: batches
@@ -978,20 +1065,8 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
             }
         }
         __syncthreads();
-        if (kPadded) {
-            sweep_flush<M, P>(smu, inv_scale, base + tile_off, g.N, pitch, accumulate);
-            if (NM == 2)
-                sweep_flush<M, P>(smu + SweepLayout<P>::Words, inv_scale, base + mesh_stride + tile_off, g.N, pitch,
-                                  accumulate);
-        } else if (sweep) {
-            flush_tile<M, TC>(lo, nullptr, nullptr, sp, inv_scale, base + tile_off, T, g.N, pitch, accumulate);
-            if (NM == 2)
-                flush_tile<M, TC>(hi, nullptr, nullptr, sp, inv_scale, base + mesh_stride + tile_off, T, g.N, pitch,
-                                  accumulate);
-        } else {
-            flush_tile<M, TC>(sp.fast ? lo : nullptr, sp.fast == 1 ? hi : nullptr, sp.fast ? nullptr : acc64, sp,
-                              inv_scale, base + m * mesh_stride + tile_off, T, g.N, pitch, accumulate);
-        }
+        flush_tile<M, TC, UNIT>(sp.fast ? lo : nullptr, sp.fast ? hi : nullptr, sp.fast ? nullptr : acc64, sp, false,
+                                inv_scale, base + m * mesh_stride + tile_off, T, g.N, pitch, accumulate);
         __syncthreads();
     }
 }
@@ -1048,7 +1123,7 @@ __global__ void __launch_bounds__(kCountThreads)
 k_paint_atomic(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
                const int64_t *__restrict__ item_off, PaintGeom g, int S, bool weighted,
                unsigned long long *__restrict__ acc, double *__restrict__ wsums,
-               double *__restrict__ wpart, unsigned *__restrict__ wmax) {
+               double *__restrict__ wpart, uint4 *__restrict__ wmax) {
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
     const int64_t beg = item_off[item], end = item_off[item + 1];
@@ -1057,6 +1132,7 @@ k_paint_atomic(const void *__restrict__ pos, const float *__restrict__ w, const 
     const float scale = ldexpf(1.0f, S);
     double sw = 0.0, sw2 = 0.0, swa = 0.0;
     float mw = 0.0f;
+    bool neg = false;
     for (int64_t i = beg + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end;
          i += (int64_t)gridDim.x * blockDim.x) {
         const Obj<R> o = load_obj<DT>(pos, w, vals, i, g);
@@ -1076,9 +1152,10 @@ k_paint_atomic(const void *__restrict__ pos, const float *__restrict__ w, const 
             sw2 += ad * ad;
             swa += fabs(ad);
             mw = fmaxf(mw, fabsf(o.a));
+            neg |= o.a < 0.0f;
         }
     }
-    flush_wsums(sw, sw2, swa, mw, weighted, item, end - beg, wsums, wpart, wmax);
+    flush_wsums(sw, sw2, swa, mw, neg, weighted, item, end - beg, wsums, wpart, wmax);
 }
 
 template <typename M>
@@ -1534,7 +1611,7 @@ int paint_classes() { return kClasses; }
 
 cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const float *vals,
                               const int64_t *item_off, int nitems, int64_t max_n, const PaintGeom &g,
-                              uint32_t *count, double *wsums, double *wpart, unsigned *wmax, cudaStream_t st) {
+                              uint32_t *count, double *wsums, double *wpart, uint4 *wmax, cudaStream_t st) {
     const bool weighted = w != nullptr || vals != nullptr || dtype == PK_F32X4;
     dim3 grid(grid_for(max_n, kCountThreads, weighted ? kWsumBlocks : 1u << 20), nitems);
 #define PK_COUNT(DT)                                                                                    \
@@ -1549,7 +1626,7 @@ cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const 
     if (weighted) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, wsums);
+        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, wsums, wmax);
     }
     return cudaGetLastError();
 }
@@ -1601,20 +1678,20 @@ size_t scan_tmp_elems(int64_t n) {
     return t + 2;
 }
 
-template <typename T>
+template <typename T, bool COPY>
 static cudaError_t scan_impl(const T *in, int64_t n, T *out, T *tmp, T *copy, int *launches, cudaStream_t st) {
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb <= 1) {
-        k_scan_blocks<T><<<1, kScanThreads, 0, st>>>(in, n, out, out + n, copy);
+        k_scan_blocks<T, COPY><<<1, kScanThreads, 0, st>>>(in, n, out, out + n, copy);
         *launches += 1;
         return cudaGetLastError();
     }
     if (nb > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_scan_blocks<T><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, out, tmp, nullptr);
+    k_scan_blocks<T, false><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, out, tmp, nullptr);
     *launches += 1;
-    cudaError_t e = scan_impl<T>(tmp, nb, tmp, tmp + nb + 1, nullptr, launches, st);
+    cudaError_t e = scan_impl<T, false>(tmp, nb, tmp, tmp + nb + 1, nullptr, launches, st);
     if (e != cudaSuccess) return e;
-    k_scan_add<T><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
+    k_scan_add<T, COPY><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -1622,12 +1699,12 @@ static cudaError_t scan_impl(const T *in, int64_t n, T *out, T *tmp, T *copy, in
 // out[0 .. n) = exclusive scan of in, out[n] = total; in[0 .. n) gets a copy of
 // out[0 .. n).  tmp: scan_tmp_elems(n).
 cudaError_t launch_scan(uint32_t *in, int64_t n, uint32_t *out, uint32_t *tmp, int *launches, cudaStream_t st) {
-    return scan_impl<uint32_t>(in, n, out, tmp, in, launches, st);
+    return scan_impl<uint32_t, true>(in, n, out, tmp, in, launches, st);
 }
 
 cudaError_t launch_scan64(const unsigned long long *in, int64_t n, unsigned long long *out,
                           unsigned long long *tmp, int *launches, cudaStream_t st) {
-    return scan_impl<unsigned long long>(in, n, out, tmp, nullptr, launches, st);
+    return scan_impl<unsigned long long, false>(in, n, out, tmp, nullptr, launches, st);
 }
 
 size_t paint_smem_bytes(int T, int window, int nmesh) {
@@ -1638,19 +1715,18 @@ size_t paint_smem_bytes(int T, int window, int nmesh) {
     return general > padded ? general : padded;
 }
 
-template <int P, int NM, typename M>
+template <int P, int NM, typename M, bool UNIT>
 static cudaError_t paint_inst(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *err, int nitems,
-                              const PaintGeom &g, int S, const unsigned *wmax, float wmax_deposit,
-                              void *mesh, long long item_stride, long long mesh_stride, int accumulate,
+                              const PaintGeom &g, int S, const uint4 *wmax, float wdep, void *mesh, long long item_stride, long long mesh_stride, int accumulate,
                               cudaStream_t st) {
     const size_t smem = paint_smem_bytes(g.T, P, NM);   // one padded mesh fits the general area
     const long long nblocks = (long long)nitems * g.ntiles;
     if (nblocks <= 0) return cudaSuccess;
     if (nblocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    auto kern = g.T == 16 ? k_paint_tiles<P, NM, M, 16> : k_paint_tiles<P, NM, M, 0>;
+    auto kern = g.T == 16 ? k_paint_tiles<P, NM, M, 16, UNIT> : k_paint_tiles<P, NM, M, 0, UNIT>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)nblocks, kPaintThreads, smem, st>>>(sorted, off, cursor, err, g, S, wmax, wmax_deposit,
+    kern<<<(unsigned)nblocks, kPaintThreads, smem, st>>>(sorted, off, cursor, err, g, S, wmax, wdep,
                                                          reinterpret_cast<M *>(mesh), item_stride,
                                                          mesh_stride, accumulate);
     return cudaGetLastError();
@@ -1658,33 +1734,32 @@ static cudaError_t paint_inst(const float4 *sorted, const uint32_t *off, const u
 
 cudaError_t launch_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *err,
                                int nitems, const PaintGeom &g, int window, int nmesh, int S, int f64,
-                               const unsigned *wmax, int unit_weights, void *mesh,
-                               long long item_stride, long long mesh_stride, int accumulate,
-                               cudaStream_t st) {
-    // Largest single deposit w W with unit weights: max W = (max per-axis weight)^3.
-    const float wdep = !unit_weights ? 0.0f : (window == 2 ? 1.0f : window == 3 ? 0.421875f : 0.2962963f);
-#define PK_PAINT_CASE(P)                                                                              \
-    if (window == P) {                                                                                \
-        if (f64) return nmesh == 2 ? paint_inst<P, 2, double>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh, \
-                                                              item_stride, mesh_stride, accumulate, st) \
-                                   : paint_inst<P, 1, double>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh, \
-                                                              item_stride, mesh_stride, accumulate, st); \
-        return nmesh == 2 ? paint_inst<P, 2, float>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh,     \
-                                                    item_stride, mesh_stride, accumulate, st)         \
-                          : paint_inst<P, 1, float>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh,     \
-                                                    item_stride, mesh_stride, accumulate, st);        \
+                               const uint4 *wmax, int unit_weights, void *mesh, long long item_stride, long long mesh_stride,
+                               int accumulate, cudaStream_t st) {
+    // The window's largest weight: (largest per-axis weight)^3.
+    const float wdep = window == 2 ? 1.0f : window == 3 ? 0.421875f : 0.2962963f;
+#define PK_PAINT_INST(P, NM, M)                                                                                  \
+    (unit_weights ? paint_inst<P, NM, M, true>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh, \
+                                               item_stride, mesh_stride, accumulate, st)                          \
+                  : paint_inst<P, NM, M, false>(sorted, off, cursor, err, nitems, g, S, wmax, wdep, mesh, \
+                                                item_stride, mesh_stride, accumulate, st))
+#define PK_PAINT_CASE(P)                                                                                         \
+    if (window == P) {                                                                                           \
+        if (f64) return nmesh == 2 ? PK_PAINT_INST(P, 2, double) : PK_PAINT_INST(P, 1, double);                  \
+        return nmesh == 2 ? PK_PAINT_INST(P, 2, float) : PK_PAINT_INST(P, 1, float);                             \
     }
     PK_PAINT_CASE(2)
     PK_PAINT_CASE(3)
     PK_PAINT_CASE(4)
 #undef PK_PAINT_CASE
+#undef PK_PAINT_INST
     return cudaErrorInvalidValue;
 }
 
 template <int DT, int P, int NM>
 static cudaError_t atomic_inst(const void *pos, const float *w, const float *vals, const int64_t *item_off, int nitems,
                                int64_t max_n, const PaintGeom &g, int S, bool weighted,
-                               unsigned long long *acc, double *wsums, double *wpart, unsigned *wmax,
+                               unsigned long long *acc, double *wsums, double *wpart, uint4 *wmax,
                                cudaStream_t st) {
     dim3 grid(grid_for(max_n, kCountThreads, weighted ? kWsumBlocks : 1u << 20), nitems);
     k_paint_atomic<DT, P, NM><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, S, weighted, acc,
@@ -1692,7 +1767,7 @@ static cudaError_t atomic_inst(const void *pos, const float *w, const float *val
     if (weighted) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, wsums);
+        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, wsums, wmax);
     }
     return cudaGetLastError();
 }
@@ -1701,7 +1776,7 @@ template <int DT>
 static cudaError_t atomic_dispatch(const void *pos, const float *w, const float *vals, const int64_t *item_off, int nitems,
                                    int64_t max_n, const PaintGeom &g, int window, int nmesh, int S,
                                    bool weighted, unsigned long long *acc, double *wsums, double *wpart,
-                                   unsigned *wmax, cudaStream_t st) {
+                                   uint4 *wmax, cudaStream_t st) {
 #define PK_ATOMIC_CASE(P)                                                                              \
     if (window == P)                                                                                   \
         return nmesh == 2 ? atomic_inst<DT, P, 2>(pos, w, vals, item_off, nitems, max_n, g, S, weighted, acc, \
@@ -1718,7 +1793,7 @@ static cudaError_t atomic_dispatch(const void *pos, const float *w, const float 
 cudaError_t launch_paint_atomic(const void *pos, int dtype, const float *w, const float *vals,
                                 const int64_t *item_off, int nitems, int64_t max_n, const PaintGeom &g,
                                 int window, int nmesh, int S, unsigned long long *acc, double *wsums,
-                                double *wpart, unsigned *wmax, cudaStream_t st) {
+                                double *wpart, uint4 *wmax, cudaStream_t st) {
     const bool weighted = w != nullptr || vals != nullptr || dtype == PK_F32X4;
     switch (dtype) {
     case PK_F32:
