@@ -431,6 +431,7 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
 
     // ---- own transform: FP32 meshes of the sizes it has kernels for ----
     if (!P->f64) P->zyx = zyx_ops(P->N);
+    if (P->zyx && !P->zyx->plan_default()) P->zyx = nullptr;
     if (!P->f64 && (P->zyx || own_fft_packed(P->N))) {
         std::vector<float> tw(2 * (size_t)P->N);
         own_fft_twiddles(P->N, tw.data());

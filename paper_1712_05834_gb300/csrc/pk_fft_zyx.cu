@@ -47,6 +47,7 @@
 #include <algorithm>
 
 #include "pk_internal.h"
+#include "pk_ylm.h"
 
 namespace pk {
 
@@ -234,7 +235,8 @@ __device__ __forceinline__ int dif_freq(int p) {
     }
 }
 
-// Shapes per mesh size.  T threads of k_fft_zy (CTAS per SM, 64 registers a
+// Shapes per mesh size (128, 192, 256 and 512 serve the survey transforms; box
+// spectra of these sizes take the packed form of pk_fft.cu).  T threads of k_fft_zy (CTAS per SM, 64 registers a
 // thread), NBY columns per y tile, TX threads of the x kernels (CTASX per SM), NX
 // columns per x tile.  About 12 to 16 complex values per thread.  At N = 2048
 // and 1024 the x tiles take 128 KB and one CTA of 1024 threads, since their runs
@@ -248,6 +250,10 @@ template <int T_, int CTAS_, int NBY_, int TX_, int CTASX_, int NX_, int LAG_>
 struct ShapeOf {
     static constexpr int T = T_, CTAS = CTAS_, NBY = NBY_, TX = TX_, CTASX = CTASX_, NX = NX_, LAG = LAG_;
 };
+template <> struct Shape<128> : ShapeOf<256, 4, 32, 256, 4, 16, 32> {};
+template <> struct Shape<192> : ShapeOf<384, 2, 16, 384, 2, 16, 32> {};
+template <> struct Shape<256> : ShapeOf<512, 2, 32, 512, 2, 16, 32> {};
+template <> struct Shape<512> : ShapeOf<512, 2, 16, 512, 2, 16, 24> {};
 template <> struct Shape<320> : ShapeOf<256, 4, 8, 320, 2, 16, 32> {};
 template <> struct Shape<384> : ShapeOf<384, 2, 8, 384, 2, 16, 32> {};
 template <> struct Shape<400> : ShapeOf<320, 3, 8, 320, 3, 8, 32> {};
@@ -265,7 +271,7 @@ struct Cfg : Shape<N> {
     static constexpr int M = N / 2, Nh = M + 1;
     // z rows: NT threads share NR rows of M complex (about 16 per thread)
     static constexpr int NT = M >= 1024 ? 64 : 32;
-    static constexpr int NR = M > 256 ? 1 : 2;
+    static constexpr int NR = M > 256 ? 1 : M > 128 ? 2 : M > 64 ? 4 : 8;
     static constexpr int RS = (M & (M - 1)) == 0 ? M : M + 16;   // shared slots per row
     static constexpr int GROUPS = Shape<N>::T / NT;              // row groups per CTA (named barriers 1 .. GROUPS)
     static constexpr int RPI = GROUPS * NR;                      // rows per z item
@@ -430,11 +436,11 @@ __device__ __forceinline__ void row_sync(int grp) {
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(NT) : "memory");
 }
 
-// One step over blocks of S points of the FFTs of rows [0, nrow) (FIRST: read
-// from g, rows gs complex apart).  The last step writes in natural order.
-template <int M, int NR, int NT, int RS, int S, bool FIRST>
-__device__ __forceinline__ void zrow_step(float2 *rows, const float2 *g, long long gs, int nrow, const float2 *ztw,
-                                          int lane, int grp) {
+// One step over blocks of S points of the FFTs of rows [0, nrow) (FIRST: values
+// from ld(row, position)).  The last step writes in natural order.
+template <int M, int NR, int NT, int RS, int S, bool FIRST, typename Ld>
+__device__ __forceinline__ void zrow_step(float2 *rows, const Ld &ld, int nrow, const float2 *ztw, int lane,
+                                          int grp) {
     constexpr int R = zradix_of(S), Q = S / R;
     constexpr int BPR = M / R;                    // butterflies per row
     constexpr int TOT = NR * BPR;
@@ -450,9 +456,8 @@ __device__ __forceinline__ void zrow_step(float2 *rows, const float2 *g, long lo
         if ((TOT % NT == 0 || beta < TOT) && r < nrow) {
             const int base = (b / Q) * S + b % Q;
             if (FIRST) {
-                const float2 *src = g + r * gs + base;
 #pragma unroll
-                for (int j = 0; j < R; ++j) v[HOLD ? s : 0][j] = __ldcs(src + Q * j);
+                for (int j = 0; j < R; ++j) v[HOLD ? s : 0][j] = ld(r, base + Q * j);
             } else {
 #pragma unroll
                 for (int j = 0; j < R; ++j) v[HOLD ? s : 0][j] = rows[r * RS + zslot_at<POW2>(zslot(base), base, Q * j)];
@@ -496,7 +501,7 @@ __device__ __forceinline__ void zrow_step(float2 *rows, const float2 *g, long lo
         }
     }
     row_sync<NT>(grp);
-    if constexpr (Q > 1) zrow_step<M, NR, NT, RS, Q, false>(rows, g, gs, nrow, ztw, lane, grp);
+    if constexpr (Q > 1) zrow_step<M, NR, NT, RS, Q, false>(rows, ld, nrow, ztw, lane, grp);
 }
 
 // D[l] and D[M-l] from u = C[l], v = C[M-l] and w = W_N^l: with s = u + conj v
@@ -517,12 +522,39 @@ __device__ __forceinline__ void split_real(float2 u, float2 v, float2 w, float2 
 // (about a second) only bounds it if that were ever wrong.
 constexpr int kMaxPolls = 1 << 20;
 
+// Y_lm(x^) along a z row as a polynomial in z: Y = (c[0] + c[1] z + .. + c[4] z^4)
+// / r^l with r^2 = x^2 + y^2 + z^2; slots 0..4: l = 2, m = slot - 2, 5..13: l = 4,
+// m = slot - 9 (the polynomials of ylm_slot in pk_survey.cu, r^2 put in).
+__device__ __forceinline__ void ylm_row(int slot, float x, float y, float *c) {
+    const float x2 = x * x, y2 = y * y, rho = x2 + y2, d = x2 - y2, xy = x * y;
+    c[0] = c[1] = c[2] = c[3] = c[4] = 0.0f;
+    switch (slot) {
+    case 0: c[0] = (float)kYa * xy; break;
+    case 1: c[1] = (float)kYa * y; break;
+    case 2: c[0] = -(float)kYb * rho; c[2] = 2.0f * (float)kYb; break;
+    case 3: c[1] = (float)kYa * x; break;
+    case 4: c[0] = (float)kYc * d; break;
+    case 5: c[0] = (float)kYd * xy * d; break;
+    case 6: c[1] = (float)kYe * y * (3.0f * x2 - y2); break;
+    case 7: c[0] = -(float)kYf * xy * rho; c[2] = 6.0f * (float)kYf * xy; break;
+    case 8: c[1] = -3.0f * (float)kYg * y * rho; c[3] = 4.0f * (float)kYg * y; break;
+    case 9: c[0] = 3.0f * (float)kYh * rho * rho; c[2] = -24.0f * (float)kYh * rho; c[4] = 8.0f * (float)kYh; break;
+    case 10: c[1] = -3.0f * (float)kYg * x * rho; c[3] = 4.0f * (float)kYg * x; break;
+    case 11: c[0] = -(float)kYi * d * rho; c[2] = 6.0f * (float)kYi * d; break;
+    case 12: c[1] = (float)kYe * x * (x2 - 3.0f * y2); break;
+    case 13: c[0] = (float)kYj * (x2 * (x2 - 3.0f * y2) - y2 * (3.0f * x2 - y2)); break;
+    }
+}
+
 // sync[0]: next ticket; sync[1 + p]: z items done in plane p.  Zero at launch;
 // the kernel that takes the x axis clears them again.  err: 4 if a wait gave up.
-template <int N>
+// SURVEY: plane p is x plane p / nslot of slot s0 + p % nslot (so the slots
+// of a plane read their source rows from L2), whose rows are formed on the way
+// in: the field D - alpha R times Y_lm(x^) of the slot (slot -1: 1).
+template <int N, bool SURVEY>
 __global__ void __launch_bounds__(Cfg<N>::T, Cfg<N>::CTAS)
-k_fft_zy(float2 *__restrict__ mesh, int planes, int ncol, int mcut, const float2 *__restrict__ twg,
-         unsigned *__restrict__ sync, int *__restrict__ err) {
+k_fft_zy(float2 *mesh, int planes, int ncol, int mcut, const float2 *__restrict__ twg, unsigned *__restrict__ sync,
+         int *__restrict__ err, SurveyRows sv) {
     using K = Cfg<N>;
     constexpr int M = K::M, Nh = K::Nh, T = K::T, NBY = K::NBY, LAG = K::LAG;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -536,6 +568,12 @@ k_fft_zy(float2 *__restrict__ mesh, int planes, int ncol, int mcut, const float2
     const unsigned per = K::ZI + ytiles;
     const unsigned total = (unsigned)(planes + LAG) * per;
     const long long plane_c = (long long)N * Nh;
+    const float alpha = SURVEY && sv.R ? (float)sv.alpha[0] : 0.0f;
+    const auto plane_at = [&](int p) -> float2 * {
+        if constexpr (!SURVEY) return mesh + (long long)p * plane_c;
+        const int i = p / sv.nslot;
+        return mesh + (long long)(p - i * sv.nslot) * sv.slot_c + (long long)i * plane_c;
+    };
     unsigned next = threadIdx.x == 0 ? atomicAdd(sync, 1u) : 0u;
     for (;;) {
         __syncthreads();                        // the previous item is done with buf and s_ticket
@@ -551,10 +589,47 @@ k_fft_zy(float2 *__restrict__ mesh, int planes, int ncol, int mcut, const float2
             const int lane = threadIdx.x % K::NT, grp = threadIdx.x / K::NT;
             const int row0 = (int)idx * K::RPI + grp * K::NR;
             const int nrow = grp < K::GROUPS ? min(K::NR, N - row0) : 0;
-            float2 *g = mesh + (long long)step * plane_c + (long long)row0 * Nh;
+            float2 *g = plane_at(step) + (long long)row0 * Nh;
             if (nrow > 0) {
                 float2 *rows = buf + (size_t)grp * K::NR * K::RS;
-                zrow_step<M, K::NR, K::NT, K::RS, M, true>(rows, g, Nh, nrow, ztw, lane, grp);
+                if constexpr (!SURVEY) {
+                    const auto ld = [&](int r, int p) { return __ldcs(g + (long long)r * Nh + p); };
+                    zrow_step<M, K::NR, K::NT, K::RS, M, true>(rows, ld, nrow, ztw, lane, grp);
+                } else {
+                    const int i = step / sv.nslot, slot = sv.s0 + step - i * sv.nslot;
+                    const long long at = (long long)i * plane_c + (long long)row0 * Nh;
+                    const float2 *D = reinterpret_cast<const float2 *>(sv.D) + at;
+                    const float2 *Rm = sv.R ? reinterpret_cast<const float2 *>(sv.R) + at : nullptr;
+                    const float x = sv.ox + (float)i * sv.H;
+                    float c[K::NR][5], rho[K::NR];
+#pragma unroll
+                    for (int r = 0; r < K::NR; ++r) {
+                        const float y = sv.oy + (float)(row0 + r) * sv.H;
+                        rho[r] = x * x + y * y;
+                        ylm_row(slot, x, y, c[r]);
+                    }
+                    const auto weight = [&](int r, int k) {       // Y_lm at z node k of the row
+                        const float z = sv.oz + (float)k * sv.H, r2 = rho[r] + z * z;
+                        const float ir = r2 > 0.0f ? rsqrtf(r2) : 0.0f;   // 0: the observer's node
+                        float inv = ir * ir;
+                        if (slot >= 5) inv *= inv;
+                        return (c[r][0] + z * (c[r][1] + z * (c[r][2] + z * (c[r][3] + z * c[r][4])))) * inv;
+                    };
+                    const auto ld = [&](int r, int p) {
+                        float2 f = __ldcg(D + (long long)r * Nh + p);
+                        if (Rm) {
+                            const float2 q = __ldcg(Rm + (long long)r * Nh + p);
+                            f.x -= alpha * q.x;
+                            f.y -= alpha * q.y;
+                        }
+                        if (slot >= 0) {
+                            f.x *= weight(K::NR == 1 ? 0 : r, 2 * p);
+                            f.y *= weight(K::NR == 1 ? 0 : r, 2 * p + 1);
+                        }
+                        return f;
+                    };
+                    zrow_step<M, K::NR, K::NT, K::RS, M, true>(rows, ld, nrow, ztw, lane, grp);
+                }
                 for (int r = 0; r < nrow; ++r) {
                     const float2 *C = rows + r * K::RS;
                     float2 *d = g + (long long)r * Nh;
@@ -586,7 +661,7 @@ k_fft_zy(float2 *__restrict__ mesh, int planes, int ncol, int mcut, const float2
             }
             __syncthreads();
             const int c0 = (int)(idx - K::ZI) * NBY;
-            float2 *g = mesh + (long long)plane * plane_c + c0;
+            float2 *g = plane_at(plane) + c0;
             const int nc = ncol - c0;           // valid columns of the tile
             const auto ld = [&](int r, int c) {
                 return c < nc ? __ldcg(g + (long long)r * Nh + c) : make_float2(0.0f, 0.0f);
@@ -803,17 +878,17 @@ cudaError_t allow_smem(F kern, size_t bytes) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <int N>
+template <int N, bool SURVEY>
 cudaError_t zy_inst(float2 *mesh, int planes, int ncol, int mcut, const float2 *tw, unsigned *sync, int *err, int nsm,
-                    cudaStream_t st) {
+                    const SurveyRows &sv, cudaStream_t st) {
     using K = Cfg<N>;
     constexpr size_t smem = zy_smem<N>();
-    cudaError_t e = allow_smem(k_fft_zy<N>, smem);
+    cudaError_t e = allow_smem(k_fft_zy<N, SURVEY>, smem);
     if (e != cudaSuccess) return e;
     const long long items = (long long)(planes + K::LAG) * (K::ZI + (ncol + K::NBY - 1) / K::NBY);
     if (items > 0x7fffffffLL) return cudaErrorInvalidValue;
     const unsigned grid = (unsigned)std::min<long long>((long long)nsm * K::CTAS, items);
-    k_fft_zy<N><<<grid, K::T, smem, st>>>(mesh, planes, ncol, mcut, tw, sync, err);
+    k_fft_zy<N, SURVEY><<<grid, K::T, smem, st>>>(mesh, planes, ncol, mcut, tw, sync, err, sv);
     return cudaGetLastError();
 }
 
@@ -888,9 +963,15 @@ struct OpsOf final : ZyxOps {
     int tile_columns(int interlaced) const override { return interlaced ? Cfg<N>::NX / 2 : Cfg<N>::NX; }
     cudaError_t zy(void *mesh, int planes, int ncol, int mcut, const void *tw, unsigned *sync, int *err, int nsm,
                    cudaStream_t st) const override {
-        return zy_inst<N>(reinterpret_cast<float2 *>(mesh), planes, ncol, mcut, reinterpret_cast<const float2 *>(tw),
-                          sync, err, nsm, st);
+        return zy_inst<N, false>(reinterpret_cast<float2 *>(mesh), planes, ncol, mcut,
+                                 reinterpret_cast<const float2 *>(tw), sync, err, nsm, SurveyRows{}, st);
     }
+    cudaError_t zy_survey(void *mesh, int nx, const SurveyRows &sv, int ncol, int mcut, const void *tw, unsigned *sync,
+                          int *err, int nsm, cudaStream_t st) const override {
+        return zy_inst<N, true>(reinterpret_cast<float2 *>(mesh), nx * sv.nslot, ncol, mcut,
+                                reinterpret_cast<const float2 *>(tw), sync, err, nsm, sv, st);
+    }
+    bool plan_default() const override { return N != 128 && N != 192 && N != 256 && N != 512; }
     cudaError_t x(void *mesh, int nmesh, long long mesh_c, int ncol, int mcut, const int *tiles, int ntiles,
                   const void *tw, unsigned *sync, int nsync, cudaStream_t st) const override {
         return x_inst<N>(reinterpret_cast<float2 *>(mesh), nmesh, mesh_c, ncol, mcut, tiles, ntiles,
@@ -939,6 +1020,10 @@ const ZyxOps *PK_ZYX_NAME(PK_ZYX_GROUP)(int N) {
     case 768: return ops_of<768>();
     case 800: return ops_of<800>();
 #elif PK_ZYX_GROUP == 1
+    case 128: return ops_of<128>();
+    case 192: return ops_of<192>();
+    case 256: return ops_of<256>();
+    case 512: return ops_of<512>();
     case 1024: return ops_of<1024>();
 #else
     case 2048: return ops_of<2048>();

@@ -145,7 +145,20 @@ cudaError_t launch_zfinish(void *mesh, int interlaced, long long item_stride_c, 
                            int nitems, int N, const void *tw, int nsm, cudaStream_t st);
 
 // ---- own FFT path (pk_fft_zyx.cu): z and y axes in one pass, then x ----
+// Rows of a survey field formed on the way into the z axis: (D - alpha R) Y_lm(x^).
+struct SurveyRows {
+    const void *D = nullptr, *R = nullptr;     // real meshes in the r2c row layout; R may be NULL
+    const double *alpha = nullptr;             // device: the factor of R
+    long long slot_c = 0;                      // complex elements between the slots' meshes
+    int s0 = -1, nslot = 1;                    // Y_lm slots s0 .. s0 + nslot - 1 (-1: weight 1)
+    float ox = 0, oy = 0, oz = 0, H = 0;       // node (i, j, k) at o + H (i, j, k), in any unit near the box edge
+};
 struct ZyxOps {
+    virtual bool plan_default() const = 0;     // box spectra of this size use it
+    // zy into mesh, the first of sv.nslot meshes, of the rows described by sv, nx x
+    // planes each; sync: 1 + nx * nslot counters.
+    virtual cudaError_t zy_survey(void *mesh, int nx, const SurveyRows &sv, int ncol, int mcut, const void *tw,
+                                  unsigned *sync, int *err, int nsm, cudaStream_t st) const = 0;
     // Columns l of one x tile (per mesh) of the fused bin pass; tile lists hold
     // ky index * 65536 + column block for the tiles with a mode m < mhi.
     virtual int tile_columns(int interlaced) const = 0;

@@ -34,6 +34,7 @@
 
 #include "pk_internal.h"
 #include "pk_plan.h"
+#include "pk_ylm.h"
 
 #ifndef M_PI
 #define M_PI 3.14159265358979323846
@@ -55,16 +56,7 @@ constexpr int kConst = 16;              // constants block: see k_survey_const
 // polynomials in x, y, z, with N_lm from (2l + 1)/(4 pi) (l - |m|)!/(l + |m|)!
 // (times 2 for m != 0).  Slot s: 0..4 -> l = 2, m = s - 2; 5..13 -> l = 4,
 // m = s - 9.
-constexpr double kYa = 1.0925484305920792;    // (1/2) sqrt(15/pi)
-constexpr double kYb = 0.31539156525252005;   // (1/4) sqrt(5/pi)
-constexpr double kYc = 0.5462742152960396;    // (1/4) sqrt(15/pi)
-constexpr double kYd = 2.5033429417967046;    // (3/4) sqrt(35/pi)
-constexpr double kYe = 1.7701307697799304;    // (3/4) sqrt(35/(2 pi))
-constexpr double kYf = 0.9461746957575601;    // (3/4) sqrt(5/pi)
-constexpr double kYg = 0.6690465435572892;    // (3/4) sqrt(5/(2 pi))
-constexpr double kYh = 0.10578554691520431;   // (3/16) sqrt(1/pi)
-constexpr double kYi = 0.47308734787878004;   // (3/8) sqrt(5/pi)
-constexpr double kYj = 0.6258357354491761;    // (3/16) sqrt(35/pi)
+using pk::kYa, pk::kYb, pk::kYc, pk::kYd, pk::kYe, pk::kYf, pk::kYg, pk::kYh, pk::kYi, pk::kYj;
 
 template <typename T>
 __host__ __device__ __forceinline__ T ylm_slot(int s, T x, T y, T z) {
@@ -270,7 +262,7 @@ k_survey_prep(const P *__restrict__ pos, long long n, const float *__restrict__ 
 
 // Constants block c[kConst]: 0 alpha, 1 norm I, 2 shot S, 3 wsum_d, 4 wsum_r,
 // 5 w2_d, 6 w2_r, 7 nsum_r, 8 nsum_d, 9 outside_d, 10 outside_r,
-// 11 rejected_d, 12 rejected_r.  Fixed-order sums of the per-CTA rows.
+// 11 rejected_d, 12 rejected_r; in the result 15: internal error flags.  Fixed-order sums of the per-CTA rows.
 __global__ void k_survey_const(const double *__restrict__ pd, int gd, const double *__restrict__ pr, int gr,
                                double *__restrict__ c) {
     __shared__ double s[2][kSums];
@@ -552,7 +544,8 @@ k_survey_bin(const C *__restrict__ A0, const C *__restrict__ S, long long stride
 // rows not in the mask and empty bins NaN; res[3 nk ..] = the constants block.
 __global__ void k_survey_final(const double *__restrict__ partial, int G, int nk,
                                const unsigned long long *__restrict__ modes, const double *__restrict__ c,
-                               unsigned mask, int subtract_shot, double *__restrict__ res) {
+                               unsigned mask, int subtract_shot, const int *__restrict__ err,
+                               double *__restrict__ res) {
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 3 * nk; k += gridDim.x * blockDim.x) {
         const int row = k / nk, b = k - row * nk;
@@ -569,7 +562,8 @@ __global__ void k_survey_final(const double *__restrict__ partial, int G, int nk
         }
         res[k] = p;
     }
-    if (blockIdx.x == 0 && threadIdx.x < kConst) res[3 * nk + threadIdx.x] = c[threadIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x < kConst)
+        res[3 * nk + threadIdx.x] = threadIdx.x == kConst - 1 ? (double)(*err & 6) : c[threadIdx.x];
 }
 
 }  // namespace
@@ -587,6 +581,13 @@ struct pk_survey_s {
     int batch = 0;                  // Y_lm-weighted meshes resident per pass
     void *a0 = nullptr;             // A_0: one mesh (complex half grid)
     void *slots = nullptr;          // batch meshes
+    // Own transforms (FP32, sizes of pk_fft_zyx.cu): NULL = cuFFT for all.
+    const pk::ZyxOps *zyx = nullptr;
+    void *tw = nullptr;             // W_N^e, e < N (float2)
+    unsigned *sync = nullptr;       // work counters of the z / y pass
+    int nsync = 0, ncol = 0;        // columns l that hold a binned mode
+    int *xtiles = nullptr;          // x tiles: those with a binned mode, then all
+    int nx_bin = 0, nx_all = 0;
     cufftHandle fft_b = 0, fft_inv = 0;   // single-mesh r2c, single-mesh c2r
     int have_b = 0, have_inv = 0;
     void *fft_work = nullptr;
@@ -671,7 +672,8 @@ void free_survey(pk_survey_s *S) {
     if (S->st || S->P) cudaStreamSynchronize(S->st);
     if (S->have_b) cufftDestroy(S->fft_b);
     if (S->have_inv) cufftDestroy(S->fft_inv);
-    void *dev[] = {S->a0, S->slots, S->fft_work, S->obj, S->stage, S->chi, S->psum, S->cst, S->partial, S->res};
+    void *dev[] = {S->a0, S->slots, S->fft_work, S->obj, S->stage, S->chi, S->psum, S->cst, S->partial, S->res, S->tw, S->sync,
+                   S->xtiles};
     for (void *d : dev)
         if (d) cudaFree(d);
     if (S->h_res) cudaFreeHost(S->h_res);
@@ -814,8 +816,35 @@ static pk_status survey_build(pk_survey_s *S, const pk_survey_config *cfg, void 
         SV_CUDA(S, cudaMemcpy(S->chi, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
     }
 
+    // ---- own transforms ----
+    if (!S->f64) S->zyx = pk::zyx_ops(S->N);
+    if (S->zyx) {
+        const int N = S->N;
+        std::vector<float> tw(2 * (size_t)N);
+        pk::own_fft_twiddles(N, tw.data());
+        SV_CUDA(S, cudaMalloc(&S->tw, sizeof(float) * tw.size()));
+        SV_CUDA(S, cudaMemcpy(S->tw, tw.data(), sizeof(float) * tw.size(), cudaMemcpyHostToDevice));
+        S->nsync = 1 + N * std::max(kSlots, S->nm);
+        SV_CUDA(S, cudaMalloc(reinterpret_cast<void **>(&S->sync), sizeof(unsigned) * S->nsync));
+        SV_CUDA(S, cudaMemset(S->sync, 0, sizeof(unsigned) * S->nsync));
+        const long long mhi = P->bg.mhi;
+        while (S->ncol < S->Nh && (long long)S->ncol * S->ncol < mhi) ++S->ncol;
+        const int w = S->zyx->tile_columns(0);
+        std::vector<int> tiles;
+        for (int all = 0; all < 2; ++all) {
+            for (int j = 0; j < N; ++j) {
+                const long long jp = j < N / 2 ? j : N - j;
+                for (int b = 0; b * w < (all ? S->Nh : S->ncol); ++b)
+                    if (all || jp * jp + (long long)b * w * b * w < mhi) tiles.push_back(j << 16 | b);
+            }
+            (all ? S->nx_all : S->nx_bin) = (int)tiles.size() - S->nx_bin;
+        }
+        SV_CUDA(S, cudaMalloc(reinterpret_cast<void **>(&S->xtiles), sizeof(int) * tiles.size()));
+        SV_CUDA(S, cudaMemcpy(S->xtiles, tiles.data(), sizeof(int) * tiles.size(), cudaMemcpyHostToDevice));
+    }
+
     // Y_lm-weighted meshes resident per pass (written by one field pass, read
-    // by one bin pass); each is transformed by its own single-mesh cuFFT call
+    // by one bin pass); with cuFFT each is transformed by its own single-mesh cuFFT call
     // (at 1024^3 a batched plan over 14 meshes measured 2x slower per mesh).
     if (nslot > 0) {
         int batch = nslot;
@@ -832,12 +861,14 @@ static pk_status survey_build(pk_survey_s *S, const pk_survey_config *cfg, void 
         long long inembed[3] = {S->N, S->N, 2LL * S->Nh};
         long long onembed[3] = {S->N, S->N, (long long)S->Nh};
         size_t work = 0, w1 = 0;
-        SV_CUFFT(S, cufftCreate(&S->fft_b));
-        S->have_b = 1;
-        SV_CUFFT(S, cufftSetAutoAllocation(S->fft_b, 0));
-        SV_CUFFT(S, cufftMakePlanMany64(S->fft_b, 3, n, inembed, 1, S->mesh_reals, onembed, 1, S->mesh_reals / 2,
-                                        S->f64 ? CUFFT_D2Z : CUFFT_R2C, 1, &w1));
-        work = std::max(work, w1);
+        if (!S->zyx) {
+            SV_CUFFT(S, cufftCreate(&S->fft_b));
+            S->have_b = 1;
+            SV_CUFFT(S, cufftSetAutoAllocation(S->fft_b, 0));
+            SV_CUFFT(S, cufftMakePlanMany64(S->fft_b, 3, n, inembed, 1, S->mesh_reals, onembed, 1, S->mesh_reals / 2,
+                                            S->f64 ? CUFFT_D2Z : CUFFT_R2C, 1, &w1));
+            work = std::max(work, w1);
+        }
         if (c.interlaced) {
             SV_CUFFT(S, cufftCreate(&S->fft_inv));
             S->have_inv = 1;
@@ -1031,14 +1062,37 @@ static pk_status survey_compute_t(pk_survey_s *S) {
     const R ox = (R)S->cfg.box_origin[0], oy = (R)S->cfg.box_origin[1], oz = (R)S->cfg.box_origin[2];
     const bool il = S->cfg.interlaced != 0;
 
+    const double L = S->cfg.box_size;
+    pk::SurveyRows rows;                    // own transforms: rows formed on the way into the z axis
+    rows.D = D;
+    rows.alpha = S->cst;
+    rows.slot_c = mr / 2;
+    // Y_lm does not depend on the unit: a power of two near the box edge keeps the
+    // fourth powers in range and the FP32 node coordinates as they are
+    const int unit = -ilogb(L);
+    rows.ox = (float)ldexp((double)(float)S->cfg.box_origin[0], unit);
+    rows.oy = (float)ldexp((double)(float)S->cfg.box_origin[1], unit);
+    rows.oz = (float)ldexp((double)(float)S->cfg.box_origin[2], unit);
+    rows.H = (float)ldexp((double)(float)(L / N), unit);
     S->seg_compute.clear();
     if (il) {
         // F = D - alpha R on both meshes, both transformed, combined into A_0
-        SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FIELD));
-        k_fkp_combine<R><<<S->nsm * 8, 256, 0, st>>>(D, Rm, (long long)S->nm * mr, S->cst);
-        SV_CUDA(S, cudaGetLastError());
-        SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FFT));
-        SV_CUFFT(S, pk::transform_meshes(P, D, S->nm));
+        if (S->zyx) {
+            SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FFT));
+            rows.R = Rm;                        // the second meshes follow the first in both catalogs
+            rows.s0 = -1;
+            rows.nslot = 1;
+            SV_CUDA(S, S->zyx->zy_survey(D, S->nm * N, rows, Nh, 0x7fffffff, S->tw, S->sync, P->d_err, S->nsm, st));
+            SV_CUDA(S, S->zyx->x(D, S->nm, mr / 2, Nh, 0x7fffffff, S->xtiles + S->nx_bin, S->nx_all, S->tw, S->sync,
+                                 S->nsync, st));
+            S->launches += 1;
+        } else {
+            SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FIELD));
+            k_fkp_combine<R><<<S->nsm * 8, 256, 0, st>>>(D, Rm, (long long)S->nm * mr, S->cst);
+            SV_CUDA(S, cudaGetLastError());
+            SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FFT));
+            SV_CUFFT(S, pk::transform_meshes(P, D, S->nm));
+        }
         C *f1 = reinterpret_cast<C *>(D);
         const R inv_n3 = (R)(1.0 / ((double)N * N * N));
         SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FIELD));
@@ -1077,7 +1131,22 @@ static pk_status survey_compute_t(pk_survey_s *S) {
         R *a0copy = (!il && first) ? A0r : nullptr;
         // compile-time slot ranges for the usual batches, else the generic kernel
         const int spec = (s0 == 0 && nb == 14) ? 1 : (s0 == 0 && nb == 5) ? 2 : (s0 == 5 && nb == 9) ? 3 : 0;
-        if (nb > 0 || a0copy) {
+        if (S->zyx) {
+            // weighting, z and y in one pass over the batch's meshes, then x
+            SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FFT));
+            rows.R = il ? nullptr : Rm;
+            const int mhi = P->bg.mhi;
+            for (int part = 0; part < 2; ++part) {
+                void *dst = part == 0 ? S->a0 : S->slots;
+                rows.s0 = part == 0 ? -1 : s0;
+                rows.nslot = part == 0 ? 1 : nb;
+                if (part == 0 ? !a0copy : nb == 0) continue;
+                SV_CUDA(S, S->zyx->zy_survey(dst, N, rows, S->ncol, mhi, S->tw, S->sync, P->d_err, S->nsm, st));
+                SV_CUDA(S, S->zyx->x(dst, rows.nslot, mr / 2, S->ncol, mhi, S->xtiles, S->nx_bin, S->tw, S->sync,
+                                     S->nsync, st));
+                S->launches += 2;
+            }
+        } else if (nb > 0 || a0copy) {
             SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FIELD));
             const R *Rsrc = il ? nullptr : Rm;
             R *a0dst = il ? nullptr : a0copy;
@@ -1099,9 +1168,9 @@ static pk_status survey_compute_t(pk_survey_s *S) {
             SV_CUDA(S, cudaGetLastError());
             S->launches += 1;
         }
-        SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FFT));
-        if (a0copy) SV_CUFFT(S, pk::transform_meshes(P, A0r, 1));
-        for (int k = 0; k < nb; ++k) {
+        if (!S->zyx) SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FFT));
+        if (a0copy && !S->zyx) SV_CUFFT(S, pk::transform_meshes(P, A0r, 1));
+        for (int k = 0; k < nb && !S->zyx; ++k) {
             R *mk = SL + (long long)k * mr;
             if (S->f64) {
                 SV_CUFFT(S, cufftExecD2Z(S->fft_b, reinterpret_cast<cufftDoubleReal *>(mk),
@@ -1127,7 +1196,7 @@ static pk_status survey_compute_t(pk_survey_s *S) {
     const int nk = g.nk;
     SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FINAL));
     k_survey_final<<<(3 * nk + 127) / 128, 128, 0, st>>>(S->partial, S->Gb, nk, P->d_modes1d, S->cst,
-                                                         S->cfg.poles_mask | 1u, S->cfg.subtract_shot, S->res);
+                                                         S->cfg.poles_mask | 1u, S->cfg.subtract_shot, P->d_err, S->res);
     SV_CUDA(S, cudaGetLastError());
     S->launches += 1;
     SV_CUDA(S, tmark(S, 1, -1));
@@ -1159,6 +1228,9 @@ pk_status pk_survey_result(pk_survey_t S, pk_survey_result_view *out) {
     pk_plan_s *P = S->P;
     const int nk = P->bg.nk;
     const double *c = S->h_res + 3 * (size_t)nk;
+    const int flags = (int)c[kConst - 1];
+    if (flags & 2) return sfail(S, PK_ECUDA, "internal: tile sort saw more copies than it counted");
+    if (flags & 4) return sfail(S, PK_ETIMEOUT, "internal: a wait inside the transform gave up");
     memset(out, 0, sizeof(*out));
     out->nk = nk;
     out->npoles = 3;
