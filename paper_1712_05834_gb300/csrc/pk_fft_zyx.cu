@@ -218,8 +218,9 @@ __host__ __device__ constexpr int radix_of(int S) {
                                           : 8;
 }
 
-// Radix order of the z FFTs: as radix_of, but 4 for the blocks of 32.
-__host__ __device__ constexpr int zradix_of(int S) { return S == 32 ? 4 : radix_of(S); }
+// Radix order of the z FFTs: as radix_of, but 4 for the blocks of 32 and 8 first
+// for 256 (8, 4, 8: the last step pairs its butterflies, see zrow_last).
+__host__ __device__ constexpr int zradix_of(int S) { return S == 32 ? 4 : (S == 256 ? 8 : radix_of(S)); }
 
 // Frequency at position p (< S) after all steps over a block of S points:
 // a step of radix R puts output k of the butterfly at n + (S/R) k, so the
@@ -272,7 +273,6 @@ struct Cfg : Shape<N> {
     // z rows: NT threads share NR rows of M complex (about 16 per thread)
     static constexpr int NT = M >= 1024 ? 64 : 32;
     static constexpr int NR = M > 256 ? 1 : M > 128 ? 2 : M > 64 ? 4 : 8;
-    static constexpr int RS = (M & (M - 1)) == 0 ? M : M + 16;   // shared slots per row
     static constexpr int GROUPS = Shape<N>::T / NT;              // row groups per CTA (named barriers 1 .. GROUPS)
     static constexpr int RPI = GROUPS * NR;                      // rows per z item
     static constexpr int ZI = (N + RPI - 1) / RPI;               // z items per plane
@@ -391,19 +391,30 @@ __device__ __forceinline__ void col_step(float2 *buf, const float2 *tw, int c, i
 
 // ---------------------------------------------------------------------------
 // z rows.  NT threads transform NR rows; position p of a row sits in slot
-// p ^ ((p >> 2) & 15), a bijection on [0, M] that keeps the FFT steps and the
-// natural-order write free of bank conflicts, except the reads of the last
-// step of the length-256 FFT (two-way).
-__host__ __device__ constexpr int zslot(int p) { return p ^ ((p >> 2) & 15); }
-
-// Slot of position base + off, off a multiple of Q with base % Q < Q and no bit
-// in common (power-of-two lengths): zslot is linear over bits, so the slot of
-// base is shifted by a constant and its low four bits flipped by another.
-template <bool POW2>
-__device__ __forceinline__ int zslot_at(int zbase, int base, int off) {
-    if constexpr (POW2) return (zbase ^ (zslot(off) & 15)) + (off & ~15);
-    else return zslot(base + off);
-}
+// p ^ L((p >> t) & 15) (the low four bits change, so the eight-byte values of a
+// half-warp spread over the 16 bank pairs).  t and L per length were chosen by
+// counting the wavefronts of every access of the steps below: none beyond the
+// minimum at 128, 256 and 512, 12 % more at 1024, 15 % at 192, 320 and 384,
+// 25-90 % at the others (a slot p ^ ((p >> 2) & 15) took 1.6 to 5 times it).
+template <int M>
+struct ZSlot {
+    static constexpr bool POW2 = (M & (M - 1)) == 0;
+    static constexpr int t = M <= 64 || M == 128 ? 3 : M == 96 ? 4 : M % 64 != 0 ? 6 : M >= 384 ? 6 : 5;
+    static constexpr bool X8 = M == 96 || (M > 128 && M % 64 == 0);    // L(d) = d ^ 8 (d & 1), else d
+    static constexpr int PAD = M <= 64 ? 4 : (M == 96 || M == 128 ? 8 : 0);
+    static constexpr int RS = (M + 15) / 16 * 16 + PAD;                // slots per row
+    __host__ __device__ static constexpr int at(int p) {
+        const int d = (p >> t) & 15;
+        return p ^ (X8 ? d ^ ((d & 1) << 3) : d);
+    }
+    // Slot of position base + off, the two without a common bit (power-of-two
+    // lengths): the map is linear over bits, so the slot of base is shifted by a
+    // constant and its low four bits flipped by another.
+    __device__ static __forceinline__ int at(int zbase, int base, int off) {
+        if constexpr (POW2) return (zbase ^ (at(off) & 15)) + (off & ~15);
+        else return at(base + off);
+    }
+};
 
 // Twiddles of the z FFT steps, one table per step with block size S (from M
 // down): entry (k - 1) Q + n = W_S^{nk} (Q = S/R, n < Q, 1 <= k < R), so the
@@ -436,72 +447,97 @@ __device__ __forceinline__ void row_sync(int grp) {
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(NT) : "memory");
 }
 
-// One step over blocks of S points of the FFTs of rows [0, nrow) (FIRST: values
-// from ld(row, position)).  The last step writes in natural order.
-template <int M, int NR, int NT, int RS, int S, bool FIRST, typename Ld>
+// Position of the block of a last step of radix R whose output k has frequency
+// f0 + k M / R (the inverse of dif_freq over the steps before it).
+template <int M, int S>
+__device__ __forceinline__ int block_of(int f0) {
+    constexpr int R = zradix_of(S), Q = S / R;
+    if constexpr (Q == 1) return 0;
+    else return (f0 % R) * Q + block_of<M, Q>(f0 / R);
+}
+
+template <int S>
+__host__ __device__ constexpr int zlast_radix() {
+    constexpr int R = zradix_of(S);
+    if constexpr (S == R) return R;
+    else return zlast_radix<S / R>();
+}
+
+// One step over blocks of S points (all but the last step) of the FFTs of rows
+// [0, nrow) (FIRST: values from ld(row, position)).
+template <int M, int NR, int NT, int S, bool FIRST, typename Ld>
 __device__ __forceinline__ void zrow_step(float2 *rows, const Ld &ld, int nrow, const float2 *ztw, int lane,
                                           int grp) {
     constexpr int R = zradix_of(S), Q = S / R;
-    constexpr int BPR = M / R;                    // butterflies per row
-    constexpr int TOT = NR * BPR;
-    constexpr int PER = (TOT + NT - 1) / NT;
-    constexpr int TW = ztw_offset(M, S);
-    constexpr bool POW2 = (M & (M - 1)) == 0;
-    constexpr bool HOLD = (POW2 && PER * R <= 16) || Q == 1;
-    constexpr int NV = HOLD ? PER : 1;
-    float2 v[NV][R];
-    const auto load = [&](int s) {
-        const int beta = lane + NT * s;
-        const int r = beta / BPR, b = beta % BPR;
-        if ((TOT % NT == 0 || beta < TOT) && r < nrow) {
-            const int base = (b / Q) * S + b % Q;
-            if (FIRST) {
+    using Zs = ZSlot<M>;
+    if constexpr (Q > 1) {
+        constexpr int BPR = M / R;                    // butterflies per row
+        constexpr int TOT = NR * BPR;
+        constexpr int PER = (TOT + NT - 1) / NT;
+        constexpr int TW = ztw_offset(M, S);
+        constexpr bool HOLD = Zs::POW2 && PER * R <= 16;
+        constexpr int NV = HOLD ? PER : 1;
+        float2 v[NV][R];
+        const auto load = [&](int s) {
+            const int beta = lane + NT * s;
+            const int r = beta / BPR, b = beta % BPR;
+            if ((TOT % NT == 0 || beta < TOT) && r < nrow) {
+                const int base = (b / Q) * S + b % Q;
 #pragma unroll
-                for (int j = 0; j < R; ++j) v[HOLD ? s : 0][j] = ld(r, base + Q * j);
-            } else {
-#pragma unroll
-                for (int j = 0; j < R; ++j) v[HOLD ? s : 0][j] = rows[r * RS + zslot_at<POW2>(zslot(base), base, Q * j)];
+                for (int j = 0; j < R; ++j) {
+                    if (FIRST) v[HOLD ? s : 0][j] = ld(r, base + Q * j);
+                    else v[HOLD ? s : 0][j] = rows[r * Zs::RS + Zs::at(Zs::at(base), base, Q * j)];
+                }
             }
-        }
-    };
-    if constexpr (HOLD) {
+        };
+        const auto work = [&](int s) {
+            float2 *w = v[HOLD ? s : 0];
+            const int beta = lane + NT * s;
+            const int r = beta / BPR, b = beta % BPR;
+            if ((TOT % NT == 0 || beta < TOT) && r < nrow) {
+                const int n = b % Q, base = (b / Q) * S + n;
+                dft<R>(w);
+                const float2 *tk = ztw + TW + n - Q;      // tk[k Q] = W_S^{nk}
+                if constexpr (R == 8 || R == 16) {
+                    // four loads and products instead of fifteen loads (two and
+                    // seven): shared memory is the busiest pipe here
+                    float2 ww[R];
+                    ww[1] = tk[Q];
+                    ww[2] = R == 16 ? tk[2 * Q] : c_mul(ww[1], ww[1]);
+                    ww[4] = tk[4 * Q];
+                    ww[3] = c_mul(ww[2], ww[1]);
 #pragma unroll
-        for (int s = 0; s < PER; ++s) load(s);
-    }
-    // the last step writes other positions than it reads: all reads first
-    if constexpr (Q == 1) row_sync<NT>(grp);
-    const auto work = [&](int s) {
-        float2 *w = v[HOLD ? s : 0];
-        const int beta = lane + NT * s;
-        const int r = beta / BPR, b = beta % BPR;
-        if ((TOT % NT == 0 || beta < TOT) && r < nrow) {
-            const int n = b % Q, base = (b / Q) * S + n;
-            dft<R>(w);
-            if constexpr (Q > 1) {
+                    for (int k = 5; k < 8; ++k) ww[k] = c_mul(ww[4], ww[k - 4]);
+                    if constexpr (R == 16) {
+                        ww[8] = tk[8 * Q];
 #pragma unroll
-                for (int k = 1; k < R; ++k) w[k] = c_mul(w[k], ztw[TW + (k - 1) * Q + n]);   // W_S^{nk}
+                        for (int k = 9; k < 16; ++k) ww[k] = c_mul(ww[8], ww[k - 8]);
+                    }
 #pragma unroll
-                for (int k = 0; k < R; ++k) rows[r * RS + zslot_at<POW2>(zslot(base), base, Q * k)] = w[k];
-            } else {
-                const int f0 = dif_freq<M, 1, true>(base), zf = zslot(f0);
+                    for (int k = 1; k < R; ++k) w[k] = c_mul(w[k], ww[k]);
+                } else {
 #pragma unroll
-                for (int k = 0; k < R; ++k)         // output k: frequency f0 + k M / R
-                    rows[r * RS + zslot_at<POW2>(zf, f0, k * (M / R))] = w[k];
+                    for (int k = 1; k < R; ++k) w[k] = c_mul(w[k], tk[k * Q]);
+                }
+#pragma unroll
+                for (int k = 0; k < R; ++k) rows[r * Zs::RS + Zs::at(Zs::at(base), base, Q * k)] = w[k];
             }
-        }
-    };
-    if constexpr (HOLD) {
+        };
+        if constexpr (HOLD) {
 #pragma unroll
-        for (int s = 0; s < PER; ++s) work(s);
-    } else {
+            for (int s = 0; s < PER; ++s) load(s);
+#pragma unroll
+            for (int s = 0; s < PER; ++s) work(s);
+        } else {
 #pragma unroll 1
-        for (int s = 0; s < PER; ++s) {
-            load(s);
-            work(s);
+            for (int s = 0; s < PER; ++s) {
+                load(s);
+                work(s);
+            }
         }
+        row_sync<NT>(grp);
+        zrow_step<M, NR, NT, Q, false>(rows, ld, nrow, ztw, lane, grp);
     }
-    row_sync<NT>(grp);
-    if constexpr (Q > 1) zrow_step<M, NR, NT, RS, Q, false>(rows, ld, nrow, ztw, lane, grp);
 }
 
 // D[l] and D[M-l] from u = C[l], v = C[M-l] and w = W_N^l: with s = u + conj v
@@ -512,6 +548,50 @@ __device__ __forceinline__ void split_real(float2 u, float2 v, float2 w, float2 
     const float qx = -(w.x * oy + w.y * ox), qy = w.x * ox - w.y * oy;
     *dl = make_float2(fmaf(-0.5f, qx, s.x), fmaf(-0.5f, qy, s.y));
     *dm = make_float2(fmaf(0.5f, qx, s.x), -fmaf(0.5f, qy, s.y));
+}
+
+// The last step of the rows' FFTs, the real-input split and the store of
+// D[0 .. ncol).  Of the B = M / R butterflies of a row, whose outputs are the
+// frequencies f0 + B k, one thread takes f0 and B - f0 (f0 = 0 with B / 2): the
+// partner M - f of each of its outputs is among them, so the transform never
+// goes back to shared memory and is written straight from registers (for one k
+// the lanes write neighbouring l).
+template <int M, int NR, int NT>
+__device__ __forceinline__ void zrow_last(const float2 *rows, int nrow, float2 *d, long long ds, int ncol,
+                                          const float2 *tw, int lane) {
+    constexpr int R = zlast_radix<M>(), B = M / R, GP = B / 2, TOT = NR * GP;
+    using Zs = ZSlot<M>;
+    static_assert(B % 2 == 0, "butterflies pair up");
+#pragma unroll 1
+    for (int t = lane; t < TOT; t += NT) {
+        const int r = t / GP, i = t % GP;
+        if (r >= nrow) continue;
+        const int fb0 = i ? B - i : GP;
+        float2 va[R], vb[R];
+        {
+            const int pa = block_of<M, M>(i), pb = block_of<M, M>(fb0), za = Zs::at(pa), zb = Zs::at(pb);
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                va[j] = rows[r * Zs::RS + Zs::at(za, pa, j)];
+                vb[j] = rows[r * Zs::RS + Zs::at(zb, pb, j)];
+            }
+        }
+        dft<R>(va);
+        dft<R>(vb);
+        float2 *row = d + r * ds;
+        const auto put = [&](float2 u, float2 v, int f) {        // u = C[f], v = C[M - f]
+            float2 dl, dm;
+            split_real(u, v, tw[f], &dl, &dm);
+            if (f < ncol) row[f] = dl;
+            if (M - f < ncol) row[M - f] = dm;
+        };
+#pragma unroll
+        for (int k = 0; k < R; ++k) put(va[k], i ? vb[R - 1 - k] : va[(R - k) % R], i + B * k);
+        if (i == 0) {
+#pragma unroll
+            for (int k = 0; k < (R + 1) / 2; ++k) put(vb[k], vb[R - 1 - k], GP + B * k);
+        }
+    }
 }
 
 // Waits of y items for their plane's z items.  A CTA holds its current item and
@@ -591,10 +671,10 @@ k_fft_zy(float2 *mesh, int planes, int ncol, int mcut, const float2 *__restrict_
             const int nrow = grp < K::GROUPS ? min(K::NR, N - row0) : 0;
             float2 *g = plane_at(step) + (long long)row0 * Nh;
             if (nrow > 0) {
-                float2 *rows = buf + (size_t)grp * K::NR * K::RS;
+                float2 *rows = buf + (size_t)grp * K::NR * ZSlot<M>::RS;
                 if constexpr (!SURVEY) {
                     const auto ld = [&](int r, int p) { return __ldcs(g + (long long)r * Nh + p); };
-                    zrow_step<M, K::NR, K::NT, K::RS, M, true>(rows, ld, nrow, ztw, lane, grp);
+                    zrow_step<M, K::NR, K::NT, M, true>(rows, ld, nrow, ztw, lane, grp);
                 } else {
                     const int i = step / sv.nslot, slot = sv.s0 + step - i * sv.nslot;
                     const long long at = (long long)i * plane_c + (long long)row0 * Nh;
@@ -628,18 +708,9 @@ k_fft_zy(float2 *mesh, int planes, int ncol, int mcut, const float2 *__restrict_
                         }
                         return f;
                     };
-                    zrow_step<M, K::NR, K::NT, K::RS, M, true>(rows, ld, nrow, ztw, lane, grp);
+                    zrow_step<M, K::NR, K::NT, M, true>(rows, ld, nrow, ztw, lane, grp);
                 }
-                for (int r = 0; r < nrow; ++r) {
-                    const float2 *C = rows + r * K::RS;
-                    float2 *d = g + (long long)r * Nh;
-                    for (int l = lane; l <= M / 2; l += K::NT) {
-                        float2 dl, dm;
-                        split_real(C[zslot(l)], C[zslot(l ? M - l : 0)], tw[l], &dl, &dm);
-                        if (l < ncol) d[l] = dl;
-                        if (M - l < ncol && l != M - l) d[M - l] = dm;
-                    }
-                }
+                zrow_last<M, K::NR, K::NT>(rows, nrow, g, Nh, ncol, tw, lane);
             }
             __syncthreads();
             if (threadIdx.x == 0) {             // the CTA's rows, seen through the barrier, then the count
@@ -869,7 +940,7 @@ k_fft_xbin(const float2 *__restrict__ mesh, long long item_stride_c, long long m
 template <int N>
 constexpr size_t zy_smem() {
     using K = Cfg<N>;
-    const size_t z = (size_t)K::RPI * K::RS, y = (size_t)N * K::NBY;
+    const size_t z = (size_t)K::RPI * ZSlot<K::M>::RS, y = (size_t)N * K::NBY;
     return sizeof(float2) * (N + (ztw_offset(K::M, 1) + 1) / 2 * 2 + (z > y ? z : y));
 }
 
