@@ -67,10 +67,10 @@ void free_plan(pk_plan_s *p) {
     if (!p) return;
     cudaStreamSynchronize(p->st);
     for (cufftHandle h : p->fft) cufftDestroy(h);
-    void *dev[] = {p->mesh, p->d_count, p->d_off, p->d_scan_tmp, p->d_sorted,
-                   p->d_stage, p->d_item_off, p->d_wsums, p->d_wpart, p->d_wmax, p->d_cw, p->d_ph,
-                   p->d_kedge, p->d_partial, p->d_sums2, p->d_res, p->d_modes1d, p->d_modes2d,
-                   p->d_err, p->d_acc, p->fft_work, p->d_xres, p->d_proj, p->d_tw};
+    void *dev[] = {p->mesh, p->d_off, p->d_scan_tmp, p->d_sorted,
+                   p->d_stage, p->d_item_off, p->d_wsums, p->d_wpart, p->d_cw, p->d_ph,
+                   p->d_kedge, p->d_partial, p->d_modes1d, p->d_modes2d,
+                   p->d_err, p->d_acc, p->fft_work, p->d_proj, p->d_tw};
     for (void *d : dev)
         if (d) cudaFree(d);
     if (p->h_res) cudaFreeHost(p->h_res);
@@ -371,13 +371,16 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
     const size_t mesh_bytes = (size_t)P->B * P->nm * P->mesh_reals * P->esz;
     PK_CUDA(P, dev_alloc(&P->mesh, mesh_bytes));
     const long long keys_all = (long long)P->B * P->nkeys;
-    PK_CUDA(P, dev_alloc(&P->d_count, sizeof(uint32_t) * keys_all));
+    // weight sums, weight maxima and key counts back to back: one memset clears
+    // what a paint starts from
+    const size_t sums_bytes = (sizeof(double) * 4 + sizeof(uint4)) * (size_t)P->B;
+    PK_CUDA(P, dev_alloc(&P->d_wsums, sums_bytes + sizeof(uint32_t) * keys_all));
+    P->d_wmax = reinterpret_cast<uint4 *>(P->d_wsums + 4 * (size_t)P->B);
+    P->d_count = reinterpret_cast<uint32_t *>(P->d_wmax + P->B);
     PK_CUDA(P, dev_alloc(&P->d_off, sizeof(uint32_t) * (keys_all + 1)));
     PK_CUDA(P, dev_alloc(&P->d_scan_tmp, sizeof(uint32_t) * scan_tmp_elems(keys_all)));
     PK_CUDA(P, dev_alloc(&P->d_item_off, sizeof(int64_t) * (P->B + 1)));
-    PK_CUDA(P, dev_alloc(&P->d_wsums, sizeof(double) * 4 * P->B));
     PK_CUDA(P, dev_alloc(&P->d_wpart, sizeof(double) * wsum_partial_elems(P->B)));
-    PK_CUDA(P, dev_alloc(&P->d_wmax, sizeof(uint4) * P->B));
     PK_CUDA(P, dev_alloc(&P->d_err, sizeof(int)));
     PK_CUDA(P, cudaMemset(P->d_err, 0, sizeof(int)));
     PK_CUDA(P, dev_alloc(&P->d_cw, P->esz * P->N));
@@ -386,10 +389,7 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
     const int occ = bin_ctas_per_sm(bg, P->f64);
     P->G_total = P->nsm * occ;
     PK_CUDA(P, dev_alloc(&P->d_partial, (size_t)(P->G_total + P->B) * bg.nh * (P->f64 ? 8 : 4)));
-    PK_CUDA(P, dev_alloc(&P->d_sums2, sizeof(double) * (size_t)(reduce_chunks(P->G_total) + P->B) * bg.nh));
-    PK_CUDA(P, dev_alloc(&P->d_res, sizeof(double) * (size_t)P->B * fg.RL));
     PK_CUDA(P, cudaMallocHost(reinterpret_cast<void **>(&P->h_res), sizeof(double) * (size_t)P->B * fg.RL));
-    PK_CUDA(P, dev_alloc(&P->d_xres, sizeof(double) * (size_t)fg.RL));
     PK_CUDA(P, dev_alloc(&P->d_proj, sizeof(double) * 3 * (size_t)nk));
     PK_CUDA(P, cudaMallocHost(reinterpret_cast<void **>(&P->h_xres), sizeof(double) * (size_t)fg.RL));
     PK_CUDA(P, cudaEventCreateWithFlags(&P->xdone, cudaEventDisableTiming));
@@ -556,13 +556,12 @@ static pk_status paint_atomic(pk_plan_s *P, const void *dpos, int dtype, const f
     const int tm = P->timing && !capturing(st);
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[0], st));
     int launches = 2;
-    PK_CUDA(P, launch_upload_i64(P->d_item_off, offsets, nitems + 1, &launches, st));
-    if (!accumulate) {
-        PK_CUDA(P, cudaMemsetAsync(P->d_wsums, 0, sizeof(double) * 4 * nitems, st));
-        PK_CUDA(P, cudaMemsetAsync(P->d_wmax, 0, sizeof(uint4) * nitems, st));
-    }
+    const int64_t *item_off = nitems > 1 ? P->d_item_off : nullptr;
+    if (item_off) PK_CUDA(P, launch_upload_i64(P->d_item_off, offsets, nitems + 1, &launches, st));
+    if (!accumulate)
+        PK_CUDA(P, cudaMemsetAsync(P->d_wsums, 0, (sizeof(double) * 4 + sizeof(uint4)) * (size_t)P->B, st));
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[1], st));   // no sort stage
-    PK_CUDA(P, launch_paint_atomic(dpos, dtype, dw, dv, P->d_item_off, nitems, max_n, P->pg, P->p, P->nm, P->S,
+    PK_CUDA(P, launch_paint_atomic(dpos, dtype, dw, dv, item_off, nitems, max_n, P->pg, P->p, P->nm, P->S,
                                    P->d_acc, P->d_wsums, P->d_wpart, P->d_wmax, st));
     if (dw != nullptr || dv != nullptr || dtype == PK_F32X4) launches += 1;   // the weight sums' reduce
     PK_CUDA(P, launch_acc_to_mesh(P->d_acc, nitems, P->nm, P->N, P->S, P->f64, P->mesh,
@@ -658,17 +657,19 @@ static pk_status paint_impl(pk_plan_s *P, const void *pos, int dtype, const floa
     const int tm = P->timing && !capturing(st);
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[0], st));
     int launches = 2;   // count, scatter
-    PK_CUDA(P, launch_upload_i64(P->d_item_off, offsets, nitems + 1, &launches, st));
-    PK_CUDA(P, cudaMemsetAsync(P->d_count, 0, sizeof(uint32_t) * nkeys, st));
-    if (!accumulate) {
-        PK_CUDA(P, cudaMemsetAsync(P->d_wsums, 0, sizeof(double) * 4 * nitems, st));
-        PK_CUDA(P, cudaMemsetAsync(P->d_wmax, 0, sizeof(uint4) * nitems, st));
+    const int64_t *item_off = nitems > 1 ? P->d_item_off : nullptr;
+    if (item_off) PK_CUDA(P, launch_upload_i64(P->d_item_off, offsets, nitems + 1, &launches, st));
+    if (accumulate) {
+        PK_CUDA(P, cudaMemsetAsync(P->d_count, 0, sizeof(uint32_t) * nkeys, st));
+    } else {
+        char *end = reinterpret_cast<char *>(P->d_count + nkeys), *beg = reinterpret_cast<char *>(P->d_wsums);
+        PK_CUDA(P, cudaMemsetAsync(beg, 0, (size_t)(end - beg), st));
     }
-    PK_CUDA(P, launch_sort_count(dpos, dtype, dw, dv, P->d_item_off, nitems, max_n, P->pg, P->d_count,
+    PK_CUDA(P, launch_sort_count(dpos, dtype, dw, dv, item_off, nitems, max_n, P->pg, P->d_count,
                                  P->d_wsums, P->d_wpart, P->d_wmax, st));
     if (dw != nullptr || dv != nullptr || dtype == PK_F32X4) launches += 1;   // the weight sums' reduce
     PK_CUDA(P, launch_scan(P->d_count, nkeys, P->d_off, P->d_scan_tmp, &launches, st));
-    PK_CUDA(P, launch_sort_scatter(dpos, dtype, dw, dv, P->d_item_off, nitems, max_n, P->pg, P->d_count,
+    PK_CUDA(P, launch_sort_scatter(dpos, dtype, dw, dv, item_off, nitems, max_n, P->pg, P->d_count,
                                    P->d_sorted, (uint32_t)ntot, P->d_err, st));
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[1], st));
     const int unit_weights = dw == nullptr && dv == nullptr && dtype != PK_F32X4;
@@ -739,7 +740,9 @@ pk_status pk_compute(pk_plan_t P) {
     const int nitems = P->npainted;
     const long long item_c = (long long)P->nm * P->mesh_reals / 2;   // complex elements
     const long long mesh_c = P->mesh_reals / 2;
-    int G = std::max(1, P->G_total / nitems);
+    // at least two of k_bin's rows per warp: fewer CTAs on small meshes leave
+    // fewer histograms to add up
+    int G = std::max(1, std::min(P->G_total / nitems, P->N * P->N / 16));
     pk_status s_ = PK_OK;
     if (P->own_fft) {
         P->transformed = 1;
@@ -806,14 +809,11 @@ pk_status pk_compute(pk_plan_t P) {
                               P->d_cw, P->d_ph, P->d_kedge, P->d_partial, st));
     }
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[5], st));
-    PK_CUDA(P, launch_bin_reduce(P->d_partial, P->f64, G, P->bg.nh, nitems, P->d_sums2, st));
-    PK_CUDA(P, launch_finalize(P->d_sums2, G, P->d_modes1d, P->d_modes2d, P->d_wsums, P->d_err, P->fg,
-                               nitems, P->d_res, st));
+    PK_CUDA(P, launch_reduce_finalize(P->d_partial, P->f64, G, P->d_modes1d, P->d_modes2d, P->d_wsums, P->d_err, P->fg,
+                                      nitems, P->h_res, -1, -1, st));
     if (tm) PK_CUDA(P, cudaEventRecord(P->tev[6], st));
     P->tev_compute = tm;
-    P->launches += 2 + reduce_launches(G);   // bin, reduce (one or two passes), finalize
-    PK_CUDA(P, cudaMemcpyAsync(P->h_res, P->d_res, sizeof(double) * (size_t)nitems * P->fg.RL,
-                               cudaMemcpyDeviceToHost, st));
+    P->launches += 2;   // bin, reduce + finalize
     // Under stream capture the results come from a later graph replay, which
     // the caller synchronizes; an event recorded into the capture could not
     // be waited on outside it.
@@ -863,12 +863,9 @@ pk_status pk_cross(pk_plan_t P, int item_a, int item_b) {
     PK_CUDA(P, launch_bin_cross(base + (size_t)item_a * item_c * csz, base + (size_t)item_b * item_c * csz, P->f64,
                                 P->cfg.interlaced, mesh_c, P->G_total, P->bg, P->d_cw, P->d_ph, P->d_kedge,
                                 P->d_partial, st));
-    PK_CUDA(P, launch_bin_reduce(P->d_partial, P->f64, P->G_total, P->bg.nh, 1, P->d_sums2, st));
-    PK_CUDA(P, launch_finalize_cross(P->d_sums2, P->G_total, P->d_modes1d, P->d_modes2d, P->d_wsums, P->d_err,
-                                     P->fg, item_a, item_b, P->d_xres, st));
-    P->launches += 2 + reduce_launches(P->G_total);
-    PK_CUDA(P, cudaMemcpyAsync(P->h_xres, P->d_xres, sizeof(double) * (size_t)P->fg.RL, cudaMemcpyDeviceToHost,
-                               st));
+    PK_CUDA(P, launch_reduce_finalize(P->d_partial, P->f64, P->G_total, P->d_modes1d, P->d_modes2d, P->d_wsums, P->d_err,
+                                      P->fg, 1, P->h_xres, item_a, item_b, st));
+    P->launches += 2;
     const int cap = capturing(st);
     if (!cap) PK_CUDA(P, cudaEventRecord(P->xdone, st));
     P->xdone_valid = !cap;

@@ -65,7 +65,8 @@ size_t scan_tmp_elems(int64_t n);
 // dst[0 .. n) = src[0 .. n) for a host array src, through kernel parameters
 // (the host array may be reused as soon as the call returns).
 cudaError_t launch_upload_i64(int64_t *dst, const int64_t *src, int n, int *launches, cudaStream_t st);
-// w: weights (normalization; NULL = 1), vals: painted values V (NULL = 1);
+// item_off: the catalogs' offsets on the device, or NULL for one catalog of max_n
+// objects.  w: weights (normalization; NULL = 1), vals: painted values V (NULL = 1);
 // each object deposits W V and the sums keep sum W, sum (W V)^2, sum |W V|.
 cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const float *vals,
                               const int64_t *item_off, int nitems, int64_t max_n, const PaintGeom &g,
@@ -109,17 +110,12 @@ cudaError_t launch_bin_cross(const void *mesh_a, const void *mesh_b, int f64, in
 size_t bin_smem_bytes(const BinGeom &g, int f64);
 int bin_ctas_per_sm(const BinGeom &g, int f64);
 int bin_threads();
-int reduce_chunks(int G);
-int reduce_launches(int G);           // k_bin_reduce launches per launch_bin_reduce
-cudaError_t launch_bin_reduce(const void *partial, int f64, int G, int nh, int nitems,
-                              double *sums2, cudaStream_t st);
-cudaError_t launch_finalize(const double *sums2, int G, const unsigned long long *modes1d,
-                            const unsigned long long *modes2d, const double *wsums, const int *err,
-                            const FinalGeom &f, int nitems, double *res, cudaStream_t st);
-
-cudaError_t launch_finalize_cross(const double *sums2, int G, const unsigned long long *modes1d,
-                                  const unsigned long long *modes2d, const double *wsums, const int *err,
-                                  const FinalGeom &f, int item_a, int item_b, double *res, cudaStream_t st);
+// Per-CTA histograms (G rows per catalog) -> result blocks in res (pinned host
+// memory): every catalog's auto power (cross_b < 0), or one cross power.
+cudaError_t launch_reduce_finalize(const void *partial, int f64, int G, const unsigned long long *modes1d,
+                                   const unsigned long long *modes2d, const double *wsums, const int *err,
+                                   const FinalGeom &f, int nitems, double *res, int cross_a, int cross_b,
+                                   cudaStream_t st);
 
 // Projected power: bin the plane / line of one catalog's transform that keeps
 // the axes in keep_mask (bit a: axis a); sums[3 b + {0,1,2}] += h, h k, h |F|^2 cw.

@@ -42,9 +42,8 @@
 //                   edges in m = |n|^2), mu bin (exact integer rule),
 //                   Legendre L_2(mu) / L_4(mu) weights; runs of equal bins merged
 //                   in registers, then per-CTA shared-memory histograms.
-//   k_bin_reduce    fixed-order FP64 sums of the per-CTA histograms in 32-row
-//                   chunks, then (in place) of the chunks.
-//   k_finalize      normalization L^3 / (sum w)^2, shot noise, multipoles.
+//   k_reduce_finalize  fixed-order FP64 sums of the per-CTA histograms, then
+//                   normalization L^3 / (sum w)^2, shot noise, multipoles.
 // Plan time (geometry only):
 //   k_geom_*        exact mode counts per bin and mean k, mean mu from integer
 //                   histograms over (m, mu bin), summed in FP64.
@@ -69,15 +68,25 @@ constexpr int kBinVec = 4;            // consecutive modes per thread
 constexpr int kScanThreads = 1024;
 constexpr int kScanPer = 4;           // elements per thread in a scan block
 constexpr int kScanTile = kScanThreads * kScanPer;
+// Up to this many blocks every block of the second scan pass adds up the totals
+// before it itself (one load a thread at most), without a scan launch between.
+constexpr int kScanDirect = 1024;
 constexpr int kClasses = 27;          // boundary classes per tile
 constexpr int kSegments = 75;         // (neighbour, class range) segments per tile
-constexpr int kReduceChunk = 32;      // per-CTA histograms summed per reduce block
 constexpr int kStage = 256;           // candidates staged in shared memory per batch (small: 6 CTAs / SM)
 constexpr int kUploadChunk = 256;     // int64 values per parameter upload (2 KB)
 // Sweep paint: tiles with at most this many candidates use branch-free
 // deposits; denser tiles (e.g. uniform lattices, ~900 candidates per 16^3
 // tile) were measured faster with deposits that skip cells outside the tile.
 constexpr int kFlatMaxCand = 640;
+
+// Objects [beg, end) of a catalog: off[item], off[item + 1], or [0, n) of the
+// only one (off NULL: nothing to upload).
+struct ItemRange {
+    int64_t beg, end;
+    __device__ __forceinline__ ItemRange(const int64_t *off, int64_t n, int item)
+        : beg(off ? off[item] : 0), end(off ? off[item + 1] : n) {}
+};
 
 // Cell coordinate s = x * (N / L) wrapped periodically into [0, N).  Written
 // with explicitly rounded intrinsics so that no FMA contraction can differ
@@ -237,7 +246,7 @@ __device__ __forceinline__ void flush_wsums(double sw, double sw2, double swa, f
 // is added to wsums[4 * item + k] (one writer per value).  wmax[item].z: the
 // mean |W V| (float bits), from which the tile paint guesses a tile's sum.
 __global__ void __launch_bounds__(256)
-k_wsum_reduce(const double *__restrict__ wpart, int nblk, const int64_t *__restrict__ item_off,
+k_wsum_reduce(const double *__restrict__ wpart, int nblk, const int64_t *__restrict__ item_off, int64_t n_one,
               double *__restrict__ wsums, uint4 *__restrict__ wmax) {
     __shared__ double red[3][256];
     const int item = blockIdx.x, t = threadIdx.x;
@@ -256,7 +265,8 @@ k_wsum_reduce(const double *__restrict__ wpart, int nblk, const int64_t *__restr
     }
     if (t < 3) wsums[4 * item + t] += red[t][0];
     if (t == 3) {
-        const float n = (float)(item_off[item + 1] - item_off[item]);
+        const ItemRange range(item_off, n_one, item);
+        const float n = (float)(range.end - range.beg);
         wmax[item].z = __float_as_uint(n > 0.0f ? (float)red[2][0] / n : 0.0f);
     }
 }
@@ -273,11 +283,12 @@ __device__ __forceinline__ int64_t sort_key(const Obj<R> &o, const PaintGeom &g,
 template <int DT, bool WEIGHTED>
 __global__ void __launch_bounds__(kCountThreads)
 k_sort_count(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
-             const int64_t *__restrict__ item_off, PaintGeom g, uint32_t *__restrict__ count,
+             const int64_t *__restrict__ item_off, int64_t n_one, PaintGeom g, uint32_t *__restrict__ count,
              double *__restrict__ wsums, double *__restrict__ wpart, uint4 *__restrict__ wmax) {
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
-    const int64_t beg = item_off[item], end = item_off[item + 1];
+    const ItemRange range(item_off, n_one, item);
+    const int64_t beg = range.beg, end = range.end;
     const int64_t kbase = (int64_t)item * g.ntiles * kClasses;
     double sw = 0.0, sw2 = 0.0, swa = 0.0;
     float mw = 0.0f;
@@ -310,11 +321,12 @@ k_sort_count(const void *__restrict__ pos, const float *__restrict__ w, const fl
 template <int DT>
 __global__ void __launch_bounds__(kCountThreads)
 k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
-               const int64_t *__restrict__ item_off, PaintGeom g, uint32_t *__restrict__ cursor,
+               const int64_t *__restrict__ item_off, int64_t n_one, PaintGeom g, uint32_t *__restrict__ cursor,
                float4 *__restrict__ sorted, uint32_t ntot, int *__restrict__ err) {
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
-    const int64_t beg = item_off[item], end = item_off[item + 1];
+    const ItemRange range(item_off, n_one, item);
+    const int64_t beg = range.beg, end = range.end;
     const int64_t kbase = (int64_t)item * g.ntiles * kClasses;
     for (int64_t i = beg + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -387,11 +399,27 @@ k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
     if (threadIdx.x == 0) bsum[blockIdx.x] = total;
 }
 
-template <typename T, bool COPY>
+// DIRECT: bsum holds the blocks' totals (every block adds up those before it);
+// else their exclusive scan with the total in bsum[nb].
+template <typename T, bool COPY, bool DIRECT>
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T *__restrict__ copy) {
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
-    const T add = bsum[blockIdx.x];
+    T add;
+    if constexpr (DIRECT) {
+        __shared__ T wsum[kScanThreads / 32];
+        T t = (T)0;
+        for (int k = threadIdx.x; k < (int)blockIdx.x; k += kScanThreads) t += bsum[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = t;
+        __syncthreads();
+        add = (T)0;
+#pragma unroll
+        for (int k = 0; k < kScanThreads / 32; ++k) add += wsum[k];
+    } else {
+        add = bsum[blockIdx.x];
+    }
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k)
         if (base + k < n) {
@@ -399,7 +427,8 @@ k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T
             out[base + k] = v;
             if constexpr (COPY) copy[base + k] = v;
         }
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = bsum[nb];
+    if (DIRECT ? blockIdx.x == nb - 1 && threadIdx.x == 0 : blockIdx.x == 0 && threadIdx.x == 0)
+        out[n] = DIRECT ? add + bsum[nb - 1] : bsum[nb];
 }
 
 // ---- tile paint ----
@@ -1121,12 +1150,13 @@ __device__ __forceinline__ void deposit_global(unsigned long long *__restrict__ 
 template <int DT, int P, int NM>
 __global__ void __launch_bounds__(kCountThreads)
 k_paint_atomic(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
-               const int64_t *__restrict__ item_off, PaintGeom g, int S, bool weighted,
+               const int64_t *__restrict__ item_off, int64_t n_one, PaintGeom g, int S, bool weighted,
                unsigned long long *__restrict__ acc, double *__restrict__ wsums,
                double *__restrict__ wpart, uint4 *__restrict__ wmax) {
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
-    const int64_t beg = item_off[item], end = item_off[item + 1];
+    const ItemRange range(item_off, n_one, item);
+    const int64_t beg = range.beg, end = range.end;
     const long long n3 = (long long)g.N * g.N * g.N;
     unsigned long long *ab = acc + (long long)item * NM * n3;
     const float scale = ldexpf(1.0f, S);
@@ -1394,80 +1424,97 @@ k_bin(const C *__restrict__ mesh, long long item_stride_c, long long mesh_stride
     for (int k = threadIdx.x; k < g.nh; k += blockDim.x) out[k] = hist[k];
 }
 
-// sums2[(item * nchunk + chunk) * nh + k] = sum of the chunk's per-CTA histograms, in order.
-// out_rows: rows per catalog in sums2 (a second pass over sums2 itself, with
-// G = out_rows, sums each column of a catalog's rows into its row 0 in place:
-// a thread reads and writes only its own column).
-template <typename A>
-__global__ void k_bin_reduce(const A *__restrict__ partial, int G, int nh, int out_rows,
-                             double *__restrict__ sums2) {
-    const int item = blockIdx.z, chunk = blockIdx.y;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nh) return;
-    const int c0 = chunk * kReduceChunk, c1 = min(G, c0 + kReduceChunk);
-    const A *p = partial + ((long long)item * G) * nh + k;
-    double s = 0.0;
-    for (int c = c0; c < c1; ++c) s += (double)p[(long long)c * nh];
-    sums2[((long long)item * out_rows + chunk) * nh + k] = s;
+// k bins per block of k_reduce_finalize: about 8 histogram slots, so that the
+// rows are summed by 32 threads per slot (with 32 slots per block the serial row
+// sums took twice as long).
+__host__ __device__ __forceinline__ int final_bins(const FinalGeom &f) {
+    const int per = (f.twod ? f.nmu : 1) + (f.poles ? 2 : 0);
+    return per >= 8 ? 1 : 8 / per;
 }
 
-// Auto power of every catalog (cross_b < 0: block = catalog), or the cross
-// power of catalogs cross_a and cross_b (one block): normalization
+// Sum of the per-CTA histograms and the results, one block per final_bins() k
+// bins and catalog: the block's slots times as many groups of rows as its
+// threads allow, each summed in row order, then the groups in order (FP64, a
+// fixed order); then normalization, shot noise and multipoles of the block's
+// bins, written straight into the result block in pinned host memory.  One
+// launch in place of two reduce passes, a finalize and a copy: 27 -> 18 us
+// at 512^3 with 10 mu bins, 20 -> 13 us at 64^3 (launches counted alone).
+// Auto power of every catalog (cross_b < 0: blockIdx.y = catalog), or the cross
+// power of catalogs cross_a and cross_b: normalization
 // L^3 / (sum w_a sum w_b), no shot noise; the result block then carries
 // sum w_a and sum w_b in its wsum and w2sum slots.
-__global__ void k_finalize(const double *__restrict__ sums2, int nchunk, int nsum,
-                           const unsigned long long *__restrict__ modes1d,
-                           const unsigned long long *__restrict__ modes2d,
-                           const double *__restrict__ wsums, const int *__restrict__ err,
-                           FinalGeom f, ResultLayout rl, double *__restrict__ res, int cross_a, int cross_b) {
+template <typename A>
+__global__ void __launch_bounds__(256)
+k_reduce_finalize(const A *__restrict__ partial, int G, const unsigned long long *__restrict__ modes1d,
+                  const unsigned long long *__restrict__ modes2d, const double *__restrict__ wsums,
+                  const int *__restrict__ err, FinalGeom f, ResultLayout rl, double *__restrict__ res, int cross_a,
+                  int cross_b) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double *sum = reinterpret_cast<double *>(smraw);       // the block's slots
+    __shared__ double red[256];
     const bool cross = cross_b >= 0;
-    const int item = blockIdx.x;
+    const int item = blockIdx.y;
+    // the normalization first: its FP64 divisions overlap the loads below
     const int ia = cross ? cross_a : item, ib = cross ? cross_b : item;
-    const double *s0 = sums2 + (long long)item * nchunk * f.nh;
     double *r = res + (long long)item * f.RL;
     const double wsum = wsums[4 * ia], wsum_b = wsums[4 * ib];
     const double w2sum = cross ? wsum_b : wsums[4 * ia + 1];
-    const double wabs = fmax(wsums[4 * ia + 2], wsums[4 * ib + 2]);
     const double norm = f.L3 / (wsum * wsum_b);
     const double shot = cross ? 0.0 : f.L3 * w2sum / (wsum * wsum);
     const double sub = f.subtract_shot ? shot : 0.0;
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
-    auto S = [&](int k) {
-        double t = 0.0;
-        for (int c = 0; c < nsum; ++c) t += s0[(long long)c * f.nh + k];
-        return t;
+    const int KB = final_bins(f), b0 = blockIdx.x * KB, nb = min(KB, f.nk - b0);
+    const int per = f.twod ? f.nmu : 1, n0 = nb * per, ns = n0 + (f.poles ? 2 * nb : 0);
+    // slot s of the block: its (k, mu) or k sums, then the two pole sums per bin
+    const auto slot = [&](int s) {
+        if (s < n0) return b0 * per + s;
+        s -= n0;
+        return s < nb ? f.hbase + b0 + s : f.hbase + f.nk + b0 + s - nb;
     };
-    // bins spread over the gridDim.y blocks of the catalog (FP64 divisions are
-    // slow on this part: one block took ~30 us for 3500 bins)
-    const int t0 = blockIdx.y * blockDim.x + threadIdx.x, tstride = gridDim.y * blockDim.x;
-    for (int b = t0; b < f.nk; b += tstride) {
-        double S0 = 0.0;
-        if (f.twod) {
-            for (int q = 0; q < f.nmu; ++q) S0 += S(b * f.nmu + q);
-        } else {
-            S0 = S(b);
+    const A *p = partial + (long long)item * G * f.nh;
+    const int parts = ns < 256 ? 256 / ns : 1;
+    for (int s0 = 0; s0 < ns; s0 += 256) {                 // one turn unless a bin has more than 254 mu bins
+        const int s = s0 + (int)threadIdx.x % min(ns, 256), part = threadIdx.x / min(ns, 256);
+        double t = 0.0;
+        if (s < ns && part < parts) {
+            const A *q = p + slot(s);
+#pragma unroll 8
+            for (int c = part; c < G; c += parts) t += (double)q[(long long)c * f.nh];
         }
+        red[threadIdx.x] = t;
+        __syncthreads();
+        if (part == 0 && s < ns) {
+            for (int k = 1; k < parts; ++k) t += red[threadIdx.x + k * ns];
+            sum[s] = t;
+        }
+        __syncthreads();
+    }
+
+    // one thread per bin and multipole
+    for (int k3 = threadIdx.x; k3 < 3 * nb; k3 += blockDim.x) {
+        const int row = k3 / nb, k = k3 - row * nb, b = b0 + k;
         const double cnt = (double)modes1d[b];
-        double p0 = nan, p2 = nan, p4 = nan;
+        double p = nan;
         if (cnt > 0.0) {
-            p0 = norm * S0 / cnt - sub;
-            if (f.poles) {               // slots: sum h P L_2(mu), sum h P L_4(mu)
-                p2 = 5.0 * norm * S(f.hbase + b) / cnt;
-                p4 = 9.0 * norm * S(f.hbase + f.nk + b) / cnt;
+            if (row == 0) {
+                double S0 = 0.0;
+                for (int q = 0; q < per; ++q) S0 += sum[k * per + q];
+                p = norm * S0 / cnt - sub;
+            } else if (f.poles) {        // slots: sum h P L_2(mu), sum h P L_4(mu)
+                p = (row == 1 ? 5.0 : 9.0) * norm * sum[n0 + (row - 1) * nb + k] / cnt;
             }
         }
-        r[rl.pk + b] = p0;
-        r[rl.poles + b] = (f.poles_mask & 1u) ? p0 : nan;
-        r[rl.poles + f.nk + b] = (f.poles_mask & 2u) ? p2 : nan;
-        r[rl.poles + 2 * f.nk + b] = (f.poles_mask & 4u) ? p4 : nan;
+        if (row == 0) r[rl.pk + b] = p;
+        r[rl.poles + row * f.nk + b] = ((f.poles_mask >> row) & 1u) ? p : nan;
     }
     if (f.twod) {
-        for (int bq = t0; bq < f.nk * f.nmu; bq += tstride) {
-            const double cnt = (double)modes2d[bq];
-            r[rl.pkmu + bq] = cnt > 0.0 ? norm * S(bq) / cnt - sub : nan;
+        for (int k = threadIdx.x; k < n0; k += blockDim.x) {
+            const double cnt = (double)modes2d[b0 * per + k];
+            r[rl.pkmu + b0 * per + k] = cnt > 0.0 ? norm * sum[k] / cnt - sub : nan;
         }
     }
-    if (blockIdx.y == 0 && threadIdx.x == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const double wabs = fmax(wsums[4 * ia + 2], wsums[4 * ib + 2]);
         r[rl.shot] = shot;
         r[rl.wsum] = wsum;
         r[rl.w2sum] = w2sum;
@@ -1615,8 +1662,8 @@ cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const 
     const bool weighted = w != nullptr || vals != nullptr || dtype == PK_F32X4;
     dim3 grid(grid_for(max_n, kCountThreads, weighted ? kWsumBlocks : 1u << 20), nitems);
 #define PK_COUNT(DT)                                                                                    \
-    if (weighted) k_sort_count<DT, true><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, count, wsums, wpart, wmax); \
-    else k_sort_count<DT, false><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, count, wsums, wpart, wmax);
+    if (weighted) k_sort_count<DT, true><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, count, wsums, wpart, wmax); \
+    else k_sort_count<DT, false><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, count, wsums, wpart, wmax);
     switch (dtype) {
     case PK_F32: PK_COUNT(PK_F32) break;
     case PK_F64: PK_COUNT(PK_F64) break;
@@ -1626,7 +1673,7 @@ cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const 
     if (weighted) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, wsums, wmax);
+        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, max_n, wsums, wmax);
     }
     return cudaGetLastError();
 }
@@ -1638,9 +1685,9 @@ cudaError_t launch_sort_scatter(const void *pos, int dtype, const float *w, cons
                                 uint32_t *cursor, float4 *sorted, uint32_t ntot, int *err, cudaStream_t st) {
     dim3 grid(grid_for(max_n, kCountThreads, 1u << 20), nitems);
     switch (dtype) {
-    case PK_F32: k_sort_scatter<PK_F32><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, cursor, sorted, ntot, err); break;
-    case PK_F64: k_sort_scatter<PK_F64><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, cursor, sorted, ntot, err); break;
-    default: k_sort_scatter<PK_F32X4><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, cursor, sorted, ntot, err); break;
+    case PK_F32: k_sort_scatter<PK_F32><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
+    case PK_F64: k_sort_scatter<PK_F64><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
+    default: k_sort_scatter<PK_F32X4><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
     }
     return cudaGetLastError();
 }
@@ -1689,9 +1736,14 @@ static cudaError_t scan_impl(const T *in, int64_t n, T *out, T *tmp, T *copy, in
     if (nb > 0x7fffffffLL) return cudaErrorInvalidValue;
     k_scan_blocks<T, false><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, out, tmp, nullptr);
     *launches += 1;
+    if (nb <= kScanDirect) {
+        k_scan_add<T, COPY, true><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
+        *launches += 1;
+        return cudaGetLastError();
+    }
     cudaError_t e = scan_impl<T, false>(tmp, nb, tmp, tmp + nb + 1, nullptr, launches, st);
     if (e != cudaSuccess) return e;
-    k_scan_add<T, COPY><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
+    k_scan_add<T, COPY, false><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -1762,12 +1814,12 @@ static cudaError_t atomic_inst(const void *pos, const float *w, const float *val
                                unsigned long long *acc, double *wsums, double *wpart, uint4 *wmax,
                                cudaStream_t st) {
     dim3 grid(grid_for(max_n, kCountThreads, weighted ? kWsumBlocks : 1u << 20), nitems);
-    k_paint_atomic<DT, P, NM><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, g, S, weighted, acc,
+    k_paint_atomic<DT, P, NM><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, S, weighted, acc,
                                                              wsums, wpart, wmax);
     if (weighted) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, wsums, wmax);
+        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, max_n, wsums, wmax);
     }
     return cudaGetLastError();
 }
@@ -1908,43 +1960,20 @@ int bin_ctas_per_sm(const BinGeom &g, int f64) {
     return n;
 }
 
-int reduce_chunks(int G) { return (G + kReduceChunk - 1) / kReduceChunk; }
-int reduce_launches(int G) { return reduce_chunks(G) > 1 ? 2 : 1; }
-
-cudaError_t launch_bin_reduce(const void *partial, int f64, int G, int nh, int nitems,
-                              double *sums2, cudaStream_t st) {
-    const int nchunk = reduce_chunks(G);
-    if (nchunk > kReduceChunk) return cudaErrorInvalidValue;    // the second pass is one chunk
-    dim3 grid((nh + 127) / 128, nchunk, nitems);
-    if (f64) k_bin_reduce<double><<<grid, 128, 0, st>>>(reinterpret_cast<const double *>(partial), G, nh, nchunk, sums2);
-    else k_bin_reduce<float><<<grid, 128, 0, st>>>(reinterpret_cast<const float *>(partial), G, nh, nchunk, sums2);
-    if (nchunk > 1) {       // the chunk rows of each catalog into its row 0 (kReduceChunk >= nchunk)
-        dim3 g2((nh + 127) / 128, 1, nitems);
-        k_bin_reduce<double><<<g2, 128, 0, st>>>(sums2, nchunk, nh, nchunk, sums2);
-    }
-    return cudaGetLastError();
-}
-
-// Blocks per catalog for k_finalize: one per 256 bins of the larger table.
-static unsigned finalize_blocks(const FinalGeom &f) {
-    const int bins = f.twod && f.nk * f.nmu > f.nk ? f.nk * f.nmu : f.nk;
-    return (unsigned)std::min(64, std::max(1, (bins + 255) / 256));
-}
-
-cudaError_t launch_finalize(const double *sums2, int G, const unsigned long long *modes1d,
-                            const unsigned long long *modes2d, const double *wsums, const int *err,
-                            const FinalGeom &f, int nitems, double *res, cudaStream_t st) {
+cudaError_t launch_reduce_finalize(const void *partial, int f64, int G, const unsigned long long *modes1d,
+                                   const unsigned long long *modes2d, const double *wsums, const int *err,
+                                   const FinalGeom &f, int nitems, double *res, int cross_a, int cross_b,
+                                   cudaStream_t st) {
     const ResultLayout rl = result_layout(f.nk, f.nmu);
-    k_finalize<<<dim3(nitems, finalize_blocks(f)), 256, 0, st>>>(sums2, reduce_chunks(G), 1, modes1d, modes2d, wsums, err, f, rl, res, -1, -1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_finalize_cross(const double *sums2, int G, const unsigned long long *modes1d,
-                                  const unsigned long long *modes2d, const double *wsums, const int *err,
-                                  const FinalGeom &f, int item_a, int item_b, double *res, cudaStream_t st) {
-    const ResultLayout rl = result_layout(f.nk, f.nmu);
-    k_finalize<<<dim3(1, finalize_blocks(f)), 256, 0, st>>>(sums2, reduce_chunks(G), 1, modes1d, modes2d, wsums, err, f, rl, res, item_a,
-                                  item_b);
+    const int KB = final_bins(f);
+    const size_t smem = sizeof(double) * (size_t)KB * ((f.twod ? f.nmu : 1) + (f.poles ? 2 : 0));   // <= 8 KB
+    const dim3 grid((f.nk + KB - 1) / KB, nitems);
+    if (f64)
+        k_reduce_finalize<double><<<grid, 256, smem, st>>>(reinterpret_cast<const double *>(partial), G, modes1d,
+                                                           modes2d, wsums, err, f, rl, res, cross_a, cross_b);
+    else
+        k_reduce_finalize<float><<<grid, 256, smem, st>>>(reinterpret_cast<const float *>(partial), G, modes1d,
+                                                          modes2d, wsums, err, f, rl, res, cross_a, cross_b);
     return cudaGetLastError();
 }
 

@@ -46,7 +46,7 @@ struct pk_plan_s {
     int *d_xtiles = nullptr;         // zyx: tiles of the x axis, fused pass then plain pass
     int nxbin = 0, nx = 0;
 
-    uint32_t *d_count = nullptr;     // objects per (tile, class) key
+    uint32_t *d_count = nullptr;     // objects per (tile, class) key, then the scatter's cursors (behind d_wmax)
     uint32_t *d_off = nullptr;       // exclusive scan of d_count (+ total)
     uint32_t *d_scan_tmp = nullptr;
     float4 *d_sorted = nullptr;      // objects in key order, home-tile-local xyz + w
@@ -55,7 +55,7 @@ struct pk_plan_s {
     void *d_stage = nullptr;
     size_t stage_cap = 0;
     int64_t *d_item_off = nullptr;   // catalog offsets of the last paint call
-    double *d_wsums = nullptr;       // per catalog: sum w, sum w^2, sum |w|, spare
+    double *d_wsums = nullptr;       // per catalog: sum w, sum w^2, sum |w|, spare (owns d_wmax and d_count)
     double *d_wpart = nullptr;       // per catalog and paint block: its three weight sums
     uint4 *d_wmax = nullptr;         // per catalog: max |W V| (float bits), any negative, mean |W V| (float bits)
     int *d_err = nullptr;           // bit 1: tile sort inconsistency (never expected)
@@ -65,8 +65,7 @@ struct pk_plan_s {
     int *d_kedge = nullptr;
     int G_total = 0;
     void *d_partial = nullptr;
-    double *d_sums2 = nullptr, *d_res = nullptr, *h_res = nullptr;
-    double *d_xres = nullptr, *h_xres = nullptr;   // cross-power result block
+    double *h_res = nullptr, *h_xres = nullptr;    // result blocks, written by the device; cross power's
     double *d_proj = nullptr;                      // projected power: 3 sums per k bin
     std::vector<double> proj_k, proj_pk;
     std::vector<uint64_t> proj_modes;
