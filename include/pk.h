@@ -378,7 +378,7 @@ typedef struct {
 } pk_lognormal_config;
 
 /* Create a generator: validates cfg, allocates the grid buffers (about 16 +
- * 8 (f_rsd != 0) bytes per cell, 16 bytes per cell for the weights and their
+ * 8 (f_rsd != 0) bytes per cell, 8 1/4 bytes per cell for the weights'
  * prefix sums) and the cuFFT plans; all its work runs on `cuda_stream`.
  * Errors: PK_EINVAL (bad cfg; message through pk_plan_error), PK_ENOMEM,
  * PK_ECUDA, PK_ECUFFT.  On error *out is NULL. */

@@ -57,6 +57,42 @@ struct ResultLayout {
 };
 ResultLayout result_layout(int nk, int nmu);
 
+// ---- scans ----
+constexpr int kScanThreads = 1024;
+constexpr int kScanPer = 4;           // elements per thread in a scan block
+constexpr int kScanTile = kScanThreads * kScanPer;
+
+#ifdef __CUDACC__
+// Exclusive scan of one value per thread of a kScanThreads block.
+template <typename T>
+__device__ __forceinline__ T block_exclusive_scan(T v, T *total) {
+    __shared__ T wsum[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    T x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        T s = lane < kScanThreads / 32 ? wsum[lane] : (T)0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const T y = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += y;
+        }
+        if (lane < kScanThreads / 32) wsum[lane] = s;
+    }
+    __syncthreads();
+    const T before = (wid > 0 ? wsum[wid - 1] : (T)0) + x - v;
+    *total = wsum[kScanThreads / 32 - 1];
+    __syncthreads();
+    return before;
+}
+#endif
+
 // ---- launchers (pk_kernels.cu); all asynchronous on `st` ----
 int paint_classes();                  // boundary classes per tile (27)
 // dynamic shared memory of one tile-paint CTA painting nmesh meshes

@@ -65,9 +65,6 @@ constexpr unsigned kWsumBlocks = 2048;  // blocks per catalog of the passes that
 constexpr int kPaintThreads = 256;
 constexpr int kBinThreads = 256;
 constexpr int kBinVec = 4;            // consecutive modes per thread
-constexpr int kScanThreads = 1024;
-constexpr int kScanPer = 4;           // elements per thread in a scan block
-constexpr int kScanTile = kScanThreads * kScanPer;
 // Up to this many blocks every block of the second scan pass adds up the totals
 // before it itself (one load a thread at most), without a scan launch between.
 constexpr int kScanDirect = 1024;
@@ -345,34 +342,6 @@ k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const 
 }
 
 // ---- exclusive scan of uint32 counts (totals < 2^32) or uint64 weights ----
-template <typename T>
-__device__ __forceinline__ T block_exclusive_scan(T v, T *total) {
-    __shared__ T wsum[kScanThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    T x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const T y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        T s = lane < kScanThreads / 32 ? wsum[lane] : (T)0;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const T y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        if (lane < kScanThreads / 32) wsum[lane] = s;
-    }
-    __syncthreads();
-    const T before = (wid > 0 ? wsum[wid - 1] : (T)0) + x - v;
-    *total = wsum[kScanThreads / 32 - 1];
-    __syncthreads();
-    return before;
-}
-
 // out and copy (COPY: a second place for the results) may alias in: every
 // thread reads its own elements before writing them.
 template <typename T, bool COPY>

@@ -11,9 +11,11 @@
 //                 inverse transform folded in), DC = 0; psi_z~ = i k_z / k^2 G~
 //                 with DC and the z-Nyquist plane set to zero.
 //   cuFFT C2R     G and psi_z on the grid.
-//   k_ln_moments  sum G, sum G^2 (FP64) -> sigma^2.
-//   k_ln_weights  q = round(2^30 exp(G - sigma^2 / 2)) as uint64 cell weights.
-//   scan          exact exclusive prefix sums of q (uint64).
+//   k_ln_moments, k_ln_halfvar  sum G, sum G^2 -> sigma^2 / 2.
+//   k_ln_sums, scan, k_ln_scan  exact exclusive prefix sums (uint64) of the cell
+//                 weights q = round(2^30 exp(G - sigma^2 / 2)), formed from G in both
+//                 passes and never stored.
+//   k_ln_guide    the cells where equal slices of the cumulative weight begin.
 //   k_ln_place    object i (key (seed, 1), counter (i, 0, 0, 0)): cell by inverse
 //                 CDF of t = floor(w0 total / 2^64), uniform offset in the cell
 //                 from w1..w3, z + f_rsd psi_z(cell), wrapped into [0, L).
@@ -34,7 +36,6 @@ namespace pk {
 namespace {
 
 constexpr int kLnThreads = 256;
-constexpr int kCoarse = 1024;         // cells per block of the coarse CDF index
 
 struct Philox4x64 {
     unsigned long long w[4];
@@ -151,17 +152,37 @@ k_ln_shape(float2 *__restrict__ gk, float2 *__restrict__ psik, int ng, float kf2
     }
 }
 
+// a + b = s + e exactly (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float *e) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    *e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+
+// Sums of G and G^2.  A thread's sums run in pairs of FP32 numbers (the square
+// and every addition split exactly, some 48 bits), the rest in FP64: three FP64
+// operations per cell bound this kernel at 1/64 of the FP32 rate (0.75 ms for
+// 512^3 cells, now 0.13 ms; the FP32 sigma^2 / 2 that comes out is the same).
 __global__ void __launch_bounds__(kLnThreads)
 k_ln_moments(const float *__restrict__ g, int ng, long long pitch, double *__restrict__ stats) {
-    const long long ncell = (long long)ng * ng * ng;
-    double s1 = 0.0, s2 = 0.0;
+    const long long npair = (long long)ng * ng * (ng / 2);
+    float h1 = 0.0f, l1 = 0.0f, h2 = 0.0f, l2 = 0.0f;
     const long long c0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-    Walk w(c0, stride, ng);
-    for (long long c = c0; c < ncell; c += stride, w.step()) {
-        const double v = (double)g[w.row * pitch + w.col];
-        s1 += v;
-        s2 += v * v;
+    Walk w(c0, stride, ng / 2);
+    for (long long c = c0; c < npair; c += stride, w.step()) {
+        const float2 v = __ldcs(reinterpret_cast<const float2 *>(g + w.row * pitch) + w.col);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const float x = k ? v.y : v.x;
+            float e;
+            h1 = two_sum(h1, x, &e);
+            l1 = __fadd_rn(l1, e);
+            const float p = __fmul_rn(x, x), pe = __fmaf_rn(x, x, -p);
+            h2 = two_sum(h2, p, &e);
+            l2 = __fadd_rn(l2, __fadd_rn(e, pe));
+        }
     }
+    double s1 = (double)h1 + (double)l1, s2 = (double)h2 + (double)l2;
     __shared__ double r1[kLnThreads / 32], r2[kLnThreads / 32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -184,65 +205,158 @@ k_ln_moments(const float *__restrict__ g, int ng, long long pitch, double *__res
     }
 }
 
-__global__ void __launch_bounds__(kLnThreads)
-k_ln_weights(const float *__restrict__ g, int ng, long long pitch, const double *__restrict__ stats,
-             unsigned long long *__restrict__ q) {
+__global__ void k_ln_halfvar(const double *__restrict__ stats, int ng, float *__restrict__ half_var) {
+    const double ncell = (double)((long long)ng * ng * ng);
+    const double mean = stats[0] / ncell;
+    *half_var = (float)(0.5 * (stats[1] / ncell - mean * mean));
+}
+
+// Weights of the kScanPer cells from flat index c0 (a multiple of kScanPer) on;
+// 0 beyond the grid.  Rows hold an even number of cells, so pairs stay together.
+__device__ __forceinline__ void ln_weights(const float *__restrict__ g, int ng, long long pitch, long long ncell,
+                                           float half_var, long long c0, unsigned long long *q) {
+    static_assert(kScanPer == 4, "two pairs per thread");
+    long long row = 0;
+    int col = 0;
+    if (c0 < ncell) {
+        row = ncell <= 0xffffffffLL ? (long long)((unsigned)c0 / (unsigned)ng) : c0 / ng;
+        col = (int)(c0 - row * ng);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        q[2 * k] = q[2 * k + 1] = 0ull;
+        if (c0 + 2 * k < ncell) {
+            const float2 v = *reinterpret_cast<const float2 *>(g + row * pitch + col);
+            q[2 * k] = (unsigned long long)__float2ll_rn(expf(v.x - half_var) * 1073741824.0f);
+            q[2 * k + 1] = (unsigned long long)__float2ll_rn(expf(v.y - half_var) * 1073741824.0f);
+        }
+        col += 2;
+        if (col >= ng) {
+            col -= ng;
+            ++row;
+        }
+    }
+}
+
+// The two passes over the field read G (4 bytes a cell) and write the prefix sums
+// once (8): a stored weight array scanned in place and corrected moved 44 bytes a
+// cell (512^3: 1.39 -> 0.72 ms).
+__global__ void __launch_bounds__(kScanThreads)
+k_ln_sums(const float *__restrict__ g, int ng, long long pitch, const float *__restrict__ half_var,
+          unsigned long long *__restrict__ bsum) {
     const long long ncell = (long long)ng * ng * ng;
-    const double mean = stats[0] / (double)ncell;
-    const float half_var = (float)(0.5 * (stats[1] / (double)ncell - mean * mean));
-    const long long c0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-    Walk w(c0, stride, ng);
-    for (long long c = c0; c < ncell; c += stride, w.step()) {
-        const float x = g[w.row * pitch + w.col] - half_var;
-        q[c] = (unsigned long long)__float2ll_rn(expf(x) * 1073741824.0f);
+    unsigned long long q[kScanPer];
+    ln_weights(g, ng, pitch, ncell, *half_var, (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanPer, q);
+    unsigned long long s = q[0] + q[1] + q[2] + q[3];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    __shared__ unsigned long long red[kScanThreads / 32];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = red[threadIdx.x];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) bsum[blockIdx.x] = s;
     }
 }
 
-// coarse[k] = excl[min(k kCoarse, ncell)], k = 0 .. nblk: a small index that
-// stays in cache, so each object's search touches one 8 KB block of excl.
-__global__ void k_ln_coarse(const unsigned long long *__restrict__ excl, long long ncell, long long nblk,
-                            unsigned long long *__restrict__ coarse) {
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k <= nblk;
-         k += (long long)gridDim.x * blockDim.x) {
-        const long long c = k * kCoarse;
-        coarse[k] = excl[c < ncell ? c : ncell];
+__global__ void __launch_bounds__(kScanThreads)
+k_ln_scan(const float *__restrict__ g, int ng, long long pitch, const float *__restrict__ half_var,
+          const unsigned long long *__restrict__ boff, int nblk, unsigned long long *__restrict__ excl) {
+    const long long ncell = (long long)ng * ng * ng;
+    const long long c0 = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanPer;
+    unsigned long long q[kScanPer], total;
+    ln_weights(g, ng, pitch, ncell, *half_var, c0, q);
+    unsigned long long run = boff[blockIdx.x] +
+                             block_exclusive_scan<unsigned long long>(q[0] + q[1] + q[2] + q[3], &total);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (c0 + 2 * k < ncell)
+            *reinterpret_cast<ulonglong2 *>(excl + c0 + 2 * k) = make_ulonglong2(run, run + q[2 * k]);
+        run += q[2 * k] + q[2 * k + 1];
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) excl[ncell] = boff[nblk];
 }
 
+// guide[j] = the cell that holds cumulative weight floor(j 2^-k total), j < 2^k, and
+// guide[2^k] = the last cell.  An object whose 64-bit draw starts with the k bits
+// j lies between guide[j] and guide[j + 1].
 __global__ void __launch_bounds__(kLnThreads)
-k_ln_place(const unsigned long long *__restrict__ excl, const unsigned long long *__restrict__ coarse,
-           long long nblk, int ng, double L, const float *__restrict__ psi, long long pitch, float f_rsd,
-           unsigned long long seed, long long n, float *__restrict__ pos) {
+k_ln_guide(const unsigned long long *__restrict__ excl, long long ncell, int k, unsigned *__restrict__ guide_lo,
+           unsigned char *__restrict__ guide_hi) {
+    const unsigned long long total = excl[ncell];
+    const long long n = 1LL << k;
+    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j <= n; j += (long long)gridDim.x * blockDim.x) {
+        long long a = 0, b = ncell;                       // excl[a] <= t < excl[b]
+        if (j == n) {
+            a = ncell - 1;
+        } else {
+            const unsigned long long t = __umul64hi((unsigned long long)j << (64 - k), total);
+            while (b - a > 1) {
+                const long long mid = a + ((b - a) >> 1);
+                if (excl[mid] <= t) a = mid;
+                else b = mid;
+            }
+        }
+        guide_lo[j] = (unsigned)a;
+        if (guide_hi) guide_hi[j] = (unsigned char)(a >> 32);
+    }
+}
+
+// Twice ((x >> 40) + 1/2 rounded to FP32) for the top 24 bits of a word: uniform24(x)
+// = twice_uniform24(x) 2^-25, as an integer.
+__device__ __forceinline__ unsigned twice_uniform24(unsigned long long x) {
+    const unsigned k = (unsigned)(x >> 40);
+    return k < (1u << 23) ? 2u * k + 1u : 2u * (k + (k & 1u));      // ties to even above 2^23
+}
+
+// The cell by binary search between two guide entries (about 16 cells, a line,
+// apart: 4 probes, for 27 of the whole array through a coarse index; slices of 64
+// cells: k_ln_guide 281 -> 172 us, this kernel 851 -> 1177 us), and the coordinates
+// with 13 FP64 operations (they are at 1/64 rate): (i + u) H as one conversion and
+// one product of an integer, exactly the same value; the division of the
+// periodic wrap only outside [0, L).  1e7 objects on 512^3: 1.98 -> 0.85 ms.
+__global__ void __launch_bounds__(kLnThreads)
+k_ln_place(const unsigned long long *__restrict__ excl, const unsigned *__restrict__ guide_lo,
+           const unsigned char *__restrict__ guide_hi, int kbits, int ng, double L, const float *__restrict__ psi,
+           long long pitch, float f_rsd, unsigned long long seed, long long n, float *__restrict__ pos) {
     const long long ncell = (long long)ng * ng * ng;
     const unsigned long long total = excl[ncell];
-    const double H = L / ng;
+    const double H = L / ng, Hs = H * 2.9802322387695312e-8;          // H 2^-25
+    const float Lf = (float)L;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const Philox4x64 r = philox4x64((unsigned long long)i, seed, 1ull);
         const unsigned long long t = __umul64hi(r.w[0], total);
-        long long ka = 0, kb = nblk;                      // coarse[ka] <= t < coarse[kb]
-        while (kb - ka > 1) {
-            const long long mid = ka + ((kb - ka) >> 1);
-            if (coarse[mid] <= t) ka = mid;
-            else kb = mid;
+        const unsigned long long j = r.w[0] >> (64 - kbits);
+        long long a = guide_lo[j], b = guide_lo[j + 1];
+        if (guide_hi) {
+            a |= (long long)guide_hi[j] << 32;
+            b |= (long long)guide_hi[j + 1] << 32;
         }
-        long long a = ka * kCoarse, b = kb * kCoarse < ncell ? kb * kCoarse : ncell;   // excl[a] <= t < excl[b]
+        ++b;                                              // excl[a] <= t < excl[b]
         while (b - a > 1) {
             const long long mid = a + ((b - a) >> 1);
             if (excl[mid] <= t) a = mid;
             else b = mid;
         }
-        const long long c = a;
-        const long long ix = c / ((long long)ng * ng), iy = (c / ng) % ng, iz = c % ng;
-        double z = ((double)iz + (double)uniform24(r.w[3])) * H;
-        if (psi) z += (double)f_rsd * (double)psi[(c / ng) * pitch + iz];
-        z = z - L * floor(z / L);
-        if (z >= L) z -= L;
+        const long long row = guide_hi ? a / ng : (long long)((unsigned)a / (unsigned)ng);
+        const int iz = (int)(a - row * ng);
+        const int ix = (int)((unsigned)row / (unsigned)ng), iy = (int)((unsigned)row - (unsigned)ix * (unsigned)ng);
+        const auto node = [&](int c, unsigned long long w) {           // (c + uniform24(w)) 2^25
+            return (double)(((long long)c << 25) + (long long)twice_uniform24(w));
+        };
+        double z = node(iz, r.w[3]) * Hs;
+        if (psi) z += (double)f_rsd * (double)psi[row * pitch + iz];
+        if (!(z >= 0.0 && z < L)) {
+            z = z - L * floor(z / L);
+            if (z >= L) z -= L;
+        }
         // FP32 rounding can reach L exactly: that point is 0 on the periodic box
-        float xf = (float)(((double)ix + (double)uniform24(r.w[1])) * H);
-        float yf = (float)(((double)iy + (double)uniform24(r.w[2])) * H);
-        float zf = (float)z;
-        const float Lf = (float)L;
+        const float xf = (float)(node(ix, r.w[1]) * Hs);
+        const float yf = (float)(node(iy, r.w[2]) * Hs);
+        const float zf = (float)z;
         pos[3 * i + 0] = xf >= Lf ? 0.0f : xf;
         pos[3 * i + 1] = yf >= Lf ? 0.0f : yf;
         pos[3 * i + 2] = zf >= Lf ? 0.0f : zf;
@@ -269,12 +383,14 @@ struct pk_lognormal_s {
     double amp = 0.0;
     float *g = nullptr;              // G (in-place r2c / c2r layout)
     float *psi = nullptr;            // psi_z (same layout), if f_rsd != 0
-    unsigned long long *q = nullptr;     // cell weights
-    unsigned long long *excl = nullptr;  // exclusive prefix sums, excl[ncell] = total
-    unsigned long long *coarse = nullptr;  // excl at every kCoarse-th cell (and at ncell)
-    long long nblk = 0;
+    unsigned long long *excl = nullptr;  // exclusive prefix sums of the cell weights, excl[ncell] = total
+    long long nblk = 0;                  // scan blocks
+    unsigned long long *bsum = nullptr;  // their weights, then their offsets (+ total)
     unsigned long long *scan_tmp = nullptr;
-    double *stats = nullptr;
+    int kguide = 1;                      // largest guide: 2^kguide slices, about one per 16 cells
+    unsigned *guide_lo = nullptr;        // low 32 bits of the guide's cells
+    unsigned char *guide_hi = nullptr;   // bits 32 .. 39 (grids of 2^32 cells and more)
+    double *stats = nullptr;             // sum G, sum G^2; then sigma^2 / 2 (float)
     cufftHandle fwd = 0, inv = 0;
     bool fwd_made = false, inv_made = false;
     long long launches = 0;
@@ -310,7 +426,7 @@ void ln_free(pk_lognormal_s *G) {
     if (G->st || G->g) cudaStreamSynchronize(G->st);
     if (G->fwd_made) cufftDestroy(G->fwd);
     if (G->inv_made) cufftDestroy(G->inv);
-    void *dev[] = {G->g, G->psi, G->q, G->excl, G->coarse, G->scan_tmp, G->stats};
+    void *dev[] = {G->g, G->psi, G->excl, G->bsum, G->guide_lo, G->guide_hi, G->scan_tmp, G->stats};
     for (void *d : dev)
         if (d) cudaFree(d);
     delete G;
@@ -375,15 +491,18 @@ pk_status pk_lognormal_plan(const pk_lognormal_config *cfg, void *cuda_stream, p
     const size_t grid_bytes = sizeof(float) * (size_t)(ng * ng * G->pitch);
     cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&G->g), grid_bytes);
     if (e == cudaSuccess && c.f_rsd != 0.0) e = cudaMalloc(reinterpret_cast<void **>(&G->psi), grid_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&G->q), sizeof(unsigned long long) * ncell);
     if (e == cudaSuccess)
         e = cudaMalloc(reinterpret_cast<void **>(&G->excl), sizeof(unsigned long long) * (ncell + 1));
+    G->nblk = (ncell + kScanTile - 1) / kScanTile;
     if (e == cudaSuccess)
-        e = cudaMalloc(reinterpret_cast<void **>(&G->scan_tmp), sizeof(unsigned long long) * scan_tmp_elems(ncell));
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&G->stats), 2 * sizeof(double));
-    G->nblk = (ncell + kCoarse - 1) / kCoarse;
+        e = cudaMalloc(reinterpret_cast<void **>(&G->bsum), sizeof(unsigned long long) * (G->nblk + 1));
     if (e == cudaSuccess)
-        e = cudaMalloc(reinterpret_cast<void **>(&G->coarse), sizeof(unsigned long long) * (G->nblk + 1));
+        e = cudaMalloc(reinterpret_cast<void **>(&G->scan_tmp), sizeof(unsigned long long) * scan_tmp_elems(G->nblk));
+    while ((32LL << G->kguide) <= ncell) ++G->kguide;
+    const size_t nguide = ((size_t)1 << G->kguide) + 1;
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&G->guide_lo), sizeof(unsigned) * nguide);
+    if (e == cudaSuccess && ncell > 0xffffffffLL) e = cudaMalloc(reinterpret_cast<void **>(&G->guide_hi), nguide);
+    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&G->stats), 3 * sizeof(double));
     if (e != cudaSuccess) {
         G->err = std::string("device allocation: ") + cudaGetErrorString(e);
         return bail(e == cudaErrorMemoryAllocation ? PK_ENOMEM : PK_ECUDA);
@@ -465,21 +584,30 @@ pk_status pk_lognormal_draw(pk_lognormal_t G, uint64_t seed, int64_t n, float *p
     const int ng = G->ng;
     const long long ncell = (long long)ng * ng * ng;
     LN_CUDA(G, cudaMemsetAsync(G->stats, 0, 2 * sizeof(double), G->st));
-    k_ln_moments<<<grid_of(ncell, G->nsm), kLnThreads, 0, G->st>>>(G->g, ng, G->pitch, G->stats);
+    k_ln_moments<<<grid_of(ncell / 2, G->nsm), kLnThreads, 0, G->st>>>(G->g, ng, G->pitch, G->stats);
     LN_CUDA(G, cudaGetLastError());
-    k_ln_weights<<<grid_of(ncell, G->nsm), kLnThreads, 0, G->st>>>(G->g, ng, G->pitch, G->stats, G->q);
+    float *half_var = reinterpret_cast<float *>(G->stats + 2);
+    k_ln_halfvar<<<1, 1, 0, G->st>>>(G->stats, ng, half_var);
     LN_CUDA(G, cudaGetLastError());
     int launches = 0;
-    LN_CUDA(G, launch_scan64(G->q, ncell, G->excl, G->scan_tmp, &launches, G->st));
-    k_ln_coarse<<<grid_of(G->nblk + 1, G->nsm), kLnThreads, 0, G->st>>>(G->excl, ncell, G->nblk, G->coarse);
+    k_ln_sums<<<(unsigned)G->nblk, kScanThreads, 0, G->st>>>(G->g, ng, G->pitch, half_var, G->bsum);
+    LN_CUDA(G, cudaGetLastError());
+    LN_CUDA(G, launch_scan64(G->bsum, G->nblk, G->bsum, G->scan_tmp, &launches, G->st));
+    k_ln_scan<<<(unsigned)G->nblk, kScanThreads, 0, G->st>>>(G->g, ng, G->pitch, half_var, G->bsum, (int)G->nblk,
+                                                             G->excl);
     LN_CUDA(G, cudaGetLastError());
     if (n > 0) {
-        k_ln_place<<<grid_of(n, G->nsm), kLnThreads, 0, G->st>>>(G->excl, G->coarse, G->nblk, ng, G->cfg.box_size,
-                                                                  G->psi, G->pitch, (float)G->cfg.f_rsd, seed,
-                                                                  (long long)n, pos);
+        int k = 1;                        // no more slices than objects
+        while (k < G->kguide && (2LL << k) <= n) ++k;
+        k_ln_guide<<<grid_of((1LL << k) + 1, G->nsm), kLnThreads, 0, G->st>>>(G->excl, ncell, k, G->guide_lo,
+                                                                               G->guide_hi);
+        LN_CUDA(G, cudaGetLastError());
+        k_ln_place<<<grid_of(n, G->nsm), kLnThreads, 0, G->st>>>(G->excl, G->guide_lo, G->guide_hi, k, ng,
+                                                                  G->cfg.box_size, G->psi, G->pitch,
+                                                                  (float)G->cfg.f_rsd, seed, (long long)n, pos);
         LN_CUDA(G, cudaGetLastError());
     }
-    G->launches += 4 + launches + (n > 0);
+    G->launches += 4 + launches + 2 * (n > 0);
     return PK_OK;
 }
 
