@@ -48,6 +48,7 @@ constexpr int kPrepCtasPerSm = 4;
 constexpr int kSums = 5;                // per catalog: sum wc, sum w^2, sum nbar wc wf^2, outside, rejected
 constexpr int kRowThreads = 256;        // warp-per-row kernels
 constexpr int kChiNodes = 8192;
+constexpr int kTrigNodes = 1440;        // quarter degrees
 constexpr double kCOverH0 = 2997.92458;
 constexpr int kConst = 16;              // constants block: see k_survey_const
 
@@ -108,28 +109,65 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Cubic Hermite interpolation of chi(z) from nodes k dz carrying (chi, dchi/dz).
-__device__ __forceinline__ double chi_of_z(const double2 *__restrict__ tab, int n, double inv_dz, double dz,
-                                           double z) {
-    double t = z * inv_dz;
-    int k = (int)t;
-    if (k > n - 2) k = n - 2;
-    if (k < 0) k = 0;
-    const double u = t - (double)k;
-    const double2 a = tab[k], b = tab[k + 1];
-    const double u2 = u * u, u3 = u2 * u;
-    const double h00 = 2.0 * u3 - 3.0 * u2 + 1.0, h10 = u3 - 2.0 * u2 + u;
-    const double h01 = -2.0 * u3 + 3.0 * u2, h11 = u3 - u2;
-    return h00 * a.x + h10 * dz * a.y + h01 * b.x + h11 * dz * b.y;
-}
-
+// FP64 runs at 1/64 of the FP32 rate on this part and bounds the conversion, so it
+// is written in few FP64 operations (some 60 per sky object; 11e6 objects 2.58 ->
+// 1.43 ms): polynomial coefficients per interval of chi(z), sines from a table
+// of quarter degrees and a short series, range tests on bit patterns.
 struct PrepArgs {
     double ox, oy, oz, L;       // box origin (observer frame), box edge
     double p0;                  // > 0: w_fkp = 1 / (1 + nbar p0)
-    const double2 *chi;         // sky input: (chi, dchi/dz) at k dz
+    const double2 *chi;         // sky input: two double2 per node k dz, the cubic's coefficients in
+                                // u = z / dz - k; then cos, sin of m / 4 degrees, m < 1440
     int nchi;
     double dz, inv_dz, zmax;
+    float zmax_f;               // the largest float <= zmax
 };
+
+// chi(z): the cubic Hermite interpolant of (chi, dchi/dz) at the nodes, as a
+// polynomial in the interval.
+__device__ __forceinline__ double chi_of_z(const PrepArgs &a, double z) {
+    const double t = z * a.inv_dz;
+    const int k = max(0, min((int)t, a.nchi - 2));
+    const double u = t - (double)k;
+    const double2 c01 = __ldg(a.chi + 2 * k), c23 = __ldg(a.chi + 2 * k + 1);
+    return fma(fma(fma(c23.y, u, c23.x), u, c01.y), u, c01.x);
+}
+
+// sin and cos of an angle in degrees: d = m / 4 + r exactly, |r| <= 1/8; table
+// entries of m / 4, the series of r's sine and cosine (next terms below 2e-19) and
+// the addition theorem, about an ulp in all.
+template <typename P>
+__device__ __forceinline__ void sincos_deg(P d, const double2 *__restrict__ trig, double *s, double *c) {
+    if (!(fabs((double)d) < 1.0e6)) {                    // also NaN
+        sincospi((double)d / 180.0, s, c);
+        return;
+    }
+    int k;
+    double r;
+    if constexpr (sizeof(P) == 4) {
+        const float kf = rintf(4.0f * d);
+        k = (int)kf;
+        r = (double)fmaf(kf, -0.25f, d);                  // exact: both are multiples of d's last place
+    } else {
+        const double kd = rint(4.0 * d);
+        k = (int)kd;
+        r = fma(kd, -0.25, d);
+    }
+    k %= 1440;
+    if (k < 0) k += 1440;
+    const double2 t = __ldg(trig + k);                    // cos, sin
+    const double th = r * 0.017453292519943295, t2 = th * th;
+    const double sr = fma(fma(t2, 1.0 / 120.0, -1.0 / 6.0) * t2, th, th);       // sin th
+    const double cr = fma(t2, 1.0 / 24.0, -0.5) * t2;                          // cos th - 1
+    *s = t.y + fma(t.y, cr, t.x * sr);
+    *c = t.x + fma(t.x, cr, -(t.y * sr));
+}
+
+// 0 <= v < L on the bit patterns of non-negative doubles (-0 counts as 0).
+__device__ __forceinline__ bool in_range(double v, double L) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    return b < (unsigned long long)__double_as_longlong(L) || (b << 1) == 0ull;
+}
 
 // Observer-frame position of object i: Cartesian input as given; sky input
 // (RA, Dec in degrees, z) through chi(z).  False (and the box origin) for a
@@ -137,25 +175,30 @@ struct PrepArgs {
 template <typename P, bool SKY>
 __device__ __forceinline__ bool observer_xyz(const P *__restrict__ pos, long long i, const PrepArgs &a, double *x,
                                              double *y, double *z) {
-    const double c0 = (double)pos[3 * i], c1 = (double)pos[3 * i + 1], c2 = (double)pos[3 * i + 2];
+    const P c0 = pos[3 * i], c1 = pos[3 * i + 1], c2 = pos[3 * i + 2];
     if (!SKY) {
-        *x = c0;
-        *y = c1;
-        *z = c2;
+        *x = (double)c0;
+        *y = (double)c1;
+        *z = (double)c2;
         return true;
     }
-    if (!(c2 >= 0.0 && c2 <= a.zmax)) {
+    bool ok;
+    if constexpr (sizeof(P) == 4) ok = c2 >= 0.0f && c2 <= a.zmax_f;
+    else ok = c2 >= 0.0 && c2 <= a.zmax;
+    if (!ok) {
         *x = a.ox;
         *y = a.oy;
         *z = a.oz;
         return false;
     }
-    const double r = chi_of_z(a.chi, a.nchi, a.inv_dz, a.dz, c2);
+    const double r = chi_of_z(a, (double)c2);
+    const double2 *trig = a.chi + 2 * a.nchi;
     double sr, cr, sd, cd;
-    sincospi(c0 / 180.0, &sr, &cr);
-    sincospi(c1 / 180.0, &sd, &cd);
-    *x = r * cd * cr;
-    *y = r * cd * sr;
+    sincos_deg<P>(c0, trig, &sr, &cr);
+    sincos_deg<P>(c1, trig, &sd, &cd);
+    const double rc = r * cd;
+    *x = rc * cr;
+    *y = rc * sr;
     *z = r * sd;
     return true;
 }
@@ -216,22 +259,25 @@ k_survey_prep(const P *__restrict__ pos, long long n, const float *__restrict__ 
               const float *__restrict__ wfkp, const float *__restrict__ nbar, PrepArgs a,
               float4 *__restrict__ out4, double *__restrict__ out3, float *__restrict__ wout,
               double *__restrict__ partial) {
-    double s_wc = 0.0, s_w2 = 0.0, s_n = 0.0, s_out = 0.0, s_rej = 0.0;
+    double s_wc = 0.0, s_w2 = 0.0, s_n = 0.0;
+    int n_out = 0, n_rej = 0, n_ok = 0;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         double wc = wcomp ? (double)wcomp[i] : 1.0;
         const double nb = nbar ? (double)nbar[i] : 0.0;
-        double wf = a.p0 > 0.0 ? 1.0 / (1.0 + nb * a.p0) : (wfkp ? (double)wfkp[i] : 1.0);
+        double wf = a.p0 > 0.0 ? 1.0 / fma(nb, a.p0, 1.0) : (wfkp ? (double)wfkp[i] : 1.0);
         double x, y, z;
         const bool ok = observer_xyz<P, SKY>(pos, i, a, &x, &y, &z);
         if (!ok) {
             wc = 0.0;
             wf = 0.0;
-            s_rej += 1.0;
+            ++n_rej;
+        } else {
+            ++n_ok;
         }
         const double bx = x - a.ox, by = y - a.oy, bz = z - a.oz;
-        if (ok && !(bx >= 0.0 && bx < a.L && by >= 0.0 && by < a.L && bz >= 0.0 && bz < a.L)) s_out += 1.0;
-        const double w = wc * wf;
+        if (ok && !(in_range(bx, a.L) && in_range(by, a.L) && in_range(bz, a.L))) ++n_out;
+        const double w = wcomp ? wc * wf : wf;
         if (F64OUT) {
             out3[3 * i] = bx;
             out3[3 * i + 1] = by;
@@ -240,10 +286,12 @@ k_survey_prep(const P *__restrict__ pos, long long n, const float *__restrict__ 
         } else {
             out4[i] = make_float4((float)bx, (float)by, (float)bz, (float)w);
         }
-        s_wc += wc;
-        s_w2 += w * w;
-        s_n += nb * wc * wf * wf;
+        if (wcomp) s_wc += wc;
+        s_w2 = fma(w, w, s_w2);
+        if (nbar) s_n = fma(nb * w, wf, s_n);
     }
+    if (!wcomp) s_wc = (double)n_ok;
+    const double s_out = (double)n_out, s_rej = (double)n_rej;
     __shared__ double red[kPrepThreads / 32][kSums];
     const double v[kSums] = {s_wc, s_w2, s_n, s_out, s_rej};
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -266,14 +314,15 @@ k_survey_prep(const P *__restrict__ pos, long long n, const float *__restrict__ 
 __global__ void k_survey_const(const double *__restrict__ pd, int gd, const double *__restrict__ pr, int gr,
                                double *__restrict__ c) {
     __shared__ double s[2][kSums];
-    const int t = threadIdx.x;
-    if (t < 2 * kSums) {
-        const int cat = t / kSums, k = t % kSums;
+    const int t = threadIdx.x, lane = t & 31;
+    if (t < 64 * kSums) {                            // one warp per sum, lanes in turn, then a fixed tree
+        const int cat = t / (32 * kSums), k = t / 32 % kSums;
         const double *p = cat == 0 ? pd : pr;
         const int g = cat == 0 ? gd : gr;
         double acc = 0.0;
-        for (int b = 0; b < g; ++b) acc += p[(long long)b * kSums + k];
-        s[cat][k] = acc;
+        for (int b = lane; b < g; b += 32) acc += p[(long long)b * kSums + k];
+        acc = warp_sum(acc);
+        if (lane == 0) s[cat][k] = acc;
     }
     __syncthreads();
     if (t == 0) {
@@ -338,11 +387,14 @@ __device__ __forceinline__ C cmulc(C a, C b) {
 }
 
 // A_0 = (F~1 + F~2 e^{i pi (i' + j' + l) / N}) / 2 on every mode with no
-// index at N/2 (zero there); F~1 <- A_0 / N^3 for the inverse transform.
+// index at N/2 (zero there); F~1 <- A_0 / N^3 for the inverse transform.  A_0
+// itself is read by the bin pass only: modes with m >= mhi are not written.
+// Four modes per lane in flight (512^3: 0.91 -> 0.32 ms).
 template <typename R, typename C>
 __global__ void __launch_bounds__(kRowThreads)
 k_survey_interlace(C *__restrict__ f1, const C *__restrict__ f2, C *__restrict__ a0, const C *__restrict__ ph,
-                   int N, int Nh, R inv_n3) {
+                   int N, int Nh, R inv_n3, int mhi) {
+    constexpr int V = 4;
     const int half = N / 2;
     const long long rows = (long long)N * N;
     const int lane = threadIdx.x & 31;
@@ -351,24 +403,38 @@ k_survey_interlace(C *__restrict__ f1, const C *__restrict__ f2, C *__restrict__
     for (long long row = w0; row < rows; row += nw) {
         const int i = (int)(row / N), j = (int)(row - (long long)i * N);
         const int ip = i < half ? i : i - N, jp = j < half ? j : j - N;
+        const int r2 = ip * ip + jp * jp;
         const bool nyq_row = i == half || j == half;
         const C rp = cmulc(ph[ip + half], ph[jp + half]);
         const long long base = row * Nh;
-        for (int l = lane; l < Nh; l += 32) {
-            C z;
-            z.x = (R)0;
-            z.y = (R)0;
-            if (!nyq_row && l != half) {
-                const C a = f1[base + l], b = f2[base + l];
-                const C t = cmulc(rp, ph[l + half]);
-                z.x = (R)0.5 * (a.x + b.x * t.x - b.y * t.y);
-                z.y = (R)0.5 * (a.y + b.x * t.y + b.y * t.x);
+        for (int l0 = lane; l0 < Nh; l0 += 32 * V) {
+            C a[V], b[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int l = l0 + 32 * v;
+                if (l < half && !nyq_row) {
+                    a[v] = f1[base + l];
+                    b[v] = __ldcs(f2 + base + l);
+                }
             }
-            a0[base + l] = z;
-            C s;
-            s.x = z.x * inv_n3;
-            s.y = z.y * inv_n3;
-            f1[base + l] = s;
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const int l = l0 + 32 * v;
+                if (l >= Nh) break;
+                C z;
+                z.x = (R)0;
+                z.y = (R)0;
+                if (l < half && !nyq_row) {
+                    const C t = cmulc(rp, ph[l + half]);
+                    z.x = (R)0.5 * (a[v].x + b[v].x * t.x - b[v].y * t.y);
+                    z.y = (R)0.5 * (a[v].y + b[v].x * t.y + b[v].y * t.x);
+                }
+                if (r2 + l * l < mhi) a0[base + l] = z;
+                C s;
+                s.x = z.x * inv_n3;
+                s.y = z.y * inv_n3;
+                f1[base + l] = s;
+            }
         }
     }
 }
@@ -547,20 +613,23 @@ __global__ void k_survey_final(const double *__restrict__ partial, int G, int nk
                                unsigned mask, int subtract_shot, const int *__restrict__ err,
                                double *__restrict__ res) {
     const double nan = __longlong_as_double(0x7ff8000000000000LL);
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 3 * nk; k += gridDim.x * blockDim.x) {
-        const int row = k / nk, b = k - row * nk;
+    // eight sums per block, 32 threads each: rows in turn, then a fixed tree
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k < 3 * nk) {
         double t = 0.0;
-        for (int q = 0; q < G; ++q) t += partial[(long long)q * 3 * nk + k];
-        const double md = (double)modes[b];
-        double p = nan;
-        if ((mask >> row) & 1u) {
-            if (md > 0.0) {
+        for (int q = lane; q < G; q += 32) t += partial[(long long)q * 3 * nk + k];
+        t = warp_sum(t);
+        if (lane == 0) {
+            const int row = k / nk, b = k - row * nk;
+            const double md = (double)modes[b];
+            double p = nan;
+            if (((mask >> row) & 1u) && md > 0.0) {
                 const double norm = c[1];
                 if (row == 0) p = t / (md * norm) - (subtract_shot ? c[2] : 0.0);
                 else p = 4.0 * M_PI * t / (md * norm);
             }
+            res[k] = p;
         }
-        res[k] = p;
     }
     if (blockIdx.x == 0 && threadIdx.x < kConst)
         res[3 * nk + threadIdx.x] = threadIdx.x == kConst - 1 ? (double)(*err & 6) : c[threadIdx.x];
@@ -595,7 +664,7 @@ struct pk_survey_s {
     int64_t obj_cap = 0;
     void *stage = nullptr;          // host inputs copied here
     size_t stage_cap = 0;
-    double2 *chi = nullptr;         // (chi, dchi/dz) at k dz
+    double2 *chi = nullptr;         // sky tables (see PrepArgs)
     double dz = 0.0;
     int G = 0;                      // prep CTAs per catalog
     double *psum = nullptr;         // [2][G][kSums]
@@ -685,14 +754,17 @@ void free_survey(pk_survey_s *S) {
 
 double inv_E(double z, double om) { return 1.0 / sqrt(om * (1.0 + z) * (1.0 + z) * (1.0 + z) + 1.0 - om); }
 
-// chi at nodes k dz by composite 8-point Gauss-Legendre quadrature, FP64.
-void chi_table(double om, double zmax, std::vector<double> &tab, double *dz_out) {
+// Tables for sky input: chi at nodes k dz by composite 8-point Gauss-Legendre
+// quadrature, FP64, as the coefficients (four per node) of the cubic Hermite
+// interpolant on [k, k + 1] dz; then cos and sin of m / 4 degrees, m < 1440.
+void sky_tables(double om, double zmax, std::vector<double> &tab, double *dz_out) {
     static const double gx[4] = {0.1834346424956498, 0.5255324099163290, 0.7966664774136267,
                                  0.9602898564975363};
     static const double gw[4] = {0.3626837833783620, 0.3137066458778873, 0.2223810344533745,
                                  0.1012285362903763};
     const double dz = zmax / (kChiNodes - 1);
-    tab.assign(2 * kChiNodes, 0.0);
+    tab.assign(4 * kChiNodes + 2 * kTrigNodes, 0.0);
+    std::vector<double> x(kChiNodes), d(kChiNodes);
     double chi = 0.0;
     for (int k = 0; k < kChiNodes; ++k) {
         const double z = k * dz;
@@ -703,10 +775,31 @@ void chi_table(double om, double zmax, std::vector<double> &tab, double *dz_out)
                 acc += gw[q] * (inv_E(mid - hw * gx[q], om) + inv_E(mid + hw * gx[q], om));
             chi += kCOverH0 * hw * acc;
         }
-        tab[2 * k] = chi;
-        tab[2 * k + 1] = kCOverH0 * inv_E(z, om);
+        x[k] = chi;
+        d[k] = kCOverH0 * inv_E(z, om) * dz;
+    }
+    for (int k = 0; k + 1 < kChiNodes; ++k) {
+        double *c = tab.data() + 4 * k;
+        const double dx = x[k + 1] - x[k];
+        c[0] = x[k];
+        c[1] = d[k];
+        c[2] = 3.0 * dx - 2.0 * d[k] - d[k + 1];
+        c[3] = d[k] + d[k + 1] - 2.0 * dx;
+    }
+    for (int m = 0; m < kTrigNodes; ++m) {
+        const int q = m / 360, r = m % 360;                // quarter turn, quarter degrees within it
+        const long double th = 3.14159265358979323846264338327950288L * r / 720.0L;
+        const double c = r == 0 ? 1.0 : (double)cosl(th), s = r == 0 ? 0.0 : (double)sinl(th);
+        tab[4 * kChiNodes + 2 * m] = q == 0 ? c : q == 1 ? -s : q == 2 ? -c : s;
+        tab[4 * kChiNodes + 2 * m + 1] = q == 0 ? s : q == 1 ? c : q == 2 ? -s : -c;
     }
     *dz_out = dz;
+}
+
+// The largest float <= v (v >= 0).
+float float_below(double v) {
+    const float f = (float)v;
+    return (double)f <= v ? f : nextafterf(f, 0.0f);
 }
 
 // Copy a host array into the staging buffer at byte offset `at` (device
@@ -811,7 +904,7 @@ static pk_status survey_build(pk_survey_s *S, const pk_survey_config *cfg, void 
     }
     if (c.omega_m > 0.0) {
         std::vector<double> tab;
-        chi_table(c.omega_m, S->cfg.zmax, tab, &S->dz);
+        sky_tables(c.omega_m, S->cfg.zmax, tab, &S->dz);
         SV_CUDA(S, cudaMalloc(reinterpret_cast<void **>(&S->chi), sizeof(double) * tab.size()));
         SV_CUDA(S, cudaMemcpy(S->chi, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
     }
@@ -961,6 +1054,7 @@ static pk_status prep_catalog(pk_survey_s *S, const pk_survey_catalog *c, int64_
     a.dz = S->dz;
     a.inv_dz = S->dz > 0.0 ? 1.0 / S->dz : 0.0;
     a.zmax = S->cfg.zmax;
+    a.zmax_f = float_below(a.zmax);
     const int64_t cap = S->obj_cap;
     float4 *o4 = S->f64 ? nullptr : reinterpret_cast<float4 *>(S->obj) + at;
     double *o3 = S->f64 ? reinterpret_cast<double *>(S->obj) + 3 * at : nullptr;
@@ -1016,7 +1110,7 @@ pk_status pk_survey_paint(pk_survey_t S, const pk_survey_catalog *data, const pk
         s = prep_catalog(S, randoms, nd, 1);
         if (s != PK_OK) return s;
     }
-    k_survey_const<<<1, 32, 0, S->st>>>(S->psum, S->G, S->psum + (size_t)S->G * kSums, S->G, S->cst);
+    k_survey_const<<<1, 64 * kSums, 0, S->st>>>(S->psum, S->G, S->psum + (size_t)S->G * kSums, S->G, S->cst);
     SV_CUDA(S, cudaGetLastError());
     S->launches += 1;
     SV_CUDA(S, tmark(S, 0, PK_SURVEY_STAGE_PAINT));
@@ -1098,7 +1192,7 @@ static pk_status survey_compute_t(pk_survey_s *S) {
         SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FIELD));
         k_survey_interlace<R, C><<<rowblocks, kRowThreads, 0, st>>>(f1, f1 + mr / 2, A0,
                                                                     reinterpret_cast<const C *>(P->d_ph), N, Nh,
-                                                                    inv_n3);
+                                                                    inv_n3, P->bg.mhi);
         SV_CUDA(S, cudaGetLastError());
         S->launches += 2;
         if (nslot > 0) {
@@ -1195,7 +1289,7 @@ static pk_status survey_compute_t(pk_survey_s *S) {
     }
     const int nk = g.nk;
     SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FINAL));
-    k_survey_final<<<(3 * nk + 127) / 128, 128, 0, st>>>(S->partial, S->Gb, nk, P->d_modes1d, S->cst,
+    k_survey_final<<<(3 * nk + 7) / 8, 256, 0, st>>>(S->partial, S->Gb, nk, P->d_modes1d, S->cst,
                                                          S->cfg.poles_mask | 1u, S->cfg.subtract_shot, P->d_err, S->res);
     SV_CUDA(S, cudaGetLastError());
     S->launches += 1;
@@ -1283,7 +1377,8 @@ pk_status pk_survey_bounds(const pk_survey_catalog *cat, double omega_m, double 
     PrepArgs a{};
     a.nchi = kChiNodes;
     a.zmax = zmax > 0.0 ? zmax : 5.0;
-    if (sky) chi_table(omega_m, a.zmax, tab, &a.dz);
+    a.zmax_f = float_below(a.zmax);
+    if (sky) sky_tables(omega_m, a.zmax, tab, &a.dz);
     a.inv_dz = a.dz > 0.0 ? 1.0 / a.dz : 0.0;
     const bool pdev = dev_ptr(cat->pos);
     // one device block: 6 results | G x 6 per-CTA partials | chi table | positions (host input)
