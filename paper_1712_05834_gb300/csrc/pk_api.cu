@@ -751,7 +751,7 @@ pk_status pk_compute(pk_plan_t P) {
             // y and x passes, then z fused into the bin pass: the meshes end up
             // holding the x/y transforms of the packed z rows
             G = std::max(1, P->G_own / nitems);
-            PK_CUDA(P, launch_fft_xy(P->mesh, nitems * P->nm, mesh_c, P->N, P->d_tw, st));
+            PK_CUDA(P, launch_fft_xy(P->mesh, nitems * P->nm, mesh_c, P->N, P->bg.mhi, P->d_tw, st));
             if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
             PK_CUDA(P, launch_zbin(P->mesh, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->d_cw, P->d_ph,
                                    P->d_tw, P->d_kedge, P->d_partial, st));

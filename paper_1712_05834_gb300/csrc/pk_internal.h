@@ -163,8 +163,9 @@ cudaError_t launch_plane_bin(const void *m1, const void *m2, int f64, int N, int
 // The meshes' z rows are read as N/2 complex values (packed real pairs).
 bool own_fft_packed(int N);
 void own_fft_twiddles(int N, float *tw);          // tw[2e], tw[2e+1] = W_N^e, e < N
-// length-N FFTs along y, then along x, of nmesh packed meshes mesh_c complex apart
-cudaError_t launch_fft_xy(void *mesh, int nmesh, long long mesh_c, int N, const void *tw, cudaStream_t st);
+// length-N FFTs along y, then along x, of nmesh packed meshes mesh_c complex apart;
+// rows (kx, ky) with kx^2 + ky^2 >= mhi are not written by the x pass
+cudaError_t launch_fft_xy(void *mesh, int nmesh, long long mesh_c, int N, int mhi, const void *tw, cudaStream_t st);
 // z transform + r2c split + the bin pass of launch_bin (FP32 form), partial
 // histograms as launch_bin writes them
 cudaError_t launch_zbin(const void *mesh, int interlaced, long long item_stride_c, long long mesh_stride_c,
