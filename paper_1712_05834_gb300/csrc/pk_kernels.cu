@@ -1358,7 +1358,7 @@ k_bin(const C *__restrict__ mesh, long long item_stride_c, long long mesh_stride
                 cur2 = key;
                 if (POLES) {
                     // FP32: mu = l rsqrt(m) from the k-bin estimate (a few ulp);
-                    // FP64: the exact quotient.  The sums are of P L_2(mu) and
+                    // FP64: l^2 / m to the last place or two.  The sums are of P L_2(mu) and
                     // P L_4(mu) themselves, not of P mu^2 and P mu^4: forming
                     // P_4 from mu moments (35 M4 - 30 M2 + 3 S0) would amplify
                     // the FP32 partial sums' rounding about forty-fold.
@@ -1367,7 +1367,13 @@ k_bin(const C *__restrict__ mesh, long long item_stride_c, long long mesh_stride
                         const float mu = (float)l * rsm;
                         mu2 = (R)(mu * mu);
                     } else {
-                        mu2 = (R)(l * l) / (R)m;
+                        // l^2 / m by two Newton steps from the FP32 reciprocal (46, then all
+                        // 53 bits): six FP64 operations for a division's thirty or so, at 1/64 rate
+                        const R dm = (R)m;
+                        R rc = (R)(rsm * rsm);
+                        rc = rc * ((R)2 - dm * rc);
+                        rc = rc * ((R)2 - dm * rc);
+                        mu2 = (R)(l * l) * rc;
                     }
                     const R t2 = pw * ((R)1.5 * mu2 - (R)0.5);
                     const R t4 = pw * (((R)4.375 * mu2 - (R)3.75) * mu2 + (R)0.375);
