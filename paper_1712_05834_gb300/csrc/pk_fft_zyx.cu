@@ -241,10 +241,13 @@ __device__ __forceinline__ int dif_freq(int p) {
 // thread), NBY columns per y tile, TX threads of the x kernels (CTASX per SM), NX
 // columns per x tile.  About 12 to 16 complex values per thread.  At N = 2048
 // and 1024 the x tiles take 128 KB and one CTA of 1024 threads, since their runs
-// along z come from device memory (64-byte runs at 1024: 9.0 against 4.1 ms
-// interlaced), while the y tiles are read from L2, where short runs cost little.
-// LAG: planes between a plane's z and y items (1024 interlaced, k_fft_zy: 8.4,
-// 7.4 and 7.6 ms at 3, 6 and 12 planes; 2048: 36.2, 36.6 and 39.4 at 1, 2 and 3).
+// along z come from device memory (32-byte runs at 1024: 5.7 against 3.8 ms
+// interlaced).  The y tiles are read from L2 in runs of 64 bytes or more: at 2048
+// that takes one 768-thread CTA per SM (k_fft_zy 29.2 ms; 32.3 with 32-byte runs
+// and two 512-thread CTAs, 58.9 with 16-byte runs), at 1024 two CTAs (6.06 ms; 6.55
+// with 128-byte runs and one).  LAG: planes between a plane's z and y items (1024
+// interlaced: 6.05, 6.06 and 6.31 ms at 4, 6 and 10 planes; 2048: 29.8 and 30.4 at
+// 1 and 2).
 template <int N>
 struct Shape;
 template <int T_, int CTAS_, int NBY_, int TX_, int CTASX_, int NX_, int LAG_>
@@ -265,7 +268,7 @@ template <> struct Shape<640> : ShapeOf<512, 2, 8, 512, 2, 8, 16> {};
 template <> struct Shape<768> : ShapeOf<512, 2, 8, 512, 2, 8, 10> {};
 template <> struct Shape<800> : ShapeOf<512, 2, 8, 512, 2, 8, 10> {};
 template <> struct Shape<1024> : ShapeOf<512, 2, 8, 1024, 1, 16, 6> {};
-template <> struct Shape<2048> : ShapeOf<512, 2, 4, 1024, 1, 8, 1> {};
+template <> struct Shape<2048> : ShapeOf<768, 1, 8, 1024, 1, 8, 1> {};
 
 template <int N>
 struct Cfg : Shape<N> {
