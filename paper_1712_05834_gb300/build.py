@@ -16,7 +16,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libpk.so")
-SOURCES = ["pk_kernels.cu", "pk_api.cu", "pk_static.cu", "pk_lognormal.cu", "pk_survey.cu", "pk_fft.cu", "pk_fft_zyx.cu"]
+SOURCES = ["pk_kernels.cu", "pk_api.cu", "pk_static.cu", "pk_lognormal.cu", "pk_survey.cu", "pk_fft.cu", "pk_fft_zyx.cu",
+           "pk_fft64.cu"]
 # sources compiled several times, once per group of template instances
 GROUPS = {"pk_fft_zyx.cu": ["-DPK_ZYX_GROUP=%d" % g for g in range(3)]}
 HEADERS = [os.path.join(ROOT, "include", "pk.h"), os.path.join(CSRC, "pk_internal.h"),

@@ -151,6 +151,11 @@ void pk::set_plan_error(const char *msg) { g_plan_error = msg ? msg : ""; }
 // single-mesh plan, else one call of the plan over one catalog's meshes
 // (count must then be nm).
 cufftResult pk::transform_meshes(pk_plan_s *P, void *first, int count) {
+    if (P->f64 && P->own_fft)
+        return launch_fft64(reinterpret_cast<double *>(first), count, P->mesh_reals, P->fft64, 0x7fffffff, P->st) ==
+                       cudaSuccess
+                   ? CUFFT_SUCCESS
+                   : CUFFT_EXEC_FAILED;
     if (ensure_cufft(P) != PK_OK) return CUFFT_ALLOC_FAILED;
     if (!P->fft_single && count != P->nm) return CUFFT_INVALID_VALUE;
     const int calls = P->fft_single ? count : 1;
@@ -429,7 +434,17 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
         PK_CUDA(P, cudaMemcpy(P->d_kedge, P->kedge.data(), sizeof(int) * (nk + 1), cudaMemcpyHostToDevice));
     }
 
-    // ---- own transform: FP32 meshes of the sizes it has kernels for ----
+    // ---- own transform: meshes of the sizes it has kernels for ----
+    if (P->f64 && fft64_plan(P->N, &P->fft64)) {
+        const size_t tw_bytes = sizeof(double) * 4 * (size_t)P->N;
+        std::vector<double> tab(4 * (size_t)P->N + (P->N + 3) / 4);
+        fft64_tables(P->fft64, tab.data(), reinterpret_cast<unsigned short *>(tab.data() + 4 * (size_t)P->N));
+        PK_CUDA(P, dev_alloc(&P->d_tw, sizeof(double) * tab.size()));
+        PK_CUDA(P, cudaMemcpy(P->d_tw, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
+        P->fft64.tw = reinterpret_cast<const double2 *>(P->d_tw);
+        P->fft64.pos = reinterpret_cast<const unsigned short *>(reinterpret_cast<const char *>(P->d_tw) + tw_bytes);
+        P->own_fft = 1;
+    }
     if (!P->f64) P->zyx = zyx_ops(P->N);
     if (P->zyx && !P->zyx->plan_default()) P->zyx = nullptr;
     if (!P->f64 && (P->zyx || own_fft_packed(P->N))) {
@@ -744,7 +759,11 @@ pk_status pk_compute(pk_plan_t P) {
     // fewer histograms to add up
     int G = std::max(1, std::min(P->G_total / nitems, P->N * P->N / 16));
     pk_status s_ = PK_OK;
-    if (P->own_fft) {
+    if (P->own_fft && P->f64) {
+        PK_CUDA(P, launch_fft64(reinterpret_cast<double *>(P->mesh), nitems * P->nm, P->mesh_reals, P->fft64, P->bg.mhi,
+                                st));
+        P->launches += 3;
+    } else if (P->own_fft) {
         P->transformed = 1;
         P->unfinished = 1;
         if (!P->zyx) {
@@ -801,7 +820,7 @@ pk_status pk_compute(pk_plan_t P) {
         }
         if (left != 0) return fail(P, PK_ECUFFT, "internal: catalog count not covered by the FFT plans");
     }
-    if (!P->own_fft) {
+    if (!P->own_fft || P->f64) {
         P->transformed = 1;
         P->unfinished = 0;
         if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));

@@ -226,6 +226,18 @@ inline const ZyxOps *zyx_ops(int N) {
     return o;
 }
 
+// ---- own FFT path of FP64 meshes (pk_fft64.cu) ----
+struct Fft64 {
+    int N, nsteps, lc;                // lc: log2 of the lines per tile
+    unsigned char radix[12];
+    const double2 *tw;                // device: W_N^e (e < N), then the same halved
+    const unsigned short *pos;        // device: place of frequency f after the steps
+};
+bool fft64_plan(int N, Fft64 *f);     // false: no own transform of this size
+void fft64_tables(const Fft64 &f, double *tw, unsigned short *pos);    // 4 N reals, N places
+// r2c of nmesh meshes in place; modes with |n|^2 >= mhi need not be transformed
+cudaError_t launch_fft64(double *mesh, int nmesh, long long mesh_reals, const Fft64 &f, int mhi, cudaStream_t st);
+
 cudaError_t launch_geom_hist(const BinGeom &g, unsigned long long *H, unsigned long long *HL,
                              cudaStream_t st);
 cudaError_t launch_geom_finalize(const BinGeom &g, const int *kedge, double kF,

@@ -693,11 +693,23 @@ __device__ __forceinline__ float cell_value<float>(unsigned lo, unsigned hi, uns
     if (sp.fast) return fmaf((float)(int)hi, sp.hi_scale, (float)lo * inv_scale);
     return ll_to_float_rn((long long)a64) * inv_scale;
 }
+// hi sh + lo sl for powers of two sl <= sh <= 2^52 sl, rounded once: 32-bit words
+// put into the low half of the double 2^52 s become 2^52 s + word s without a
+// conversion, and the sum of the offsets leaves again in the first of the two
+// additions (exact).  Conversions and products took twice as many operations of
+// the FP64 pipe, which bounds the write-out of FP64 meshes.
+__device__ __forceinline__ double words_value(unsigned lo, int hi, float sl, float sh) {
+    const int el = ((__float_as_int(sl) >> 23) + (1023 - 127 + 52)) << 20;
+    const int eh = ((__float_as_int(sh) >> 23) + (1023 - 127 + 52)) << 20;
+    const double off = __hiloint2double(eh, 0x80000000) + __hiloint2double(el, 0);
+    return (__hiloint2double(eh, hi ^ 0x80000000) - off) + __hiloint2double(el, (int)lo);
+}
+
 template <>
 __device__ __forceinline__ double cell_value<double>(unsigned lo, unsigned hi, unsigned long long a64,
                                                      const Split &sp, float inv_scale) {
-    if (sp.fast) return fma((double)(int)hi, (double)sp.hi_scale, (double)lo * (double)inv_scale);
-    return __ll2double_rn((long long)a64) * (double)inv_scale;
+    if (sp.fast) return words_value(lo, (int)hi, inv_scale, sp.hi_scale);
+    return words_value((unsigned)a64, (int)(a64 >> 32), inv_scale, inv_scale * 4294967296.0f);
 }
 
 // 2^k for -126 <= k <= 127, exactly (the fixed-point scales: S <= 40, B <= 22).
@@ -1334,7 +1346,7 @@ k_bin(const C *__restrict__ mesh, long long item_stride_c, long long mesh_stride
                     }
                 }
                 R pw = (CROSS ? z.x * y.x + z.y * y.y : z.x * z.x + z.y * z.y) * rowcw * scw[l + (l >> 2)];
-                pw *= (R)((l != 0 && l != half) ? 2 : 1) * (R)(live ? 1 : 0);
+                pw *= !live ? (R)0 : (l != 0 && l != half) ? (R)2 : (R)1;
                 int key = b;
                 if (TWOD) {
                     // mu bin: FP32 estimate, then one exact integer step each way

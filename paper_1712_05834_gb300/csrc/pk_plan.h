@@ -33,12 +33,14 @@ struct pk_plan_s {
     int fft_single = 0;              // one single-mesh plan, one call per mesh (large meshes)
     void *fft_work = nullptr;
     // Own transform: packed (pk_fft.cu: y and x passes, then z fused into the bin)
-    // or zyx (pk_fft_zyx.cu: z and y in one pass, then x fused into the bin).
-    int own_fft = 0;                 // pk_compute uses it (FP32 form, supported N)
+    // or zyx (pk_fft_zyx.cu: z and y in one pass, then x fused into the bin); FP64
+    // meshes: pk_fft64.cu, then the bin pass.
+    int own_fft = 0;                 // pk_compute uses it (supported N)
     int own_selectable = 0;          // pk_use_own_fft(plan, 1) accepts it
     const pk::ZyxOps *zyx = nullptr; // zyx form; NULL: packed
     int unfinished = 0;              // meshes hold the transform without its last axis
     int G_own = 0;                   // fused last-axis CTAs for one catalog (zyx: 0 = x, then k_bin)
+    pk::Fft64 fft64{};               // FP64 form: steps and tables (both in d_tw)
     void *d_tw = nullptr;            // W_N^e, e < N (float2)
     unsigned *d_sync = nullptr;      // zyx: ticket and plane counters of the z / y pass
     int nsync = 0;
