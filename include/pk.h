@@ -6,7 +6,7 @@
  *
  *   paint     objects -> mesh with a CIC / TSC / PCS window, optionally a
  *             second mesh shifted by half a cell (interlacing)      Sec. 3.3.1-3.3.2
- *   r2c FFT   real mesh -> complex half grid (cuFFT)                Sec. 3.3.1
+ *   r2c FFT   real mesh -> complex half grid                        Sec. 3.3.1
  *   compensate + interlace: divide by prod_i sinc^p(pi k_i / 2 k_N),
  *             average the two meshes with the half-cell phase       Eq. window-deconvolution
  *   bin       |delta(k)|^2 into k bins, (k, mu) bins about the z axis,
@@ -73,10 +73,11 @@ typedef enum {
  * (cuFFT R2C otherwise; see pk_use_own_fft); bins summed per CTA in
  * FP32 with shared-memory atomics, whose order (and so the last bits of
  * P(k)) can vary between runs, then across CTAs in FP64.
- * PK_MESH_F64: cuFFT D2Z; bins summed in FP64. */
+ * PK_MESH_F64: the library's own FP64 r2c transform for even nmesh from 32 to
+ * 2048 with prime factors up to 7, cuFFT D2Z otherwise; bins summed in FP64. */
 typedef enum {
     PK_MESH_F32 = 0,   /* FP32 mesh, FP32 per-mode arithmetic                   */
-    PK_MESH_F64 = 1    /* FP64 mesh, cuFFT D2Z, FP64 per-mode arithmetic        */
+    PK_MESH_F64 = 1    /* FP64 mesh, FP64 transform and per-mode arithmetic     */
 } pk_precision;
 
 /* How pk_paint deposits the window weights.  Both give int64 fixed-point
@@ -278,7 +279,8 @@ pk_status pk_mesh(pk_plan_t plan, int item, int mesh, void *dst);
  * r2c transform and bins it without writing it) and 320, 384, 400, 480, 500,
  * 600, 640, 768, 800, 1024, 2048 (z and y in one pass over device memory, then
  * x, at 1024 and 2048 in the bin pass).  on = 0: cuFFT's in-place R2C, then the
- * bin pass.  Both give the same result within FP32 rounding.  After a compute
+ * bin pass.  Both give the same result within FP32 rounding (FP64 meshes: the
+ * own FP64 transform or cuFFT's D2Z, within FP64 rounding).  After a compute
  * that did not write the transform itself, pk_cross and pk_projected first
  * write it into the meshes (one extra pass).  Takes effect at the next
  * pk_compute.

@@ -439,7 +439,7 @@ def pk_enable_timing(plan, on=True):
 
 def pk_use_own_fft(plan, on=True):
     """Select the r2c transform of the next pk_compute: the library's own FFT
-    kernels (y and x passes, then z fused into the bin pass) or cuFFT's R2C."""
+    kernels or cuFFT's R2C."""
     _check(load().pk_use_own_fft(plan, int(bool(on))), plan)
 
 

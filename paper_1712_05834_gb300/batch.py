@@ -10,7 +10,8 @@ whose batch holds all of its catalogs, back to back in one device buffer:
   * one pk_paint_many per class: one count / scan / scatter / tile-paint
     launch set (or one atomic-paint launch and one conversion launch) over
     every catalog of the class;
-  * one batched cuFFT call over every mesh of the class;
+  * one transform of every mesh of the class (own kernels, or a batched cuFFT
+    call);
   * one bin launch (persistent CTAs, a fixed share per catalog), one reduce
     and one finalize launch over every catalog of the class.
 

@@ -1251,11 +1251,14 @@ __device__ __forceinline__ int isqrt_floor(int x) {
 // shared histogram when its bin changes.  CROSS: the meshes of a second
 // catalog at meshb; each mode contributes Re(delta_a conj(delta_b)) instead
 // of |delta|^2.  MU32: the mu-bin test q^2 m <= nmu^2 l^2 fits in 32 bits.
-template <bool IL, bool TWOD, bool POLES, typename R, typename C, typename A, bool CROSS = false, bool MU32 = true>
-__global__ void __launch_bounds__(kBinThreads, sizeof(R) == 4 ? 5 : 1)
-k_bin(const C *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
-      const R *__restrict__ cw, const C *__restrict__ ph, const int *__restrict__ kedge, A *__restrict__ partial,
-      const C *__restrict__ meshb) {
+template <bool IL, bool TWOD, bool POLES, bool CROSS, bool MU32>
+__global__ void __launch_bounds__(kBinThreads, 5)
+k_bin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
+      const float *__restrict__ cw, const float2 *__restrict__ ph, const int *__restrict__ kedge,
+      float *__restrict__ partial, const float2 *__restrict__ meshb) {
+    using R = float;
+    using C = float2;
+    using A = float;
     using SM = BinSmem<R, C, A>;
     extern __shared__ __align__(16) unsigned char smraw[];
     A *hist = reinterpret_cast<A *>(smraw);
@@ -1369,24 +1372,12 @@ k_bin(const C *__restrict__ mesh, long long item_stride_c, long long mesh_stride
                 run2 = new2 ? pw : run2 + pw;
                 cur2 = key;
                 if (POLES) {
-                    // FP32: mu = l rsqrt(m) from the k-bin estimate (a few ulp);
-                    // FP64: l^2 / m to the last place or two.  The sums are of P L_2(mu) and
-                    // P L_4(mu) themselves, not of P mu^2 and P mu^4: forming
-                    // P_4 from mu moments (35 M4 - 30 M2 + 3 S0) would amplify
+                    // mu = l rsqrt(m) from the k-bin estimate (a few ulp).  The sums are
+                    // of P L_2(mu) and P L_4(mu) themselves, not of P mu^2 and P mu^4:
+                    // forming P_4 from mu moments (35 M4 - 30 M2 + 3 S0) would amplify
                     // the FP32 partial sums' rounding about forty-fold.
-                    R mu2;
-                    if (sizeof(R) == 4) {
-                        const float mu = (float)l * rsm;
-                        mu2 = (R)(mu * mu);
-                    } else {
-                        // l^2 / m by two Newton steps from the FP32 reciprocal (46, then all
-                        // 53 bits): six FP64 operations for a division's thirty or so, at 1/64 rate
-                        const R dm = (R)m;
-                        R rc = (R)(rsm * rsm);
-                        rc = rc * ((R)2 - dm * rc);
-                        rc = rc * ((R)2 - dm * rc);
-                        mu2 = (R)(l * l) * rc;
-                    }
+                    const float mu = (float)l * rsm;
+                    const R mu2 = mu * mu;
                     const R t2 = pw * ((R)1.5 * mu2 - (R)0.5);
                     const R t4 = pw * (((R)4.375 * mu2 - (R)3.75) * mu2 + (R)0.375);
                     const bool new1 = b != cur1;
@@ -1408,6 +1399,211 @@ k_bin(const C *__restrict__ mesh, long long item_stride_c, long long mesh_stride
     }
     __syncthreads();
     A *out = partial + ((long long)item * gridDim.x + blockIdx.x) * g.nh;
+    for (int k = threadIdx.x; k < g.nh; k += blockDim.x) out[k] = hist[k];
+}
+
+// Shared memory of k_bin_f64: hist[nh], weights (cw, twice where a mode stands for
+// two) at l + l/4, phases e^{i pi s / N} (|s| <= N/2) at k + k/4 with k = s + N/2,
+// edge pairs.
+struct Bin64Smem {
+    __host__ __device__ static size_t off_cw(const BinGeom &g) { return align_up((size_t)g.nh * sizeof(double), 16); }
+    __host__ __device__ static size_t off_ph(const BinGeom &g) {
+        return align_up(off_cw(g) + ((size_t)g.Nh + (g.Nh >> 2) + 1) * sizeof(double), 16);
+    }
+    __host__ __device__ static size_t off_edge(const BinGeom &g) {
+        return off_ph(g) + ((size_t)g.N + 1 + (g.N >> 2) + 1) * sizeof(double2);
+    }
+    __host__ __device__ static size_t bytes(const BinGeom &g) { return align_up(off_edge(g) + (size_t)g.nk * sizeof(int2), 16); }
+};
+
+// An integer 0 <= v < 2^32 as a double by one addition (the conversion
+// instruction has the FP64 pipe's rate as well, and a longer latency).
+__device__ __forceinline__ double u32_to_double(unsigned v) {
+    return __hiloint2double(0x43300000, (int)v) - 4503599627370496.0;
+}
+// A normal float as a double, by its bits.
+__device__ __forceinline__ double float_bits_to_double(float f) {
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+}
+
+// The bin pass of FP64 meshes: as k_bin, laid out for the FP64 pipe (two
+// operations per SM and clock), which bounds it (85 % of its rate):
+//   * 19 FP64 operations per mode with interlacing and multipoles: the phase of
+//     a mode is one table entry (its arguments add up: i' + j' + l, folded by
+//     e^{i pi} = -1), weights of 1 or 2 stand in the cw table, Legendre sums are
+//     one FMA each, and l^2 / m comes from the FP32 reciprocal r by
+//     r (1 + e + e^2), e = 1 - m r (the geometric series of 1 / (m r); e^3 <
+//     2^-60).
+//   * Runs of kBinVec modes of four rows are dealt to the lanes without gaps: with
+//     a row per warp a third of the lanes idled at the rows' ends, and an FP64
+//     instruction costs the same with half of its lanes off.
+// Two interlaced meshes, multipoles (k_bin in FP64 before): 64^3 49 -> 18 us, 256^3
+// 512 -> 311 us, 512^3 3.25 -> 1.86 ms.  Eight rows a turn: 31, 283 us, 1.87 ms, but
+// 400^3 1.03 ms for 0.94.
+template <bool IL, bool TWOD, bool POLES, bool CROSS, bool MU32>
+__global__ void __launch_bounds__(kBinThreads, 2)
+k_bin_f64(const double2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
+          const double *__restrict__ cw, const double2 *__restrict__ ph, const int *__restrict__ kedge,
+          double *__restrict__ partial, const double2 *__restrict__ meshb) {
+    using SM = Bin64Smem;
+    constexpr int kRows = 4;                          // rows per warp and turn
+    extern __shared__ __align__(16) unsigned char smraw[];
+    double *hist = reinterpret_cast<double *>(smraw);
+    double *scw = reinterpret_cast<double *>(smraw + SM::off_cw(g));
+    double2 *sph = reinterpret_cast<double2 *>(smraw + SM::off_ph(g));
+    int2 *sedge = reinterpret_cast<int2 *>(smraw + SM::off_edge(g));
+    const int half = g.N / 2, N = g.N, Nh = g.Nh;
+    for (int k = threadIdx.x; k < g.nh; k += blockDim.x) hist[k] = 0.0;
+    for (int k = threadIdx.x; k < Nh; k += blockDim.x) scw[k + (k >> 2)] = (k != 0 && k != half ? 2.0 : 1.0) * cw[k];
+    for (int k = threadIdx.x; IL && k <= N; k += blockDim.x) sph[k + (k >> 2)] = ph[k];
+    for (int k = threadIdx.x; k < g.nk; k += blockDim.x) sedge[k] = make_int2(kedge[k], kedge[k + 1]);
+    __syncthreads();
+
+    const int item = blockIdx.y;
+    const double2 *m1 = mesh + (long long)item * item_stride_c;
+    const double2 *m2 = m1 + mesh_stride_c;
+    const double2 *n1 = CROSS ? meshb : m1;
+    const double2 *n2 = n1 + mesh_stride_c;
+    const int nk = g.nk, nmu = g.nmu, hbase = g.hbase;
+    const float kscale = g.kscale, koff = g.koff;
+    const int lane = threadIdx.x & 31;
+    const int wpb = blockDim.x >> 5;
+    const int rows = N * N;
+    // Turn k of W warps covers W groups of rows, shifted so that a warp moves on by
+    // 5/8 of a plane per turn: W = 152 x 16 groups are whole planes for powers of
+    // two, and it would meet the same ky, short rows or long ones, on every turn.
+    const int W = gridDim.x * wpb, w0 = blockIdx.x * wpb + (threadIdx.x >> 5);
+    const int gp = (N + kRows - 1) / kRows, shift = (5 * gp / 8 + gp - W % gp) % gp % W;
+    for (int first = 0, w = w0; first * kRows < rows; first += W, w = w + shift < W ? w + shift : w + shift - W) {
+        const int row0 = (first + w) * kRows;
+        if (row0 >= rows) continue;
+        // lane r < kRows: row row0 + r, its l range, runs and weight
+        int r2 = 0, llo = 0, lhi = 0, s0 = 0;
+        double rowcw = 0.0;
+        if (lane < kRows && row0 + lane < rows) {
+            const int i = (row0 + lane) / N, j = row0 + lane - i * N;
+            const int ip = i < half ? i : i - N;
+            const int jp = j < half ? j : j - N;
+            r2 = ip * ip + jp * jp;
+            s0 = ip + jp;
+            if (r2 < g.mhi) {
+                lhi = min(Nh, isqrt_floor(g.mhi - 1 - r2) + 1);
+                llo = g.mlo > r2 ? isqrt_floor(g.mlo - r2 - 1) + 1 : 0;
+                if (r2 == 0 && llo == 0) llo = 1;
+                rowcw = cw[i] * cw[j] * (IL ? 0.25 : 1.0);
+            }
+        }
+        int incl = max(lhi - llo + kBinVec - 1, 0) / kBinVec;      // runs of this and the lanes before it
+#pragma unroll
+        for (int d = 1; d < kRows; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, kRows - 1);
+        for (int t0 = 0; t0 < total; t0 += 32) {
+            const int t = t0 + lane;
+            int r = 0;                                             // rows whose runs all lie before run t
+#pragma unroll
+            for (int d = kRows / 2; d; d >>= 1)
+                if (t >= __shfl_sync(0xffffffffu, incl, r + d - 1)) r += d;
+            const int before = __shfl_sync(0xffffffffu, incl, max(r - 1, 0));
+            const int rr2 = __shfl_sync(0xffffffffu, r2, r), rs = __shfl_sync(0xffffffffu, s0, r);
+            const int end = __shfl_sync(0xffffffffu, lhi, r);
+            const int l0 = __shfl_sync(0xffffffffu, llo, r) + kBinVec * (t - (r ? before : 0));
+            const double rcw = __shfl_sync(0xffffffffu, rowcw, r);
+            if (t >= total) continue;
+            const int cnt = end - l0;                              // modes of this run: min(cnt, kBinVec)
+            const long long base = (long long)(row0 + r) * Nh + l0;
+            double2 a[kBinVec], b2[kBinVec], ca[CROSS ? kBinVec : 1], cb2[CROSS && IL ? kBinVec : 1];
+#pragma unroll
+            for (int v = 0; v < kBinVec; ++v) {
+                const long long at = base + min(v, cnt - 1);       // the tail re-reads the last mode
+                a[v] = __ldcs(m1 + at);
+                if (IL) b2[v] = __ldcs(m2 + at);
+                if (CROSS) {
+                    ca[CROSS ? v : 0] = __ldcs(n1 + at);
+                    if (IL) cb2[CROSS && IL ? v : 0] = __ldcs(n2 + at);
+                }
+            }
+            int cur2 = -1, cur1 = -1;                              // open register runs
+            double run2 = 0.0, runm2 = 0.0, runm4 = 0.0;
+#pragma unroll
+            for (int v = 0; v < kBinVec; ++v) {
+                const bool live = v < cnt;
+                const int l = min(l0 + v, end - 1);
+                const int m = rr2 + l * l;
+                const float rsm = rsqrtf((float)m);                // bins: as k_bin
+                int b = (int)((float)m * rsm * kscale - koff);
+                b = min(max(b, 0), nk - 1);
+                {
+                    const int2 e = sedge[b];
+                    b += (int)(m >= e.y) - (int)(m < e.x);
+                }
+                double2 z = a[v], y;
+                if (CROSS) y = ca[CROSS ? v : 0];
+                if (IL) {
+                    int s = rs + l, flip = 0;                      // -N <= s <= 3 N / 2
+                    if (s > half) s -= N, flip ^= 0x80000000;
+                    if (s > half) s -= N, flip ^= 0x80000000;
+                    if (s < -half) s += N, flip ^= 0x80000000;
+                    s += half;
+                    double2 w = sph[s + (s >> 2)];
+                    w.x = __hiloint2double(__double2hiint(w.x) ^ flip, __double2loint(w.x));
+                    w.y = __hiloint2double(__double2hiint(w.y) ^ flip, __double2loint(w.y));
+                    z.x = fma(b2[v].x, w.x, fma(-b2[v].y, w.y, z.x));
+                    z.y = fma(b2[v].x, w.y, fma(b2[v].y, w.x, z.y));
+                    if (CROSS) {
+                        const double2 u = cb2[CROSS && IL ? v : 0];
+                        y.x = fma(u.x, w.x, fma(-u.y, w.y, y.x));
+                        y.y = fma(u.x, w.y, fma(u.y, w.x, y.y));
+                    }
+                }
+                const double p2 = CROSS ? fma(z.x, y.x, z.y * y.y) : fma(z.x, z.x, z.y * z.y);
+                const double pw = live ? p2 * (rcw * scw[l + (l >> 2)]) : 0.0;
+                int key = b;
+                if (TWOD) {
+                    int q = (int)((float)(nmu * l) * rsm);
+                    q = min(max(q, 0), nmu - 1);
+                    if (MU32) {
+                        const unsigned rhs = (unsigned)(nmu * nmu) * (unsigned)(l * l);
+                        q -= (int)(q > 0 && (unsigned)(q * q) * (unsigned)m > rhs);
+                        q += (int)(q < nmu - 1 && (unsigned)((q + 1) * (q + 1)) * (unsigned)m <= rhs);
+                    } else {
+                        const long long rhs = (long long)nmu * nmu * l * l;
+                        q -= (int)(q > 0 && (long long)q * q * m > rhs);
+                        q += (int)(q < nmu - 1 && (long long)(q + 1) * (q + 1) * m <= rhs);
+                    }
+                    key = b * nmu + q;
+                }
+                const bool new2 = key != cur2;
+                if (new2 && cur2 >= 0) atomicAdd(hist + cur2, run2);
+                run2 = new2 ? pw : run2 + pw;
+                cur2 = key;
+                if (POLES) {
+                    const double rc = float_bits_to_double(rsm * rsm);
+                    const double e = fma(-u32_to_double((unsigned)m), rc, 1.0);
+                    const double q = u32_to_double((unsigned)(l * l)) * rc;
+                    const double mu2 = fma(q, fma(e, e, e), q);
+                    const bool new1 = b != cur1;
+                    if (new1 && cur1 >= 0) {
+                        atomicAdd(hist + hbase + cur1, runm2);
+                        atomicAdd(hist + hbase + nk + cur1, runm4);
+                    }
+                    runm2 = fma(pw, fma(1.5, mu2, -0.5), new1 ? 0.0 : runm2);
+                    runm4 = fma(pw, fma(fma(4.375, mu2, -3.75), mu2, 0.375), new1 ? 0.0 : runm4);
+                    cur1 = b;
+                }
+            }
+            atomicAdd(hist + cur2, run2);
+            if (POLES) {
+                atomicAdd(hist + hbase + cur1, runm2);
+                atomicAdd(hist + hbase + nk + cur1, runm4);
+            }
+        }
+    }
+    __syncthreads();
+    double *out = partial + ((long long)item * gridDim.x + blockIdx.x) * g.nh;
     for (int k = threadIdx.x; k < g.nh; k += blockDim.x) out[k] = hist[k];
 }
 
@@ -1867,34 +2063,47 @@ cudaError_t launch_acc_to_mesh(unsigned long long *acc, int nitems, int nmesh, i
 }
 
 size_t bin_smem_bytes(const BinGeom &g, int f64) {
-    return f64 ? BinSmem<double, double2, double>::bytes(g) : BinSmem<float, float2, float>::bytes(g);
+    return f64 ? Bin64Smem::bytes(g) : BinSmem<float, float2, float>::bytes(g);
+}
+
+// Histograms that a plan may ask for: up to 200 KB with one entry per l in both
+// tables (the phases that k_bin_f64 holds beyond that, 20 KB at 2048, fit above it).
+bool bin_smem_allowed(const BinGeom &g, int f64) {
+    return (f64 ? BinSmem<double, double2, double>::bytes(g) : BinSmem<float, float2, float>::bytes(g)) <= 200 * 1024;
 }
 
 int bin_threads() { return kBinThreads; }
 
-template <bool IL, bool TWOD, bool POLES, typename R, typename C, typename A, bool CROSS>
+// The pass of either form, chosen by the types.
+template <bool IL, bool TWOD, bool POLES, typename R, typename C, bool CROSS, bool MU32>
+static auto bin_kernel() {
+    if constexpr (sizeof(R) == 4) return k_bin<IL, TWOD, POLES, CROSS, MU32>;
+    else return k_bin_f64<IL, TWOD, POLES, CROSS, MU32>;
+}
+
+template <bool IL, bool TWOD, bool POLES, typename R, typename C, bool CROSS>
 static cudaError_t bin_inst(const void *mesh, long long item_stride_c, long long mesh_stride_c,
                             int nitems, int G, const BinGeom &g, const void *cw, const void *ph,
                             const int *kedge, void *partial, const void *meshb, cudaStream_t st) {
-    const size_t smem = BinSmem<R, C, A>::bytes(g);
-    auto kern = (g.mu32 || !TWOD) ? k_bin<IL, TWOD, POLES, R, C, A, CROSS, true>
-                                  : k_bin<IL, TWOD, POLES, R, C, A, CROSS, false>;
+    const size_t smem = bin_smem_bytes(g, sizeof(R) == 8);
+    auto kern = (g.mu32 || !TWOD) ? bin_kernel<IL, TWOD, POLES, R, C, CROSS, true>()
+                                  : bin_kernel<IL, TWOD, POLES, R, C, CROSS, false>();
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid(G, nitems);
     kern<<<grid, kBinThreads, smem, st>>>(reinterpret_cast<const C *>(mesh), item_stride_c,
                                           mesh_stride_c, g, reinterpret_cast<const R *>(cw),
                                           reinterpret_cast<const C *>(ph), kedge,
-                                          reinterpret_cast<A *>(partial), reinterpret_cast<const C *>(meshb));
+                                          reinterpret_cast<R *>(partial), reinterpret_cast<const C *>(meshb));
     return cudaGetLastError();
 }
 
-template <typename R, typename C, typename A, bool CROSS>
+template <typename R, typename C, bool CROSS>
 static cudaError_t bin_dispatch(const void *mesh, int il, long long is, long long ms, int nitems,
                                 int G, const BinGeom &g, const void *cw, const void *ph,
                                 const int *kedge, void *partial, const void *meshb, cudaStream_t st) {
     const int key = (il ? 4 : 0) | (g.twod ? 2 : 0) | (g.poles ? 1 : 0);
-#define PK_BIN(a, b, c) bin_inst<a, b, c, R, C, A, CROSS>(mesh, is, ms, nitems, G, g, cw, ph, kedge, partial, meshb, st)
+#define PK_BIN(a, b, c) bin_inst<a, b, c, R, C, CROSS>(mesh, is, ms, nitems, G, g, cw, ph, kedge, partial, meshb, st)
     switch (key) {
     case 0: return PK_BIN(false, false, false);
     case 1: return PK_BIN(false, false, true);
@@ -1913,21 +2122,20 @@ cudaError_t launch_bin(const void *mesh, int f64, int interlaced, long long item
                        const BinGeom &g, const void *cw, const void *ph, const int *kedge,
                        void *partial, cudaStream_t st) {
     if (f64)
-        return bin_dispatch<double, double2, double, false>(mesh, interlaced, item_stride_c, mesh_stride_c,
-                                                             nitems, ctas_per_item, g, cw, ph, kedge, partial,
-                                                             nullptr, st);
-    return bin_dispatch<float, float2, float, false>(mesh, interlaced, item_stride_c, mesh_stride_c, nitems,
-                                                     ctas_per_item, g, cw, ph, kedge, partial, nullptr, st);
+        return bin_dispatch<double, double2, false>(mesh, interlaced, item_stride_c, mesh_stride_c, nitems,
+                                                    ctas_per_item, g, cw, ph, kedge, partial, nullptr, st);
+    return bin_dispatch<float, float2, false>(mesh, interlaced, item_stride_c, mesh_stride_c, nitems,
+                                              ctas_per_item, g, cw, ph, kedge, partial, nullptr, st);
 }
 
 cudaError_t launch_bin_cross(const void *mesh_a, const void *mesh_b, int f64, int interlaced,
                              long long mesh_stride_c, int ctas, const BinGeom &g, const void *cw,
                              const void *ph, const int *kedge, void *partial, cudaStream_t st) {
     if (f64)
-        return bin_dispatch<double, double2, double, true>(mesh_a, interlaced, 0, mesh_stride_c, 1, ctas, g, cw,
-                                                            ph, kedge, partial, mesh_b, st);
-    return bin_dispatch<float, float2, float, true>(mesh_a, interlaced, 0, mesh_stride_c, 1, ctas, g, cw, ph,
-                                                    kedge, partial, mesh_b, st);
+        return bin_dispatch<double, double2, true>(mesh_a, interlaced, 0, mesh_stride_c, 1, ctas, g, cw, ph, kedge,
+                                                   partial, mesh_b, st);
+    return bin_dispatch<float, float2, true>(mesh_a, interlaced, 0, mesh_stride_c, 1, ctas, g, cw, ph, kedge,
+                                             partial, mesh_b, st);
 }
 
 int bin_ctas_per_sm(const BinGeom &g, int f64) {
@@ -1935,11 +2143,11 @@ int bin_ctas_per_sm(const BinGeom &g, int f64) {
     const size_t smem = bin_smem_bytes(g, f64);
     cudaError_t e;
     if (f64) {
-        auto k = k_bin<true, true, true, double, double2, double>;
+        auto k = k_bin_f64<true, true, true, false, true>;
         set_smem(k, smem);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kBinThreads, smem);
     } else {
-        auto k = k_bin<true, true, true, float, float2, float>;
+        auto k = k_bin<true, true, true, false, true>;
         set_smem(k, smem);
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kBinThreads, smem);
     }
