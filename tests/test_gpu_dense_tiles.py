@@ -58,3 +58,34 @@ def test_cells_match_the_oracle(N, window, interlaced, kind, place):
         reach = sum(np.roll(count, (i, j, k), (0, 1, 2)) for i in range(-2, 3) for j in range(-2, 3) for k in range(-2, 3))
         tol = 2e-6 * total + 2.0 ** -24 * total + 2.0 ** -23 * reach + 1e-6 * np.abs(amp).max()
         assert np.all(np.abs(mesh - ref) <= tol), np.max(np.abs(mesh - ref) / tol)
+
+
+@pytest.mark.parametrize("N,window,interlaced,n", [(64, "cic", False, 64_000), (64, "pcs", True, 63_999),
+                                                   (48, "tsc", True, 27_000), (24, "pcs", False, 8_000)])
+def test_default_tile_of_small_meshes(N, window, interlaced, n):
+    """Plans reserved for 1000 objects a tile or more take tiles of 8 where those of 16
+    (12 at 24) would leave SMs idle; against both tiles asked for and one object fewer
+    reserved.  Tiles hold positions as FP32 offsets below 32, rounded by 2^-20 at most,
+    on either side: with window slopes of at most 1 along three axes and deposits
+    rounded to 2^-22, 6e-6 for each object that reaches a cell, and 2^-23 of the cell."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1712_05834_gb300 as pk
+    pk.build()
+    L = 300.0
+    pos = (torch.rand((n, 3), generator=torch.Generator().manual_seed(N + n)) * L).cuda()
+    got = []
+    for capacity, tile in ((n, 0), (n - 1, 0), (n, 8), (n, 12 if N == 24 else 16)):
+        plan = pk.pk_plan(pk.make_config(L, N, window, interlaced=interlaced, dk=0.1, capacity=capacity, tile=tile))
+        try:
+            pk.pk_paint(plan, pos)
+            got.append([pk.pk_mesh(plan, 0, m, N) for m in range(2 if interlaced else 1)])
+        finally:
+            pk.pk_destroy(plan)
+    c = np.floor(pos.cpu().numpy().astype(np.float64) * N / L).astype(int) % N
+    count = np.bincount((c[:, 0] * N + c[:, 1]) * N + c[:, 2], minlength=N ** 3).reshape(N, N, N)
+    reach = sum(np.roll(count, (i, j, k), (0, 1, 2)) for i in range(-2, 3) for j in range(-2, 3) for k in range(-2, 3))
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.all(np.abs(a - b) <= 6e-6 * reach + 2.0 ** -23 * np.abs(b))
