@@ -216,6 +216,7 @@ template <int LEN, int NB>
 __global__ void __launch_bounds__(AxisCfg<LEN>::T, AxisCfg<LEN>::MINB)
 k_fft_axis(float2 *__restrict__ mesh, long long mesh_c, long long outer_stride, long long astride, int mcut,
            const float2 *__restrict__ twg) {
+    grid_wait(twg);
     extern __shared__ __align__(16) unsigned char smraw[];
     float2 *tw = reinterpret_cast<float2 *>(smraw);
     float2 *buf = tw + LEN;
@@ -245,8 +246,8 @@ cudaError_t axis_inst(float2 *mesh, int nmesh, long long mesh_c, int mhi, const 
     const long long Nh = LEN / 2 + 1;
     const unsigned grid = (unsigned)nmesh * LEN * ((LEN / 2) / NB);
     // y: lines (x, n) with stride Nh; then x: lines (y, n) with stride N Nh
-    kern<<<grid, T, smem, st>>>(mesh, mesh_c, (long long)LEN * Nh, Nh, 0, tw);
-    kern<<<grid, T, smem, st>>>(mesh, mesh_c, Nh, (long long)LEN * Nh, mhi, tw);
+    chained(kern, grid, T, smem, st)(mesh, mesh_c, (long long)LEN * Nh, Nh, 0, tw);
+    chained(kern, grid, T, smem, st)(mesh, mesh_c, Nh, (long long)LEN * Nh, mhi, tw);
     return cudaGetLastError();
 }
 
@@ -521,6 +522,7 @@ __global__ void __launch_bounds__(32 * ZRows<M>::WPB)
 k_zbin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
        const float *__restrict__ cw, const float2 *__restrict__ ph, const float2 *__restrict__ twg,
        const int *__restrict__ kedge, float *__restrict__ partial) {
+    grid_wait(mesh, cw, ph, twg, kedge);
     constexpr int NR = IL ? 4 : 2, RS = ZRows<M>::RS, PPC = ZRows<M>::WPB, N = 2 * M,
                   Nh = M + 1;
     using SM = ZSmem<M, NR>;
@@ -573,6 +575,7 @@ template <int M, int NR>
 __global__ void __launch_bounds__(32 * ZRows<M>::WPB)
 k_zfinish(float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c,
           const float2 *__restrict__ twg) {
+    grid_wait(twg);
     constexpr int RS = ZRows<M>::RS, PPC = ZRows<M>::WPB, N = 2 * M, Nh = M + 1;
     using SM = ZSmem<M, NR>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -623,7 +626,7 @@ cudaError_t zbin_inst(const void *mesh, long long is, long long ms, int nitems, 
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid(G, nitems);
-    kern<<<grid, 32 * ZRows<M>::WPB, smem, st>>>(
+    chained(kern, grid, 32 * ZRows<M>::WPB, smem, st)(
         reinterpret_cast<const float2 *>(mesh), is, ms, g, reinterpret_cast<const float *>(cw),
         reinterpret_cast<const float2 *>(ph), reinterpret_cast<const float2 *>(tw), kedge,
         reinterpret_cast<float *>(partial));
@@ -663,7 +666,7 @@ cudaError_t zfinish_inst(void *mesh, long long is, long long ms, int nitems, int
         occ = 1;
     }
     dim3 grid((unsigned)(nsm > 0 ? nsm : 1) * occ, nitems);
-    kern<<<grid, 32 * ZRows<M>::WPB, smem, st>>>(reinterpret_cast<float2 *>(mesh), is, ms,
+    chained(kern, grid, 32 * ZRows<M>::WPB, smem, st)(reinterpret_cast<float2 *>(mesh), is, ms,
                                                  reinterpret_cast<const float2 *>(tw));
     return cudaGetLastError();
 }

@@ -245,6 +245,7 @@ __device__ __forceinline__ void flush_wsums(double sw, double sw2, double swa, f
 __global__ void __launch_bounds__(256)
 k_wsum_reduce(const double *__restrict__ wpart, int nblk, const int64_t *__restrict__ item_off, int64_t n_one,
               double *__restrict__ wsums, uint4 *__restrict__ wmax) {
+    grid_wait(wpart, item_off);
     __shared__ double red[3][256];
     const int item = blockIdx.x, t = threadIdx.x;
     double a[3] = {0.0, 0.0, 0.0};
@@ -282,6 +283,7 @@ __global__ void __launch_bounds__(kCountThreads)
 k_sort_count(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
              const int64_t *__restrict__ item_off, int64_t n_one, PaintGeom g, uint32_t *__restrict__ count,
              double *__restrict__ wsums, double *__restrict__ wpart, uint4 *__restrict__ wmax) {
+    grid_wait(pos, w, vals, item_off);
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
     const ItemRange range(item_off, n_one, item);
@@ -320,6 +322,7 @@ __global__ void __launch_bounds__(kCountThreads)
 k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const float *__restrict__ vals,
                const int64_t *__restrict__ item_off, int64_t n_one, PaintGeom g, uint32_t *__restrict__ cursor,
                float4 *__restrict__ sorted, uint32_t ntot, int *__restrict__ err) {
+    grid_wait(pos, w, vals, item_off);
     using R = typename PosReal<DT>::type;
     const int item = blockIdx.y;
     const ItemRange range(item_off, n_one, item);
@@ -347,6 +350,7 @@ k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const 
 template <typename T, bool COPY>
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
+    grid_wait(in);
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
     T v[kScanPer];
     T s = 0;
@@ -373,6 +377,7 @@ k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
 template <typename T, bool COPY, bool DIRECT>
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T *__restrict__ copy) {
+    grid_wait(bsum);
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
     T add;
     if constexpr (DIRECT) {
@@ -882,6 +887,7 @@ __global__ void __launch_bounds__(kPaintThreads)
 k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ off,
               const uint32_t *__restrict__ cursor, int *__restrict__ err, PaintGeom g, int S, const uint4 *__restrict__ wmaxs, float wdep, M *__restrict__ mesh,
               long long item_stride, long long mesh_stride, int accumulate) {
+    grid_wait(sorted, off, cursor, wmaxs);
     extern __shared__ __align__(16) unsigned smu[];   // lo[T^3], hi[T^3] or acc64[T^3]; cand[kStage]
     __shared__ uint32_t s_beg[kSegments];
     __shared__ uint32_t s_pre[kSegments + 1];
@@ -1307,6 +1313,7 @@ __global__ void __launch_bounds__(kBinThreads, 5)
 k_bin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
       const float *__restrict__ cw, const float2 *__restrict__ ph, const int *__restrict__ kedge,
       float *__restrict__ partial, const float2 *__restrict__ meshb) {
+    grid_wait(mesh, cw, ph, kedge, meshb);
     using R = float;
     using C = float2;
     using A = float;
@@ -1497,6 +1504,7 @@ __global__ void __launch_bounds__(kBinThreads, 2)
 k_bin_f64(const double2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
           const double *__restrict__ cw, const double2 *__restrict__ ph, const int *__restrict__ kedge,
           double *__restrict__ partial, const double2 *__restrict__ meshb) {
+    grid_wait(mesh, cw, ph, kedge, meshb);
     using SM = Bin64Smem;
     constexpr int kRows = 4;                          // rows per warp and turn
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -1683,6 +1691,7 @@ k_reduce_finalize(const A *__restrict__ partial, int G, const unsigned long long
                   const unsigned long long *__restrict__ modes2d, const double *__restrict__ wsums,
                   const int *__restrict__ err, FinalGeom f, ResultLayout rl, double *__restrict__ res, int cross_a,
                   int cross_b) {
+    grid_wait(partial, modes1d, modes2d, wsums, err);
     extern __shared__ __align__(16) unsigned char smraw[];
     double *sum = reinterpret_cast<double *>(smraw);       // the block's slots
     __shared__ double red[256];
@@ -1896,8 +1905,8 @@ cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const 
     const bool weighted = w != nullptr || vals != nullptr || dtype == PK_F32X4;
     dim3 grid(grid_for(max_n, kCountThreads, weighted ? kWsumBlocks : 1u << 20), nitems);
 #define PK_COUNT(DT)                                                                                    \
-    if (weighted) k_sort_count<DT, true><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, count, wsums, wpart, wmax); \
-    else k_sort_count<DT, false><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, count, wsums, wpart, wmax);
+    if (weighted) chained(k_sort_count<DT, true>, grid, kCountThreads, 0, st)(pos, w, vals, item_off, max_n, g, count, wsums, wpart, wmax); \
+    else chained(k_sort_count<DT, false>, grid, kCountThreads, 0, st)(pos, w, vals, item_off, max_n, g, count, wsums, wpart, wmax);
     switch (dtype) {
     case PK_F32: PK_COUNT(PK_F32) break;
     case PK_F64: PK_COUNT(PK_F64) break;
@@ -1907,7 +1916,7 @@ cudaError_t launch_sort_count(const void *pos, int dtype, const float *w, const 
     if (weighted) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, max_n, wsums, wmax);
+        chained(k_wsum_reduce, nitems, 256, 0, st)(wpart, (int)grid.x, item_off, max_n, wsums, wmax);
     }
     return cudaGetLastError();
 }
@@ -1919,9 +1928,9 @@ cudaError_t launch_sort_scatter(const void *pos, int dtype, const float *w, cons
                                 uint32_t *cursor, float4 *sorted, uint32_t ntot, int *err, cudaStream_t st) {
     dim3 grid(grid_for(max_n, kCountThreads, 1u << 20), nitems);
     switch (dtype) {
-    case PK_F32: k_sort_scatter<PK_F32><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
-    case PK_F64: k_sort_scatter<PK_F64><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
-    default: k_sort_scatter<PK_F32X4><<<grid, kCountThreads, 0, st>>>(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
+    case PK_F32: chained(k_sort_scatter<PK_F32>, grid, kCountThreads, 0, st)(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
+    case PK_F64: chained(k_sort_scatter<PK_F64>, grid, kCountThreads, 0, st)(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
+    default: chained(k_sort_scatter<PK_F32X4>, grid, kCountThreads, 0, st)(pos, w, vals, item_off, max_n, g, cursor, sorted, ntot, err); break;
     }
     return cudaGetLastError();
 }
@@ -1963,21 +1972,21 @@ template <typename T, bool COPY>
 static cudaError_t scan_impl(const T *in, int64_t n, T *out, T *tmp, T *copy, int *launches, cudaStream_t st) {
     const int64_t nb = (n + kScanTile - 1) / kScanTile;
     if (nb <= 1) {
-        k_scan_blocks<T, COPY><<<1, kScanThreads, 0, st>>>(in, n, out, out + n, copy);
+        chained(k_scan_blocks<T, COPY>, 1, kScanThreads, 0, st)(in, n, out, out + n, copy);
         *launches += 1;
         return cudaGetLastError();
     }
     if (nb > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_scan_blocks<T, false><<<(unsigned)nb, kScanThreads, 0, st>>>(in, n, out, tmp, nullptr);
+    chained(k_scan_blocks<T, false>, (unsigned)nb, kScanThreads, 0, st)(in, n, out, tmp, nullptr);
     *launches += 1;
     if (nb <= kScanDirect) {
-        k_scan_add<T, COPY, true><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
+        chained(k_scan_add<T, COPY, true>, (unsigned)nb, kScanThreads, 0, st)(out, n, tmp, (int)nb, copy);
         *launches += 1;
         return cudaGetLastError();
     }
     cudaError_t e = scan_impl<T, false>(tmp, nb, tmp, tmp + nb + 1, nullptr, launches, st);
     if (e != cudaSuccess) return e;
-    k_scan_add<T, COPY, false><<<(unsigned)nb, kScanThreads, 0, st>>>(out, n, tmp, (int)nb, copy);
+    chained(k_scan_add<T, COPY, false>, (unsigned)nb, kScanThreads, 0, st)(out, n, tmp, (int)nb, copy);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -2012,7 +2021,7 @@ static cudaError_t paint_inst(const float4 *sorted, const uint32_t *off, const u
     auto kern = g.T == 16 ? k_paint_tiles<P, NM, M, 16, UNIT> : k_paint_tiles<P, NM, M, 0, UNIT>;
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)nblocks, kPaintThreads, smem, st>>>(sorted, off, cursor, err, g, S, wmax, wdep,
+    chained(kern, (unsigned)nblocks, kPaintThreads, smem, st)(sorted, off, cursor, err, g, S, wmax, wdep,
                                                          reinterpret_cast<M *>(mesh), item_stride,
                                                          mesh_stride, accumulate);
     return cudaGetLastError();
@@ -2053,7 +2062,7 @@ static cudaError_t atomic_inst(const void *pos, const float *w, const float *val
     if (weighted) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        k_wsum_reduce<<<nitems, 256, 0, st>>>(wpart, (int)grid.x, item_off, max_n, wsums, wmax);
+        chained(k_wsum_reduce, nitems, 256, 0, st)(wpart, (int)grid.x, item_off, max_n, wsums, wmax);
     }
     return cudaGetLastError();
 }
@@ -2142,7 +2151,7 @@ static cudaError_t bin_inst(const void *mesh, long long item_stride_c, long long
     cudaError_t e = set_smem(kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid(G, nitems);
-    kern<<<grid, kBinThreads, smem, st>>>(reinterpret_cast<const C *>(mesh), item_stride_c,
+    chained(kern, grid, kBinThreads, smem, st)(reinterpret_cast<const C *>(mesh), item_stride_c,
                                           mesh_stride_c, g, reinterpret_cast<const R *>(cw),
                                           reinterpret_cast<const C *>(ph), kedge,
                                           reinterpret_cast<R *>(partial), reinterpret_cast<const C *>(meshb));
@@ -2215,10 +2224,10 @@ cudaError_t launch_reduce_finalize(const void *partial, int f64, int G, const un
     const size_t smem = sizeof(double) * (size_t)KB * ((f.twod ? f.nmu : 1) + (f.poles ? 2 : 0));   // <= 8 KB
     const dim3 grid((f.nk + KB - 1) / KB, nitems);
     if (f64)
-        k_reduce_finalize<double><<<grid, 256, smem, st>>>(reinterpret_cast<const double *>(partial), G, modes1d,
+        chained(k_reduce_finalize<double>, grid, 256, smem, st)(reinterpret_cast<const double *>(partial), G, modes1d,
                                                            modes2d, wsums, err, f, rl, res, cross_a, cross_b);
     else
-        k_reduce_finalize<float><<<grid, 256, smem, st>>>(reinterpret_cast<const float *>(partial), G, modes1d,
+        chained(k_reduce_finalize<float>, grid, 256, smem, st)(reinterpret_cast<const float *>(partial), G, modes1d,
                                                           modes2d, wsums, err, f, rl, res, cross_a, cross_b);
     return cudaGetLastError();
 }
