@@ -65,10 +65,12 @@ constexpr int kScanTile = kScanThreads * kScanPer;
 #ifdef __CUDACC__
 // Launches whose overhead overlaps the kernel before (programmatic dependent launch):
 // the kernel begins with grid_wait(), which returns when every kernel before it on the
-// stream has ended and its writes can be seen.  Grids of kChainedCtas or fewer only: a
-// 64^3 catalog 86 -> 72 us, weighted 100^3 halos 121 -> 104, 2e6 objects at 256^3 241 ->
-// 231; with every grid 256^3 took 246 us, 1e7 objects at 512^3 2.31 ms for 2.01.
-constexpr unsigned kChainedCtas = 1216;
+// stream has ended and its writes can be seen.  Grids up to kChainedCtas; those up to
+// kEarlyCtas also let the next kernel's CTAs in as soon as all of their own have
+// started: a 64^3 catalog 86 -> 72 us, weighted 100^3 halos 121 -> 104, 2e6 objects at
+// 256^3 241 -> 219 (231 with only those chained; early entry at every size: 246, and 1e7
+// objects at 512^3 2.31 ms for 2.01).
+constexpr unsigned kChainedCtas = 8192, kEarlyCtas = 1216;
 template <typename... Args>
 struct ChainedLaunch {
     void (*kernel)(Args...);
@@ -97,10 +99,9 @@ ChainedLaunch<Args...> chained(void (*kernel)(Args...), dim3 grid, dim3 block, s
 // first knows after the wait, so that no load through them can move above it.
 template <typename... P>
 __device__ __forceinline__ void grid_wait(P &...p) {
-    if ((unsigned long long)gridDim.x * gridDim.y <= kChainedCtas) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    }
+    const unsigned long long ctas = (unsigned long long)gridDim.x * gridDim.y;
+    if (ctas <= kChainedCtas) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (ctas <= kEarlyCtas) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int zero;
     asm volatile("mov.b32 %0, 0;" : "=r"(zero)::"memory");
     ((p = (P)((const char *)p + zero)), ...);
