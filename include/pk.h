@@ -560,8 +560,10 @@ pk_status pk_survey_bounds(const pk_survey_catalog *cat, double omega_m, double 
 typedef enum {
     PK_SURVEY_STAGE_PREP = 0,    /* catalog conversion + sums (pk_survey_paint)     */
     PK_SURVEY_STAGE_PAINT = 1,   /* tile sort + paint of both catalogs              */
-    PK_SURVEY_STAGE_FFT = 2,     /* every cuFFT call of pk_survey_compute           */
-    PK_SURVEY_STAGE_FIELD = 3,   /* FKP combine, interlacing, Y_lm weighting         */
+    PK_SURVEY_STAGE_FFT = 2,     /* every transform of pk_survey_compute (own sizes:
+                                    with the FKP combine and Y_lm weighting)        */
+    PK_SURVEY_STAGE_FIELD = 3,   /* FKP combine, interlacing, Y_lm weighting, where
+                                    passes of their own (else 0)                    */
     PK_SURVEY_STAGE_BIN = 4,     /* per-mode sums of A_0 and the Y_lm transforms     */
     PK_SURVEY_STAGE_FINAL = 5,   /* row reduce + normalization                      */
     PK_SURVEY_NSTAGES = 6
