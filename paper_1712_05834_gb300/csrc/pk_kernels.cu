@@ -407,7 +407,10 @@ k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T
 
 // ---- tile paint ----
 // Per-axis B-spline weights of order P at node-relative coordinate u (cells):
-// nodes base .. base + P - 1.
+// nodes base .. base + P - 1.  Every multiply-add is written out: left to the
+// compiler, 0.75 - g g was contracted in some instances of k_paint_tiles and not
+// in others, so that an object's cells depended on the instance (weighted or
+// not, one mesh or two, tile edge) that painted them.
 template <int P>
 __device__ __forceinline__ void spline_weights(float u, int &base, float *wt) {
     if (P == 2) {                       // CIC
@@ -422,7 +425,7 @@ __device__ __forceinline__ void spline_weights(float u, int &base, float *wt) {
         base = (int)f0;
         const float a = 0.5f - g, b = 0.5f + g;
         wt[0] = 0.5f * a * a;
-        wt[1] = 0.75f - g * g;
+        wt[1] = __fmaf_rn(-g, g, 0.75f);
         wt[2] = 0.5f * b * b;
     } else {                            // PCS
         const float f0 = floorf(u);
@@ -430,8 +433,8 @@ __device__ __forceinline__ void spline_weights(float u, int &base, float *wt) {
         base = (int)f0 - 1;
         const float f2 = f * f, r2 = r * r;
         wt[0] = (1.0f / 6.0f) * r2 * r;
-        wt[1] = (1.0f / 6.0f) * (4.0f - 6.0f * f2 + 3.0f * f2 * f);
-        wt[2] = (1.0f / 6.0f) * (4.0f - 6.0f * r2 + 3.0f * r2 * r);
+        wt[1] = (1.0f / 6.0f) * __fmaf_rn(3.0f * f2, f, __fmaf_rn(-6.0f, f2, 4.0f));
+        wt[2] = (1.0f / 6.0f) * __fmaf_rn(3.0f * r2, r, __fmaf_rn(-6.0f, r2, 4.0f));
         wt[3] = (1.0f / 6.0f) * f2 * f;
     }
 }

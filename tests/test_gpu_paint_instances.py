@@ -1,0 +1,43 @@
+"""An object's deposits do not depend on which instance of the tile paint serves the
+call: painted with unit weights or with an array of ones, in tiles of few objects or
+many, the cells of the FP64 mesh form (window weights and one rounding per deposit,
+summed as integers) are the same bits.  With and without the interlaced mesh a tile
+looks at more or fewer candidates, and the split of its deposits into two words may
+round one of them the other way: a unit of 2^-32 for each object that reaches a cell."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _cells(pk, pos, w, N, window, interlaced):
+    plan = pk.pk_plan(pk.make_config(100.0, N, window, interlaced=interlaced, dk=0.2, precision="f64"))
+    try:
+        pk.pk_paint(plan, pos, w)
+        return [pk.pk_mesh(plan, 0, m, N, f64=True) for m in range(2 if interlaced else 1)]
+    finally:
+        pk.pk_destroy(plan)
+
+
+# 96: tiles of 16 known at compile time; 72: of 12.  The counts put some 30, 240 and
+# 2000 objects into a tile: staged at once, in batches, and cells of 64 bits.
+@pytest.mark.parametrize("window", ["cic", "tsc", "pcs"])
+@pytest.mark.parametrize("N,n", [(96, 6001), (96, 200_003), (72, 50_001), (72, 430_001), (48, 100_003)])
+def test_ones_and_unit_weights_paint_the_same_cells(window, N, n):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1712_05834_gb300 as pk
+    pk.build()
+    pos = (torch.rand((n, 3), generator=torch.Generator().manual_seed(n), dtype=torch.float64) * 100.0).cuda()
+    ones = torch.ones(n, device="cuda")
+    c = np.floor(pos.cpu().numpy() * (N / 100.0)).astype(int) % N
+    count = np.bincount((c[:, 0] * N + c[:, 1]) * N + c[:, 2], minlength=N ** 3).reshape(N, N, N)
+    reach = sum(np.roll(count, (i, j, k), (0, 1, 2)) for i in range(-2, 3) for j in range(-2, 3) for k in range(-2, 3))
+    first = []
+    for interlaced in (True, False):
+        unit, weighted = (_cells(pk, pos, w, N, window, interlaced) for w in (None, ones))
+        for a, b in zip(unit, weighted):
+            assert np.array_equal(a, b), (interlaced, int((a != b).sum()))
+        first.append(unit[0])
+    assert np.all(np.abs(first[0] - first[1]) <= 2.0 ** -32 * reach)
