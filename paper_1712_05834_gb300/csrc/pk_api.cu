@@ -292,7 +292,7 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
 
     int rlo, rhi;
     window_reach(P->p, c.interlaced, &rlo, &rhi);
-    int T = choose_tile(P->N, rhi - rlo, c.tile);
+    const int T = choose_tile(P->N, rhi - rlo, c.tile);
     if (T <= 0)
         return fail(P, PK_EINVAL, "tile must divide nmesh, be >= the window reach and fit in shared memory");
     const double L = c.box_size;
@@ -308,15 +308,6 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
     PK_CUDA(P, cudaDeviceGetAttribute(&P->nsm, cudaDevAttrMultiProcessorCount, P->device));
 
     // ---- paint geometry ----
-    // Tiles on less than half of the SMs, each with 1000 objects or more: tiles of 8 (one
-    // catalog at 64^3, us a spectrum, tiles of 16 and 8: 2.5e5 CIC 114 and 88, weighted PCS
-    // interlaced 162 and 131; 1e5 88 and 82, 107 and 102; 6e4 82 and 77, 92 and 88; 2e4 70
-    // and 76, 74 and 78).  At 80^3 they lose for PCS (2.5e5: 131 and 146), from 128^3 on
-    // for all (sort and paint of 1e6 TSC interlaced 107 and 130).
-    if (c.tile <= 0 && T > 8 && P->N % 8 == 0 && rhi - rlo <= 8) {
-        const long long ntile = (long long)(P->N / T) * (P->N / T) * (P->N / T) * P->B;
-        if (2 * ntile < P->nsm && c.capacity >= 1000 * ntile) T = 8;
-    }
     PaintGeom &pg = P->pg;
     pg.invH = (float)((double)P->N / c.box_size);
     pg.invH_lo = (float)((double)P->N / c.box_size - (double)pg.invH);
