@@ -452,13 +452,19 @@ struct Split {
     int fast;         // 1: split when needed; 0: this tile uses 64-bit shared atomics instead
 };
 
-// round(vxy wz) as a two's complement word.  UNIT: in [0, 2^23), by one FMA
-// against 2^23, whose bits hold the integer; else any |v| < 2^31, by a conversion
-// (16 lanes a clock on this part, hidden behind the shared atomics).
+// round(vxy wz) as a two's complement word, the exact product rounded once.  UNIT:
+// in [0, 2^23), by one FMA against 2^23, whose bits hold the integer.  Else any |v| <
+// 2^31: below 2^22 by an FMA against 1.5 2^23; from there on the FP32 product holds
+// two binary places at most and is converted (a product converted at any size was
+// rounded twice).
 template <bool UNIT>
 __device__ __forceinline__ unsigned quantize(float vxy, float wz) {
-    if constexpr (UNIT) return __float_as_uint(fmaf(vxy, wz, 8388608.0f)) - 0x4B000000u;
-    else return (unsigned)__float2int_rn(vxy * wz);
+    if constexpr (UNIT) {
+        return __float_as_uint(fmaf(vxy, wz, 8388608.0f)) - 0x4B000000u;
+    } else {
+        const unsigned q = __float_as_uint(fmaf(vxy, wz, 12582912.0f)) - 0x4B400000u;
+        return q + (1u << 22) < (1u << 23) ? q : (unsigned)__float2int_rn(vxy * wz);
+    }
 }
 
 // MODE 2: the tile's cells fit one word each (see the sweep in k_paint_tiles):

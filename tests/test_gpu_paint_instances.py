@@ -41,3 +41,28 @@ def test_ones_and_unit_weights_paint_the_same_cells(window, N, n):
             assert np.array_equal(a, b), (interlaced, int((a != b).sum()))
         first.append(unit[0])
     assert np.all(np.abs(first[0] - first[1]) <= 2.0 ** -32 * reach)
+
+
+# FP32 form: deposits of an array of ones are below 2^22, where each is the exact product
+# rounded once, as with unit weights; of minus ones, the negative (ties go to even).
+@pytest.mark.parametrize("window", ["cic", "tsc", "pcs"])
+@pytest.mark.parametrize("N,n", [(96, 6001), (96, 200_003), (72, 50_001), (40, 30_001)])
+@pytest.mark.parametrize("interlaced", [False, True])
+def test_ones_in_the_fp32_form(window, N, n, interlaced):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1712_05834_gb300 as pk
+    pk.build()
+    pos = (torch.rand((n, 3), generator=torch.Generator().manual_seed(n)) * 100.0).cuda()
+    got = []
+    for w in (None, torch.ones(n, device="cuda"), -torch.ones(n, device="cuda")):
+        plan = pk.pk_plan(pk.make_config(100.0, N, window, interlaced=interlaced, dk=0.2))
+        try:
+            pk.pk_paint(plan, pos, w)
+            got.append([pk.pk_mesh(plan, 0, m, N) for m in range(2 if interlaced else 1)])
+        finally:
+            pk.pk_destroy(plan)
+    for unit, ones, minus in zip(*got):
+        assert np.array_equal(unit, ones), int((unit != ones).sum())
+        assert np.array_equal(unit, -minus), int((unit != -minus).sum())
