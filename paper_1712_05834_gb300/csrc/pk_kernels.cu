@@ -265,7 +265,8 @@ k_wsum_reduce(const double *__restrict__ wpart, int nblk, const int64_t *__restr
     if (t == 3) {
         const ItemRange range(item_off, n_one, item);
         const float n = (float)(range.end - range.beg);
-        wmax[item].z = __float_as_uint(n > 0.0f ? (float)red[2][0] / n : 0.0f);
+        // ten bits of it: the rounding of the sum, and so the order of the objects, is not seen
+        wmax[item].z = __float_as_uint(n > 0.0f ? (float)red[2][0] / n : 0.0f) & 0xffffe000u;
     }
 }
 
@@ -1028,11 +1029,16 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
             if (dense)
                 atomicAdd(s_blk + block_of<P>(v.x, v.y, v.z, T > 16), UNIT ? 1u : __float2uint_ru(fabsf(v.w) * blk_scale));
         };
-        float sum_abs = 0.0f;
+        // |W V| in units rounded up, as integers: the sum, and so the path taken, does
+        // not depend on the order of the candidates (NaN: far too much)
+        unsigned long long sum_abs = 0ull;
+        const auto add_abs = [&](float w) {
+            if (!UNIT) sum_abs += fabsf(w) < 4.29e9f ? (unsigned long long)__float2uint_ru(fabsf(w)) : 1ull << 40;
+        };
         if (kPadded) {
             for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
                 const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
-                if (!UNIT) sum_abs += fabsf(v.w);
+                add_abs(v.w);
                 count(v);
                 sweep_deposit<P, UNIT>(smu, v.x, v.y, v.z, v.w);
                 if (NM == 2)
@@ -1044,7 +1050,7 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
             const bool flat = !dense && total <= (uint32_t)kFlatMaxCand;
             for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
                 const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
-                if (!UNIT) sum_abs += fabsf(v.w);
+                add_abs(v.w);
                 count(v);
                 if (flat) {
                     deposit_flat<P, TC, UNIT>(smu, 0, trash, T, v.x, v.y, v.z, v.w);
@@ -1075,16 +1081,16 @@ k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ of
         } else if constexpr (UNIT) {
             __syncthreads();
         } else {
-            __shared__ float s_abs[kPaintThreads / 32];
+            __shared__ unsigned long long s_abs[kPaintThreads / 32];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sum_abs += __shfl_down_sync(0xffffffffu, sum_abs, o);
             if ((threadIdx.x & 31) == 0) s_abs[threadIdx.x >> 5] = sum_abs;
             __syncthreads();
-            float t = 0.0f;
+            unsigned long long t = 0ull;
 #pragma unroll
             for (int k = 0; k < kPaintThreads / 32; ++k) t += s_abs[k];
             // every cell: sum of round(w W V 2^S) <= wdep sum |W V| 2^S + candidates / 2
-            fits = t * wdep + ncf < cell_max;
+            fits = (float)t * wdep + ncf < cell_max;
         }
         if (fits) {
             const Split none{};

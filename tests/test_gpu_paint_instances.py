@@ -66,3 +66,34 @@ def test_ones_in_the_fp32_form(window, N, n, interlaced):
     for unit, ones, minus in zip(*got):
         assert np.array_equal(unit, ones), int((unit != ones).sum())
         assert np.array_equal(unit, -minus), int((unit != -minus).sum())
+
+
+def test_cells_at_the_limit_of_one_word_do_not_depend_on_the_order():
+    """A tile whose sum of |W| is at the limit up to which its cells are kept in one word
+    (2^22 sum W + n = 4.29e9): whatever order its objects come in, it is painted the same
+    way, and its cells are the same bits."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1712_05834_gb300 as pk
+    pk.build()
+    N, n, light = 64, 1000, 20_000
+    rng = np.random.default_rng(7)
+    pos = np.concatenate([2.0 + 11.0 * rng.random((n, 3)), 34.0 + 11.0 * rng.random((light, 3))]).astype(np.float32)
+    w = np.concatenate([rng.uniform(0.9, 1.1, n), np.full(light, 0.01)]).astype(np.float32)
+    w[:n] *= np.float32((4.29e9 - n) / 2.0 ** 22 / w[:n].astype(np.float64).sum())
+    w[0] += np.float32((4.29e9 - n) / 2.0 ** 22 - w[:n].astype(np.float64).sum())
+    plan = pk.pk_plan(pk.make_config(float(N), N, "cic", dk=0.2))
+    try:
+        for step in range(-24, 25):
+            wk = w.copy()
+            wk[0] += np.float32(step * 2.0 ** -15)                # 128 units of 2^-22
+            first = None
+            for _ in range(4):
+                o = rng.permutation(n + light)
+                pk.pk_paint(plan, torch.from_numpy(pos[o]).cuda(), torch.from_numpy(wk[o]).cuda())
+                cells = pk.pk_mesh(plan, 0, 0, N)
+                first = cells if first is None else first
+                assert np.array_equal(first, cells), (step, int((first != cells).sum()))
+    finally:
+        pk.pk_destroy(plan)
