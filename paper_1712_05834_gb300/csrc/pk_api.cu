@@ -70,7 +70,7 @@ void free_plan(pk_plan_s *p) {
     void *dev[] = {p->mesh, p->d_off, p->d_scan_tmp, p->d_sorted,
                    p->d_stage, p->d_item_off, p->d_wsums, p->d_wpart, p->d_cw, p->d_ph,
                    p->d_kedge, p->d_partial, p->d_modes1d, p->d_modes2d,
-                   p->d_err, p->d_acc, p->fft_work, p->d_proj, p->d_tw};
+                   p->d_err, p->d_acc, p->fft_work, p->d_proj, p->d_tw, p->d_sync, p->d_xtiles};
     for (void *d : dev)
         if (d) cudaFree(d);
     if (p->h_res) cudaFreeHost(p->h_res);
