@@ -741,6 +741,7 @@ static pk_status finish_transform(pk_plan_s *P, int nitems) {
                                   nitems, P->N, P->d_tw, P->nsm, P->st));
     P->launches += 1;
     P->unfinished = 0;
+    P->sync_used = 0;
     return PK_OK;
 }
 
@@ -778,6 +779,7 @@ pk_status pk_compute(pk_plan_t P) {
         } else {
             // z and y axes, then x fused into the bin pass (or, where its
             // histogram does not fit beside a tile, x in place and k_bin)
+            PK_CUDA(P, zyx_counters(P->d_sync, P->nsync, &P->sync_used, st));
             PK_CUDA(P, P->zyx->zy(P->mesh, nitems * P->nm * P->N, P->fft_ncol, P->bg.mhi, P->d_tw, P->d_sync,
                                   P->d_err, P->nsm, st));
             P->launches += 1;
@@ -787,6 +789,7 @@ pk_status pk_compute(pk_plan_t P) {
                 PK_CUDA(P, P->zyx->xbin(P->mesh, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->fft_ncol,
                                         P->d_xtiles, P->nxbin, P->d_cw, P->d_ph, P->d_tw, P->d_kedge, P->d_partial,
                                         P->d_sync, P->nsync, st));
+                P->sync_used = 0;
             } else {
                 if (pk_status s = finish_transform(P, nitems); s != PK_OK) return s;
                 if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));

@@ -260,6 +260,15 @@ struct ZyxOps {
 protected:
     ~ZyxOps() = default;
 };
+// The counters of the z / y pass before a launch of it: zero at first and again after
+// every x axis pass; cleared here if the pass that should have done so was never launched
+// (the z / y pass would find its last ticket given out and leave the mesh as it is).
+// *used: set until the x axis pass is on the stream.
+inline cudaError_t zyx_counters(unsigned *sync, int nsync, int *used, cudaStream_t st) {
+    const cudaError_t e = *used ? cudaMemsetAsync(sync, 0, sizeof(unsigned) * nsync, st) : cudaSuccess;
+    *used = 1;
+    return e;
+}
 const ZyxOps *zyx_ops_group0(int N);
 const ZyxOps *zyx_ops_group1(int N);
 const ZyxOps *zyx_ops_group2(int N);

@@ -43,7 +43,7 @@ struct pk_plan_s {
     pk::Fft64 fft64{};               // FP64 form: steps and tables (both in d_tw)
     void *d_tw = nullptr;            // W_N^e, e < N (float2)
     unsigned *d_sync = nullptr;      // zyx: ticket and plane counters of the z / y pass
-    int nsync = 0;
+    int nsync = 0, sync_used = 0;    // sync_used: see zyx_counters
     int fft_ncol = 0;                // zyx: columns l that hold a binned mode
     int *d_xtiles = nullptr;         // zyx: tiles of the x axis, fused pass then plain pass
     int nxbin = 0, nx = 0;

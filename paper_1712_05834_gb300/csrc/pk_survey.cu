@@ -654,7 +654,8 @@ struct pk_survey_s {
     const pk::ZyxOps *zyx = nullptr;
     void *tw = nullptr;             // W_N^e, e < N (float2)
     unsigned *sync = nullptr;       // work counters of the z / y pass
-    int nsync = 0, ncol = 0;        // columns l that hold a binned mode
+    int nsync = 0, sync_used = 0;   // sync_used: see zyx_counters
+    int ncol = 0;                   // columns l that hold a binned mode
     int *xtiles = nullptr;          // x tiles: those with a binned mode, then all
     int nx_bin = 0, nx_all = 0;
     cufftHandle fft_b = 0, fft_inv = 0;   // single-mesh r2c, single-mesh c2r
@@ -1176,9 +1177,11 @@ static pk_status survey_compute_t(pk_survey_s *S) {
             rows.R = Rm;                        // the second meshes follow the first in both catalogs
             rows.s0 = -1;
             rows.nslot = 1;
+            SV_CUDA(S, pk::zyx_counters(S->sync, S->nsync, &S->sync_used, st));
             SV_CUDA(S, S->zyx->zy_survey(D, S->nm * N, rows, Nh, 0x7fffffff, S->tw, S->sync, P->d_err, S->nsm, st));
             SV_CUDA(S, S->zyx->x(D, S->nm, mr / 2, Nh, 0x7fffffff, S->xtiles + S->nx_bin, S->nx_all, S->tw, S->sync,
                                  S->nsync, st));
+            S->sync_used = 0;
             S->launches += 1;
         } else {
             SV_CUDA(S, tmark(S, 1, PK_SURVEY_STAGE_FIELD));
@@ -1235,9 +1238,11 @@ static pk_status survey_compute_t(pk_survey_s *S) {
                 rows.s0 = part == 0 ? -1 : s0;
                 rows.nslot = part == 0 ? 1 : nb;
                 if (part == 0 ? !a0copy : nb == 0) continue;
+                SV_CUDA(S, pk::zyx_counters(S->sync, S->nsync, &S->sync_used, st));
                 SV_CUDA(S, S->zyx->zy_survey(dst, N, rows, S->ncol, mhi, S->tw, S->sync, P->d_err, S->nsm, st));
                 SV_CUDA(S, S->zyx->x(dst, rows.nslot, mr / 2, S->ncol, mhi, S->xtiles, S->nx_bin, S->tw, S->sync,
                                      S->nsync, st));
+                S->sync_used = 0;
                 S->launches += 2;
             }
         } else if (nb > 0 || a0copy) {
