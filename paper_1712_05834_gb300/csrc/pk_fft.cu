@@ -216,7 +216,7 @@ template <int LEN, int NB>
 __global__ void __launch_bounds__(AxisCfg<LEN>::T, AxisCfg<LEN>::MINB)
 k_fft_axis(float2 *__restrict__ mesh, long long mesh_c, long long outer_stride, long long astride, int mcut,
            const float2 *__restrict__ twg) {
-    grid_wait(twg);
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     float2 *tw = reinterpret_cast<float2 *>(smraw);
     float2 *buf = tw + LEN;
@@ -519,10 +519,10 @@ __device__ __forceinline__ void bin_pair(const float2 *rows, int i, int j, int p
 // r2 = kx'^2 + ky'^2 puts no mode into a bin (their rows are not read).
 template <bool IL, bool TWOD, bool POLES, bool MU32, int M>
 __global__ void __launch_bounds__(32 * ZRows<M>::WPB)
-k_zbin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
-       const float *__restrict__ cw, const float2 *__restrict__ ph, const float2 *__restrict__ twg,
-       const int *__restrict__ kedge, float *__restrict__ partial) {
-    grid_wait(mesh, cw, ph, twg, kedge);
+k_zbin(const float2 *mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
+       const float *cw, const float2 *ph, const float2 *__restrict__ twg, const int *kedge,
+       float *__restrict__ partial) {
+    grid_wait();
     constexpr int NR = IL ? 4 : 2, RS = ZRows<M>::RS, PPC = ZRows<M>::WPB, N = 2 * M,
                   Nh = M + 1;
     using SM = ZSmem<M, NR>;
@@ -575,7 +575,7 @@ template <int M, int NR>
 __global__ void __launch_bounds__(32 * ZRows<M>::WPB)
 k_zfinish(float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c,
           const float2 *__restrict__ twg) {
-    grid_wait(twg);
+    grid_wait();
     constexpr int RS = ZRows<M>::RS, PPC = ZRows<M>::WPB, N = 2 * M, Nh = M + 1;
     using SM = ZSmem<M, NR>;
     extern __shared__ __align__(16) unsigned char smraw[];

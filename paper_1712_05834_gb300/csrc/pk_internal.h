@@ -95,8 +95,12 @@ template <typename... Args>
 ChainedLaunch<Args...> chained(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t st) {
     return {kernel, grid, block, smem, st};
 }
-// p: the kernel's read-only pointers.  They get an offset (zero) that the compiler
-// first knows after the wait, so that no load through them can move above it.
+// Such a kernel begins before the kernel ahead of it has ended, so what a kernel of the
+// same call wrote is not constant over its lifetime: it is read through plain pointers
+// (const without __restrict__, no __ldg), not through the read-only path.
+// p: pointers to the caller's data, constant from before the call on and read through
+// that path; they get an offset (zero) that the compiler first knows after the wait, so
+// that no load through them can move above it.
 template <typename... P>
 __device__ __forceinline__ void grid_wait(P &...p) {
     const unsigned long long ctas = (unsigned long long)gridDim.x * gridDim.y;

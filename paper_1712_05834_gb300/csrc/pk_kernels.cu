@@ -243,9 +243,9 @@ __device__ __forceinline__ void flush_wsums(double sw, double sw2, double swa, f
 // is added to wsums[4 * item + k] (one writer per value).  wmax[item].z: the
 // mean |W V| (float bits), from which the tile paint guesses a tile's sum.
 __global__ void __launch_bounds__(256)
-k_wsum_reduce(const double *__restrict__ wpart, int nblk, const int64_t *__restrict__ item_off, int64_t n_one,
+k_wsum_reduce(const double *wpart, int nblk, const int64_t *__restrict__ item_off, int64_t n_one,
               double *__restrict__ wsums, uint4 *__restrict__ wmax) {
-    grid_wait(wpart, item_off);
+    grid_wait(item_off);
     __shared__ double red[3][256];
     const int item = blockIdx.x, t = threadIdx.x;
     double a[3] = {0.0, 0.0, 0.0};
@@ -351,7 +351,7 @@ k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const 
 template <typename T, bool COPY>
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
-    grid_wait(in);
+    grid_wait();
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
     T v[kScanPer];
     T s = 0;
@@ -377,8 +377,8 @@ k_scan_blocks(const T *in, int64_t n, T *out, T *bsum, T *copy) {
 // else their exclusive scan with the total in bsum[nb].
 template <typename T, bool COPY, bool DIRECT>
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_add(T *__restrict__ out, int64_t n, const T *__restrict__ bsum, int nb, T *__restrict__ copy) {
-    grid_wait(bsum);
+k_scan_add(T *__restrict__ out, int64_t n, const T *bsum, int nb, T *__restrict__ copy) {
+    grid_wait();
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
     T add;
     if constexpr (DIRECT) {
@@ -760,7 +760,7 @@ __device__ __forceinline__ int seg_dz(int s) { return s % 3 - 1; }
 
 // Candidate k of the tile (k < s_pre[kSegments]) in this tile's frame
 // (segment shift added), weight scaled by 2^S.
-__device__ __forceinline__ float4 fetch_candidate(const float4 *__restrict__ sorted, const uint32_t *s_beg,
+__device__ __forceinline__ float4 fetch_candidate(const float4 *sorted, const uint32_t *s_beg,
                                                   const uint32_t *s_pre, int T, uint32_t k, float scale) {
     int lo_s = 0, hi_s = kSegments;                   // s_pre[lo_s] <= k < s_pre[hi_s]
     while (hi_s - lo_s > 1) {
@@ -768,13 +768,13 @@ __device__ __forceinline__ float4 fetch_candidate(const float4 *__restrict__ sor
         if (s_pre[mid] <= k) lo_s = mid;
         else hi_s = mid;
     }
-    const float4 v = __ldg(sorted + s_beg[lo_s] + (k - s_pre[lo_s]));
+    const float4 v = sorted[s_beg[lo_s] + (k - s_pre[lo_s])];
     return make_float4(v.x + (float)(seg_dx(lo_s) * T), v.y + (float)(seg_dy(lo_s) * T),
                        v.z + (float)(seg_dz(lo_s) * T), v.w * scale);
 }
 
 // Copy candidates [k0, k0 + n) of the tile into shared memory.
-__device__ __forceinline__ void stage_candidates(const float4 *__restrict__ sorted, const uint32_t *s_beg,
+__device__ __forceinline__ void stage_candidates(const float4 *sorted, const uint32_t *s_beg,
                                                  const uint32_t *s_pre, int T, uint32_t k0, uint32_t n,
                                                  float scale, float4 *cand) {
     for (uint32_t j = threadIdx.x; j < n; j += blockDim.x)
@@ -894,10 +894,10 @@ __host__ __device__ constexpr int paint_cell_words(int T) { return (2 * T * T * 
 // TC > 0: the tile edge is the compile-time constant TC (index math in shifts).
 template <int P, int NM, typename M, int TC, bool UNIT>
 __global__ void __launch_bounds__(kPaintThreads)
-k_paint_tiles(const float4 *__restrict__ sorted, const uint32_t *__restrict__ off,
-              const uint32_t *__restrict__ cursor, int *__restrict__ err, PaintGeom g, int S, const uint4 *__restrict__ wmaxs, float wdep, M *__restrict__ mesh,
+k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *__restrict__ err, PaintGeom g,
+              int S, const uint4 *wmaxs, float wdep, M *__restrict__ mesh,
               long long item_stride, long long mesh_stride, int accumulate) {
-    grid_wait(sorted, off, cursor, wmaxs);
+    grid_wait();
     extern __shared__ __align__(16) unsigned smu[];   // lo[T^3], hi[T^3] or acc64[T^3]; cand[kStage]
     __shared__ uint32_t s_beg[kSegments];
     __shared__ uint32_t s_pre[kSegments + 1];
@@ -1325,10 +1325,9 @@ __device__ __forceinline__ int isqrt_floor(int x) {
 // of |delta|^2.  MU32: the mu-bin test q^2 m <= nmu^2 l^2 fits in 32 bits.
 template <bool IL, bool TWOD, bool POLES, bool CROSS, bool MU32>
 __global__ void __launch_bounds__(kBinThreads, 5)
-k_bin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
-      const float *__restrict__ cw, const float2 *__restrict__ ph, const int *__restrict__ kedge,
-      float *__restrict__ partial, const float2 *__restrict__ meshb) {
-    grid_wait(mesh, cw, ph, kedge, meshb);
+k_bin(const float2 *mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
+      const float *cw, const float2 *ph, const int *kedge, float *__restrict__ partial, const float2 *meshb) {
+    grid_wait();
     using R = float;
     using C = float2;
     using A = float;
@@ -1516,10 +1515,9 @@ __device__ __forceinline__ double float_bits_to_double(float f) {
 // 400^3 1.03 ms for 0.94.
 template <bool IL, bool TWOD, bool POLES, bool CROSS, bool MU32>
 __global__ void __launch_bounds__(kBinThreads, 2)
-k_bin_f64(const double2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
-          const double *__restrict__ cw, const double2 *__restrict__ ph, const int *__restrict__ kedge,
-          double *__restrict__ partial, const double2 *__restrict__ meshb) {
-    grid_wait(mesh, cw, ph, kedge, meshb);
+k_bin_f64(const double2 *mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
+          const double *cw, const double2 *ph, const int *kedge, double *__restrict__ partial, const double2 *meshb) {
+    grid_wait();
     using SM = Bin64Smem;
     constexpr int kRows = 4;                          // rows per warp and turn
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -1702,11 +1700,10 @@ __host__ __device__ __forceinline__ int final_bins(const FinalGeom &f) {
 // sum w_a and sum w_b in its wsum and w2sum slots.
 template <typename A>
 __global__ void __launch_bounds__(256)
-k_reduce_finalize(const A *__restrict__ partial, int G, const unsigned long long *__restrict__ modes1d,
-                  const unsigned long long *__restrict__ modes2d, const double *__restrict__ wsums,
-                  const int *__restrict__ err, FinalGeom f, ResultLayout rl, double *__restrict__ res, int cross_a,
+k_reduce_finalize(const A *partial, int G, const unsigned long long *__restrict__ modes1d,
+                  const unsigned long long *__restrict__ modes2d, const double *wsums, const int *err, FinalGeom f, ResultLayout rl, double *__restrict__ res, int cross_a,
                   int cross_b) {
-    grid_wait(partial, modes1d, modes2d, wsums, err);
+    grid_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     double *sum = reinterpret_cast<double *>(smraw);       // the block's slots
     __shared__ double red[256];
