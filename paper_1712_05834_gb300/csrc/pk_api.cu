@@ -353,7 +353,7 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
     bg.mhi = P->kedge[nk];
     bg.mu32 = (double)(nmu + 1) * (nmu + 1) * (double)(bg.mhi + 1) < 4294967295.0 &&
               (double)nmu * nmu * (double)(P->N / 2) * (P->N / 2) < 4294967295.0;
-    if (!bin_smem_allowed(bg, P->f64))
+    if (bin_smem_bytes(bg, P->f64) > 200 * 1024)
         return fail(P, PK_EINVAL, "too many (k, mu) bins for the per-CTA histogram");
 
     FinalGeom &fg = P->fg;

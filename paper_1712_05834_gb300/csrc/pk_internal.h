@@ -192,7 +192,6 @@ cudaError_t launch_bin_cross(const void *mesh_a, const void *mesh_b, int f64, in
                              long long mesh_stride_c, int ctas, const BinGeom &g, const void *cw,
                              const void *ph, const int *kedge, void *partial, cudaStream_t st);
 size_t bin_smem_bytes(const BinGeom &g, int f64);
-bool bin_smem_allowed(const BinGeom &g, int f64);   // small enough for a plan
 int bin_ctas_per_sm(const BinGeom &g, int f64);
 int bin_threads();
 // Per-CTA histograms (G rows per catalog) -> result blocks in res (pinned host

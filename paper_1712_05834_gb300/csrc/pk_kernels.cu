@@ -1474,20 +1474,6 @@ k_bin(const float2 *mesh, long long item_stride_c, long long mesh_stride_c, BinG
     for (int k = threadIdx.x; k < g.nh; k += blockDim.x) out[k] = hist[k];
 }
 
-// Shared memory of k_bin_f64: hist[nh], weights (cw, twice where a mode stands for
-// two) at l + l/4, phases e^{i pi s / N} (|s| <= N/2) at k + k/4 with k = s + N/2,
-// edge pairs.
-struct Bin64Smem {
-    __host__ __device__ static size_t off_cw(const BinGeom &g) { return align_up((size_t)g.nh * sizeof(double), 16); }
-    __host__ __device__ static size_t off_ph(const BinGeom &g) {
-        return align_up(off_cw(g) + ((size_t)g.Nh + (g.Nh >> 2) + 1) * sizeof(double), 16);
-    }
-    __host__ __device__ static size_t off_edge(const BinGeom &g) {
-        return off_ph(g) + ((size_t)g.N + 1 + (g.N >> 2) + 1) * sizeof(double2);
-    }
-    __host__ __device__ static size_t bytes(const BinGeom &g) { return align_up(off_edge(g) + (size_t)g.nk * sizeof(int2), 16); }
-};
-
 // An integer 0 <= v < 2^32 as a double by one addition (the conversion
 // instruction has the FP64 pipe's rate as well, and a longer latency).
 __device__ __forceinline__ double u32_to_double(unsigned v) {
@@ -1503,7 +1489,8 @@ __device__ __forceinline__ double float_bits_to_double(float f) {
 // operations per SM and clock), which bounds it (85 % of its rate):
 //   * 19 FP64 operations per mode with interlacing and multipoles: the phase of
 //     a mode is one table entry (its arguments add up: i' + j' + l, folded by
-//     e^{i pi} = -1), weights of 1 or 2 stand in the cw table, Legendre sums are
+//     e^{i pi} = -1 and e^{-ix} = conj e^{ix} into 0 .. N/2, so that the tables take
+//     k_bin's places), weights of 1 or 2 stand in the cw table, Legendre sums are
 //     one FMA each, and l^2 / m comes from the FP32 reciprocal r by
 //     r (1 + e + e^2), e = 1 - m r (the geometric series of 1 / (m r); e^3 <
 //     2^-60).
@@ -1518,7 +1505,7 @@ __global__ void __launch_bounds__(kBinThreads, 2)
 k_bin_f64(const double2 *mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g,
           const double *cw, const double2 *ph, const int *kedge, double *__restrict__ partial, const double2 *meshb) {
     grid_wait();
-    using SM = Bin64Smem;
+    using SM = BinSmem<double, double2, double>;
     constexpr int kRows = 4;                          // rows per warp and turn
     extern __shared__ __align__(16) unsigned char smraw[];
     double *hist = reinterpret_cast<double *>(smraw);
@@ -1528,7 +1515,7 @@ k_bin_f64(const double2 *mesh, long long item_stride_c, long long mesh_stride_c,
     const int half = g.N / 2, N = g.N, Nh = g.Nh;
     for (int k = threadIdx.x; k < g.nh; k += blockDim.x) hist[k] = 0.0;
     for (int k = threadIdx.x; k < Nh; k += blockDim.x) scw[k + (k >> 2)] = (k != 0 && k != half ? 2.0 : 1.0) * cw[k];
-    for (int k = threadIdx.x; IL && k <= N; k += blockDim.x) sph[k + (k >> 2)] = ph[k];
+    for (int k = threadIdx.x; IL && k < Nh; k += blockDim.x) sph[k + (k >> 2)] = ph[k + half];
     for (int k = threadIdx.x; k < g.nk; k += blockDim.x) sedge[k] = make_int2(kedge[k], kedge[k + 1]);
     __syncthreads();
 
@@ -1615,14 +1602,14 @@ k_bin_f64(const double2 *mesh, long long item_stride_c, long long mesh_stride_c,
                 double2 z = a[v], y;
                 if (CROSS) y = ca[CROSS ? v : 0];
                 if (IL) {
-                    int s = rs + l, flip = 0;                      // -N <= s <= 3 N / 2
+                    int s = rs + l, flip = 0, conj = 0;            // -N <= s <= 3 N / 2
                     if (s > half) s -= N, flip ^= 0x80000000;
                     if (s > half) s -= N, flip ^= 0x80000000;
                     if (s < -half) s += N, flip ^= 0x80000000;
-                    s += half;
+                    if (s < 0) s = -s, conj = 0x80000000;
                     double2 w = sph[s + (s >> 2)];
                     w.x = __hiloint2double(__double2hiint(w.x) ^ flip, __double2loint(w.x));
-                    w.y = __hiloint2double(__double2hiint(w.y) ^ flip, __double2loint(w.y));
+                    w.y = __hiloint2double(__double2hiint(w.y) ^ flip ^ conj, __double2loint(w.y));
                     z.x = fma(b2[v].x, w.x, fma(-b2[v].y, w.y, z.x));
                     z.y = fma(b2[v].x, w.y, fma(b2[v].y, w.x, z.y));
                     if (CROSS) {
@@ -2135,13 +2122,7 @@ cudaError_t launch_acc_to_mesh(unsigned long long *acc, int nitems, int nmesh, i
 }
 
 size_t bin_smem_bytes(const BinGeom &g, int f64) {
-    return f64 ? Bin64Smem::bytes(g) : BinSmem<float, float2, float>::bytes(g);
-}
-
-// Histograms that a plan may ask for: up to 200 KB with one entry per l in both
-// tables (the phases that k_bin_f64 holds beyond that, 20 KB at 2048, fit above it).
-bool bin_smem_allowed(const BinGeom &g, int f64) {
-    return (f64 ? BinSmem<double, double2, double>::bytes(g) : BinSmem<float, float2, float>::bytes(g)) <= 200 * 1024;
+    return f64 ? BinSmem<double, double2, double>::bytes(g) : BinSmem<float, float2, float>::bytes(g);
 }
 
 int bin_threads() { return kBinThreads; }
