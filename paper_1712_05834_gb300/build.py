@@ -21,7 +21,7 @@ SOURCES = ["pk_kernels.cu", "pk_api.cu", "pk_static.cu", "pk_lognormal.cu", "pk_
 # sources compiled several times, once per group of template instances
 GROUPS = {"pk_fft_zyx.cu": ["-DPK_ZYX_GROUP=%d" % g for g in range(3)]}
 HEADERS = [os.path.join(ROOT, "include", "pk.h"), os.path.join(CSRC, "pk_internal.h"),
-           os.path.join(CSRC, "pk_plan.h"), os.path.join(CSRC, "pk_ylm.h")]
+           os.path.join(CSRC, "pk_plan.h"), os.path.join(CSRC, "pk_ylm.h"), os.path.join(CSRC, "pk_sums.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

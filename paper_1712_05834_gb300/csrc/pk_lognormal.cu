@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "pk_internal.h"
+#include "pk_sums.h"
 
 namespace pk {
 namespace {
@@ -152,21 +153,15 @@ k_ln_shape(float2 *__restrict__ gk, float2 *__restrict__ psik, int ng, float kf2
     }
 }
 
-// a + b = s + e exactly (Knuth's two-sum).
-__device__ __forceinline__ float two_sum(float a, float b, float *e) {
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    *e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-    return s;
-}
-
-// Sums of G and G^2.  A thread's sums run in pairs of FP32 numbers (the square
-// and every addition split exactly, some 48 bits), the rest in FP64: three FP64
-// operations per cell bound this kernel at 1/64 of the FP32 rate (0.75 ms for
-// 512^3 cells, now 0.13 ms; the FP32 sigma^2 / 2 that comes out is the same).
+// Sums of G and G^2.  A thread's sums run in FP32 numbers (pk_sums.h; G's in pairs: its
+// mean is zero but for rounding, and enters squared), the rest in FP64: three FP64
+// operations per cell bound this kernel at 1/64 of the FP32 rate (512^3 cells 0.75 ms,
+// now 0.19 ms; sums of squares in two parts took 0.13 ms and lost 5e-15, see there).
 __global__ void __launch_bounds__(kLnThreads)
 k_ln_moments(const float *__restrict__ g, int ng, long long pitch, double *__restrict__ stats) {
     const long long npair = (long long)ng * ng * (ng / 2);
-    float h1 = 0.0f, l1 = 0.0f, h2 = 0.0f, l2 = 0.0f;
+    float h1 = 0.0f, l1 = 0.0f;
+    SquareSum squares;
     const long long c0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
     Walk w(c0, stride, ng / 2);
     for (long long c = c0; c < npair; c += stride, w.step()) {
@@ -177,12 +172,10 @@ k_ln_moments(const float *__restrict__ g, int ng, long long pitch, double *__res
             float e;
             h1 = two_sum(h1, x, &e);
             l1 = __fadd_rn(l1, e);
-            const float p = __fmul_rn(x, x), pe = __fmaf_rn(x, x, -p);
-            h2 = two_sum(h2, p, &e);
-            l2 = __fadd_rn(l2, __fadd_rn(e, pe));
+            squares.add(x);
         }
     }
-    double s1 = (double)h1 + (double)l1, s2 = (double)h2 + (double)l2;
+    double s1 = (double)h1 + (double)l1, s2 = squares.value();
     __shared__ double r1[kLnThreads / 32], r2[kLnThreads / 32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
