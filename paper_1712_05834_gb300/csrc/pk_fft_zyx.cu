@@ -694,9 +694,11 @@ k_fft_zy(float2 *mesh, int planes, int ncol, int mcut, const float2 *__restrict_
                     const auto weight = [&](int r, int k) {       // Y_lm at z node k of the row
                         const float z = sv.oz + (float)k * sv.H, r2 = rho[r] + z * z;
                         const float ir = r2 > 0.0f ? rsqrtf(r2) : 0.0f;   // 0: the observer's node
-                        float inv = ir * ir;
-                        if (slot >= 5) inv *= inv;
-                        return (c[r][0] + z * (c[r][1] + z * (c[r][2] + z * (c[r][3] + z * c[r][4])))) * inv;
+                        // r^-4 as two factors: a node 2e-10 box edges from the observer, who
+                        // sits on it but for FP32 rounding, would have an infinite one
+                        const float inv = ir * ir;
+                        const float y = (c[r][0] + z * (c[r][1] + z * (c[r][2] + z * (c[r][3] + z * c[r][4])))) * inv;
+                        return slot >= 5 ? y * inv : y;
                     };
                     const auto ld = [&](int r, int p) {
                         float2 f = __ldcg(D + (long long)r * Nh + p);
