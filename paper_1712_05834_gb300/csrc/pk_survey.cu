@@ -1162,9 +1162,12 @@ static pk_status survey_compute_t(pk_survey_s *S) {
     rows.D = D;
     rows.alpha = S->cst;
     rows.slot_c = mr / 2;
-    // Y_lm does not depend on the unit: a power of two near the box edge keeps the
-    // fourth powers in range and the FP32 node coordinates as they are
-    const int unit = -ilogb(L);
+    // Y_lm does not depend on the unit: a power of two near the largest node coordinate
+    // keeps the fourth powers in range (also of an observer 1e10 box edges away) and the
+    // FP32 node coordinates as they are
+    double far = L;
+    for (double o : S->cfg.box_origin) far = std::max(far, fabs(o));
+    const int unit = -ilogb(far);
     rows.ox = (float)ldexp((double)(float)S->cfg.box_origin[0], unit);
     rows.oy = (float)ldexp((double)(float)S->cfg.box_origin[1], unit);
     rows.oz = (float)ldexp((double)(float)S->cfg.box_origin[2], unit);

@@ -34,3 +34,30 @@ def test_multipoles_are_finite(N, L, node, interlaced):
     for row in range(3):
         err = np.abs(got["poles"][row] - ref["poles"][row])[ok]
         assert np.all(err <= 1e-4 * raw), (row, float(np.max(err / raw)))
+
+
+def test_observer_very_far_away():
+    """2e10 box edges along z, as a program that wants the plane-parallel limit may ask
+    for: fourth powers of the distance would leave the FP32 range in units of the box."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1712_05834_gb300 as pk
+    pk.build()
+    N, L, far = 128, 1000.0, 2.0 ** 44
+    g = torch.Generator().manual_seed(3)
+    dev = lambda n: (L * torch.rand((n, 3), generator=g, dtype=torch.float64) +
+                     torch.tensor([-500.0, -500.0, far], dtype=torch.float64)).cuda()
+    data = pk.survey_catalog(dev(40_000), nbar=torch.full((40_000,), 1e-4, device="cuda"))
+    rand = pk.survey_catalog(dev(120_000), nbar=torch.full((120_000,), 1e-4, device="cuda"))
+    out = []
+    for precision in ("f32", "f64"):
+        cfg = pk.make_survey_config(L, (-500.0, -500.0, far), N, "tsc", False, dk=0.02, precision=precision)
+        with pk.ConvolvedFFTPower(cfg) as power:
+            out.append(power.run(data, rand))
+    got, ref = out
+    ok = ref["modes"] > 0
+    raw = np.abs(ref["poles"][0][ok] + ref["shot_noise"])
+    for row in range(3):
+        err = np.abs(got["poles"][row] - ref["poles"][row])[ok]
+        assert np.all(err <= 1e-4 * raw), (row, float(np.max(err / raw)))
