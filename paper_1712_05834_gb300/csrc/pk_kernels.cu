@@ -441,11 +441,11 @@ __device__ __forceinline__ void spline_weights(float u, int &base, float *wt) {
 }
 
 // Fixed-point split of one tile: deposit q = round(v) (v = w W 2^S) is held as
-// hi * 2^B + lo with lo in [0, 2^B]; the cell keeps sum(lo) and sum(hi) in two
-// uint32 words.  With at most `ncand` deposits per cell, sum(lo) <=
+// hi * 2^B + lo with lo in [0, 2^B) (FP64 meshes: [0, 2^B]); the cell keeps sum(lo) and
+// sum(hi) in two uint32 words.  With at most `ncand` deposits per cell, sum(lo) <=
 // ncand 2^B < 2^32 and |sum(hi)| <= ncand (hmax + 1) < 2^31 by construction.
 struct Split {
-    int B;            // split bit (1 .. 22)
+    int B;            // split bit (1 .. 30, FP64 meshes 1 .. 22)
     float twoB;       // 2^B
     unsigned twoB_u;  // 2^B as an integer
     float inv2B;      // 2^-B
@@ -453,26 +453,34 @@ struct Split {
     int fast;         // 1: split when needed; 0: this tile uses 64-bit shared atomics instead
 };
 
-// round(vxy wz) as a two's complement word, the exact product rounded once.  UNIT:
-// in [0, 2^23), by one FMA against 2^23, whose bits hold the integer.  Else any |v| <
-// 2^31: below 2^22 by an FMA against 1.5 2^23; from there on the FP32 product holds
-// two binary places at most and is converted (a product converted at any size was
-// rounded twice).
+// round(vxy wz) as a two's complement word, the exact product rounded once, where
+// fma_exact says so: one FMA against 2^23 (UNIT: [0, 2^23)) or 1.5 2^23 ([-2^22,
+// 2^22)), whose bits hold the integer.
+template <bool UNIT>
+__device__ __forceinline__ unsigned quantize_fma(float vxy, float wz) {
+    return __float_as_uint(fmaf(vxy, wz, UNIT ? 8388608.0f : 12582912.0f)) - (UNIT ? 0x4B000000u : 0x4B400000u);
+}
+template <bool UNIT>
+__device__ __forceinline__ bool fma_exact(unsigned q) {
+    return (UNIT ? q : q + (1u << 22)) < (1u << 23);
+}
+// Any |v| < 2^31 (UNIT: deposits known to be below 2^23): from 2^22 on the FP32 product
+// holds two binary places at most and is converted (a product converted at any size
+// was rounded twice).
 template <bool UNIT>
 __device__ __forceinline__ unsigned quantize(float vxy, float wz) {
-    if constexpr (UNIT) {
-        return __float_as_uint(fmaf(vxy, wz, 8388608.0f)) - 0x4B000000u;
-    } else {
-        const unsigned q = __float_as_uint(fmaf(vxy, wz, 12582912.0f)) - 0x4B400000u;
-        return q + (1u << 22) < (1u << 23) ? q : (unsigned)__float2int_rn(vxy * wz);
-    }
+    const unsigned q = quantize_fma<UNIT>(vxy, wz);
+    return UNIT || fma_exact<UNIT>(q) ? q : (unsigned)__float2int_rn(vxy * wz);
 }
 
 // MODE 2: the tile's cells fit one word each (see the sweep in k_paint_tiles):
 // one rounding and one 32-bit shared atomic per cell.  MODE 1: lo words with a
 // split into hi * 2^B + lo for the rare large or negative deposit.  MODE 0:
-// 64-bit shared atomics (dense tiles).
-template <int P, int MODE, int TC = 0, bool UNIT = true>
+// 64-bit shared atomics (dense tiles).  Meshes of M = float: the same integer in
+// every mode, so that a cell does not depend on the way its tile is painted.
+// (M = double has modes 0 and 1 only; the split rounds deposits from 2^B on to FP32
+// first.)
+template <int P, int MODE, int TC, bool UNIT, typename M>
 __device__ __forceinline__ void deposit(unsigned *lo, unsigned *hi, unsigned long long *acc64,
                                         const Split &sp, int T, float x, float y, float z, float ws) {
     int bx, by, bz;
@@ -497,6 +505,22 @@ __device__ __forceinline__ void deposit(unsigned *lo, unsigned *hi, unsigned lon
                 if ((unsigned)cz >= (unsigned)T) continue;
                 if (MODE == 2) {
                     atomicAdd(lo + row + cz, quantize<UNIT>(vxy, wz[c]));
+                } else if (MODE == 1 && sizeof(M) == 4) {
+                    // lo and hi words of the integer (beyond 2^31, where FP32 products are
+                    // multiples of 256, split as they are: exact for B <= 30)
+                    unsigned q = quantize_fma<UNIT>(vxy, wz[c]);
+                    int hf = 0;
+                    if (__builtin_expect(!fma_exact<UNIT>(q), 0)) {
+                        float v = vxy * wz[c];
+                        if (fabsf(v) >= 2147483648.0f) {
+                            const float h = floorf(v * sp.inv2B);
+                            v = fmaf(-h, sp.twoB, v);
+                            hf = (int)h;
+                        }
+                        q = (unsigned)__float2int_rn(v);
+                    }
+                    atomicAdd(lo + row + cz, q & (sp.twoB_u - 1u));
+                    if (q >= sp.twoB_u || hf != 0) atomicAdd(hi + row + cz, (unsigned)(((int)q >> sp.B) + hf));
                 } else if (MODE == 1) {
                     // 2^23 + round(v) in one FMA; its bits minus 0x4B000000 are
                     // round(v) whenever 0 <= round(v) < 2^B (B <= 22): the
@@ -514,7 +538,8 @@ __device__ __forceinline__ void deposit(unsigned *lo, unsigned *hi, unsigned lon
                             atomicAdd(hi + row + cz, (unsigned)(__float_as_int(hf + 12582912.0f) - 0x4B400000));
                     }
                 } else {
-                    const long long q = __float2ll_rn(vxy * wz[c]);
+                    const unsigned f = quantize_fma<UNIT>(vxy, wz[c]);
+                    const long long q = sizeof(M) == 4 && fma_exact<UNIT>(f) ? (long long)(int)f : __float2ll_rn(vxy * wz[c]);
                     if (q) atomicAdd(acc64 + row + cz, (unsigned long long)q);
                 }
             }
@@ -712,18 +737,15 @@ __device__ __forceinline__ float ll_to_float_rn(long long q) {
     return q < 0 ? -f : f;
 }
 
-// Cell value in weight units from its fixed-point words.  FP32: the fast path
-// rounds hi 2^(B-S) + lo 2^-S within one ulp (a fixed function of the integer
-// words, so still bit-reproducible); the 64-bit path is rounded exactly.
-// FP64: exact in both paths (the cell integer has far fewer than 53 bits).
+// Cell value in weight units from its fixed-point words: the cell's integer rounded
+// once, as in one-word cells (FP64: exact, it has far fewer than 53 bits).
 template <typename M>
 __device__ __forceinline__ M cell_value(unsigned lo, unsigned hi, unsigned long long a64, const Split &sp,
                                         float inv_scale);
 template <>
 __device__ __forceinline__ float cell_value<float>(unsigned lo, unsigned hi, unsigned long long a64,
                                                    const Split &sp, float inv_scale) {
-    if (sp.fast) return fmaf((float)(int)hi, sp.hi_scale, (float)lo * inv_scale);
-    return ll_to_float_rn((long long)a64) * inv_scale;
+    return ll_to_float_rn(sp.fast ? ((long long)(int)hi << sp.B) + (long long)lo : (long long)a64) * inv_scale;
 }
 // hi sh + lo sl for powers of two sl <= sh <= 2^52 sl, rounded once: 32-bit words
 // put into the low half of the double 2^52 s become 2^52 s + word s without a
@@ -781,20 +803,20 @@ __device__ __forceinline__ void stage_candidates(const float4 *sorted, const uin
         cand[j] = fetch_candidate(sorted, s_beg, s_pre, T, k0 + j, scale);
 }
 
-template <int P, int MODE, int TC>
+template <int P, int MODE, int TC, bool UNIT, typename M>
 __device__ __forceinline__ void deposit_staged(const float4 *cand, uint32_t n, unsigned *lo, unsigned *hi,
                                                unsigned long long *acc64, const Split &sp, int T, float sh) {
     for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
         const float4 v = cand[j];
-        deposit<P, MODE, TC>(lo, hi, acc64, sp, T, v.x + sh, v.y + sh, v.z + sh, v.w);
+        deposit<P, MODE, TC, UNIT, M>(lo, hi, acc64, sp, T, v.x + sh, v.y + sh, v.z + sh, v.w);
     }
 }
 
-template <int P, int TC>
+template <int P, int TC, bool UNIT, typename M>
 __device__ __forceinline__ void deposit_any(const float4 *cand, uint32_t n, unsigned *lo, unsigned *hi,
                                             unsigned long long *acc64, const Split &sp, int T, float sh) {
-    if (sp.fast) deposit_staged<P, 1, TC>(cand, n, lo, hi, acc64, sp, T, sh);
-    else deposit_staged<P, 0, TC>(cand, n, lo, hi, acc64, sp, T, sh);
+    if (sp.fast) deposit_staged<P, 1, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, sh);
+    else deposit_staged<P, 0, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, sh);
 }
 
 // Write one tile's cells to the mesh (r2c layout, rows of T cells along z at
@@ -1000,13 +1022,16 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
     const float cell_max = sgn ? 2.145e9f : 4.29e9f;      // 2^31, 2^32, less 1e-3 for rounding
     const float mean = UNIT ? (dmax + 1.0f) * ncf : ncf * __uint_as_float(wm.z) * wdep * scale;
     if (!UNIT && mean > 0.9f * cell_max) sweep = false;
+    // FP64 meshes: only where every deposit is below the general path's 2^B, which
+    // rounds no other way
+    if (sizeof(M) == 8) sweep = sweep && UNIT && dmax < (float)(1u << max(min(22, 31 - ceil_log2(max(total, 1u))), 0)) - 1.0f;
     // A tile whose candidates in all pass that bound, but by no more than ten times, is
     // swept with its candidates counted per block (|W V| in steps of max |W V| / 1024,
     // rounded up): 2 x 2 x 2 blocks bound a cell, 64 (CIC) or 512 cells of the tile's 16^3 and more.
     // Such tiles took the general path: 6.7e7 clustered objects at 512^3 (2000 a tile),
     // us: CIC 1133 -> 758, TSC interlaced 5255 -> 2197, weighted PCS interlaced 12363 ->
     // 5064; 1.3e5 at 64^3, TSC interlaced: 84 -> 27.
-    const bool dense = !sweep && mean < 10.0f * cell_max && ncf < 4.0e6f && dmax < (UNIT ? 8388607.0f : 1.07e9f);
+    const bool dense = sizeof(M) == 4 && !sweep && mean < 10.0f * cell_max && ncf < 4.0e6f && dmax < (UNIT ? 8388607.0f : 1.07e9f);
     const float blk_scale = UNIT ? 1.0f : 1024.0f / (wmax * scale);
     if (sweep || dense) {
         // TSC and PCS sweeps of 16^3 tiles deposit into the padded layout
@@ -1057,9 +1082,9 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
                     if (NM == 2) deposit_flat<P, TC, UNIT>(smu, T3, trash, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
                 } else {
                     const Split none{};
-                    deposit<P, 2, TC, UNIT>(lo, nullptr, nullptr, none, T, v.x, v.y, v.z, v.w);
+                    deposit<P, 2, TC, UNIT, float>(lo, nullptr, nullptr, none, T, v.x, v.y, v.z, v.w);
                     if (NM == 2)
-                        deposit<P, 2, TC, UNIT>(hi, nullptr, nullptr, none, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
+                        deposit<P, 2, TC, UNIT, float>(hi, nullptr, nullptr, none, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
                 }
             }
         }
@@ -1115,7 +1140,9 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
     Split sp;
     {
         const unsigned nc = total > 0u ? total : 1u;
-        sp.B = min(22, 31 - ceil_log2(nc));
+        // FP32: sums of nc words below 2^B stay below 2^32; FP64: the split that its
+        // rounding has always had
+        sp.B = sizeof(M) == 4 ? min(30, 32 - ceil_log2(nc)) : min(22, 31 - ceil_log2(nc));
         sp.twoB = __uint_as_float((unsigned)(127 + max(sp.B, 0)) << 23);
         sp.twoB_u = 1u << max(sp.B, 0);
         sp.inv2B = __uint_as_float((unsigned)(127 - max(sp.B, 0)) << 23);
@@ -1136,14 +1163,14 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
         __syncthreads();
         const float sh = m ? 0.5f : 0.0f;
         if (staged_once) {
-            deposit_any<P, TC>(cand, total, lo, hi, acc64, sp, T, sh);
+            deposit_any<P, TC, UNIT, M>(cand, total, lo, hi, acc64, sp, T, sh);
         } else {
             for (uint32_t k0 = 0; k0 < total; k0 += kStage) {     // dense tile: batches
                 const uint32_t n = min((uint32_t)kStage, total - k0);
                 __syncthreads();                                  // previous batch consumed
                 stage_candidates(sorted, s_beg, s_pre, T, k0, n, scale, cand);
                 __syncthreads();
-                deposit_any<P, TC>(cand, n, lo, hi, acc64, sp, T, sh);
+                deposit_any<P, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, sh);
             }
         }
         __syncthreads();

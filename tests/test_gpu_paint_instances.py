@@ -97,3 +97,39 @@ def test_cells_at_the_limit_of_one_word_do_not_depend_on_the_order():
                 assert np.array_equal(first, cells), (step, int((first != cells).sum()))
     finally:
         pk.pk_destroy(plan)
+
+
+@pytest.mark.parametrize("window", ["cic", "tsc", "pcs"])
+@pytest.mark.parametrize("N,n,clump", [(96, 100_003, 0), (96, 400_003, 0), (96, 100_003, 3000), (72, 200_003, 2000),
+                                       (34, 20_003, 0)])
+@pytest.mark.parametrize("kind", ["unit", "positive", "mixed", "heavy"])
+def test_fp32_cells_do_not_depend_on_the_way_a_tile_is_painted(window, N, n, clump, kind):
+    """One object far from the others and heavier by 1e4 to 1e9 has their tiles painted
+    the general way (split into two words, or 64-bit cells) where they are swept with
+    one-word cells without it; a cell is the sum of the same integers rounded once."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_1712_05834_gb300 as pk
+    pk.build()
+    rng = np.random.default_rng(n + clump)
+    L = float(N)
+    pos = rng.random((n, 3)) * L * np.array([0.5, 1.0, 1.0])
+    if clump:
+        pos[:clump] = np.array([5.3, 6.1, 40.7]) + 0.3 * rng.standard_normal((clump, 3))
+    w = {"unit": np.ones(n), "positive": rng.uniform(0.5, 1.5, n), "mixed": rng.normal(0.0, 1.0, n),
+         "heavy": rng.uniform(5.0, 40.0, n)}[kind]
+    pos = np.concatenate([pos, [[0.75 * L, 0.5 * L, 0.5 * L]]]).astype(np.float32)
+    got = []
+    for far in (0.0, 1e4, 1e9):
+        wk = torch.from_numpy(np.append(w, far).astype(np.float32)).cuda()
+        plan = pk.pk_plan(pk.make_config(L, N, window, interlaced=True, dk=0.2))
+        try:
+            pk.pk_paint(plan, torch.from_numpy(pos).cuda(), wk)
+            got.append([pk.pk_mesh(plan, 0, m, N) for m in range(2)])
+        finally:
+            pk.pk_destroy(plan)
+    x = slice(0, N // 2 + 6)                             # without the far object's cells
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.array_equal(a[x], b[x]), int((a[x] != b[x]).sum())
