@@ -589,22 +589,42 @@ __device__ __forceinline__ void deposit_flat(unsigned *sm, int cell0, unsigned t
     }
 }
 
-// Blocks of a tile and its surroundings: `width` cells along each axis, from -width
-// on.  A cell's deposits come from an open interval of P cells per axis, so with
-// blocks of P cells or more from at most 2 x 2 x 2 neighbouring ones.  Width 2 for
-// CIC and 4 for TSC and PCS at edges up to 16, twice that up to 28: at most
-// kBlocks<P> per axis, whose counters fit beside the cells without costing a CTA
-// per SM (TSC blocks of 3 cells did: 816 -> 858 us for 2e7 objects at 512^3).
+// Blocks of a tile and its surroundings: 2^SH cells along each axis (twice that in
+// tiles wider than 16), from one block below the tile on, at most NB per axis.  A
+// cell's deposits come from an open interval of P cells per axis, so from SPAN
+// neighbouring blocks at most.
+template <int SH_, int NB_, int SPAN_, int SPAN_WIDE_>
+struct Blocks {
+    static constexpr int NB = NB_, Count = NB * NB * NB;
+    __device__ static __forceinline__ int of(float x, float y, float z, bool wide) {
+        const int sh = wide ? SH_ + 1 : SH_;
+        const auto along = [&](float v) { return min(max(__float2int_rd(v) + (1 << sh), 0) >> sh, NB - 1); };
+        return (along(x) * NB + along(y)) * NB + along(z);
+    }
+    // The largest sum of the counters that one cell's deposits come from, of this
+    // thread's share of the cells.
+    __device__ static __forceinline__ float most(const unsigned *blk, bool wide) {
+        const int span = wide ? SPAN_WIDE_ : SPAN_, ends = NB - span + 1;
+        float m = 0.0f;
+        for (int c = threadIdx.x; c < ends * ends * ends; c += blockDim.x) {
+            const unsigned *b = blk + (c / (ends * ends) * NB + c / ends % ends) * NB + c % ends;
+            float n = 0.0f;
+            for (int i = 0; i < span; ++i)
+                for (int j = 0; j < span; ++j)
+                    for (int k = 0; k < span; ++k) n += (float)b[(i * NB + j) * NB + k];
+            m = fmaxf(m, n);
+        }
+        return m;
+    }
+};
+// Counters that fit beside the cells without costing a CTA per SM (TSC blocks of 3 cells
+// did: 816 -> 858 us for 2e7 objects at 512^3), and those that take the cells' place:
+// 2 x 2 x 2 blocks are 64 cells (CIC) or 512, 3 x 3 x 3 are 216.  The smaller windows lie
+// within the larger ones: what fits by the larger fits by the smaller.
 template <int P>
-constexpr int kBlocks = P == 2 ? 10 : 6;                  // (the same for TSC and PCS)
+using CoarseBlocks = typename std::conditional<P == 2, Blocks<1, 10, 2, 2>, Blocks<2, 6, 2, 2>>::type;
 template <int P>
-__device__ __forceinline__ int block_of(float x, float y, float z, bool wide) {
-    const int sh = (P == 2 ? 1 : 2) + (wide ? 1 : 0);
-    const auto along = [&](float v) {
-        return min(max(__float2int_rd(v) + (1 << sh), 0) >> sh, kBlocks<P> - 1);
-    };
-    return (along(x) * kBlocks<P> + along(y)) * kBlocks<P> + along(z);
-}
+using FineBlocks = typename std::conditional<P == 2, Blocks<1, 10, 2, 2>, Blocks<1, 10, 3, 2>>::type;
 
 // ---- one-sweep paint of 16^3 tiles into a padded layout (unit weights, TSC and PCS) ----
 // Shared layout: cell (x, y, z) of the tile's mesh m at word
@@ -720,7 +740,7 @@ __device__ __forceinline__ void sweep_flush(const unsigned *sm, bool sgn, float 
 
 // Correctly rounded int64 -> float without the 64-bit conversion instruction.
 __device__ __forceinline__ float ll_to_float_rn(long long q) {
-    if (q == 0) return 0.0f;
+    if (q == (long long)(int)q) return (float)(int)q;
     const unsigned long long u = q < 0 ? 0ull - (unsigned long long)q : (unsigned long long)q;
     const int nb = 64 - __clzll((long long)u);
     float f;
@@ -1027,19 +1047,54 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
     if (sizeof(M) == 8) sweep = sweep && UNIT && dmax < (float)(1u << max(min(22, 31 - ceil_log2(max(total, 1u))), 0)) - 1.0f;
     // A tile whose candidates in all pass that bound, but by no more than ten times, is
     // swept with its candidates counted per block (|W V| in steps of max |W V| / 1024,
-    // rounded up): 2 x 2 x 2 blocks bound a cell, 64 (CIC) or 512 cells of the tile's 16^3 and more.
+    // rounded up): the blocks that a cell's deposits come from bound it.
     // Such tiles took the general path: 6.7e7 clustered objects at 512^3 (2000 a tile),
     // us: CIC 1133 -> 758, TSC interlaced 5255 -> 2197, weighted PCS interlaced 12363 ->
     // 5064; 1.3e5 at 64^3, TSC interlaced: 84 -> 27.
+    // One candidate in eight tells first whether that would be in vain (not for CIC, whose
+    // sweep costs little more); then, and where it was, all candidates are counted in
+    // smaller blocks before anything is deposited.  Without that, crowded tiles were swept
+    // in vain before they took the general path: fifty blobs of 2000 objects (0.6 cells
+    // wide) at 64^3, interlaced, us a spectrum, general path alone, swept in vain, now: TSC
+    // 320, 363, 315; PCS 440, 656, 458; 3e6 such objects at 128^3: 835, 894, 790; 1360, 1614,
+    // 1356; 3e7 at 256^3: 4059, 3447, 2500; 7184, 4604, 3450.
     const bool dense = sizeof(M) == 4 && !sweep && mean < 10.0f * cell_max && ncf < 4.0e6f && dmax < (UNIT ? 8388607.0f : 1.07e9f);
     const float blk_scale = UNIT ? 1.0f : 1024.0f / (wmax * scale);
-    if (sweep || dense) {
+    const bool wide = T > 16;
+    using Coarse = CoarseBlocks<P>;
+    using Fine = FineBlocks<P>;
+    static_assert(Fine::Count <= kStage * (int)(sizeof(float4) / sizeof(unsigned)), "counters in the smallest tile's memory");
+    const auto blocks_fit = [&](float n) {               // n: largest count of a cell's blocks
+        // every cell: sum of round(w W V 2^S) <= wdep sum |W V| 2^S + candidates
+        return UNIT ? n * (dmax + 1.0f) < cell_max
+                    : n * (wmax * scale * wdep * (1.0f / 1024.0f)) * 1.00001f + ncf < cell_max;
+    };
+    const auto steps = [&](float w) { return UNIT ? 1u : __float2uint_ru(fabsf(w) * blk_scale); };
+    // Largest count of a cell's blocks B over candidates 0, stride, 2 stride, ..
+    const auto count_blocks = [&](auto B, uint32_t stride) {
+        for (int c = threadIdx.x; c < B.Count; c += blockDim.x) smu[c] = 0u;
+        __syncthreads();
+        for (uint32_t k = threadIdx.x * stride; k < total; k += blockDim.x * stride) {
+            const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
+            atomicAdd(smu + B.of(v.x, v.y, v.z, wide), steps(v.w));
+        }
+        __syncthreads();
+        return B.most(smu, wide);
+    };
+    bool known = UNIT && sweep;                           // every cell is known to fit
+    bool look = false;                                    // count in the smaller blocks first
+    if (P > 2 && dense) look = __syncthreads_or(!blocks_fit(8.0f * count_blocks(Coarse{}, 8u)));
+#pragma unroll 1
+    while (sweep || dense) {
+        if (look) {
+            known = !__syncthreads_or(!blocks_fit(count_blocks(Fine{}, 1u)));
+            if (!known) break;
+        }
+        const bool counted = dense && !known;
         // TSC and PCS sweeps of 16^3 tiles deposit into the padded layout
         // (SweepLayout); CIC keeps the compact one
         constexpr bool kPadded = TC == 16 && (P == 4 || P == 3);
         // block counters behind the cells (the staging area is unused here)
-        constexpr int kBlk = kBlocks<P>;
-        static_assert(kBlk * kBlk * kBlk * sizeof(unsigned) <= kStage * sizeof(float4), "counters in the staging area");
         unsigned *s_blk = smu + (kPadded ? NM * SweepLayout<P>::Words : paint_cell_words(T));
         {
             uint4 *z4 = reinterpret_cast<uint4 *>(smu);
@@ -1047,24 +1102,19 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
             const int n4 = nw / 4;
             for (int c = threadIdx.x; c < n4; c += blockDim.x) z4[c] = make_uint4(0u, 0u, 0u, 0u);
             for (int c = 4 * n4 + threadIdx.x; c < nw; c += blockDim.x) smu[c] = 0u;
-            for (int c = threadIdx.x; dense && c < kBlk * kBlk * kBlk; c += blockDim.x) s_blk[c] = 0u;
+            for (int c = threadIdx.x; counted && c < Coarse::Count; c += blockDim.x) s_blk[c] = 0u;
         }
         __syncthreads();
-        const auto count = [&](const float4 &v) {
-            if (dense)
-                atomicAdd(s_blk + block_of<P>(v.x, v.y, v.z, T > 16), UNIT ? 1u : __float2uint_ru(fabsf(v.w) * blk_scale));
-        };
-        // |W V| in units rounded up, as integers: the sum, and so the path taken, does
-        // not depend on the order of the candidates (NaN: far too much)
+        // |W V| in units rounded up, as integers (NaN: far too much)
         unsigned long long sum_abs = 0ull;
-        const auto add_abs = [&](float w) {
-            if (!UNIT) sum_abs += fabsf(w) < 4.29e9f ? (unsigned long long)__float2uint_ru(fabsf(w)) : 1ull << 40;
+        const auto account = [&](const float4 &v) {
+            if (!UNIT) sum_abs += fabsf(v.w) < 4.29e9f ? (unsigned long long)__float2uint_ru(fabsf(v.w)) : 1ull << 40;
+            if (counted) atomicAdd(s_blk + Coarse::of(v.x, v.y, v.z, wide), steps(v.w));
         };
         if (kPadded) {
             for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
                 const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
-                add_abs(v.w);
-                count(v);
+                account(v);
                 sweep_deposit<P, UNIT>(smu, v.x, v.y, v.z, v.w);
                 if (NM == 2)
                     sweep_deposit<P, UNIT>(smu + SweepLayout<P>::Words, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
@@ -1075,8 +1125,7 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
             const bool flat = !dense && total <= (uint32_t)kFlatMaxCand;
             for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
                 const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
-                add_abs(v.w);
-                count(v);
+                account(v);
                 if (flat) {
                     deposit_flat<P, TC, UNIT>(smu, 0, trash, T, v.x, v.y, v.z, v.w);
                     if (NM == 2) deposit_flat<P, TC, UNIT>(smu, T3, trash, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
@@ -1088,24 +1137,11 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
                 }
             }
         }
-        bool fits = true;
-        if (dense) {
-            __syncthreads();
-            bool over = false;
-            for (int c = threadIdx.x; c < (kBlk - 1) * (kBlk - 1) * (kBlk - 1); c += blockDim.x) {
-                const int bx = c / ((kBlk - 1) * (kBlk - 1)), by = c / (kBlk - 1) % (kBlk - 1);
-                const unsigned *b = s_blk + (bx * kBlk + by) * kBlk + c % (kBlk - 1);
-                float n = 0.0f;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) n += (float)b[((k >> 2) * kBlk + (k >> 1 & 1)) * kBlk + (k & 1)];
-                // every cell: sum of round(w W V 2^S) <= wdep sum |W V| 2^S + candidates
-                over |= !(UNIT ? n * (dmax + 1.0f) < cell_max
-                               : n * (wmax * scale * wdep * (1.0f / 1024.0f)) * 1.00001f + ncf < cell_max);
-            }
-            fits = !__syncthreads_or(over);
-        } else if constexpr (UNIT) {
-            __syncthreads();
-        } else {
+        __syncthreads();
+        if (known) {
+        } else if (dense) {
+            known = !__syncthreads_or(!blocks_fit(Coarse::most(s_blk, wide)));
+        } else if constexpr (!UNIT) {
             __shared__ unsigned long long s_abs[kPaintThreads / 32];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sum_abs += __shfl_down_sync(0xffffffffu, sum_abs, o);
@@ -1114,10 +1150,11 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
             unsigned long long t = 0ull;
 #pragma unroll
             for (int k = 0; k < kPaintThreads / 32; ++k) t += s_abs[k];
+            __syncthreads();                              // read before a second sweep's sum
             // every cell: sum of round(w W V 2^S) <= wdep sum |W V| 2^S + candidates / 2
-            fits = (float)t * wdep + ncf < cell_max;
+            known = (float)t * wdep + ncf < cell_max;
         }
-        if (fits) {
+        if (known) {
             const Split none{};
             if (kPadded) {
                 sweep_flush<M, P, UNIT>(smu, sgn, inv_scale, base + tile_off, g.N, pitch, accumulate);
@@ -1133,8 +1170,10 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
             }
             return;
         }
-        __syncthreads();                                  // s_abs read; the cells are zeroed again below
+        if ((P == 2 && dense) || ncf >= 4.0e6f) break;    // the same blocks; beyond the counters' range
+        look = true;
     }
+    __syncthreads();                                      // the cells are zeroed again below
 
     // General path: one mesh per pass over staged candidates.
     Split sp;
@@ -2032,7 +2071,7 @@ size_t paint_smem_bytes(int T, int window, int nmesh) {
     const size_t general = (size_t)paint_cell_words(T) * sizeof(unsigned) + (size_t)kStage * sizeof(float4);
     const size_t words = window == 4   ? (size_t)nmesh * SweepLayout<4>::Words
                          : window == 3 ? (size_t)nmesh * SweepLayout<3>::Words : 0;
-    const size_t padded = T == 16 && words ? (words + kBlocks<3> * kBlocks<3> * kBlocks<3>) * sizeof(unsigned) : 0;
+    const size_t padded = T == 16 && words ? (words + CoarseBlocks<3>::Count) * sizeof(unsigned) : 0;
     return general > padded ? general : padded;
 }
 
