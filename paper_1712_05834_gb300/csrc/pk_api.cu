@@ -292,7 +292,7 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
 
     int rlo, rhi;
     window_reach(P->p, c.interlaced, &rlo, &rhi);
-    const int T = choose_tile(P->N, rhi - rlo, c.tile);
+    int T = choose_tile(P->N, rhi - rlo, c.tile);
     if (T <= 0)
         return fail(P, PK_EINVAL, "tile must divide nmesh, be >= the window reach and fit in shared memory");
     const double L = c.box_size;
@@ -309,12 +309,26 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
 
     // ---- paint geometry ----
     PaintGeom &pg = P->pg;
+    // Tiles of 16 on less than half of the SMs (meshes up to 64^3), each with 1000 objects
+    // or more: painted as halves along each axis, eight CTAs to a tile, with positions
+    // held in the whole tile's frame, so that the cells are the same bits (not with FP64
+    // meshes, where the split of a deposit, and so its rounding, goes by the number of
+    // candidates).  us a spectrum, whole tiles and halves: 64^3 CIC 6.4e4 objects 85 and 75,
+    // 1e5 95 and 76, 1e6 277 and 127, weighted PCS interlaced 135 and 101, 173 and 118, 531
+    // and 342; 48^3 2.7e4 75 and 72, 98 and 97; 32^3 8e3 74 and 67, 97 and 80.  With fewer
+    // objects there is little to divide (2e4 at 64^3 lost 5 us to the eight times as many
+    // keys).
+    pg.flog = 0;
+    if (c.tile <= 0 && T == 16 && !P->f64) {
+        const long long ntile = (long long)(P->N / T) * (P->N / T) * (P->N / T) * P->B;
+        if (2 * ntile < P->nsm && c.capacity >= 1000 * ntile) pg.flog = 1, T = 8;
+    }
     pg.invH = (float)((double)P->N / c.box_size);
     pg.invH_lo = (float)((double)P->N / c.box_size - (double)pg.invH);
     pg.invHd = (double)P->N / c.box_size;
     pg.N = P->N;
     pg.T = T;
-    pg.inv_T = ((1u << 20) + T - 1) / T;
+    pg.inv_F = ((1u << 20) + (T << pg.flog) - 1) / (T << pg.flog);
     pg.ntx = P->N / T;
     pg.lo = rlo;
     pg.hi = rhi;

@@ -23,8 +23,10 @@ struct PaintGeom {
     double invHd;       // N / L in FP64
     int N;              // cells per side
     int T;              // tile edge (divides N, T >= hi - lo)
-    unsigned inv_T;     // ceil(2^20 / T): cell / T = cell * inv_T >> 20 exactly for
-                        // cell < 4096 (the excess, below 2^-8, is less than 1 / T)
+    int flog;           // 1: tiles are halves (along each axis) of frames of 2 T cells, in
+                        // which positions are held; 0: a tile is its own frame
+    unsigned inv_F;     // ceil(2^20 / F), F = T << flog: cell / F = cell * inv_F >> 20 exactly
+                        // for cell < 4096 (the excess, below 2^-8, is less than 1 / F)
     int ntx;            // tiles per side = N / T
     int lo, hi;         // reach of the window support relative to floor(s)
     long long ntiles;   // ntx^3 tiles per catalog

@@ -170,16 +170,29 @@ __device__ __forceinline__ Obj<typename PosReal<DT>::type> load_obj(const void *
 // Home tile and boundary class of one object.  Along each axis the class is
 // 0 if the window reaches the tile below (c + lo < 0), 2 if it reaches the
 // tile above (c + hi >= T), else 1; T >= hi - lo keeps these disjoint.
-template <typename R>
-__device__ __forceinline__ void home_key(const Obj<R> &o, const PaintGeom &g, int *tile3, int *cls) {
+// u: the coordinate in the tile's frame (the tile, or the pair of tiles it is half
+// of).  Halves, and what reaches across their seam, go by u, which the deposits are
+// made of; what reaches into other frames goes by the cell of s, as with whole
+// frames, so that both paint the same cells.
+template <typename R, bool WANT_U>
+__device__ __forceinline__ void home_key(const Obj<R> &o, const PaintGeom &g, int *tile3, float *u, int *cls) {
     int c = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
+        const int F = g.T << g.flog;
         const int cell = min((int)o.s[a], g.N - 1);        // s >= 0: truncation is the floor
-        const int t = (int)(((unsigned)cell * g.inv_T) >> 20);      // cell / T (see PaintGeom)
-        const int cl = cell - t * g.T;
+        int t = (int)(((unsigned)cell * g.inv_F) >> 20);            // cell / F (see PaintGeom)
+        const int cl = cell - t * F;
+        if (g.flog || WANT_U) u[a] = (float)(o.s[a] - (R)(t * F)) + o.e[a];
+        bool below = cl < -g.lo, above = cl >= F - g.hi;
+        if (g.flog) {
+            const int cu = min(max(__float2int_rd(u[a]), 0), F - 1);
+            t = 2 * t + (cu >= g.T);
+            if (cu >= g.T) below = cu - g.T < -g.lo;
+            else above = cu >= g.T - g.hi;
+        }
         tile3[a] = t;
-        c = c * 3 + (cl < -g.lo ? 0 : (cl >= g.T - g.hi ? 2 : 1));
+        c = c * 3 + (below ? 0 : above ? 2 : 1);
     }
     *cls = c;
 }
@@ -271,10 +284,10 @@ k_wsum_reduce(const double *wpart, int nblk, const int64_t *__restrict__ item_of
 }
 
 // Key of an object: (catalog, home tile, boundary class).
-template <typename R>
-__device__ __forceinline__ int64_t sort_key(const Obj<R> &o, const PaintGeom &g, int64_t kbase, int *t3) {
-    int cls;
-    home_key<R>(o, g, t3, &cls);
+template <typename R, bool WANT_U>
+__device__ __forceinline__ int64_t sort_key(const Obj<R> &o, const PaintGeom &g, int64_t kbase, float *u) {
+    int t3[3], cls;
+    home_key<R, WANT_U>(o, g, t3, u, &cls);
     return kbase + (((int64_t)t3[0] * g.ntx + t3[1]) * g.ntx + t3[2]) * kClasses + cls;
 }
 
@@ -296,8 +309,8 @@ k_sort_count(const void *__restrict__ pos, const float *__restrict__ w, const fl
     for (int64_t i = beg + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end;
          i += (int64_t)gridDim.x * blockDim.x) {
         const Obj<R> o = load_obj<DT>(pos, w, vals, i, g);
-        int t3[3];
-        atomicAdd(count + sort_key<R>(o, g, kbase, t3), 1u);   // result unused: a reduction
+        float u[3];
+        atomicAdd(count + sort_key<R, false>(o, g, kbase, u), 1u);   // result unused: a reduction
         if (WEIGHTED) {
             const double ad = (double)o.a;
             sw += (double)o.w;
@@ -332,16 +345,14 @@ k_sort_scatter(const void *__restrict__ pos, const float *__restrict__ w, const 
     for (int64_t i = beg + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end;
          i += (int64_t)gridDim.x * blockDim.x) {
         const Obj<R> o = load_obj<DT>(pos, w, vals, i, g);
-        int t3[3];
-        const int64_t key = sort_key<R>(o, g, kbase, t3);
+        float u[3];
+        const int64_t key = sort_key<R, true>(o, g, kbase, u);
         const uint32_t slot = atomicAdd(cursor + key, 1u);
         if (slot >= ntot) {                      // count and scatter disagree: never write
             atomicOr(err, 2);
             continue;
         }
-        sorted[slot] = make_float4((float)(o.s[0] - (R)(t3[0] * g.T)) + o.e[0],
-                                   (float)(o.s[1] - (R)(t3[1] * g.T)) + o.e[1],
-                                   (float)(o.s[2] - (R)(t3[2] * g.T)) + o.e[2], o.a);
+        sorted[slot] = make_float4(u[0], u[1], u[2], o.a);
     }
 }
 
@@ -800,10 +811,31 @@ __device__ __forceinline__ int seg_dx(int s) { const int ax = s / 15; return ax 
 __device__ __forceinline__ int seg_dy(int s) { const int ay = (s / 3) % 5; return ay == 0 ? -1 : (ay == 4 ? 1 : 0); }
 __device__ __forceinline__ int seg_dz(int s) { return s % 3 - 1; }
 
+// Where a tile lies in its frame: the tile itself, or (half > 0) a pair of tiles along
+// each axis, of which it is the lower or the upper one.  Coordinates of candidates, and
+// their shifts to the second mesh, are rounded in the frame; at() then takes the frame
+// coordinate to the tile's, exactly (in an upper half it is 5 or more).
+template <int TC>
+struct TileFrame {
+    int T, bits;                                      // bits 0 .. 2: upper half along x, y, z; 3: halves
+    __device__ __forceinline__ TileFrame(int T_, int flog, int tx, int ty, int tz)
+        : T(T_), bits(flog ? 8 | (tx & 1) | (ty & 1) << 1 | (tz & 1) << 2 : 0) {}
+    // Neighbour d's frame relative to this one, in cells.
+    __device__ __forceinline__ float shift(int d, int axis) const {
+        if (TC > 0) return (float)(d * TC);
+        return (float)(bits & 8 ? (((bits >> axis & 1) + d) >> 1) * 2 * T : d * T);
+    }
+    __device__ __forceinline__ float at(float v, int axis) const {
+        if (TC > 0) return v;
+        return bits >> axis & 1 ? v - (float)T : v;
+    }
+};
+
 // Candidate k of the tile (k < s_pre[kSegments]) in this tile's frame
 // (segment shift added), weight scaled by 2^S.
+template <int TC>
 __device__ __forceinline__ float4 fetch_candidate(const float4 *sorted, const uint32_t *s_beg,
-                                                  const uint32_t *s_pre, int T, uint32_t k, float scale) {
+                                                  const uint32_t *s_pre, const TileFrame<TC> &fr, uint32_t k, float scale) {
     int lo_s = 0, hi_s = kSegments;                   // s_pre[lo_s] <= k < s_pre[hi_s]
     while (hi_s - lo_s > 1) {
         const int mid = (lo_s + hi_s) >> 1;
@@ -811,32 +843,33 @@ __device__ __forceinline__ float4 fetch_candidate(const float4 *sorted, const ui
         else hi_s = mid;
     }
     const float4 v = sorted[s_beg[lo_s] + (k - s_pre[lo_s])];
-    return make_float4(v.x + (float)(seg_dx(lo_s) * T), v.y + (float)(seg_dy(lo_s) * T),
-                       v.z + (float)(seg_dz(lo_s) * T), v.w * scale);
+    return make_float4(v.x + fr.shift(seg_dx(lo_s), 0), v.y + fr.shift(seg_dy(lo_s), 1), v.z + fr.shift(seg_dz(lo_s), 2),
+                       v.w * scale);
 }
 
 // Copy candidates [k0, k0 + n) of the tile into shared memory.
+template <int TC>
 __device__ __forceinline__ void stage_candidates(const float4 *sorted, const uint32_t *s_beg,
-                                                 const uint32_t *s_pre, int T, uint32_t k0, uint32_t n,
+                                                 const uint32_t *s_pre, const TileFrame<TC> &fr, uint32_t k0, uint32_t n,
                                                  float scale, float4 *cand) {
     for (uint32_t j = threadIdx.x; j < n; j += blockDim.x)
-        cand[j] = fetch_candidate(sorted, s_beg, s_pre, T, k0 + j, scale);
+        cand[j] = fetch_candidate(sorted, s_beg, s_pre, fr, k0 + j, scale);
 }
 
 template <int P, int MODE, int TC, bool UNIT, typename M>
 __device__ __forceinline__ void deposit_staged(const float4 *cand, uint32_t n, unsigned *lo, unsigned *hi,
-                                               unsigned long long *acc64, const Split &sp, int T, float sh) {
+                                               unsigned long long *acc64, const Split &sp, int T, const TileFrame<TC> &fr, float sh) {
     for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
         const float4 v = cand[j];
-        deposit<P, MODE, TC, UNIT, M>(lo, hi, acc64, sp, T, v.x + sh, v.y + sh, v.z + sh, v.w);
+        deposit<P, MODE, TC, UNIT, M>(lo, hi, acc64, sp, T, fr.at(v.x + sh, 0), fr.at(v.y + sh, 1), fr.at(v.z + sh, 2), v.w);
     }
 }
 
 template <int P, int TC, bool UNIT, typename M>
 __device__ __forceinline__ void deposit_any(const float4 *cand, uint32_t n, unsigned *lo, unsigned *hi,
-                                            unsigned long long *acc64, const Split &sp, int T, float sh) {
-    if (sp.fast) deposit_staged<P, 1, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, sh);
-    else deposit_staged<P, 0, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, sh);
+                                            unsigned long long *acc64, const Split &sp, int T, const TileFrame<TC> &fr, float sh) {
+    if (sp.fast) deposit_staged<P, 1, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, fr, sh);
+    else deposit_staged<P, 0, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, fr, sh);
 }
 
 // Write one tile's cells to the mesh (r2c layout, rows of T cells along z at
@@ -959,6 +992,7 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
     const int tz = (int)(t - tq * ntx);
     const int tx = (int)(tq / ntx);
     const int ty = (int)(tq - (unsigned)tx * ntx);
+    const TileFrame<TC> fr(T, g.flog, tx, ty, tz);
     const uint4 wm = wmaxs[item];
 
     // Segments: neighbour offset d (per axis -1, 0, +1) with the classes of
@@ -1075,8 +1109,8 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
         for (int c = threadIdx.x; c < B.Count; c += blockDim.x) smu[c] = 0u;
         __syncthreads();
         for (uint32_t k = threadIdx.x * stride; k < total; k += blockDim.x * stride) {
-            const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
-            atomicAdd(smu + B.of(v.x, v.y, v.z, wide), steps(v.w));
+            const float4 v = fetch_candidate(sorted, s_beg, s_pre, fr, k, scale);
+            atomicAdd(smu + B.of(fr.at(v.x, 0), fr.at(v.y, 1), fr.at(v.z, 2), wide), steps(v.w));
         }
         __syncthreads();
         return B.most(smu, wide);
@@ -1109,11 +1143,11 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
         unsigned long long sum_abs = 0ull;
         const auto account = [&](const float4 &v) {
             if (!UNIT) sum_abs += fabsf(v.w) < 4.29e9f ? (unsigned long long)__float2uint_ru(fabsf(v.w)) : 1ull << 40;
-            if (counted) atomicAdd(s_blk + Coarse::of(v.x, v.y, v.z, wide), steps(v.w));
+            if (counted) atomicAdd(s_blk + Coarse::of(fr.at(v.x, 0), fr.at(v.y, 1), fr.at(v.z, 2), wide), steps(v.w));
         };
         if (kPadded) {
             for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
-                const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
+                const float4 v = fetch_candidate(sorted, s_beg, s_pre, fr, k, scale);
                 account(v);
                 sweep_deposit<P, UNIT>(smu, v.x, v.y, v.z, v.w);
                 if (NM == 2)
@@ -1124,16 +1158,17 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
             const unsigned trash = (unsigned)(2 * T3) + (threadIdx.x & 31);
             const bool flat = !dense && total <= (uint32_t)kFlatMaxCand;
             for (uint32_t k = threadIdx.x; k < total; k += blockDim.x) {
-                const float4 v = fetch_candidate(sorted, s_beg, s_pre, T, k, scale);
+                const float4 v = fetch_candidate(sorted, s_beg, s_pre, fr, k, scale);
                 account(v);
+                const float x = fr.at(v.x, 0), y = fr.at(v.y, 1), z = fr.at(v.z, 2);
+                const float x2 = fr.at(v.x + 0.5f, 0), y2 = fr.at(v.y + 0.5f, 1), z2 = fr.at(v.z + 0.5f, 2);
                 if (flat) {
-                    deposit_flat<P, TC, UNIT>(smu, 0, trash, T, v.x, v.y, v.z, v.w);
-                    if (NM == 2) deposit_flat<P, TC, UNIT>(smu, T3, trash, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
+                    deposit_flat<P, TC, UNIT>(smu, 0, trash, T, x, y, z, v.w);
+                    if (NM == 2) deposit_flat<P, TC, UNIT>(smu, T3, trash, T, x2, y2, z2, v.w);
                 } else {
                     const Split none{};
-                    deposit<P, 2, TC, UNIT, float>(lo, nullptr, nullptr, none, T, v.x, v.y, v.z, v.w);
-                    if (NM == 2)
-                        deposit<P, 2, TC, UNIT, float>(hi, nullptr, nullptr, none, T, v.x + 0.5f, v.y + 0.5f, v.z + 0.5f, v.w);
+                    deposit<P, 2, TC, UNIT, float>(lo, nullptr, nullptr, none, T, x, y, z, v.w);
+                    if (NM == 2) deposit<P, 2, TC, UNIT, float>(hi, nullptr, nullptr, none, T, x2, y2, z2, v.w);
                 }
             }
         }
@@ -1190,7 +1225,7 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
         sp.fast = sp.B >= 1 && hmax < 4194304.0f && (float)nc * (hmax + 1.0f) < 2.0e9f;
     }
     const bool staged_once = total <= (uint32_t)kStage;
-    if (staged_once) stage_candidates(sorted, s_beg, s_pre, T, 0u, total, scale, cand);
+    if (staged_once) stage_candidates(sorted, s_beg, s_pre, fr, 0u, total, scale, cand);
 #pragma unroll 1
     for (int m = 0; m < NM; ++m) {
         {
@@ -1202,14 +1237,14 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
         __syncthreads();
         const float sh = m ? 0.5f : 0.0f;
         if (staged_once) {
-            deposit_any<P, TC, UNIT, M>(cand, total, lo, hi, acc64, sp, T, sh);
+            deposit_any<P, TC, UNIT, M>(cand, total, lo, hi, acc64, sp, T, fr, sh);
         } else {
             for (uint32_t k0 = 0; k0 < total; k0 += kStage) {     // dense tile: batches
                 const uint32_t n = min((uint32_t)kStage, total - k0);
                 __syncthreads();                                  // previous batch consumed
-                stage_candidates(sorted, s_beg, s_pre, T, k0, n, scale, cand);
+                stage_candidates(sorted, s_beg, s_pre, fr, k0, n, scale, cand);
                 __syncthreads();
-                deposit_any<P, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, sh);
+                deposit_any<P, TC, UNIT, M>(cand, n, lo, hi, acc64, sp, T, fr, sh);
             }
         }
         __syncthreads();
