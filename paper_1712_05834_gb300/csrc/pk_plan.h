@@ -39,6 +39,7 @@ struct pk_plan_s {
     int own_selectable = 0;          // pk_use_own_fft(plan, 1) accepts it
     const pk::ZyxOps *zyx = nullptr; // zyx form; NULL: packed
     int unfinished = 0;              // meshes hold the transform without its last axis
+    int wants_transform = 0;         // cross or projected power has been asked for (see finish_transform)
     int G_own = 0;                   // fused last-axis CTAs for one catalog (zyx: 0 = x, then k_bin)
     pk::Fft64 fft64{};               // FP64 form: steps and tables (both in d_tw)
     void *d_tw = nullptr;            // W_N^e, e < N (float2)
