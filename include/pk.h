@@ -282,8 +282,8 @@ pk_status pk_mesh(pk_plan_t plan, int item, int mesh, void *dst);
  * bin pass.  Both give the same result within FP32 rounding (FP64 meshes: the
  * own FP64 transform or cuFFT's D2Z, within FP64 rounding).  After a compute
  * that did not write the transform itself, pk_cross and pk_projected first
- * write it into the meshes (one extra pass).  Takes effect at the next
- * pk_compute.
+ * write it into the meshes (one extra pass; at 1024 and 2048 later computes of
+ * the plan then write it themselves).  Takes effect at the next pk_compute.
  * Errors: PK_EINVAL (on = 1 other than for the FP32 mesh form with nmesh 128,
  * 192, 256, 512, 1024 or 2048). */
 pk_status pk_use_own_fft(pk_plan_t plan, int on);

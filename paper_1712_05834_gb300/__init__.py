@@ -371,7 +371,7 @@ def pk_compute(plan):
 def _arr(ptr, n, dtype=np.float64):
     if not ptr or n == 0:
         return None
-    # one copy into a buffer of its own; np.ctypeslib.as_array and astype took 2.3 us an array for 1.0
+    # a writable copy through bytes: 1.0 us an array, np.ctypeslib.as_array and astype took 2.3
     return np.frombuffer(bytearray(ctypes.string_at(ptr, 8 * n)), dtype)
 
 

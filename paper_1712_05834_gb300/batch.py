@@ -12,8 +12,8 @@ whose batch holds all of its catalogs, back to back in one device buffer:
     every catalog of the class;
   * one transform of every mesh of the class (own kernels, or a batched cuFFT
     call);
-  * one bin launch (persistent CTAs, a fixed share per catalog), one reduce
-    and one finalize launch over every catalog of the class.
+  * one bin launch (persistent CTAs, a fixed share per catalog) and one launch
+    that sums and normalizes over every catalog of the class.
 
 The whole sequence for all classes is captured once into a CUDA graph on the
 runner's stream and replayed per evaluation; the graph re-reads the position

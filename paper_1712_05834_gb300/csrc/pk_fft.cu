@@ -674,9 +674,9 @@ cudaError_t zfinish_inst(void *mesh, long long is, long long ms, int nitems, int
 }  // namespace
 
 // Measured on a GB300 (FFT + bin): 32 catalogs of 128^3 0.40 against 0.56 ms
-// with cuFFT, 24 of 192^3 1.07 against 1.35 ms, 512^3 1.24 against 1.84 ms.
+// with cuFFT, 24 of 192^3 1.07 against 1.35 ms, 512^3 1.16 against 1.84 ms.
 // Against the z-and-y-in-one-pass form of pk_fft_zyx.cu (interlaced at 512^3
-// 1.24 against 1.28 ms, one mesh of 256^3 0.099 against 0.144 ms): these sizes
+// 1.16 against 1.23 ms, one mesh of 256^3 0.098 against 0.125 ms): these sizes
 // stay packed, where the fused z pass works warp by warp without CTA barriers.
 bool own_fft_packed(int N) { return N == 128 || N == 192 || N == 256 || N == 512; }
 

@@ -24,10 +24,15 @@
 //                interlace combine, sinc^p compensation, k bin, mu bin,
 //                Legendre sums; the r2c transform is never written.  Measured
 //                against k_fft_x + k_bin (ms, with k_fft_zy): 1024 interlaced
-//                11.1 against 12.0, 2048 58.3 against 62.1; 640 interlaced 4.5
-//                against 4.1, 480 1.96 against 1.74 (its bin pass idles half
-//                of the threads at the edge of the sphere), so the smaller
-//                sizes take the two kernels.
+//                10.0 against 10.4, one mesh 5.66 against 5.70, 2048 51.5 against
+//                54.3; 640 interlaced 4.5 against 4.1, 480 1.96 against 1.74 (the
+//                bin pass idles half of the threads at the edge of the sphere), so
+//                the smaller sizes take the two kernels.
+//
+// Sizes: each is an instance to compile and to measure; 320 to 800 are those with factors
+// 2, 3 and 5 that the workloads and tests here use.  Others (432, 576, 720, 864, 960, 1000,
+// and all with a factor 7) have no instance and go to cuFFT, as do the smaller ones but
+// 128, 192 and 256 (pk_fft.cu).
 //
 // Only modes with m = |n|^2 < mhi enter a bin: columns l with l^2 >= mhi are
 // neither transformed along y nor read, the y pass does not write rows ky with
@@ -245,7 +250,8 @@ __device__ __forceinline__ int dif_freq(int p) {
 // and two 512-thread CTAs, 58.9 with 16-byte runs), at 1024 two CTAs (6.06 ms; 6.55
 // with 128-byte runs and one).  LAG: planes between a plane's z and y items (1024
 // interlaced: 6.05, 6.06 and 6.31 ms at 4, 6 and 10 planes; 2048: 29.8 and 30.4 at
-// 1 and 2).
+// 1 and 2; at 512, 8 planes 1060 us, 24 774, 64 858; the other sizes are set between
+// those, not swept).
 template <int N>
 struct Shape;
 template <int T_, int CTAS_, int NBY_, int TX_, int CTASX_, int NX_, int LAG_>

@@ -1,5 +1,5 @@
-// pk_internal.h -- declarations shared by the two translation units of
-// libpk.so (host API in pk_api.cu, kernels in pk_kernels.cu).  Not installed.
+// pk_internal.h -- declarations shared by the translation units of libpk.so.  Not
+// installed.
 #pragma once
 
 #include <cuda_runtime.h>

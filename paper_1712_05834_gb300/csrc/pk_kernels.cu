@@ -10,7 +10,7 @@
 //   k_wsum_reduce   weighted catalogs: the paint blocks' rows of weight sums
 //                   added in a fixed order (run-to-run identical sums).
 //   k_scan_*        exclusive scan of the key counts (uint32).
-//   k_sort_scatter  write one float4 (home-tile-local x, y, z, w) per object
+//   k_sort_scatter  write one float4 (x, y, z in the home tile's frame, w) per object
 //                   at its key's cursor, advanced by the write (the scan
 //                   leaves the offsets in the counts' place, too): the
 //                   order inside a key is whatever order the cursors are
@@ -27,8 +27,10 @@
 //                   every cell of the tile, one sweep over the candidates
 //                   deposits both interlaced meshes, branch-free in sparse
 //                   tiles; else one mesh per pass over staged candidates.
-//                   Integer adds are order-free: the mesh is
-//                   bit-identical run to run and for any object order.
+//                   Integer adds are order-free, and an FP32 cell is the same
+//                   integers rounded once either way: the mesh is bit-identical
+//                   run to run, for any object order, tile size of the plan's
+//                   choice and batch.
 //   k_paint_atomic  the variant without a sort: one thread per object adds
 //                   each deposit with a 64-bit global atomic into a dense
 //                   int64 accumulator per mesh (as order-free as the tiles);
@@ -1061,8 +1063,9 @@ k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor,
     // weights: the sum of the candidates' |W V| bounds every cell; it is taken
     // during the sweep, and a tile whose cells might pass 2^31, or 2^32 where no
     // W V is negative (S = 22: sum |W V| above 1022 for CIC, 2424 for TSC, 3451
-    // for PCS), is painted again the general way.  A tile that the catalog's
-    // mean |W V| says will not fit skips the sweep.
+    // for PCS), is counted in blocks (below) and painted again, swept if those fit,
+    // else the general way.  A tile that the catalog's mean |W V| says will not fit
+    // skips the sweep.
     //
     // Weighted catalogs used to stage their candidates and take one pass per
     // mesh; unit weights needed deposits below the general path's 2^B, so at
