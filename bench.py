@@ -382,7 +382,7 @@ def measure_2048(pk, torch, stream, world, steps=5, warmup=2):
     L = 2000, PCS + interlacing on N = 2048 (FP32 mesh, int64 fixed-point
     paint, FP32 per-CTA bin partials summed in FP64), (k, mu) bins dk = 0.005
     x 10, multipoles; then the same catalog in the FP64 mesh form (FP64 mesh,
-    D2Z, FP64 sums), whose result is the reference of the per-bin error."""
+    own transform, FP64 sums), whose result is the reference of the per-bin error."""
     import synth
     L, N, dk = 2000.0, 2048, 0.005
     pos = synth.zeldovich_lattice(1024, L, synth.seed_for(3), device="cuda")
@@ -425,7 +425,7 @@ def measure_2048(pk, torch, stream, world, steps=5, warmup=2):
 
 def measure_fp64_form(pk, torch, stream, pos, flush, steps=10, warmup=3):
     """The FP64 mesh form of the main workload (FP64 deposits from the int64
-    fixed-point cells, FP64 mesh, D2Z, FP64 per-mode arithmetic and sums),
+    fixed-point cells, FP64 mesh and transform, FP64 per-mode arithmetic and sums),
     timed like the main line (L2 flushed between steps)."""
     cfg = pk.make_config(L_BOX, NMESH, "tsc", interlaced=True, dk=DK, nmu=NMU, precision="f64")
     plan = pk.pk_plan(cfg, stream)
@@ -454,7 +454,7 @@ def measure_fp64_form(pk, torch, stream, pos, flush, steps=10, warmup=3):
     ms = statistics.median(times)
     return {"ms_per_step": ms, "pk_per_s": 1e3 / ms, "stage_ms_median": {k: statistics.median(v) for k, v in
                                                                            stages.items()},
-            "form": "FP64 mesh, int64 fixed-point paint, D2Z, FP64 per-mode arithmetic and bin sums"}, res
+            "form": "FP64 mesh, int64 fixed-point paint, FP64 transform, per-mode arithmetic and bin sums"}, res
 
 
 def max_rel_diff(a, b):
