@@ -969,8 +969,14 @@ __device__ __forceinline__ void flush_tile(const unsigned *lo, const unsigned *h
 __host__ __device__ constexpr int paint_cell_words(int T) { return (2 * T * T * T + 3) & ~3; }
 
 // TC > 0: the tile edge is the compile-time constant TC (index math in shifts).
+// CTAs per SM: as many as the shared memory of tiles of 16 lets in, and their registers;
+// left to itself the compiler spilled for more (general path, weighted, 3e7 objects at
+// 256^3, interlaced: TSC 3603 -> 3337 us, PCS 7103 -> 6214; 2048^3 lattice 74.3 -> 73.8 ms).
+// Other tiles: its choice (asked for 5 or 6 CTAs, halves of tiles lost up to 35 %).
+template <int P, int NM, int TC>
+constexpr int kPaintCtas = TC != 16 ? 0 : NM == 1 || P == 2 ? 6 : P == 3 ? 5 : 4;
 template <int P, int NM, typename M, int TC, bool UNIT>
-__global__ void __launch_bounds__(kPaintThreads)
+__global__ void __launch_bounds__(kPaintThreads, kPaintCtas<P, NM, TC>)
 k_paint_tiles(const float4 *sorted, const uint32_t *off, const uint32_t *cursor, int *__restrict__ err, PaintGeom g,
               int S, const uint4 *wmaxs, float wdep, M *__restrict__ mesh,
               long long item_stride, long long mesh_stride, int accumulate) {
