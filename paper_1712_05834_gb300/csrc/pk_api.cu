@@ -486,11 +486,9 @@ static pk_status plan_build(pk_plan_s *P, const pk_config *cfg) {
                 }
                 return (int)tiles.size() - before;
             };
-            P->nxbin = add_tiles(P->zyx->tile_columns(c.interlaced));
-            P->nx = c.interlaced ? add_tiles(P->zyx->tile_columns(0)) : P->nxbin;
+            P->nx = add_tiles(P->zyx->tile_columns());
             PK_CUDA(P, dev_alloc(&P->d_xtiles, sizeof(int) * tiles.size()));
             PK_CUDA(P, cudaMemcpy(P->d_xtiles, tiles.data(), sizeof(int) * tiles.size(), cudaMemcpyHostToDevice));
-            P->G_own = std::min(std::min(P->G_total, P->nsm * P->zyx->xbin_ctas_per_sm(bg, c.interlaced)), P->nxbin);
         }
     }
 
@@ -745,8 +743,7 @@ pk_status pk_paint_values(pk_plan_t P, const void *pos, int dtype, const float *
 static pk_status take_last_axis(pk_plan_s *P, int nitems) {
     if (P->zyx)
         PK_CUDA(P, P->zyx->x(P->mesh, nitems * P->nm, P->mesh_reals / 2, P->fft_ncol, P->bg.mhi,
-                             P->cfg.interlaced ? P->d_xtiles + P->nxbin : P->d_xtiles, P->nx, P->d_tw, P->d_sync,
-                             P->nsync, P->st));
+                             P->d_xtiles, P->nx, P->d_tw, P->d_sync, P->nsync, P->st));
     else
         PK_CUDA(P, launch_zfinish(P->mesh, P->cfg.interlaced, (long long)P->nm * P->mesh_reals / 2, P->mesh_reals / 2,
                                   nitems, P->N, P->d_tw, P->nsm, P->st));
@@ -757,13 +754,9 @@ static pk_status take_last_axis(pk_plan_s *P, int nitems) {
 }
 
 // After a compute with the last axis fused into the bins the meshes lack it; the calls
-// that read the transform itself get it taken in place first (once per compute).  A plan
-// that has been asked for it takes x and the bins in two passes from then on (zyx
-// form): two catalogs and their cross power at 1024^3, interlaced, 30.4 ms, 36.2 with x
-// taken twice.
+// that read the transform itself get it taken in place first (once per compute).
 static pk_status finish_transform(pk_plan_s *P) {
     if (!P->unfinished) return PK_OK;
-    P->wants_transform = 1;
     return take_last_axis(P, P->computed);
 }
 
@@ -799,25 +792,15 @@ pk_status pk_compute(pk_plan_t P) {
                                    P->d_tw, P->d_kedge, P->d_partial, st));
             P->launches += 2;   // the two axis passes
         } else {
-            // z and y axes, then x fused into the bin pass (or, where its histogram does
-            // not fit beside a tile or the transform is wanted, x in place and k_bin)
+            // z and y axes, x in place, then k_bin
             PK_CUDA(P, zyx_counters(P->d_sync, P->nsync, &P->sync_used, st));
             PK_CUDA(P, P->zyx->zy(P->mesh, nitems * P->nm * P->N, P->fft_ncol, P->bg.mhi, P->d_tw, P->d_sync,
                                   P->d_err, P->nsm, st));
             P->launches += 1;
-            if (P->G_own > 0 && !P->wants_transform) {
-                if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
-                G = std::max(1, P->G_own / nitems);
-                PK_CUDA(P, P->zyx->xbin(P->mesh, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->fft_ncol,
-                                        P->d_xtiles, P->nxbin, P->d_cw, P->d_ph, P->d_tw, P->d_kedge, P->d_partial,
-                                        P->d_sync, P->nsync, st));
-                P->sync_used = 0;
-            } else {
-                if (pk_status s = take_last_axis(P, nitems); s != PK_OK) return s;
-                if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
-                PK_CUDA(P, launch_bin(P->mesh, P->f64, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->d_cw,
-                                      P->d_ph, P->d_kedge, P->d_partial, st));
-            }
+            if (pk_status s = take_last_axis(P, nitems); s != PK_OK) return s;
+            if (tm) PK_CUDA(P, cudaEventRecord(P->tev[4], st));
+            PK_CUDA(P, launch_bin(P->mesh, P->f64, P->cfg.interlaced, item_c, mesh_c, nitems, G, P->bg, P->d_cw,
+                                  P->d_ph, P->d_kedge, P->d_partial, st));
         }
     } else if ((s_ = ensure_cufft(P)) != PK_OK) {
         return s_;

@@ -16,18 +16,12 @@
 //                L2 (129 MB) and overwrite them there: device memory sees one
 //                read and one write for two axes (512^3: 2.1 GB counted, where
 //                two passes move 4.3).
-//   k_fft_x      the x axis, written back in place; k_bin then bins the modes.
-//   k_fft_xbin   (N = 1024, 2048, unless a pass needs the transform itself) x
-//                axis and the bin pass: one CTA per tile of columns (ky, l0 ..)
-//                (two interlaced meshes share a tile) takes the length-N FFTs
-//                along x in shared memory and bins the modes from there:
-//                interlace combine, sinc^p compensation, k bin, mu bin,
-//                Legendre sums; the r2c transform is never written.  Measured
-//                against k_fft_x + k_bin (ms, with k_fft_zy): 1024 interlaced
-//                10.0 against 10.4, one mesh 5.66 against 5.70, 2048 51.5 against
-//                54.3; 640 interlaced 4.5 against 4.1, 480 1.96 against 1.74 (the
-//                bin pass idles half of the threads at the edge of the sphere), so
-//                the smaller sizes take the two kernels.
+//   k_fft_x      the x axis, written back in place; k_bin then bins the modes.  A
+//                pass that took x and binned from shared memory at 1024 and 2048
+//                was faster (1024 interlaced 10.0 ms for 10.4, 2048 51.5 for 54.3,
+//                with k_fft_zy) but less exact: a CTA's FP32 sums ran over more
+//                modes, the rms error of P_2 on a lattice of 512^3 objects at 1024
+//                was 1.7e-6 of P_0 for 3.2e-7, at 2048 1.1e-5 for 2.3e-6.
 //
 // Sizes: each is an instance to compile and to measure; 320 to 800 are those with factors
 // 2, 3 and 5 that the workloads and tests here use.  Others (432, 576, 720, 864, 960, 1000,
@@ -284,7 +278,6 @@ struct Cfg : Shape<N> {
     static constexpr int RPI = GROUPS * NR;                      // rows per z item
     static constexpr int ZI = (N + RPI - 1) / RPI;               // z items per plane
     static_assert(NT == 32 || GROUPS <= 15, "named barriers are 1 .. 15");
-    static constexpr bool FUSE = N >= 1024;                      // k_fft_xbin
 };
 
 // ---------------------------------------------------------------------------
@@ -768,8 +761,7 @@ __device__ __forceinline__ void clear_sync(unsigned *sync, int n) {
 
 // A value of a run along z at an x line's point: the runs of a tile are 64 or 128
 // bytes, planes apart, and the tiles beside it are in flight too, so the L2 is
-// told to fetch 256 bytes around (k_fft_xbin 4.12 -> 3.77 ms at 1024^3 interlaced,
-// 22.5 -> 21.0 ms at 2048^3).
+// told to fetch 256 bytes around.
 __device__ __forceinline__ float2 load_run(const float2 *p) {
     float2 v;
     asm volatile("ld.global.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
@@ -799,159 +791,6 @@ k_fft_x(float2 *__restrict__ mesh, long long mesh_c, int ncol, int mcut, const i
         if (c < nc && ip * ip + r2 < mcut) g[f * ps + c] = v;
     };
     col_step<N, NX, K::TX, false, N, true, false>(buf, tw, threadIdx.x % NX, threadIdx.x / NX, ld, st);
-}
-
-// Shared memory of k_fft_xbin: the twiddles, the tile, then the histogram,
-// the cw and phase tables and the k-bin edges.
-template <int N>
-struct XSmem {
-    __host__ __device__ static constexpr size_t al(size_t x) { return (x + 15) / 16 * 16; }
-    __host__ __device__ static constexpr size_t off_buf() { return al(sizeof(float2) * N); }
-    __host__ __device__ static constexpr size_t off_hist() { return off_buf() + al(sizeof(float2) * N * Cfg<N>::NX); }
-    __host__ __device__ static size_t off_cw(const BinGeom &g) { return off_hist() + al(sizeof(float) * g.nh); }
-    __host__ __device__ static size_t off_ph(const BinGeom &g) { return off_cw(g) + al(sizeof(float) * Cfg<N>::Nh); }
-    __host__ __device__ static size_t off_edge(const BinGeom &g) { return off_ph(g) + al(sizeof(float2) * Cfg<N>::Nh); }
-    __host__ __device__ static size_t bytes(const BinGeom &g) { return off_edge(g) + al(sizeof(int2) * g.nk); }
-};
-
-// x FFT + bin over the tiles of one catalog per blockIdx.y.  Bin pass: a
-// thread takes one column l and runs of four kx with their mirror images -kx:
-// both modes have the same m, k bin, mu bin and Legendre weights, so the key
-// arithmetic is done once for the pair, and a run is summed in registers until
-// its key changes.  |kx| = 0 and N/2 occur once.
-template <int N, bool IL, bool TWOD, bool POLES>
-__global__ void __launch_bounds__(Cfg<N>::TX, Cfg<N>::CTASX)
-k_fft_xbin(const float2 *__restrict__ mesh, long long item_stride_c, long long mesh_stride_c, BinGeom g, int ncol,
-           const int *__restrict__ tiles, int ntiles, const float *__restrict__ cw, const float2 *__restrict__ ph,
-           const float2 *__restrict__ twg, const int *__restrict__ kedge, float *__restrict__ partial,
-           unsigned *__restrict__ sync, int nsync) {
-    using K = Cfg<N>;
-    using SM = XSmem<N>;
-    constexpr int M = K::M, Nh = K::Nh, NX = K::NX, TX = K::TX, CM = IL ? NX / 2 : NX;
-    using Tl = Tile<NX, IL>;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    float2 *tw = reinterpret_cast<float2 *>(smraw);
-    float2 *buf = reinterpret_cast<float2 *>(smraw + SM::off_buf());
-    float *hist = reinterpret_cast<float *>(smraw + SM::off_hist());
-    float *scw = reinterpret_cast<float *>(smraw + SM::off_cw(g));
-    float2 *sph = reinterpret_cast<float2 *>(smraw + SM::off_ph(g));
-    int2 *sedge = reinterpret_cast<int2 *>(smraw + SM::off_edge(g));
-    for (int e = threadIdx.x; e < N; e += TX) tw[e] = twg[e];
-    for (int k = threadIdx.x; k < g.nh; k += TX) hist[k] = 0.0f;
-    for (int k = threadIdx.x; k < Nh; k += TX) {
-        scw[k] = cw[k];                          // cw[N/2] = the Nyquist index
-        sph[k] = ph[k + M];                      // e^{+i pi k / N}
-    }
-    for (int k = threadIdx.x; k < g.nk; k += TX) sedge[k] = make_int2(kedge[k], kedge[k + 1]);
-    clear_sync(sync, nsync);
-
-    const int nk = g.nk, nmu = g.nmu, hbase = g.hbase;
-    const float kscale = g.kscale, koff = g.koff;
-    const long long ps = (long long)N * Nh;
-    const float2 *base = mesh + (long long)blockIdx.y * item_stride_c;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int tile = tiles[t];
-        const int j = tile >> 16, c0 = (tile & 0xffff) * CM, nc = ncol - c0;
-        const float2 *gt = base + (long long)j * Nh + c0;
-        __syncthreads();                         // tables filled; the previous tile is binned
-        const auto ld = [&](int r, int c) {
-            const int cc = IL ? c % CM : c;
-            const float2 *p = gt + r * ps + cc;
-            if (IL && c >= CM) p += mesh_stride_c;
-            return cc < nc ? load_run(p) : make_float2(0.0f, 0.0f);
-        };
-        const auto st = [&](int f, int c, float2 v) { buf[Tl::slot(f, c)] = v; };
-        col_step<N, NX, TX, IL, N, true, true>(buf, tw, threadIdx.x % NX, threadIdx.x / NX, ld, st);
-        __syncthreads();
-
-        const int c = threadIdx.x % CM, l = c0 + c;
-        const int jp = j < M ? j : j - N, ja = j < M ? j : N - j;
-        const int r2 = jp * jp + l * l;
-        if (c < nc && r2 < g.mhi) {
-            const float rowcw = scw[ja] * scw[l] * (IL ? 0.25f : 1.0f) * ((l != 0 && l != M) ? 2.0f : 1.0f);
-            float2 rph = make_float2(1.0f, 0.0f);
-            if (IL) {
-                const float2 py = sph[ja];
-                rph = c_mul(make_float2(py.x, jp < 0 ? -py.y : py.y), sph[l]);
-            }
-            const unsigned rhs = (unsigned)(nmu * nmu) * (unsigned)(l * l);
-            for (int i0 = 4 * (threadIdx.x / CM); i0 <= M; i0 += 4 * (TX / CM)) {
-                if (i0 * i0 + r2 >= g.mhi) break;
-                int cur2 = -1, cur1 = -1;                 // open register runs
-                float run2 = 0.0f, runm2 = 0.0f, runm4 = 0.0f;
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    const int i = min(i0 + v, M);
-                    const int m = r2 + i * i;
-                    const bool live = i0 + v <= M && m < g.mhi && m >= g.mlo && m != 0;
-                    // k bin: FP32 estimate, then one exact step against the edges
-                    const float rsm = rsqrtf((float)max(m, 1));
-                    int b = (int)((float)m * rsm * kscale - koff);
-                    b = min(max(b, 0), nk - 1);
-                    {
-                        const int2 e = sedge[b];
-                        b += (int)(m >= e.y) - (int)(m < e.x);
-                        b = min(max(b, 0), nk - 1);
-                    }
-                    const int ib = i ? N - i : 0;          // row of -kx (row N/2: kx = -N/2)
-                    float2 zp = buf[Tl::slot(i == M ? 0 : i, c)], zm = buf[Tl::slot(ib, c)];
-                    if (IL) {
-                        const float2 yp = buf[Tl::slot(i == M ? 0 : i, c + CM)], ym = buf[Tl::slot(ib, c + CM)];
-                        const float2 px = sph[i];
-                        const float2 tp = c_mul(rph, px), tm = c_mul(rph, make_float2(px.x, -px.y));
-                        zp.x += yp.x * tp.x - yp.y * tp.y;
-                        zp.y += yp.x * tp.y + yp.y * tp.x;
-                        zm.x += ym.x * tm.x - ym.y * tm.y;
-                        zm.y += ym.x * tm.y + ym.y * tm.x;
-                    }
-                    float pw = i != M ? zp.x * zp.x + zp.y * zp.y : 0.0f;
-                    if (i != 0) pw += zm.x * zm.x + zm.y * zm.y;
-                    pw = live ? pw * (rowcw * scw[i]) : 0.0f;
-                    int key = b;
-                    if (TWOD) {
-                        // mu bin: FP32 estimate, then one exact integer step each way
-                        int q = (int)((float)(nmu * l) * rsm);
-                        q = min(max(q, 0), nmu - 1);
-                        if (g.mu32) {
-                            q -= (int)(q > 0 && (unsigned)(q * q) * (unsigned)m > rhs);
-                            q += (int)(q < nmu - 1 && (unsigned)((q + 1) * (q + 1)) * (unsigned)m <= rhs);
-                        } else {
-                            const long long rl = (long long)nmu * nmu * l * l;
-                            q -= (int)(q > 0 && (long long)q * q * m > rl);
-                            q += (int)(q < nmu - 1 && (long long)(q + 1) * (q + 1) * m <= rl);
-                        }
-                        key = b * nmu + q;
-                    }
-                    const bool new2 = key != cur2;
-                    if (new2 && cur2 >= 0) atomicAdd(hist + cur2, run2);
-                    run2 = new2 ? pw : run2 + pw;
-                    cur2 = key;
-                    if (POLES) {
-                        const float mu = (float)l * rsm;
-                        const float mu2 = mu * mu;
-                        const float t2 = pw * (1.5f * mu2 - 0.5f);
-                        const float t4 = pw * ((4.375f * mu2 - 3.75f) * mu2 + 0.375f);
-                        const bool new1 = b != cur1;
-                        if (new1 && cur1 >= 0) {
-                            atomicAdd(hist + hbase + cur1, runm2);
-                            atomicAdd(hist + hbase + nk + cur1, runm4);
-                        }
-                        runm2 = new1 ? t2 : runm2 + t2;
-                        runm4 = new1 ? t4 : runm4 + t4;
-                        cur1 = b;
-                    }
-                }
-                atomicAdd(hist + cur2, run2);
-                if (POLES) {
-                    atomicAdd(hist + hbase + cur1, runm2);
-                    atomicAdd(hist + hbase + nk + cur1, runm4);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    float *out = partial + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * g.nh;
-    for (int k = threadIdx.x; k < g.nh; k += TX) out[k] = hist[k];
 }
 
 // ---------------------------------------------------------------- host --
@@ -993,64 +832,10 @@ cudaError_t x_inst(float2 *mesh, int nmesh, long long mesh_c, int ncol, int mcut
     return cudaGetLastError();
 }
 
-struct XbinArgs {
-    const float2 *mesh;
-    long long is, ms;
-    int nitems, G, ncol;
-    const int *tiles;
-    int ntiles;
-    const float *cw;
-    const float2 *ph, *tw;
-    const int *kedge;
-    float *partial;
-    unsigned *sync;
-    int nsync;
-};
-
-template <int N, bool IL, bool TWOD, bool POLES>
-cudaError_t xbin_inst(const XbinArgs &a, const BinGeom &g, cudaStream_t st) {
-    const size_t smem = XSmem<N>::bytes(g);
-    cudaError_t e = allow_smem(k_fft_xbin<N, IL, TWOD, POLES>, smem);
-    if (e != cudaSuccess) return e;
-    k_fft_xbin<N, IL, TWOD, POLES><<<dim3(a.G, a.nitems), Cfg<N>::TX, smem, st>>>(
-        a.mesh, a.is, a.ms, g, a.ncol, a.tiles, a.ntiles, a.cw, a.ph, a.tw, a.kedge, a.partial, a.sync, a.nsync);
-    return cudaGetLastError();
-}
-
-template <int N>
-cudaError_t xbin_dispatch(const XbinArgs &a, int il, const BinGeom &g, cudaStream_t st) {
-    const int key = (il ? 4 : 0) | (g.twod ? 2 : 0) | (g.poles ? 1 : 0);
-    switch (key) {
-    case 0: return xbin_inst<N, false, false, false>(a, g, st);
-    case 1: return xbin_inst<N, false, false, true>(a, g, st);
-    case 2: return xbin_inst<N, false, true, false>(a, g, st);
-    case 3: return xbin_inst<N, false, true, true>(a, g, st);
-    case 4: return xbin_inst<N, true, false, false>(a, g, st);
-    case 5: return xbin_inst<N, true, false, true>(a, g, st);
-    case 6: return xbin_inst<N, true, true, false>(a, g, st);
-    default: return xbin_inst<N, true, true, true>(a, g, st);
-    }
-}
-
-template <int N>
-int xbin_occ(const BinGeom &g, int il) {
-    const size_t smem = XSmem<N>::bytes(g);
-    const void *k = il ? reinterpret_cast<const void *>(k_fft_xbin<N, true, true, true>)
-                       : reinterpret_cast<const void *>(k_fft_xbin<N, false, true, true>);
-    int n = 0;
-    if (smem > 227 * 1024 ||
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, Cfg<N>::TX, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return n;
-}
-
 // One size's launchers.
 template <int N>
 struct OpsOf final : ZyxOps {
-    int tile_columns(int interlaced) const override { return interlaced ? Cfg<N>::NX / 2 : Cfg<N>::NX; }
+    int tile_columns() const override { return Cfg<N>::NX; }
     cudaError_t zy(void *mesh, int planes, int ncol, int mcut, const void *tw, unsigned *sync, int *err, int nsm,
                    cudaStream_t st) const override {
         return zy_inst<N, false>(reinterpret_cast<float2 *>(mesh), planes, ncol, mcut,
@@ -1066,20 +851,6 @@ struct OpsOf final : ZyxOps {
                   const void *tw, unsigned *sync, int nsync, cudaStream_t st) const override {
         return x_inst<N>(reinterpret_cast<float2 *>(mesh), nmesh, mesh_c, ncol, mcut, tiles, ntiles,
                          reinterpret_cast<const float2 *>(tw), sync, nsync, st);
-    }
-    int xbin_ctas_per_sm(const BinGeom &g, int interlaced) const override {
-        if constexpr (Cfg<N>::FUSE) return xbin_occ<N>(g, interlaced);
-        else return 0;
-    }
-    cudaError_t xbin(const void *mesh, int interlaced, long long item_stride_c, long long mesh_stride_c, int nitems,
-                     int ctas_per_item, const BinGeom &g, int ncol, const int *tiles, int ntiles, const void *cw,
-                     const void *ph, const void *tw, const int *kedge, void *partial, unsigned *sync, int nsync,
-                     cudaStream_t st) const override {
-        const XbinArgs a{reinterpret_cast<const float2 *>(mesh), item_stride_c, mesh_stride_c, nitems, ctas_per_item,
-                         ncol, tiles, ntiles, reinterpret_cast<const float *>(cw), reinterpret_cast<const float2 *>(ph),
-                         reinterpret_cast<const float2 *>(tw), kedge, reinterpret_cast<float *>(partial), sync, nsync};
-        if constexpr (Cfg<N>::FUSE) return xbin_dispatch<N>(a, interlaced, g, st);
-        else return cudaErrorInvalidValue;
     }
 };
 

@@ -242,25 +242,18 @@ struct ZyxOps {
     // planes each; sync: 1 + nx * nslot counters.
     virtual cudaError_t zy_survey(void *mesh, int nx, const SurveyRows &sv, int ncol, int mcut, const void *tw,
                                   unsigned *sync, int *err, int nsm, cudaStream_t st) const = 0;
-    // Columns l of one x tile (per mesh) of the fused bin pass; tile lists hold
+    // Columns l of one x tile; tile lists hold
     // ky index * 65536 + column block for the tiles with a mode m < mhi.
-    virtual int tile_columns(int interlaced) const = 0;
+    virtual int tile_columns() const = 0;
     // z and y axes of `planes` consecutive x planes; only columns l < ncol and
     // rows with ky^2 + l^2 below mcut are transformed.  sync: 1 + planes
-    // counters, zero on entry, cleared by the next x or xbin.  err: 4 if a wait
+    // counters, zero on entry, cleared by the next x.  err: 4 if a wait
     // gave up.
     virtual cudaError_t zy(void *mesh, int planes, int ncol, int mcut, const void *tw, unsigned *sync, int *err,
                            int nsm, cudaStream_t st) const = 0;
-    // x axis of nmesh meshes in place (tiles: tile_columns(0) wide).
+    // x axis of nmesh meshes in place (tiles: tile_columns() wide).
     virtual cudaError_t x(void *mesh, int nmesh, long long mesh_c, int ncol, int mcut, const int *tiles, int ntiles,
                           const void *tw, unsigned *sync, int nsync, cudaStream_t st) const = 0;
-    // x axis + the bin pass of launch_bin, partial histograms as launch_bin
-    // writes them.
-    virtual cudaError_t xbin(const void *mesh, int interlaced, long long item_stride_c, long long mesh_stride_c,
-                             int nitems, int ctas_per_item, const BinGeom &g, int ncol, const int *tiles, int ntiles,
-                             const void *cw, const void *ph, const void *tw, const int *kedge, void *partial,
-                             unsigned *sync, int nsync, cudaStream_t st) const = 0;
-    virtual int xbin_ctas_per_sm(const BinGeom &g, int interlaced) const = 0;   // 0: no xbin (or its shared memory does not fit)
 
 protected:
     ~ZyxOps() = default;

@@ -39,15 +39,14 @@ struct pk_plan_s {
     int own_selectable = 0;          // pk_use_own_fft(plan, 1) accepts it
     const pk::ZyxOps *zyx = nullptr; // zyx form; NULL: packed
     int unfinished = 0;              // meshes hold the transform without its last axis
-    int wants_transform = 0;         // cross or projected power has been asked for (see finish_transform)
-    int G_own = 0;                   // fused last-axis CTAs for one catalog (zyx: 0 = x, then k_bin)
+    int G_own = 0;                   // packed form: fused last-axis CTAs for one catalog
     pk::Fft64 fft64{};               // FP64 form: steps and tables (both in d_tw)
     void *d_tw = nullptr;            // W_N^e, e < N (float2)
     unsigned *d_sync = nullptr;      // zyx: ticket and plane counters of the z / y pass
     int nsync = 0, sync_used = 0;    // sync_used: see zyx_counters
     int fft_ncol = 0;                // zyx: columns l that hold a binned mode
-    int *d_xtiles = nullptr;         // zyx: tiles of the x axis, fused pass then plain pass
-    int nxbin = 0, nx = 0;
+    int *d_xtiles = nullptr;         // zyx: tiles of the x axis
+    int nx = 0;
 
     uint32_t *d_count = nullptr;     // objects per (tile, class) key, then the scatter's cursors (behind d_wmax)
     uint32_t *d_off = nullptr;       // exclusive scan of d_count (+ total)

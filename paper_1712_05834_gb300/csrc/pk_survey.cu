@@ -923,7 +923,7 @@ static pk_status survey_build(pk_survey_s *S, const pk_survey_config *cfg, void 
         SV_CUDA(S, cudaMemset(S->sync, 0, sizeof(unsigned) * S->nsync));
         const long long mhi = P->bg.mhi;
         while (S->ncol < S->Nh && (long long)S->ncol * S->ncol < mhi) ++S->ncol;
-        const int w = S->zyx->tile_columns(0);
+        const int w = S->zyx->tile_columns();
         std::vector<int> tiles;
         for (int all = 0; all < 2; ++all) {
             for (int j = 0; j < N; ++j) {

@@ -23,8 +23,7 @@ struct Refusing final : pk::ZyxOps {
     mutable int refuse = 1;
     cudaError_t no() const { refuse = 0; return cudaErrorInvalidConfiguration; }
     bool plan_default() const override { return real->plan_default(); }
-    int tile_columns(int il) const override { return real->tile_columns(il); }
-    int xbin_ctas_per_sm(const pk::BinGeom &g, int il) const override { return real->xbin_ctas_per_sm(g, il); }
+    int tile_columns() const override { return real->tile_columns(); }
     cudaError_t zy_survey(void *m, int nx, const pk::SurveyRows &sv, int nc, int mc, const void *tw, unsigned *s, int *e,
                           int nsm, cudaStream_t st) const override {
         return real->zy_survey(m, nx, sv, nc, mc, tw, s, e, nsm, st);
@@ -36,11 +35,6 @@ struct Refusing final : pk::ZyxOps {
     cudaError_t x(void *m, int n, long long mc, int nc, int mcut, const int *t, int nt, const void *tw, unsigned *s, int ns,
                   cudaStream_t st) const override {
         return refuse ? no() : real->x(m, n, mc, nc, mcut, t, nt, tw, s, ns, st);
-    }
-    cudaError_t xbin(const void *m, int il, long long is, long long ms, int ni, int cpi, const pk::BinGeom &g, int nc,
-                     const int *t, int nt, const void *cw, const void *ph, const void *tw, const int *ke, void *pa,
-                     unsigned *s, int ns, cudaStream_t st) const override {
-        return refuse ? no() : real->xbin(m, il, is, ms, ni, cpi, g, nc, t, nt, cw, ph, tw, ke, pa, s, ns, st);
     }
 };
 
@@ -86,7 +80,7 @@ int main(int argc, char **argv) {
 '''
 
 
-@pytest.mark.parametrize("N", [320, 1024])       # x, then bins; x fused with the bins
+@pytest.mark.parametrize("N", [320, 1024])
 def test_compute_after_a_refused_launch(N, tmp_path):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():

@@ -1,7 +1,6 @@
-"""A plan of 1024^3 that is asked for cross or projected power, which read the transform
-itself, writes it once from then on: its next compute takes x and the bins in two passes
-(4 launches for 3) and the cross power no longer takes the x axis again (2 launches
-for 3).  Spectra of both ways agree to the FP32 sums' order."""
+"""Cross and projected power of 1024^3 read the transform that the compute has written (x
+in place, then the bins: 4 launches) and take no axis again; spectra of repeated
+passes agree to the FP32 sums' order."""
 import numpy as np
 import pytest
 
@@ -31,8 +30,7 @@ def test_the_x_axis_is_taken_once(what):
             counts.append((b - a, pk.pk_launch_count(plan) - b))
     finally:
         pk.pk_destroy(plan)
-    assert counts[0][0] == 3 and counts[1][0] == counts[2][0] == 4, counts
-    assert counts[0][1] == counts[1][1] + 1 == counts[2][1] + 1, counts
+    assert counts[0] == counts[1] == counts[2] and counts[0][0] == 4, counts
     shot = L ** 3 / n
     for k in (1, 2):
         for x, y in zip(auto[0], auto[k]):
