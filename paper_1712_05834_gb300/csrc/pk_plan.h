@@ -33,7 +33,7 @@ struct pk_plan_s {
     int fft_single = 0;              // one single-mesh plan, one call per mesh (large meshes)
     void *fft_work = nullptr;
     // Own transform: packed (pk_fft.cu: y and x passes, then z fused into the bin)
-    // or zyx (pk_fft_zyx.cu: z and y in one pass, then x fused into the bin); FP64
+    // or zyx (pk_fft_zyx.cu: z and y in one pass, then x); FP64
     // meshes: pk_fft64.cu, then the bin pass.
     int own_fft = 0;                 // pk_compute uses it (supported N)
     int own_selectable = 0;          // pk_use_own_fft(plan, 1) accepts it
